@@ -163,11 +163,10 @@ typedef struct {
                              a push sent more than 0.5 % of a species (at least
                              1024 particles) down the escape path              */
   int64_t step;           /* completed time steps                                 */
-  int64_t n_push_mid_drain; /* species pushes that took the kernel variant which
-                             deposits its deferred shape-changing particles
-                             between chunks (chosen when the previous push of
-                             the species averaged more than 168 of them per
-                             work item, e.g. fast beams)                      */
+  int64_t n_push_mid_drain; /* species pushes made while the species' last count
+                             read back averaged more than 168 particles per
+                             work item changing their shape support (e.g. fast
+                             beams)                                            */
   int64_t n_adj_escaped;  /* particle adjoints since pic_adjoint_begin computed
                              on the global-memory path: the particle had moved
                              more than 2 cells out of the tile it was sorted

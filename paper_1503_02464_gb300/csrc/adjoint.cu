@@ -651,9 +651,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_adj_push2d(cons
 }
 
 // Work items of a recorded particle buffer (the sort in effect when it was
-// recorded): item i covers slots [work_pb[i], min(work_pb[i] + chunk,
-// tile_start[t + 1])) of tile t = work_tile[i] (-1: none); nsub blocks share
-// an item, kAdjSub slots each.
+// recorded): item i covers the work_item_slots slots from work_pb[i] (fewer
+// at the end of the run) of tile t = work_tile[i] (-1: none); nsub blocks
+// share an item, kAdjSub slots each.
 struct AdjWork {
   const int32_t *work_tile;
   const int64_t *work_pb;
@@ -681,7 +681,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
   if (t < 0) return;
   const int64_t te = w.tile_start[t + 1];
   const int64_t ib = w.work_pb[item];
-  const int64_t ie = ib + w.chunk < te ? ib + w.chunk : te;
+  const int64_t len = work_item_slots(te - w.tile_start[t], w.chunk);
+  const int64_t ie = ib + len < te ? ib + len : te;
   const int64_t pb = ib + (int64_t)(blockIdx.x % w.nsub) * kAdjSub;
   if (pb >= ie) return;
   const int64_t pe = pb + kAdjSub < ie ? pb + kAdjSub : ie;

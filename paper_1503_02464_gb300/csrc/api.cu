@@ -36,16 +36,14 @@ struct Species {
   int32_t *rank = nullptr;
   int64_t *tile_start = nullptr;
   pic::WorkSplit work;          // push work items (tile pieces of at most work.chunk slots)
-  float *tq = nullptr;          // per-item deposit bound carried between pushes
   // escapes of the last push, read back without blocking (adaptive sort)
-  unsigned long long *esc_host = nullptr;  // page-locked: [0] escapes, [1] deferred deposit jobs
+  unsigned long long *esc_host = nullptr;  // page-locked: [0] escapes, [1] particles whose support changed
   cudaEvent_t esc_ev = nullptr;
   bool esc_pending = false;
-  bool mid_drain = false;       // push variant draining its job queue between chunks
+  bool crowded = false;         // the last count read averaged more than kCrowdedJobs such particles per item
   bool fast = false;            // the last escape count read was above 1/8 of the early-sort threshold
   int count_age = 0;            // steps since an escape count was last read
   int64_t esc_step = -1;        // step of the push whose escape count is being read back
-  bool fresh = true;            // sorted since the last push
   bool need_sort = true;
   int64_t sorted_at = -1;  // step count at the last sort
   int64_t sorts = 0;       // sorts so far (names the slot order in effect)
@@ -125,7 +123,7 @@ struct pic_handle {
   int64_t step = 0;
   int64_t launches = 0;
   int64_t adaptive_sorts = 0;  // sorts triggered by escapes rather than by the cadence
-  int64_t mid_drain_pushes = 0;  // species pushes launched with the between-chunk drain variant
+  int64_t crowded_pushes = 0;  // pushes of crowded species (pic_diag's n_push_mid_drain)
   std::string err;
   bool profiling = false;
   std::vector<TimerRec> timers;
@@ -346,7 +344,6 @@ int sort_species(pic_handle *h, Species &s) {
   s.need_sort = false;
   s.sorted_at = h->step;
   s.sorts++;
-  s.fresh = true;
   return PIC_OK;
 }
 
@@ -676,7 +673,6 @@ int pic_destroy(pic_handle *h) {
     cudaFree(s.d_count);
     cudaFree(s.rank);
     cudaFree(s.work.work_pb);  // with tile_start and work_tile
-    cudaFree(s.tq);
     cudaFreeHost(s.esc_host);
     if (s.esc_ev) cudaEventDestroy(s.esc_ev);
   }
@@ -723,8 +719,8 @@ int pic_add_species(pic_handle *h, double q, double m, int64_t capacity, int *sp
   if (e == cudaSuccess) e = cudaMalloc(&s.rank, (size_t)(s.slots > 0 ? s.slots : 1) * sizeof(int32_t));
   // Work items: pieces of at most `chunk` slots per tile, chunk sized so that
   // a species spread over few tiles (a thin slab, a small grid) still gives
-  // about 16 blocks per SM, never below 512 slots and never above the
-  // fixed-point window's limit (kMaxWindowSlots).
+  // about 16 blocks per SM, never below 512 slots and never above what the
+  // push kernel holds in shared memory.
   {
     int dev = 0, nsm = 1;
     cudaGetDevice(&dev);
@@ -732,10 +728,10 @@ int pic_add_species(pic_handle *h, double q, double m, int64_t capacity, int *sp
     int64_t chunk = s.slots / (16 * (int64_t)(nsm > 0 ? nsm : 1));
     chunk = (chunk + 255) / 256 * 256;
     chunk = chunk < 512 ? 512 : chunk;
-    s.work.chunk = chunk > pic::kMaxWindowSlots ? pic::kMaxWindowSlots : chunk;
+    const int64_t cap = pic::push_item_cap(h->g);
+    s.work.chunk = chunk > cap ? cap : chunk;
     s.work.nwork = s.slots / s.work.chunk + 1 + h->g.ntiles;
   }
-  if (e == cudaSuccess) e = cudaMalloc(&s.tq, (size_t)2 * s.work.nwork * sizeof(float));
   if (e == cudaSuccess) e = cudaMallocHost(&s.esc_host, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.esc_ev, cudaEventDisableTiming);
   // the sort's outputs in one allocation (one copy for a tape entry):
@@ -751,7 +747,6 @@ int pic_add_species(pic_handle *h, double q, double m, int64_t capacity, int *sp
     cudaFree(s.d_count);
     cudaFree(s.rank);
     cudaFree(s.work.work_pb);  // with tile_start and work_tile
-    cudaFree(s.tq);
     cudaFreeHost(s.esc_host);
     if (s.esc_ev) cudaEventDestroy(s.esc_ev);
     s = Species{};
@@ -1244,9 +1239,7 @@ int pic_step(pic_handle *h, int nsteps) {
           // (a count from before the last sort says nothing about the order now)
           many_escapes = s.esc_step >= s.sorted_at && s.esc_host[0] > lim;
           s.fast = s.esc_host[0] > lim / 8;
-          // many particles changing shape support per step (fast beams): the
-          // push variant that drains its deferred-job queue between chunks
-          s.mid_drain = s.esc_host[1] > (unsigned long long)pic::kPushQueueMidDrain * (unsigned long long)s.work.nwork;
+          s.crowded = s.esc_host[1] > (unsigned long long)pic::kCrowdedJobs * (unsigned long long)s.work.nwork;
         } else {
           cudaGetLastError();  // not ready: not an error
           s.count_age++;
@@ -1278,12 +1271,11 @@ int pic_step(pic_handle *h, int nsteps) {
       Timed tm(h, pic::KC_PUSH);
       int nl = 0;
       CK(h,
-         pic::launch_push(h->g, h->E, h->B, h->J, s.buf[s.cur], s.tile_start, s.work, s.tq, s.fresh ? 1 : 0,
-                          s.rank, h->esc_count, s.q, s.m, h->ctr, h->st, &nl, s.mid_drain ? 1 : 0),
+         pic::launch_push(h->g, h->E, h->B, h->J, s.buf[s.cur], s.tile_start, s.work, s.rank, h->esc_count, s.q,
+                          s.m, h->ctr, h->st, &nl),
          "push");
-      s.fresh = false;
       h->launches += nl;
-      if (s.mid_drain) h->mid_drain_pushes++;
+      if (s.crowded) h->crowded_pushes++;
       if (s.esc_host && !s.esc_pending) {
         CK(h, cudaMemcpyAsync(s.esc_host, h->esc_count, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                               h->st),
@@ -1468,7 +1460,7 @@ int pic_diag(pic_handle *h, pic_diag_t *out) {
   out->n_clamped = (int64_t)c.clamped;
   out->n_absorbed = (int64_t)c.absorbed;
   out->n_sorts_adaptive = h->adaptive_sorts;
-  out->n_push_mid_drain = h->mid_drain_pushes;
+  out->n_push_mid_drain = h->crowded_pushes;
   out->n_adj_escaped = (int64_t)adj_esc;
   out->step = h->step;
   if (c.error & pic::kErrBounds) return fail(h, PIC_EOVERFLOW, "an index outside its buffer was caught (checked build)");

@@ -104,16 +104,26 @@ template <class R, int ORDER> struct DepositAxis {
   static constexpr int NW = ORDER + 2;
   int rel;
   R S0[NW], DS[NW];
+  // From the old and new offsets f, fn and the cell shift s.
   __device__ __forceinline__ void set(R f, int s, R fn) {
     if (ORDER == 2) {
       const int h0 = f >= R(0.5), h1 = fn >= R(0.5);
-      const int k = s + h1 - h0;  // nearest node moves by k (|k| <= 1 under the Courant limit)
-      const R d0 = f - R(h0);     // old position from N0, in [-1/2, 1/2)
-      const R e1 = fn - R(h1);    // new position from its own nearest node
+      set_nodes(f - R(h0), s + h1 - h0, fn - R(h1));
+      rel += h0;
+    } else {
+      set_nodes(f, s, fn);
+    }
+  }
+  // From the offsets d0, e1 of the old and new position from their own
+  // nearest nodes (TSC, in [-1/2, 1/2)) or in their cells (CIC), k apart
+  // (|k| <= 1 under the Courant limit); rel is then relative to the old
+  // nearest node or cell.
+  __device__ __forceinline__ void set_nodes(R d0, int k, R e1) {
+    if (ORDER == 2) {
       R w0[3];
       tsc3<R>(d0, w0);
       if (k == 0) {
-        rel = h0 - 1;
+        rel = -1;
         const R dl = e1 - d0, sg = d0 + e1, hd = R(0.5) * dl;
         S0[0] = w0[0];
         S0[1] = w0[1];
@@ -123,7 +133,7 @@ template <class R, int ORDER> struct DepositAxis {
         DS[2] = hd * (sg + R(1));
         S0[NW - 1] = DS[NW - 1] = R(0);
       } else if (k > 0) {
-        rel = h0 - 1;
+        rel = -1;
         const R g0 = R(0.5) - d0, g1 = e1 + R(0.5);
         S0[0] = w0[0];
         S0[1] = w0[1];
@@ -134,7 +144,7 @@ template <class R, int ORDER> struct DepositAxis {
         DS[2] = g1 * (R(1) - g1) + R(0.5) * g0 * (R(2) - g0);
         DS[3] = R(0.5) * g1 * g1;
       } else {
-        rel = h0 - 2;
+        rel = -2;
         const R g0 = R(0.5) + d0, g1 = R(0.5) - e1;
         S0[0] = R(0);
         S0[1] = w0[0];
@@ -146,30 +156,30 @@ template <class R, int ORDER> struct DepositAxis {
         DS[3] = R(-0.5) * g0 * g0;
       }
     } else {
-      if (s == 0) {
+      if (k == 0) {
         rel = 0;
-        const R dl = fn - f;
-        S0[0] = R(1) - f;
-        S0[1] = f;
+        const R dl = e1 - d0;
+        S0[0] = R(1) - d0;
+        S0[1] = d0;
         S0[2] = R(0);
         DS[0] = -dl;
         DS[1] = dl;
         DS[2] = R(0);
-      } else if (s > 0) {
+      } else if (k > 0) {
         rel = 0;
-        const R g0 = R(1) - f, g1 = fn;
+        const R g0 = R(1) - d0, g1 = e1;
         S0[0] = g0;
-        S0[1] = f;
+        S0[1] = d0;
         S0[2] = R(0);
         DS[0] = -g0;
         DS[1] = g0 - g1;
         DS[2] = g1;
       } else {
         rel = -1;
-        const R g0 = f, g1 = R(1) - fn;
+        const R g0 = d0, g1 = R(1) - e1;
         S0[0] = R(0);
-        S0[1] = R(1) - f;
-        S0[2] = f;
+        S0[1] = R(1) - d0;
+        S0[2] = d0;
         DS[0] = g1;
         DS[1] = g0 - g1;
         DS[2] = -g0;

@@ -126,10 +126,20 @@ enum KernelClass {
 // drift allowance is one cell.
 void push_tile_shape(int dims, int tile[3]);
 size_t push_smem_bytes(const Grid &g);
-// Work items of the push kernel: each tile's slot run is cut into pieces of
-// at most `chunk` slots; item i covers slots [work_pb[i], min(work_pb[i] +
-// chunk, tile_start[t + 1])) of tile t = work_tile[i] (-1: no work).  nwork
-// bounds the item count (slots / chunk + 1 + ntiles).
+// Most slots a work item of the push may hold (its chunk is at most this).
+int64_t push_item_cap(const Grid &g);
+// Work items of the push kernel: each tile's slot run is cut into the fewest
+// pieces of at most `chunk` slots (a multiple of 4), all of them
+// work_item_slots(run, chunk) long but the last; item i starts at slot
+// work_pb[i] of tile work_tile[i] (-1: no work).  nwork bounds the item count
+// (slots / chunk + 1 + ntiles).
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int64_t work_item_slots(int64_t run, int64_t chunk) {
+  const int64_t pieces = (run + chunk - 1) / chunk;
+  return pieces > 1 ? ((run + pieces - 1) / pieces + 3) / 4 * 4 : run;
+}
 struct WorkSplit {
   int64_t chunk = 0;
   int64_t nwork = 0;
@@ -137,23 +147,15 @@ struct WorkSplit {
   int64_t *work_pb = nullptr;
 };
 
-// Tile kernel (one block per work item) + escape kernel.  tq (2 floats per
-// work item) carries the bound of the FP32 fixed-point deposit from one step
-// to the next; fresh = 1 on the first push after a sort (tq is recomputed
-// from the particles).
+// Tile kernel (one block per work item) + escape kernel.
 // esc_list (one int per slot) is scratch for particles deferred to the
 // escape kernel; esc_count (two counters) receives their number and the
-// number of deferred deposit jobs (particles whose shape support changed)
-// of the launch.  mid_drain selects the kernel variant that deposits those
-// jobs between chunks when its queue fills (3D): the caller turns it on for
-// a species whose last push averaged more than kPushQueueMidDrain jobs per
-// work item.
-constexpr int kPushQueueCap = 224;      // deferred deposit jobs a work item queues at a time
-constexpr int kPushQueueMidDrain = 168;  // 3/4 of the queue
+// number of particles whose shape support changed in the launch.
+constexpr int kCrowdedJobs = 168;  // such particles per work item above which a species counts as crowded (pic_diag)
 cudaError_t launch_push(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
-                        const int64_t *tile_start, const WorkSplit &ws, float *tq, int fresh, int32_t *esc_list,
+                        const int64_t *tile_start, const WorkSplit &ws, int32_t *esc_list,
                         unsigned long long *esc_count, double q, double m, Counters *ctr, cudaStream_t st,
-                        int *nlaunch, int mid_drain);
+                        int *nlaunch);
 
 // Diagnostics charge density of particles sorted by tile (exact 64-bit
 // fixed-point window sums; adds into rho).

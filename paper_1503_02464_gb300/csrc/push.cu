@@ -6,19 +6,10 @@
 // Cell tiles are 8x8x4 in 3D, 16x16 in 2D.  The sort keeps each tile's
 // particles in one contiguous, 4-aligned slot range and cuts that range into
 // work items of bounded size; one thread block takes one work item.  The
-// block stages E and B of the tile plus guard cells in shared memory and
-// accumulates J of the tile plus guard with shared-memory atomics (fixed
-// point in FP32 runs), then adds its J window to the global J (one atomic per
-// non-zero value).
-//
-// Particles stream through a 256-slot shared staging chunk, loaded with
-// coalesced accesses in slot order.  The deposit runs in a permuted order that
-// gives the 32 lanes of a warp particles eight slots apart: slots are
-// cell-sorted, so lanes then sit in different cells and their shared atomics
-// hit different addresses and banks.  FP32 3D runs gather and push in slot
-// order first (lanes of a warp in a few cells read the same field nodes),
-// write the new state to global memory and leave a deposit job for the
-// permuted phase after a block barrier (see k_push).
+// block stages E and B of the tile plus guard cells in shared memory, pushes
+// all its particles, and then deposits them by groups that share a nearest
+// node (see k_push) into a J window in shared memory (fixed point in FP32
+// runs), which it adds to the global J.
 //
 // A particle that has drifted more than D = 1 cell outside its tile since the
 // last sort is not handled here: its slot is appended to an escape list and
@@ -41,31 +32,56 @@ __device__ __forceinline__ int wrap_near(int i, int n) {
 }
 constexpr int32_t kEscFlag = 0x40000000;  // set in `cell` while a particle waits for the escape kernel
 
-// Compile-time tile and window geometry.
+// Compile-time tile and window geometry.  E, B and J share one window: the
+// nodes -O .. (last) around the tile that the gather of a particle up to D
+// cells outside it reaches, and that its deposit reaches when its nearest
+// node stays within D cells of the tile over the move (a particle that moves
+// further takes the escape path).
 template <int DIM, int ORDER> struct Geo {
   static constexpr int TX = DIM == 3 ? 8 : 16;
   static constexpr int TY = DIM == 3 ? 8 : 16;
   static constexpr int TZ = DIM == 3 ? 4 : 1;
   static constexpr int D = 1;  // drift allowance (cells)
   static constexpr int LOE = 1, HIE = ORDER == 2 ? 2 : 1;  // gather reach below / above the cell
-  static constexpr int LOJ = ORDER == 2 ? 2 : 1, HIJ = ORDER == 2 ? 3 : 2;  // deposit reach
+  static constexpr int O = D + LOE;                        // window index of the tile's first node
   static constexpr int EX = TX + 2 * D + LOE + HIE;
   static constexpr int EY = TY + 2 * D + LOE + HIE;
   static constexpr int EZ = DIM == 3 ? TZ + 2 * D + LOE + HIE : 1;
-  static constexpr int JX = TX + 2 * D + LOJ + HIJ;
-  static constexpr int JY = TY + 2 * D + LOJ + HIJ;
-  static constexpr int JZ = DIM == 3 ? TZ + 2 * D + LOJ + HIJ : 1;
   static constexpr int EN = EX * EY * EZ;
-  // J window plane stride.  For 3D TSC it is padded from 15 x 15 = 225 to 231
-  // nodes: the deposit's atomics come from 32 lanes in 32 neighbouring cells,
-  // each offset by its particle's stencil start, and with 231 those addresses
-  // fall on fewer shared banks twice (a count over thermal-plasma tiles: 2.6
-  // -> 2.2 wavefronts per atomic instruction).  The padding nodes stay zero.
-  static constexpr int JP = (DIM == 3 && ORDER == 2) ? JX * JY + 6 : JX * JY;
-  static constexpr int JN = JP * JZ;
-  static constexpr int JS = JN + (ORDER == 2 ? 32 : 0);  // word-array stride of the shared J window (TSC: + 32 scratch words)
-  static constexpr int NS = ORDER + 1;  // gather stencil width
-  static constexpr int NW = ORDER + 2;  // deposit stencil width
+  static constexpr int JS = EN + 32;    // word-array stride of the fixed-point J window (32 scratch words)
+  static constexpr int NS = ORDER + 1;  // gather stencil width, and that of a settled deposit
+  static constexpr int NW = ORDER + 2;  // general deposit stencil width
+  // Groups: the nearest node (TSC) or the cell (CIC) of a particle's old
+  // position, -D .. T - 1 + D (+ 1 for nodes) on every axis.
+  static constexpr int KX = TX + 2 * D + (ORDER == 2 ? 1 : 0);
+  static constexpr int KY = TY + 2 * D + (ORDER == 2 ? 1 : 0);
+  static constexpr int KZ = DIM == 3 ? TZ + 2 * D + (ORDER == 2 ? 1 : 0) : 1;
+  static constexpr int KN = KX * KY * KZ;
+  static constexpr int KT = KN + 7;  // and the particles whose support changes, by the axes that do (mask 1..7)
+};
+
+// Shared memory of k_push, and the most slots a work item may hold (CAP): a
+// block keeps the deposit jobs of its whole item, so that the particles of
+// one node meet whatever their slots.  FP32 3D items hold a full 8x8x4 tile
+// of the 8-per-cell plasma with room to spare at two blocks per SM.
+constexpr int kTaskLen = 8;  // particles one thread sums at a time
+template <class R, int DIM, int ORDER> struct Lay {
+  using G = Geo<DIM, ORDER>;
+  static constexpr bool F32 = sizeof(R) == 4;
+  static constexpr int CAP = F32 ? (DIM == 3 ? 2176 : 2048) : (DIM == 3 ? 2432 : 1664);
+  static constexpr int BLOCKS = F32 ? (DIM == 3 ? 2 : 3) : (DIM == 3 ? 1 : 2);  // per SM
+  static constexpr int NJ = DIM == 3 ? 7 : 6;  // job: old and new offsets per axis, weight (2D3V: and vz)
+  static constexpr int MAXT = CAP / kTaskLen + G::KN;
+  static constexpr size_t align16(size_t b) { return (b + 15) / 16 * 16; }
+  // E and B, then (once every particle is pushed) the J window
+  static constexpr size_t kWin = align16(6 * G::EN * sizeof(R) > 24 * G::JS ? 6 * G::EN * sizeof(R) : 24 * G::JS);
+  static constexpr size_t kJob = kWin;                                  // [NJ][CAP] R
+  static constexpr size_t kTag = kJob + align16(NJ * CAP * sizeof(R));  // [CAP] u32
+  static constexpr size_t kOrder = kTag + 4 * CAP;                      // [CAP] u16
+  static constexpr size_t kCount = align16(kOrder + 2 * CAP);           // [KT] u32, then [KT + 1] u16 and the tasks
+  static constexpr size_t kTask = kCount + 2 * (G::KT + 1);             // [MAXT] u16
+  static constexpr size_t kEnd = kTask + 2 * MAXT > kCount + 4 * G::KT ? kTask + 2 * MAXT : kCount + 4 * G::KT;
+  static_assert(G::KT < 1024 && CAP < 4096 && CAP % 32 == 0, "tag packing");
 };
 
 // Division by a runtime constant (Granlund-Montgomery): q = (umulhi(n,m) + n) >> l.
@@ -97,15 +113,13 @@ template <class R> struct PushArgs {
   R *u[3];
   const R *w;
   const int64_t *tile_start;
-  double qabs;                      // |q|
+  float qabs;                       // |q|
   const int32_t *work_tile;         // work item -> tile (-1: none)
   const int64_t *work_pb;           // work item -> first slot
-  int64_t chunk;                    // slots per work item at most
-  float *tq;                        // per item: [2i] sum |w|, [2i+1] sum |w| min(1, |u|) (FP32 runs)
-  int fresh;                        // tile contents changed (sorted) since tq was written
+  int64_t chunk;                    // slots per work item at most (work_item_slots)
   int32_t *esc_list;                // slots deferred to k_push_escaped
   unsigned long long *esc_count;
-  unsigned long long *q_jobs;       // deferred deposit jobs of this launch (counted at each drain)
+  unsigned long long *q_jobs;       // particles of this launch whose shape support changes
   R qmh;      // q dt / (2 m)
   R dtdx[3];  // dt / dx_a
   R jfac[3];  // -q dx_a / dt  (Esirkepov running-sum scale, times w)
@@ -152,24 +166,23 @@ __device__ __forceinline__ R gsum(const R *__restrict__ F, const R *wx, const R 
 // atomics are compare-and-swap loops costing several shared-memory
 // wavefronts each, integer shared atomics are single native operations, and
 // integer sums are exact and independent of order.  A contribution v becomes
-// the integer X = rint(v * 2^K), K chosen per tile from a bound on |J| at any
-// node: each Esirkepov contribution of a particle satisfies |v| <= |q w| |v_p|
-// and Boris raises |u| by at most |q/m| dt |E|, so
-//   |J_node| <= Q = sum over the tile's particles of |q w| min(1, |u| + |q/m| dt Emax)
-// with Emax bounding |E| over the tile's field window; 2^K keeps Q 2^K below
+// the integer X = rint(v * 2^K), K chosen per work item from a bound on |J|
+// at any node: each Esirkepov contribution of a particle satisfies
+// |v| <= |q w| |v_p|, so |J_node| <= Q = sum over the item's particles of
+// |q w| min(1, |u|) with u the momentum after the push; 2^K keeps Q 2^K below
 // 2^kLimitLog2.  X is kept as two signed 32-bit words, X = hi * 2^16 + lo
 // with |lo| <= 2^15, both found with FP32 FMAs and adds only (adding
 // 1.5 * 2^(23 + s) rounds a float of magnitude below 2^(22 + s) to a multiple
 // of 2^s held in the low mantissa bits), because float-to-64-bit conversions
-// run on the slow FP64 pipe.  With
-// |X| < 2^37 the hi sums cannot overflow, and the lo sums cannot overflow for
-// fewer than 65,536 contributions per node.  FP64 runs use plain double
-// shared atomics, keeping FP64 rounding.
+// run on the slow FP64 pipe.  With |X| < 2^37 the hi sums cannot overflow, and
+// the lo sums cannot overflow for fewer than 65,536 contributions per node (an
+// item holds at most Lay::CAP particles).  FP64 runs use plain double shared
+// atomics, keeping FP64 rounding.
 template <class R> struct WinAcc;
 template <> struct WinAcc<float> {
   int *w;       // [3][2][jn]: per component lo words, then hi words
-  int jn;       // word stride: the window's nodes (then, for TSC, 32 scratch words)
-  int dummy;    // TSC: this lane's scratch word (past the nodes, bank = lane)
+  int jn;       // word stride: the window's nodes, then 32 scratch words
+  int dummy;    // this lane's scratch word (past the nodes)
   float scale;  // 2^K
   float unit;   // 2^-K
   static constexpr int kLimitLog2 = 37;
@@ -182,7 +195,6 @@ template <> struct WinAcc<float> {
   // the second FMA gives X - hi 2^16 with one rounding, |.| <= 2^15, and a
   // round-to-nearest conversion gives the integer lo (one instruction where
   // adding and removing the 1.5 * 2^23 magic took two).
-  template <bool kScratch>
   __device__ __forceinline__ void add(int comp, int idx, float p, float q) const {
     const float y = fmaf(p, q, kMagicHi);
     const float r = y - kMagicHi;  // hi 2^16, exact
@@ -190,16 +202,23 @@ template <> struct WinAcc<float> {
     const int hi = __float_as_int(y) - __float_as_int(kMagicHi);
     const int lo = __float2int_rn(lf);  // round to nearest even, as the 2^23 magic would
     // Both words are added unconditionally: a branch around the pair (or a
-    // predicate on it) cost more than the adds.  With kScratch (TSC) a zero
-    // contribution goes to the lane's own scratch word instead of the node,
-    // so that it does not collide with the other lanes' nodes in their
-    // banks (for CIC's smaller stencils the select costs more than it
-    // saves).  Warps whose particles all deposit nothing skip the whole
-    // stencil instead (deposit_particle).
-    const int at = (!kScratch || (hi | lo)) ? idx : dummy;
+    // predicate on it) cost more than the adds.  A zero contribution goes to
+    // the lane's own scratch word instead of the node, so that it does not
+    // collide with the other lanes' nodes in their banks (and an outer node
+    // past the window's end, whose contributions are all zero, is not
+    // touched).
+    const int at = (hi | lo) ? idx : dummy;
     const unsigned s = (unsigned)__cvta_generic_to_shared(w + comp * 2 * jn + at);
     asm volatile("red.shared.add.s32 [%0], %1;\n\tred.shared.add.s32 [%2], %3;" ::"r"(s), "r"(lo),
                  "r"(s + 4u * (unsigned)jn), "r"(hi));
+  }
+  // The largest power of two (within 2^+-100) that keeps Q 2^K below 2^kLimitLog2.
+  __device__ __forceinline__ void set_scale(float Q) {
+    const int e2 = (int)(__float_as_uint(Q) >> 23) - 126;  // Q < 2^e2
+    int K = Q > 0.f ? kLimitLog2 - e2 : 100;
+    K = K > 100 ? 100 : (K < -100 ? -100 : K);
+    scale = __int_as_float((127 + K) << 23);
+    unit = __int_as_float((127 - K) << 23);
   }
   __device__ __forceinline__ float get(int comp, int idx) const {
     const int *b = w + comp * 2 * jn + idx;
@@ -212,7 +231,6 @@ template <> struct WinAcc<double> {
   int dummy;  // (unused)
   double scale;  // 1: contributions are passed unscaled
   double unit;
-  template <bool kScratch>
   __device__ __forceinline__ void add(int comp, int idx, double p, double q) const {
     const double x = p * q;
     if (x != 0.0) atomicAdd(w + comp * jn + idx, x);
@@ -269,7 +287,7 @@ __device__ __forceinline__ void deposit_win(const WinAcc<R> &acc, int base, cons
 #pragma unroll
         for (int a = 0; a < M; ++a) {
           if (a == M - 1 && !lx) continue;
-          acc.template add<ORDER == 2>(0, base + c * SZ + b * SY + a, Px[a], br);
+          acc.add(0, base + c * SZ + b * SY + a, Px[a], br);
         }
       }
     }
@@ -283,7 +301,7 @@ __device__ __forceinline__ void deposit_win(const WinAcc<R> &acc, int base, cons
 #pragma unroll
         for (int b = 0; b < M; ++b) {
           if (b == M - 1 && !ly) continue;
-          acc.template add<ORDER == 2>(1, base + c * SZ + b * SY + a, Py[b], br);
+          acc.add(1, base + c * SZ + b * SY + a, Py[b], br);
         }
       }
     }
@@ -299,7 +317,7 @@ __device__ __forceinline__ void deposit_win(const WinAcc<R> &acc, int base, cons
 #pragma unroll
         for (int c = 0; c < M; ++c) {
           if (c == M - 1 && !lz) continue;
-          acc.template add<ORDER == 2>(2, base + c * SZ + b * SY + a, Pz[c], br);
+          acc.add(2, base + c * SZ + b * SY + a, Pz[c], br);
         }
       }
     }
@@ -314,12 +332,12 @@ __device__ __forceinline__ void deposit_win(const WinAcc<R> &acc, int base, cons
 #pragma unroll
       for (int a = 0; a < M; ++a) {
         if (a == M - 1 && !lx) continue;
-        acc.template add<ORDER == 2>(0, base + b * SY + a, Px[a], hy);
+        acc.add(0, base + b * SY + a, Px[a], hy);
       }
 #pragma unroll
       for (int a = 0; a < NW; ++a) {
         if (a == NW - 1 && !lx) continue;
-        acc.template add<ORDER == 2>(2, base + b * SY + a, qwvz, X.S0[a] * hy + X.DS[a] * ty);
+        acc.add(2, base + b * SY + a, qwvz, X.S0[a] * hy + X.DS[a] * ty);
       }
     }
 #pragma unroll
@@ -329,24 +347,9 @@ __device__ __forceinline__ void deposit_win(const WinAcc<R> &acc, int base, cons
 #pragma unroll
       for (int b = 0; b < M; ++b) {
         if (b == M - 1 && !ly) continue;
-        acc.template add<ORDER == 2>(1, base + b * SY + a, Py[b], hx);
+        acc.add(1, base + b * SY + a, Py[b], hx);
       }
     }
-  }
-}
-
-// A deposit job: the particle's cell relative to the tile (l in [-1, 16] on
-// every axis) and its cell shift (s in {-1, 0, 1}), 5 + 2 bits per axis, and
-// bit 30 set so that a job is never 0.
-__device__ __forceinline__ int pack_job(const int l[3], const int s[3]) {
-  return (1 << 30) | (l[0] + 1) | ((l[1] + 1) << 5) | ((l[2] + 1) << 10) | ((s[0] + 1) << 15) |
-         ((s[1] + 1) << 17) | ((s[2] + 1) << 19);
-}
-__device__ __forceinline__ void unpack_job(int j, int l[3], int s[3]) {
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    l[d] = ((j >> (5 * d)) & 31) - 1;
-    s[d] = ((j >> (15 + 2 * d)) & 3) - 1;
   }
 }
 
@@ -364,17 +367,11 @@ __device__ __forceinline__ void unpack_job(int j, int l[3], int s[3]) {
 // continuity equation with rho = sum q w S (to FP32 round-off of S).
 template <class R, int ORDER> struct SettledAxis {
   static constexpr int NS = ORDER + 1;
-  int rel;    // first support node relative to the old cell
   R S0[NS], DS[NS];
-  R dl;       // displacement in cells
-  // false when the support changes (then nothing is set)
-  __device__ __forceinline__ bool set(R f0, int s, R f1) {
+  // offsets of the two positions from their nearest node (TSC) or in the cell (CIC)
+  __device__ __forceinline__ void set(R d0, R d1) {
+    const R dl = d1 - d0;
     if (ORDER == 2) {
-      const int h0 = f0 >= R(0.5), h1 = f1 >= R(0.5);
-      if (s + h1 != h0) return false;
-      rel = h0 - 1;
-      const R d0 = f0 - R(h0), d1 = f1 - R(h1);  // both from the same node
-      dl = d1 - d0;
       const R sg = d0 + d1;
       tsc3<R>(d0, S0);
       const R hd = R(0.5) * dl;
@@ -382,227 +379,182 @@ template <class R, int ORDER> struct SettledAxis {
       DS[1] = -dl * sg;
       DS[2] = hd * (sg + R(1));
     } else {
-      if (s != 0) return false;
-      rel = 0;
-      S0[0] = R(1) - f0;
-      S0[1] = f0;
-      dl = f1 - f0;
+      S0[0] = R(1) - d0;
+      S0[1] = d0;
       DS[0] = -dl;
       DS[NS - 1] = dl;
     }
-    return true;
-  }
-  __device__ __forceinline__ void zero() {
-    rel = 0;
-    dl = R(0);
-#pragma unroll
-    for (int k = 0; k < NS; ++k) S0[k] = DS[k] = R(0);
-    S0[0] = R(1);
   }
 };
 
-// Add the contribution p q (window units) at the shared byte address sa of
-// its low word; the high word lies JS words further.  Same split as
-// WinAcc<float>::add, without the scratch-word select, so that the address
-// is one base register plus a compile-time offset for the whole stencil.
-template <int JS> __device__ __forceinline__ void fx_add(unsigned sa, float p, float q) {
-  const float y = fmaf(p, q, WinAcc<float>::kMagicHi);
-  const float r = y - WinAcc<float>::kMagicHi;
-  const float lf = fmaf(p, q, -r);
-  const int hi = __float_as_int(y) - __float_as_int(WinAcc<float>::kMagicHi);
-  const int lo = __float2int_rn(lf);
-  asm volatile("red.shared.add.s32 [%0], %1;\n\tred.shared.add.s32 [%2], %3;" ::"r"(sa), "r"(lo),
-               "r"(sa + 4u * (unsigned)JS), "r"(hi));
-}
-
-// One contribution p q to component comp at node offset off (compile-time)
-// from the stencil's first node.  FP32: fixed point at the byte address
-// base + ...; FP64: a double shared atomic at the node (zero skipped), as in
-// WinAcc<double>.
-template <class R, int JS> struct SettledSink;
-template <int JS> struct SettledSink<float, JS> {
-  unsigned sb;  // byte address of the Jx low word of the stencil's first node
-  __device__ __forceinline__ void add(int comp, int off, float p, float q) const {
-    fx_add<JS>(sb + 8u * (unsigned)JS * (unsigned)comp + 4u * (unsigned)off, p, q);
-  }
-};
-template <int JS> struct SettledSink<double, JS> {
-  double *w;  // Jx value of the stencil's first node (components JS doubles apart)
-  __device__ __forceinline__ void add(int comp, int off, double p, double q) const {
-    const double x = p * q;
-    if (x != 0.0) atomicAdd(w + comp * JS + off, x);
-  }
-};
-
-// Esirkepov deposit of a settled particle on its ORDER + 1 support nodes per
-// axis (compile-time strides SY, SZ in nodes).  Same brackets as deposit_win:
-// Jx gets Px (S0y S0z + DSy S0z/2 + S0y DSz/2 + DSy DSz/3), cyclic; in 2D3V
+// The settled contributions of the particles of one node, summed in
+// registers: add() one particle, flush() the sums into the J window once per
+// group.  Same brackets as deposit_win: Jx gets
+// Px (S0y S0z + DSy S0z/2 + S0y DSz/2 + DSy DSz/3), cyclic; in 2D3V
 // Jz = q w vz (S0x S0y + DSx S0y/2 + S0x DSy/2 + DSx DSy/3).  The running
 // sums of DS along an axis end at -DS[last] (the whole sum vanishes).
-template <class R, int ORDER, int DIM, int SY, int SZ, int JS>
-__device__ __forceinline__ void deposit_settled_win(const SettledSink<R, JS> &out, const SettledAxis<R, ORDER> &X,
-                                                    const SettledAxis<R, ORDER> &Y, const SettledAxis<R, ORDER> &Z,
-                                                    R cx, R cy, R cz, R qwvz) {
-  constexpr int NS = ORDER + 1, M = ORDER;
-  R Px[M], Py[M], Pz[M];
-  {
-    R ra = R(0), rb = R(0), rc = R(0);
+template <class R, int DIM, int ORDER> struct GroupSum {
+  static constexpr int NS = ORDER + 1, M = ORDER;
+  static constexpr int NA = DIM == 3 ? M * NS * NS : M * NS;  // Jx, Jy sums
+  static constexpr int NZ = DIM == 3 ? M * NS * NS : NS * NS;  // Jz sums
+  R jx[NA], jy[NA], jz[NZ];
+  __device__ __forceinline__ void clear() {
 #pragma unroll
-    for (int k = 0; k < M - 1; ++k) {
-      ra += X.DS[k];
-      rb += Y.DS[k];
-      rc += Z.DS[k];
-      Px[k] = cx * ra;
-      Py[k] = cy * rb;
-      Pz[k] = cz * rc;
-    }
-    Px[M - 1] = -cx * X.DS[NS - 1];
-    Py[M - 1] = -cy * Y.DS[NS - 1];
-    Pz[M - 1] = -cz * Z.DS[NS - 1];
+    for (int i = 0; i < NA; ++i) jx[i] = jy[i] = R(0);
+#pragma unroll
+    for (int i = 0; i < NZ; ++i) jz[i] = R(0);
   }
-  if (DIM == 3) {
-    R hz[NS], tz[NS], hx[NS], tx[NS];
+  __device__ __forceinline__ void add(const SettledAxis<R, ORDER> &X, const SettledAxis<R, ORDER> &Y,
+                                      const SettledAxis<R, ORDER> &Z, R cx, R cy, R cz, R qwvz) {
+    R Px[M], Py[M], Pz[M];
+    {
+      R ra = R(0), rb = R(0), rc = R(0);
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      hz[k] = Z.S0[k] + R(0.5) * Z.DS[k];
-      tz[k] = R(0.5) * Z.S0[k] + Z.DS[k] * R(1.0 / 3.0);
-      hx[k] = X.S0[k] + R(0.5) * X.DS[k];
-      tx[k] = R(0.5) * X.S0[k] + X.DS[k] * R(1.0 / 3.0);
+      for (int k = 0; k < M - 1; ++k) {
+        ra += X.DS[k];
+        rb += Y.DS[k];
+        Px[k] = cx * ra;
+        Py[k] = cy * rb;
+        if (DIM == 3) {
+          rc += Z.DS[k];
+          Pz[k] = cz * rc;
+        }
+      }
+      Px[M - 1] = -cx * X.DS[NS - 1];
+      Py[M - 1] = -cy * Y.DS[NS - 1];
+      if (DIM == 3) Pz[M - 1] = -cz * Z.DS[NS - 1];
     }
+    if constexpr (DIM == 3) {
+      R hz[NS], tz[NS], hx[NS], tx[NS];
 #pragma unroll
-    for (int c = 0; c < NS; ++c)
+      for (int k = 0; k < NS; ++k) {
+        hz[k] = Z.S0[k] + R(0.5) * Z.DS[k];
+        tz[k] = R(0.5) * Z.S0[k] + Z.DS[k] * R(1.0 / 3.0);
+        hx[k] = X.S0[k] + R(0.5) * X.DS[k];
+        tx[k] = R(0.5) * X.S0[k] + X.DS[k] * R(1.0 / 3.0);
+      }
+#pragma unroll
+      for (int c = 0; c < NS; ++c)
+#pragma unroll
+        for (int b = 0; b < NS; ++b) {
+          const R br = Y.S0[b] * hz[c] + Y.DS[b] * tz[c];
+#pragma unroll
+          for (int a = 0; a < M; ++a) jx[(c * NS + b) * M + a] += Px[a] * br;
+        }
+#pragma unroll
+      for (int c = 0; c < NS; ++c)
+#pragma unroll
+        for (int a = 0; a < NS; ++a) {
+          const R br = Z.S0[c] * hx[a] + Z.DS[c] * tx[a];
+#pragma unroll
+          for (int b = 0; b < M; ++b) jy[(c * NS + a) * M + b] += Py[b] * br;
+        }
 #pragma unroll
       for (int b = 0; b < NS; ++b) {
-        const R br = Y.S0[b] * hz[c] + Y.DS[b] * tz[c];
+        const R hy = Y.S0[b] + R(0.5) * Y.DS[b];
+        const R ty = R(0.5) * Y.S0[b] + Y.DS[b] * R(1.0 / 3.0);
 #pragma unroll
-        for (int a = 0; a < M; ++a) out.add(0, c * SZ + b * SY + a, Px[a], br);
+        for (int a = 0; a < NS; ++a) {
+          const R br = X.S0[a] * hy + X.DS[a] * ty;
+#pragma unroll
+          for (int c = 0; c < M; ++c) jz[(b * NS + a) * M + c] += Pz[c] * br;
+        }
       }
+    } else {
 #pragma unroll
-    for (int c = 0; c < NS; ++c)
+      for (int b = 0; b < NS; ++b) {
+        const R hy = Y.S0[b] + R(0.5) * Y.DS[b];
+        const R ty = R(0.5) * Y.S0[b] + Y.DS[b] * R(1.0 / 3.0);
+#pragma unroll
+        for (int a = 0; a < M; ++a) jx[b * M + a] += Px[a] * hy;
+#pragma unroll
+        for (int a = 0; a < NS; ++a) jz[b * NS + a] += qwvz * (X.S0[a] * hy + X.DS[a] * ty);
+      }
 #pragma unroll
       for (int a = 0; a < NS; ++a) {
-        const R br = Z.S0[c] * hx[a] + Z.DS[c] * tx[a];
+        const R hx = X.S0[a] + R(0.5) * X.DS[a];
 #pragma unroll
-        for (int b = 0; b < M; ++b) out.add(1, c * SZ + b * SY + a, Py[b], br);
-      }
-#pragma unroll
-    for (int b = 0; b < NS; ++b) {
-      const R hy = Y.S0[b] + R(0.5) * Y.DS[b];
-      const R ty = R(0.5) * Y.S0[b] + Y.DS[b] * R(1.0 / 3.0);
-#pragma unroll
-      for (int a = 0; a < NS; ++a) {
-        const R br = X.S0[a] * hy + X.DS[a] * ty;
-#pragma unroll
-        for (int c = 0; c < M; ++c) out.add(2, c * SZ + b * SY + a, Pz[c], br);
+        for (int b = 0; b < M; ++b) jy[a * M + b] += Py[b] * hx;
       }
     }
-  } else {
+  }
+  // SY, SZ: the window's row and plane strides; the sink adds at a
+  // compile-time node offset from the stencil's first node
+  template <int SY, int SZ, class Sink> __device__ __forceinline__ void flush(const Sink &out) const {
+    if constexpr (DIM == 3) {
 #pragma unroll
-    for (int b = 0; b < NS; ++b) {
-      const R hy = Y.S0[b] + R(0.5) * Y.DS[b];
-      const R ty = R(0.5) * Y.S0[b] + Y.DS[b] * R(1.0 / 3.0);
+      for (int c = 0; c < NS; ++c)
 #pragma unroll
-      for (int a = 0; a < M; ++a) out.add(0, b * SY + a, Px[a], hy);
+        for (int b = 0; b < NS; ++b)
 #pragma unroll
-      for (int a = 0; a < NS; ++a) out.add(2, b * SY + a, qwvz, X.S0[a] * hy + X.DS[a] * ty);
-    }
+          for (int a = 0; a < M; ++a) out.add(0, c * SZ + b * SY + a, jx[(c * NS + b) * M + a]);
 #pragma unroll
-    for (int a = 0; a < NS; ++a) {
-      const R hx = X.S0[a] + R(0.5) * X.DS[a];
+      for (int c = 0; c < NS; ++c)
 #pragma unroll
-      for (int b = 0; b < M; ++b) out.add(1, b * SY + a, Py[b], hx);
+        for (int a = 0; a < NS; ++a)
+#pragma unroll
+          for (int b = 0; b < M; ++b) out.add(1, c * SZ + b * SY + a, jy[(c * NS + a) * M + b]);
+#pragma unroll
+      for (int b = 0; b < NS; ++b)
+#pragma unroll
+        for (int a = 0; a < NS; ++a)
+#pragma unroll
+          for (int c = 0; c < M; ++c) out.add(2, c * SZ + b * SY + a, jz[(b * NS + a) * M + c]);
+    } else {
+#pragma unroll
+      for (int b = 0; b < NS; ++b) {
+#pragma unroll
+        for (int a = 0; a < M; ++a) out.add(0, b * SY + a, jx[b * M + a]);
+#pragma unroll
+        for (int a = 0; a < NS; ++a) out.add(2, b * SY + a, jz[b * NS + a]);
+      }
+#pragma unroll
+      for (int a = 0; a < NS; ++a)
+#pragma unroll
+        for (int b = 0; b < M; ++b) out.add(1, b * SY + a, jy[a * M + b]);
     }
   }
-}
-
-// Deposit of a particle whose support did not change.  Returns false,
-// depositing nothing, when the support changes on some axis: such a particle
-// takes the general ORDER + 2 node stencil (deposit_particle), through the
-// block's queue of deferred jobs.
-template <class R, int DIM, int ORDER>
-__device__ __forceinline__ bool deposit_settled(const PushArgs<R> &a, const WinAcc<R> &acc, const int l[3],
-                                                const int s[3], const R f[3], const R fn[3], R w, R vz) {
-  using G = Geo<DIM, ORDER>;
-  SettledAxis<R, ORDER> X, Y, Z;
-  bool ok = X.set(f[0], s[0], fn[0]);
-  ok = Y.set(f[1], s[1], fn[1]) && ok;
-  if (DIM == 3) ok = Z.set(f[2], s[2], fn[2]) && ok;
-  else Z.zero();
-  if (!ok) return false;
-  // a warp whose settled particles neither move nor (2D3V) carry vz deposits nothing
-  const bool moves = w != R(0) && (X.dl != R(0) || Y.dl != R(0) || (DIM == 3 ? Z.dl != R(0) : vz != R(0)));
-  if (!__any_sync(__activemask(), moves)) return true;
-  constexpr int oJ = G::D + G::LOJ;
-#ifdef PIC_CHECKED
-  {
-    const int rel[3] = {X.rel, Y.rel, Z.rel};
-    constexpr int JW[3] = {G::JX, G::JY, G::JZ};
-    bool in = true;
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) in = in && l[d] + rel[d] + oJ >= 0 && l[d] + rel[d] + oJ + ORDER < JW[d];
-    if (!PIC_CHECK(in, a.ctr)) return true;
-  }
-#endif
-  const int jb = (l[0] + X.rel + oJ) + (l[1] + Y.rel + oJ) * G::JX + (DIM == 3 ? (l[2] + Z.rel + oJ) * G::JP : 0);
-  SettledSink<R, G::JS> out;
-  if constexpr (sizeof(R) == 4) out.sb = (unsigned)__cvta_generic_to_shared(acc.w) + 4u * (unsigned)jb;
-  else out.w = acc.w + jb;
-  const R ws = w * acc.scale;
-  deposit_settled_win<R, ORDER, DIM, G::JX, G::JP, G::JS>(out, X, Y, Z, a.jfac[0] * ws, a.jfac[1] * ws,
-                                                           a.jfac[2] * ws, a.qz * ws * vz);
-  return true;
-}
-
-// Deferred deposit jobs of particles whose support changes: up to kQCap
-// entries in shared memory, appended by warps through a shared counter and
-// deposited once, at the end of the work item, by all threads together
-// (dq_drain), so that the general stencil runs on full warps instead of on
-// the few lanes of every warp that hold such a particle.  A job that finds
-// the queue full is deposited on the spot.
-constexpr int kQCap = kPushQueueCap;
-// A chunk after which the queue could not take another chunk's worth of jobs
-// (1.5 times what the last chunk added) drains it, the whole block taking
-// one job per thread, so that plasmas whose particles change support often
-// (fast beams) do not overflow it and deposit in divergent lanes.  A plasma
-// with few such particles drains once, at the end of the work item: every
-// drain costs a partly idle block-wide pass.
-template <class R> struct DepQueue {
-  int *job;  // [kQCap] packed cell and shift (pack_job) | axes whose support changes << 22
-  R *f;      // [7][kQCap]: old offsets x y z, new offsets x y z, weight (2D3V: vz in the old z slot)
-  int *tail;  // shared counter of appended jobs
 };
 
-// Append this lane's job; false when the queue is full.
-template <class R>
-__device__ __forceinline__ bool dq_push(const DepQueue<R> &q, int job, const R f[3], const R fn[3], R w, R vz,
-                                        bool twod) {
-  const unsigned act = __activemask();
-  const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
-  int base = 0;
-  if (lane == leader) base = atomicAdd(q.tail, __popc(act));
-  base = __shfl_sync(act, base, leader);
-  const int at = base + __popc(act & ((1u << lane) - 1u));
-  if (at >= kQCap) return false;
-  q.job[at] = job;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    q.f[d * kQCap + at] = (twod && d == 2) ? vz : f[d];
-    q.f[(3 + d) * kQCap + at] = fn[d];
+// Where a group's sums go.  FP32: the fixed-point pair of WinAcc<float>::add
+// at one base register plus a compile-time offset; FP64: a double shared
+// atomic (zero skipped).
+template <class R, int JS> struct GroupSink;
+template <int JS> struct GroupSink<float, JS> {
+  unsigned sb;  // byte address of the Jx low word of the stencil's first node
+  __device__ __forceinline__ void add(int comp, int off, float v) const {
+    const float y = v + WinAcc<float>::kMagicHi;
+    const float lf = v - (y - WinAcc<float>::kMagicHi);
+    const int hi = __float_as_int(y) - __float_as_int(WinAcc<float>::kMagicHi);
+    const int lo = __float2int_rn(lf);
+    const unsigned sa = sb + 8u * (unsigned)JS * (unsigned)comp + 4u * (unsigned)off;
+    asm volatile("red.shared.add.s32 [%0], %1;\n\tred.shared.add.s32 [%2], %3;" ::"r"(sa), "r"(lo),
+                 "r"(sa + 4u * (unsigned)JS), "r"(hi));
   }
-  q.f[6 * kQCap + at] = w;
-  return true;
-}
+};
+template <int JS> struct GroupSink<double, JS> {
+  double *w;  // Jx value of the stencil's first node (components JS doubles apart)
+  __device__ __forceinline__ void add(int comp, int off, double v) const {
+    if (v != 0.0) atomicAdd(w + comp * JS + off, v);
+  }
+};
 
-// The axes (bit d) on which a particle's shape support changes over a move.
-template <class R, int ORDER>
-__device__ __forceinline__ int support_change(const R f[3], const int s[3], const R fn[3]) {
-  int m = 0;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const bool ch = ORDER == 2 ? (s[d] + (fn[d] >= R(0.5)) != (f[d] >= R(0.5))) : s[d] != 0;
-    m |= ch ? 1 << d : 0;
-  }
-  return m;
+// A particle's tag, left by the push for the deposit: its group (10 bits),
+// for a particle whose support changes the move of its nearest node (CIC: of
+// its cell) as 1 + {-1, 0, 1} in 2 bits per axis, its rank within its sort
+// key (12 bits), and kTagChange or kTagIdle.
+constexpr uint32_t kTagChange = 1u << 30, kTagIdle = 1u << 31;
+
+// How many deposit tasks a group of c particles makes: pieces of kTaskLen,
+// and one for the rest, counted by length class in 10-bit fields (class 0 the
+// longest).  The threads of a warp take tasks of one class, so that their
+// loops have about the same length.
+__device__ __forceinline__ int task_class(unsigned rest) {
+  return rest >= 6 ? 1 : rest == 5 ? 2 : rest == 4 ? 3 : rest >= 2 ? 4 : 5;
+}
+__device__ __forceinline__ unsigned long long task_counts(unsigned c) {
+  const unsigned full = c / kTaskLen, rest = c % kTaskLen;
+  return (unsigned long long)full + (rest ? 1ull << (10 * task_class(rest)) : 0ull);
 }
 
 // The per-particle physics shared by the tile kernel and the escape kernel:
@@ -635,145 +587,50 @@ __device__ __forceinline__ void push_move(const PushArgs<R> &a, R u[3], const R 
   }
 }
 
-// Esirkepov deposit of one particle's move into the J window (§2 eq. 4 and
-// the continuity equation): l is its cell relative to the tile, s its cell
-// shift, f -> fn its offsets before and after the move, w its weight, vz its
-// velocity along z (the 2D3V Jz term).  Returns false when the checked build
-// finds the stencil outside the window (nothing deposited).
+// One block per work item.  In order: the E, B window is staged; every
+// particle of the item is gathered, pushed, moved and written back, leaving
+// its deposit job and tag in shared memory; the jobs are counting-sorted by
+// nearest node (indices only); the settled jobs are deposited a group at a
+// time, summed in registers, and those whose support changes one by one on
+// the general stencil; the J window is added to global J.
+//
+// What bounds it: instruction issue and shared-memory wavefronts, not HBM.
+// Depositing each particle by itself cost 54 contributions of seven
+// instructions, two of them shared reductions of 3.2 wavefronts (1884
+// instructions per 32 particles, 36 % of the time in reductions); a group sum
+// costs one FMA per contribution and the seven instructions once per group of
+// up to kTaskLen particles.  3D TSC FP32 thermal plasma at 8 per cell, 16.8M
+// particles (ncu): 1.655 -> 1.110 ms, 1626 instructions, reduction wavefronts
+// 210 M -> 63 M; 256^3 (134M particles): 14.0 -> 9.4 ms per push; FP64 64^3:
+// 4.26 -> 3.03 ms (no compare-and-swap loop per contribution).
 template <class R, int DIM, int ORDER>
-__device__ __forceinline__ bool deposit_particle(const PushArgs<R> &a, const WinAcc<R> &acc, const int l[3],
-                                                 const int s[3], const R f[3], const R fn[3], R w, R vz) {
+__global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(const PushArgs<R> a) {
   using G = Geo<DIM, ORDER>;
-  // A particle that keeps its place (and, in 2D3V, has vz = 0) or has no
-  // weight deposits nothing; a warp of such particles (a cold target before
-  // the pulse reaches it) skips the stencil with a uniform branch.
-  const unsigned act = __activemask();
-  const bool moves = w != R(0) && ((s[0] | s[1] | s[2]) != 0 || f[0] != fn[0] || f[1] != fn[1] ||
-                                   (DIM == 3 ? f[2] != fn[2] : vz != R(0)));
-  if (!__any_sync(act, moves)) return true;
-  DepositAxis<R, ORDER> dx, dy, dz;
-  dx.set(f[0], s[0], fn[0]);
-  dy.set(f[1], s[1], fn[1]);
-  if (DIM == 3) dz.set(f[2], s[2], fn[2]);
-  else dz.zero();
-  constexpr int oJ = G::D + G::LOJ;
-#ifdef PIC_CHECKED
-  {
-    // every deposit stencil inside the J window (checked builds)
-    const int rel[3] = {dx.rel, dy.rel, dz.rel};
-    constexpr int JW[3] = {G::JX, G::JY, G::JZ};
-    bool ok = true;
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) ok = ok && l[d] + rel[d] + oJ >= 0 && l[d] + rel[d] + oJ + G::NW - 1 < JW[d];
-    if (!PIC_CHECK(ok, a.ctr)) return false;
-  }
-#endif
-  const int jb = (l[0] + dx.rel + oJ) + (l[1] + dy.rel + oJ) * G::JX +
-                 (DIM == 3 ? (l[2] + dz.rel + oJ) * G::JP : 0);
-  const R ws = w * acc.scale;  // fixed-point units folded into the factors
-  // does some lane of this warp use the last stencil node of an axis?
-  const bool lx = __any_sync(act, dx.S0[G::NW - 1] != R(0) || dx.DS[G::NW - 1] != R(0));
-  const bool ly = __any_sync(act, dy.S0[G::NW - 1] != R(0) || dy.DS[G::NW - 1] != R(0));
-  const bool lz = DIM == 3 && __any_sync(act, dz.S0[G::NW - 1] != R(0) || dz.DS[G::NW - 1] != R(0));
-  deposit_win<R, ORDER, DIM, G::JX, G::JP>(acc, jb, dx, dy, dz, a.jfac[0] * ws, a.jfac[1] * ws,
-                                                    a.jfac[2] * ws, a.qz * ws * vz, lx, ly, lz);
-  return true;
-}
-
-// Deposit the n <= kQCap queued jobs on the general stencil, one per thread
-// (with `reset`, the queue is emptied for the jobs of the next chunks).
-// The jobs are first ordered by the axes on which their support changes
-// (a counting sort into `order`, kQCap ints of shared memory), so that the
-// lanes of a warp mostly share that set and the warp-uniform skip of the
-// outer stencil shell in deposit_particle drops the axes that did not
-// change.  Block-wide: every thread of the block calls it.
-template <class R, int DIM, int ORDER>
-__device__ __forceinline__ void dq_drain(const PushArgs<R> &a, const WinAcc<R> &acc, const DepQueue<R> &q, int n,
-                                         int *order, bool reset) {
-  __shared__ int s_cls[8];
-  const int i = threadIdx.x;
-  if (i < 8) s_cls[i] = 0;
-  __syncthreads();
-  // every thread has read the count: the queue may start over (appends
-  // resume only after the next chunk's barriers)
-  if (reset && i == 0) *q.tail = 0;
-  int cls = 0, rank = 0;
-  if (i < n) {
-    cls = (q.job[i] >> 22) & 7;
-    rank = atomicAdd(&s_cls[cls], 1);
-  }
-  __syncthreads();
-  if (i < n) {
-    int start = 0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) start += c < cls ? s_cls[c] : 0;
-    order[start + rank] = i;
-  }
-  __syncthreads();
-  if (i >= n) return;
-  const int at = order[i];
-  int l[3], sh[3];
-  unpack_job(q.job[at] & ((1 << 22) - 1), l, sh);
-  R f[3], fn[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    f[d] = (DIM == 2 && d == 2) ? R(0) : q.f[d * kQCap + at];
-    fn[d] = q.f[(3 + d) * kQCap + at];
-  }
-  const R vz = DIM == 2 ? q.f[2 * kQCap + at] : R(0);
-  deposit_particle<R, DIM, ORDER>(a, acc, l, sh, f, fn, q.f[6 * kQCap + at], vz);
-}
-
-// MID: drain the queue between chunks when it fills (for plasmas whose
-// particles change support often; see the launcher).
-template <class R, int DIM, int ORDER, bool MID>
-// Blocks per SM the register allocation is held to: FP32 3D TSC windows
-// fill half the shared memory (two blocks); the 3D CIC windows leave room for
-// three, which fit at 72 registers (1.27x faster than two); FP32 2D windows
-// are small, and at 64 registers four blocks fit (1.46x faster on a 2D slab
-// than two); none of these spill.  FP64 runs are bound by the FP64 pipe
-// whatever their occupancy.
-__global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? (DIM == 2 ? 4 : (ORDER == 1 ? 3 : 2)) : 1)
-    k_push(const PushArgs<R> a) {
-  using G = Geo<DIM, ORDER>;
-  constexpr int NS = G::NS;
-  static_assert(G::TX + G::D < 31 && G::TY + G::D < 31 && G::TZ + G::D < 31, "deposit job packing");
+  using L = Lay<R, DIM, ORDER>;
+  constexpr int NS = G::NS, CAP = L::CAP;
+  constexpr int SY = G::EX, SZ = G::EX * G::EY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R *sF = reinterpret_cast<R *>(smem_raw);    // 6 * EN: Ex Ey Ez Bx By Bz
-  // J window: 24 bytes per node (3 components x 8 bytes of fixed point)
-  unsigned char *sJraw = smem_raw + 6 * G::EN * sizeof(R);
-  R *sOff = reinterpret_cast<R *>(sJraw + 24 * G::JS);  // DIM x 256
-  R *sU = sOff + DIM * kThreads;              // 3 x 256
-  R *sW = sU + 3 * kThreads;                  // 256
-  int32_t *sCell = reinterpret_cast<int32_t *>(sW + kThreads);  // 256
-  int32_t *sJob = sCell + kThreads;  // FP32 3D: 256 deposit jobs
-  // queue of deferred deposit jobs (after the jobs in 3D FP32, after the cells otherwise)
-  constexpr bool kSplitLayout = DIM == 3 && sizeof(R) == 4;
-  // the settled stencils and the queue: all but FP64 2D, whose kernel is
-  // bound by the FP64 pipe in its gather and lost occupancy to the extra
-  // registers and shared memory (measured 2.22 -> 1.91 G particle-steps/s
-  // on the 2D laser slab)
-  constexpr bool kSettled = !(sizeof(R) == 8 && DIM == 2);
-  constexpr int kQJobBytes = 4 * kQCap;  // a multiple of 8: the R array that follows stays aligned
-  DepQueue<R> dq;
-  dq.job = sCell + (kSplitLayout ? 2 : 1) * kThreads;
-  dq.f = reinterpret_cast<R *>(reinterpret_cast<char *>(dq.job) + kQJobBytes);
-  __shared__ int s_qtail;
-  dq.tail = &s_qtail;
-  int q_prev = 0;  // jobs queued at the end of the previous chunk (the same in every thread)
-  __shared__ unsigned int s_clamp;
-  __shared__ double s_scale;
-  __shared__ unsigned int s_emax[3];
-  __shared__ float s_qsum, s_wsum, s_q1;
-  float emax[3] = {0.f, 0.f, 0.f};
+  R *sF = reinterpret_cast<R *>(smem_raw);  // 6 * EN: Ex Ey Ez Bx By Bz, then the J window
+  R *sJob = reinterpret_cast<R *>(smem_raw + L::kJob);
+  uint32_t *sTag = reinterpret_cast<uint32_t *>(smem_raw + L::kTag);
+  uint16_t *sOrder = reinterpret_cast<uint16_t *>(smem_raw + L::kOrder);
+  uint32_t *sCount = reinterpret_cast<uint32_t *>(smem_raw + L::kCount);
+  uint16_t *sStart = reinterpret_cast<uint16_t *>(smem_raw + L::kCount);  // over the counts, once read
+  uint16_t *sTask = reinterpret_cast<uint16_t *>(smem_raw + L::kTask);
+  __shared__ unsigned int s_clamp, s_absorbed, s_next;
+  __shared__ float s_q;
+  __shared__ unsigned int s_wsum[kThreads / 32];
+  __shared__ unsigned long long s_wcls[kThreads / 32];
 
   const int wi = blockIdx.x;  // work item
   const int t = a.work_tile[wi];
   if (t < 0) return;
   const int64_t pb = a.work_pb[wi];
-  const int64_t pe = pb + a.chunk < a.tile_start[t + 1] ? pb + a.chunk : a.tile_start[t + 1];
-  if (pb >= pe) return;
-  const int tid = threadIdx.x;
+  const int64_t run_b = a.tile_start[t], run_e = a.tile_start[t + 1];
+  const int64_t len = work_item_slots(run_e - run_b, a.chunk);
+  const int n = (int)(run_e - pb < len ? run_e - pb : len);
+  if (n <= 0) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int t0[3];
   {
     const int tx = t % a.ntile[0];
@@ -782,320 +639,393 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? (DIM == 2 ? 4 : (OR
     t0[1] = (r % a.ntile[1]) * G::TY;
     t0[2] = (r / a.ntile[1]) * G::TZ;
   }
+  // this thread's particles are slots tid, tid + 256, ...: each is loaded one
+  // pass ahead of its use
+  int c_next = -1;
+  R f_next[3], u_next[3], w_next = R(0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) f_next[d] = u_next[d] = R(0);
+  auto fetch = [&](int s) {
+    const int64_t p = pb + s;
+    c_next = a.cell[p];
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) f_next[d] = a.off[d][p];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) u_next[d] = a.u[d][p];
+    w_next = a.w[p];
+  };
+  if (tid < n) fetch(tid);
 
   // ---- stage E, B of the tile + guard (periodic wrap of global indices) ----
   for (int q = tid; q < G::EN; q += kThreads) {
     const int x = q % G::EX;
     const int y = (q / G::EX) % G::EY;
     const int z = q / (G::EX * G::EY);
-    const int gi = wrap_near(t0[0] - G::D - G::LOE + x, a.n[0]);
-    const int gj = wrap_near(t0[1] - G::D - G::LOE + y, a.n[1]);
-    const int gk = DIM == 3 ? wrap_near(t0[2] - G::D - G::LOE + z, a.n[2]) : 0;
+    const int gi = wrap_near(t0[0] - G::O + x, a.n[0]);
+    const int gj = wrap_near(t0[1] - G::O + y, a.n[1]);
+    const int gk = DIM == 3 ? wrap_near(t0[2] - G::O + z, a.n[2]) : 0;
     const int64_t g = gi + (int64_t)a.n[0] * (gj + (int64_t)a.n[1] * gk);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const R ev = a.E[c][g];
-      sF[c * G::EN + q] = ev;
+      sF[c * G::EN + q] = a.E[c][g];
       sF[(3 + c) * G::EN + q] = a.B[c][g];
-      emax[c] = fmax(emax[c], fabs((float)ev));
     }
   }
-  for (int q = tid; q < 6 * G::JS; q += kThreads) reinterpret_cast<int *>(sJraw)[q] = 0;  // 24 B per node
+  for (int q = tid; q < G::KT; q += kThreads) sCount[q] = 0;
   if (tid == 0) {
-    s_clamp = 0;
-    s_qtail = 0;
-    s_emax[0] = s_emax[1] = s_emax[2] = 0u;
-    s_qsum = 0.f;
-    s_wsum = 0.f;
-    s_q1 = 0.f;
+    s_clamp = s_absorbed = s_next = 0;
+    s_q = 0.f;
   }
   __syncthreads();
-  if (sizeof(R) == 4) {
-    // fixed-point scale: bound Q on |J| at any node of the window (see WinAcc)
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-      if (emax[c] > 0.f) atomicMax(&s_emax[c], __float_as_uint(emax[c]));
-    __syncthreads();
-    const float ex = __uint_as_float(s_emax[0]), ey = __uint_as_float(s_emax[1]), ez = __uint_as_float(s_emax[2]);
-    const float kick = (float)(2.0 * fabs((double)a.qmh)) * sqrtf(ex * ex + ey * ey + ez * ez);
-    if (a.fresh) {
-      // tile contents are new (sorted): bound from the particles themselves
-      float qs = 0.f, w0 = 0.f;
-      for (int64_t p = pb + tid; p < pe; p += kThreads) {
-        if (a.cell[p] < 0) continue;
-        const float ux = (float)a.u[0][p], uy = (float)a.u[1][p], uz = (float)a.u[2][p];
-        const float aw = fabsf((float)a.w[p]);
-        qs += aw * fminf(1.f, sqrtf(ux * ux + uy * uy + uz * uz) + kick);
-        w0 += aw;
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        qs += __shfl_down_sync(0xffffffffu, qs, o);
-        w0 += __shfl_down_sync(0xffffffffu, w0, o);
-      }
-      if ((tid & 31) == 0) {
-        if (qs > 0.f) atomicAdd(&s_qsum, qs);
-        if (w0 > 0.f) atomicAdd(&s_wsum, w0);
-      }
-    } else if (tid == 0) {
-      // |u| min'ed at 1 from the previous push, plus the kick of this step:
-      // sum |w| min(1, |u| + kick) <= sum |w| min(1, |u|) + kick sum |w|
-      s_wsum = a.tq[2 * wi];
-      s_qsum = a.tq[2 * wi + 1] + kick * s_wsum;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      // 1.01: room for the FP32 rounding of the sums above
-      const double Q = 1.01 * a.qabs * (double)s_qsum;
-      int e2 = 0;
-      if (Q > 0.0) frexp(Q, &e2);  // Q < 2^e2
-      int K = Q > 0.0 ? WinAcc<float>::kLimitLog2 - e2 : 100;
-      K = K > 100 ? 100 : (K < -100 ? -100 : K);
-      s_scale = ldexp(1.0, K);
-    }
-  } else if (tid == 0) {
-    s_scale = 1.0;
-  }
-  __syncthreads();
-  WinAcc<R> acc;
-  acc.w = reinterpret_cast<decltype(acc.w)>(sJraw);
-  acc.jn = G::JS;
-  acc.dummy = G::JN + (tid & 31);
-  acc.scale = (R)s_scale;
-  acc.unit = (R)(1.0 / s_scale);
 
-  // Slot assignment.  The deposit runs on the lane-spreading permutation e
-  // (bijective; lane l of warp w takes slot 8l + ((w + l/4) mod 8)): the
-  // slots are cell-sorted, so a warp's lanes sit about one cell apart and
-  // their atomics hit different nodes.  In 3D the gather and push run first
-  // on slot tid instead, where a warp's lanes sit in a few neighbouring cells
-  // and mostly read the same field nodes (shared-memory broadcasts instead of
-  // bank conflicts on the 162-node TSC gather); each pushed particle then
-  // writes its new state to global memory and leaves a deposit job behind
-  // (old offsets in sU, new ones in sOff, tile cell and cell shift packed in
-  // sJob) for the deposit phase after a block barrier.  In 2D the gather is a third of that, and FP64 runs are bound by
-  // the FP64 pipe: there the extra barrier and staging traffic cost more than
-  // they save, so one thread pushes and deposits slot e.
-  constexpr bool kSplit = DIM == 3 && sizeof(R) == 4;
-  const int lane = tid & 31, warp = tid >> 5;
-  const int e = 8 * lane + ((warp + (lane >> 2)) & 7);
-  const int ep = kSplit ? tid : e;  // slot gathered and pushed by this thread
+  // ---- gather, Boris, move, write back; leave a deposit job and its tag.
+  // The slots are cell-sorted, so a warp's lanes sit in a few neighbouring
+  // cells and mostly read the same field nodes (shared-memory broadcasts).
   unsigned my_clamp = 0, my_absorbed = 0;
-  float my_q1 = 0.f;
-
-  for (int64_t c0 = pb; c0 < pe; c0 += kThreads) {
-    const int cn = (int)(pe - c0 < kThreads ? pe - c0 : kThreads);
-    // coalesced load of the chunk, slot order
-    if (tid < cn) {
-      const int64_t p = c0 + tid;
-      sCell[tid] = a.cell[p];
+  float my_q = 0.f;  // bound on this thread's part of |J| at any node: sum |w| min(1, |u|)
+  for (int s = tid; s < n; s += kThreads) {
+    const int c = c_next;
+    R f[3], u[3];
 #pragma unroll
-      for (int d = 0; d < DIM; ++d) sOff[d * kThreads + tid] = a.off[d][p];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) sU[d * kThreads + tid] = a.u[d][p];
-      sW[tid] = a.w[p];
+    for (int d = 0; d < 3; ++d) {
+      f[d] = f_next[d];
+      u[d] = u_next[d];
     }
-    __syncthreads();
-    // ---- gather, Boris, move (and, in 2D, deposit) of slot ep ----
-    if (ep < cn) {
-      int job = 0;
-      const int c = sCell[ep];
-      if (c >= 0) {
-        // decode the cell and its position relative to the tile
-        const uint32_t r0 = a.dn0.div((uint32_t)c);
-        int ci[3];
-        ci[0] = c - (int)r0 * a.n[0];
-        if (DIM == 3) {
-          const uint32_t r1 = a.dn1.div(r0);
-          ci[1] = (int)r0 - (int)r1 * a.n[1];
-          ci[2] = (int)r1;
-        } else {
-          ci[1] = (int)r0;
-          ci[2] = 0;
+    const R w = w_next;
+    if (s + kThreads < n) fetch(s + kThreads);
+    uint32_t tag = kTagIdle;
+    if (c >= 0) do {  // (a single pass, left early by particles that do not deposit)
+      const int64_t p = pb + s;
+      // decode the cell and its position relative to the tile
+      const uint32_t r0 = a.dn0.div((uint32_t)c);
+      int ci[3];
+      ci[0] = c - (int)r0 * a.n[0];
+      if (DIM == 3) {
+        const uint32_t r1 = a.dn1.div(r0);
+        ci[1] = (int)r0 - (int)r1 * a.n[1];
+        ci[2] = (int)r1;
+      } else {
+        ci[1] = (int)r0;
+        ci[2] = 0;
+      }
+      int l[3] = {0, 0, 0};
+      bool inw = true;
+      constexpr int TT[3] = {G::TX, G::TY, G::TZ};
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) {
+        int dl = ci[d] - t0[d];
+        if (dl > TT[d] - 1 + G::D) dl -= a.n[d];
+        if (dl < -G::D) dl += a.n[d];
+        l[d] = dl;
+        inw = inw && dl >= -G::D && dl <= TT[d] - 1 + G::D;
+      }
+      R fn[3], ig = R(0), d0[3], d1[3];
+      int sh[3], k[3] = {0, 0, 0}, key[3] = {0, 0, 0};
+      if (inw) {
+        // ---- gather (§2: g-weighted average of the grid fields) ----
+        GatherAxis<R, ORDER> gx, gy, gz;
+        gx.set(f[0], a.ec);
+        gy.set(f[1], a.ec);
+        gz.set(f[2], a.ec);
+#ifdef PIC_CHECKED
+        {
+          // every gather stencil inside the E/B window (checked builds)
+          const GatherAxis<R, ORDER> *ga[3] = {&gx, &gy, &gz};
+          constexpr int EW[3] = {G::EX, G::EY, G::EZ};
+          bool ok = true;
+#pragma unroll
+          for (int d = 0; d < DIM; ++d) {
+            const int lo = l[d] + (ga[d]->relp < ga[d]->reld ? ga[d]->relp : ga[d]->reld) + G::O;
+            const int hi = l[d] + (ga[d]->relp > ga[d]->reld ? ga[d]->relp : ga[d]->reld) + G::O + NS - 1;
+            ok = ok && lo >= 0 && hi < EW[d];
+          }
+          if (!PIC_CHECK(ok, a.ctr)) break;  // leaves the particle as it was
         }
-        int l[3] = {0, 0, 0};
-        bool inw = true;
-        constexpr int TT[3] = {G::TX, G::TY, G::TZ};
+#endif
+        const int xp = l[0] + gx.relp + G::O, xd = l[0] + gx.reld + G::O;
+        const int yp = (l[1] + gy.relp + G::O) * SY, yd = (l[1] + gy.reld + G::O) * SY;
+        const int zp = DIM == 3 ? (l[2] + gz.relp + G::O) * SZ : 0;
+        const int zd = DIM == 3 ? (l[2] + gz.reld + G::O) * SZ : 0;
+        R E[3], B[3];
+        E[0] = gsum<R, NS, DIM, SY, SZ>(sF + 0 * G::EN + xd + yp + zp, gx.wd, gy.wp, gz.wp);
+        E[1] = gsum<R, NS, DIM, SY, SZ>(sF + 1 * G::EN + xp + yd + zp, gx.wp, gy.wd, gz.wp);
+        E[2] = gsum<R, NS, DIM, SY, SZ>(sF + 2 * G::EN + xp + yp + zd, gx.wp, gy.wp, gz.wd);
+        B[0] = gsum<R, NS, DIM, SY, SZ>(sF + 3 * G::EN + xp + yd + zd, gx.wp, gy.wd, gz.wd);
+        B[1] = gsum<R, NS, DIM, SY, SZ>(sF + 4 * G::EN + xd + yp + zd, gx.wd, gy.wp, gz.wd);
+        B[2] = gsum<R, NS, DIM, SY, SZ>(sF + 5 * G::EN + xd + yd + zp, gx.wd, gy.wd, gz.wp);
+
+        // ---- Boris push (§2 eq. 3) and leap-frog move ----
+        unsigned clamp = 0;
+        push_move<R, ORDER, DIM>(a, u, E, B, f, fn, sh, ig, clamp);
+        // offsets from the nearest node (TSC) or in the cell (CIC), before
+        // and after, and how far that node or cell moved
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          if (d >= DIM) {
+            d0[d] = d1[d] = R(0);
+            continue;
+          }
+          const int h0 = ORDER == 2 && f[d] >= R(0.5), h1 = ORDER == 2 && fn[d] >= R(0.5);
+          d0[d] = f[d] - R(h0);
+          d1[d] = fn[d] - R(h1);
+          k[d] = sh[d] + h1 - h0;
+          key[d] = l[d] + h0 + G::D;
+          constexpr int KK[3] = {G::KX, G::KY, G::KZ};
+          inw = inw && key[d] + k[d] >= 0 && key[d] + k[d] < KK[d];
+        }
+        if (inw) my_clamp += clamp;  // (the escape kernel counts its own)
+      }
+      if (!inw) {
+        // defer to k_push_escaped (state left untouched)
+        a.cell[p] = c | kEscFlag;
+        const unsigned act = __activemask();
+        const int leader = __ffs(act) - 1;
+        unsigned long long slot = 0;
+        if (lane == leader) slot = atomicAdd(a.esc_count, (unsigned long long)__popc(act));
+        slot = __shfl_sync(act, slot, leader) + __popc(act & ((1u << lane) - 1u));
+        a.esc_list[slot] = (int32_t)p;
+        break;
+      }
+
+      // ---- the new state ----
+      int nc = -1;  // removed at an absorbing wall after depositing its move
+      if (outside_walls<R>(a.absorb, ci[0] + sh[0], fn[0], a.n[0])) {
+        ++my_absorbed;
+      } else {
+        nc = c;
+        const int i0 = ci[0] + sh[0];
+        nc += sh[0] + (i0 < 0 ? a.n[0] : (i0 >= a.n[0] ? -a.n[0] : 0));
+        const int i1 = ci[1] + sh[1];
+        nc += (sh[1] + (i1 < 0 ? a.n[1] : (i1 >= a.n[1] ? -a.n[1] : 0))) * a.n[0];
+        if (DIM == 3) {
+          const int i2 = ci[2] + sh[2];
+          nc += (sh[2] + (i2 < 0 ? a.n[2] : (i2 >= a.n[2] ? -a.n[2] : 0))) * a.n[0] * a.n[1];
+        }
+      }
+      a.cell[p] = nc;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) a.off[d][p] = fn[d];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) a.u[d][p] = u[d];
+
+      // ---- the deposit job ----
+      // A particle that keeps its place (and, in 2D3V, has vz = 0) or has no
+      // weight deposits nothing (a cold target before the pulse reaches it).
+      const R vz = u[2] * ig;
+      const bool change = (k[0] | k[1] | k[2]) != 0;
+      if (w == R(0) || !(change || d0[0] != d1[0] || d0[1] != d1[1] || (DIM == 3 ? d0[2] != d1[2] : vz != R(0)))) break;
+      sJob[0 * CAP + s] = d0[0];
+      sJob[1 * CAP + s] = d0[1];
+      sJob[2 * CAP + s] = d1[0];
+      sJob[3 * CAP + s] = d1[1];
+      sJob[4 * CAP + s] = w;
+      if (DIM == 3) {
+        sJob[5 * CAP + s] = d0[2];
+        sJob[(L::NJ - 1) * CAP + s] = d1[2];
+      } else {
+        sJob[5 * CAP + s] = vz;
+      }
+      const uint32_t group = (uint32_t)(key[0] + G::KX * (key[1] + G::KY * key[2]));
+      uint32_t sort_key = group;
+      tag = group;
+      if (change) {
+        sort_key = G::KN - 1 + (k[0] != 0) + 2 * (k[1] != 0) + 4 * (k[2] != 0);
+        tag |= (uint32_t)((k[0] + 1) << 10 | (k[1] + 1) << 12 | (k[2] + 1) << 14) | kTagChange;
+      }
+      tag |= atomicAdd(&sCount[sort_key], 1u) << 16;
+      if (sizeof(R) == 4)
+        my_q += fabsf((float)w) * fminf(1.f, sqrtf((float)(u[0] * u[0] + u[1] * u[1] + u[2] * u[2])));
+    } while (0);
+    sTag[s] = tag;
+  }
+  if (sizeof(R) == 4) {
+    for (int o = 16; o > 0; o >>= 1) my_q += __shfl_xor_sync(0xffffffffu, my_q, o);
+    if (lane == 0 && my_q > 0.f) atomicAdd(&s_q, my_q);
+  }
+  if (my_clamp) atomicAdd(&s_clamp, my_clamp);
+  if (my_absorbed) atomicAdd(&s_absorbed, my_absorbed);
+  __syncthreads();
+  if (tid == 0) {
+    if (s_clamp) atomicAdd(&a.ctr->clamped, (unsigned long long)s_clamp);
+    if (s_absorbed) atomicAdd(&a.ctr->absorbed, (unsigned long long)s_absorbed);
+  }
+
+  // ---- counting sort of the jobs: key starts, and the deposit tasks.  Each
+  // thread takes KPT consecutive keys; one block scan carries the job count
+  // and the task counts of every length class.
+  constexpr int KPT = (G::KT + kThreads - 1) / kThreads;
+  uint32_t cnt[KPT], sum = 0;
+  unsigned long long cls = 0;
+#pragma unroll
+  for (int i = 0; i < KPT; ++i) {
+    const int q = tid * KPT + i;
+    cnt[i] = q < G::KT ? sCount[q] : 0u;
+    sum += cnt[i];
+    if (q < G::KN) cls += task_counts(cnt[i]);
+  }
+  const uint32_t sum0 = sum;
+  const unsigned long long cls0 = cls;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, sum, o);
+    const unsigned long long x = __shfl_up_sync(0xffffffffu, cls, o);
+    if (lane >= o) {
+      sum += v;
+      cls += x;
+    }
+  }
+  if (lane == 31) {
+    s_wsum[warp] = sum;
+    s_wcls[warp] = cls;
+  }
+  // the J window replaces E and B
+  for (int q = tid; q < (int)(L::kWin / 16); q += kThreads) reinterpret_cast<int4 *>(smem_raw)[q] = int4{0, 0, 0, 0};
+  __syncthreads();
+  uint32_t at = sum - sum0, njob = 0;
+  unsigned long long pos = cls - cls0, all = 0;
+#pragma unroll
+  for (int i = 0; i < kThreads / 32; ++i) {
+    const uint32_t v = s_wsum[i];
+    const unsigned long long x = s_wcls[i];
+    if (i < warp) {
+      at += v;
+      pos += x;
+    }
+    njob += v;
+    all += x;
+  }
+  if (njob == 0) return;  // nothing moved: no current
+  int ntask = 0;
+  {
+    int first[6];  // this thread's next task of each class; a class follows the longer ones
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      first[q] = ntask + (int)((pos >> (10 * q)) & 1023u);
+      ntask += (int)((all >> (10 * q)) & 1023u);
+    }
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+      const int q = tid * KPT + i;
+      if (q <= G::KT) sStart[q] = (uint16_t)at;
+      if (q < G::KN && cnt[i] > 0) {
+        const unsigned full = cnt[i] / kTaskLen, rest = cnt[i] % kTaskLen;
+        for (unsigned j = 0; j < full; ++j) sTask[first[0]++] = (uint16_t)((at + j * kTaskLen) | (kTaskLen - 1) << 12);
+        if (rest) {
+          const int cl = task_class(rest);
+          int where = 0;
+#pragma unroll
+          for (int z = 1; z < 6; ++z)
+            if (z == cl) where = first[z]++;
+          sTask[where] = (uint16_t)((at + full * kTaskLen) | (rest - 1) << 12);
+        }
+      }
+      at += cnt[i];
+    }
+  }
+  __syncthreads();
+  for (int s = tid; s < n; s += kThreads) {
+    const uint32_t tag = sTag[s];
+    if (tag & kTagIdle) continue;
+    uint32_t sort_key = tag & 1023u;
+    if (tag & kTagChange)
+      sort_key = G::KN - 1 + (((tag >> 10) & 3u) != 1u) + 2 * (((tag >> 12) & 3u) != 1u) + 4 * (((tag >> 14) & 3u) != 1u);
+    const uint32_t q = sStart[sort_key] + ((tag >> 16) & 4095u);
+    if (!PIC_CHECK(q < (uint32_t)CAP, a.ctr)) continue;
+    sOrder[q] = (uint16_t)s;
+  }
+  WinAcc<R> acc;
+  acc.w = reinterpret_cast<decltype(acc.w)>(smem_raw);
+  acc.jn = sizeof(R) == 4 ? G::JS : G::EN;
+  acc.dummy = G::EN + lane;
+  acc.scale = acc.unit = R(1);
+  if constexpr (sizeof(R) == 4) acc.set_scale(1.01f * a.qabs * s_q);  // 1.01: room for the FP32 rounding of the sum
+  __syncthreads();
+
+  // ---- deposit: warps take the next 32 tasks, longest first, then the next
+  // 32 particles whose support changes (in order of the axes that do)
+  const int ntask32 = (ntask + 31) & ~31, nset = sStart[G::KN];
+  const int nunit = ntask32 + (int)njob - nset;
+  if (tid == 0 && (int)njob > nset) atomicAdd(a.q_jobs, (unsigned long long)((int)njob - nset));
+  const R jf0 = a.jfac[0] * acc.scale, jf1 = a.jfac[1] * acc.scale, jf2 = a.jfac[2] * acc.scale;
+  const R jz = a.qz * acc.scale;  // 2D3V
+  for (;;) {
+    unsigned base = 0;
+    if (lane == 0) base = atomicAdd(&s_next, 32u);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if ((int)base >= nunit) break;
+    const int unit = (int)base + lane;
+    if ((int)base < ntask32) {
+      if (unit >= ntask) continue;
+      const unsigned tk = sTask[unit];
+      int j = tk & 4095u;
+      const int je = j + (int)(tk >> 12) + 1;
+      int s = sOrder[j];
+      const uint32_t group = sTag[s] & 1023u;
+      const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
+      // the stencil's first node: one below the nearest node (TSC), the cell's (CIC)
+      constexpr int o = ORDER == 2 ? 0 : 1;
+      const int jb = (kx + o) + (ky + o) * SY + (DIM == 3 ? (kz + o) * SZ : 0);
+      GroupSum<R, DIM, ORDER> g;
+      g.clear();
+      while (true) {
+        SettledAxis<R, ORDER> X, Y, Z;
+        X.set(sJob[s], sJob[2 * CAP + s]);
+        Y.set(sJob[CAP + s], sJob[3 * CAP + s]);
+        const R w = sJob[4 * CAP + s];
+        R qwvz = R(0);
+        if (DIM == 3) Z.set(sJob[5 * CAP + s], sJob[(L::NJ - 1) * CAP + s]);
+        else qwvz = jz * w * sJob[5 * CAP + s];
+        if (++j < je) s = sOrder[j];
+        g.add(X, Y, Z, jf0 * w, jf1 * w, jf2 * w, qwvz);
+        if (j >= je) break;
+      }
+      GroupSink<R, sizeof(R) == 4 ? G::JS : G::EN> out;
+      if constexpr (sizeof(R) == 4) out.sb = (unsigned)__cvta_generic_to_shared(acc.w) + 4u * (unsigned)jb;
+      else out.w = acc.w + jb;
+      g.template flush<SY, SZ>(out);
+    } else {
+      if (unit >= nunit) continue;
+      const int s = sOrder[nset + unit - ntask32];
+      const uint32_t tag = sTag[s];
+      const int group = tag & 1023u;
+      const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
+      DepositAxis<R, ORDER> X, Y, Z;
+      X.set_nodes(sJob[s], (int)((tag >> 10) & 3u) - 1, sJob[2 * CAP + s]);
+      Y.set_nodes(sJob[CAP + s], (int)((tag >> 12) & 3u) - 1, sJob[3 * CAP + s]);
+      const R w = sJob[4 * CAP + s];
+      R qwvz = R(0);
+      if (DIM == 3) {
+        Z.set_nodes(sJob[5 * CAP + s], (int)((tag >> 14) & 3u) - 1, sJob[(L::NJ - 1) * CAP + s]);
+      } else {
+        Z.zero();
+        qwvz = jz * w * sJob[5 * CAP + s];
+      }
+      const int bx = kx + 1 + X.rel, by = ky + 1 + Y.rel, bz = DIM == 3 ? kz + 1 + Z.rel : 0;
+#ifdef PIC_CHECKED
+      {
+        // the nodes that receive a current inside the window (checked builds)
+        const DepositAxis<R, ORDER> *da[3] = {&X, &Y, &Z};
+        const int b0[3] = {bx, by, bz};
+        constexpr int JW[3] = {G::EX, G::EY, G::EZ};
+        bool ok = true;
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
-          int dl = ci[d] - t0[d];
-          if (dl > TT[d] - 1 + G::D) dl -= a.n[d];
-          if (dl < -G::D) dl += a.n[d];
-          l[d] = dl;
-          inw = inw && dl >= -G::D && dl <= TT[d] - 1 + G::D;
+          const bool last = da[d]->S0[G::NW - 1] != R(0) || da[d]->DS[G::NW - 1] != R(0);
+          ok = ok && b0[d] >= 0 && b0[d] + G::NW - 2 + (last ? 1 : 0) < JW[d];
         }
-        if (!inw) {
-          // defer to k_push_escaped (state left untouched)
-          if (kSplit) a.cell[c0 + ep] = c | kEscFlag;
-          else sCell[ep] = c | kEscFlag;
-          const unsigned long long slot = atomicAdd(a.esc_count, 1ull);
-          a.esc_list[slot] = (int32_t)(c0 + ep);
-          my_q1 += fabsf((float)sW[ep]);  // its new |u| is not known here: bound by 1
-        } else do {  // (a single pass: the checked build leaves it early on a bad index)
-          R f[3], u[3];
-#pragma unroll
-          for (int d = 0; d < 3; ++d) {
-            f[d] = d < DIM ? sOff[d * kThreads + ep] : R(0);
-            u[d] = sU[d * kThreads + ep];
-          }
-          // ---- gather (§2: g-weighted average of the grid fields) ----
-          GatherAxis<R, ORDER> gx, gy, gz;
-          gx.set(f[0], a.ec);
-          gy.set(f[1], a.ec);
-          gz.set(f[2], a.ec);
-          constexpr int oE = G::D + G::LOE;
-#ifdef PIC_CHECKED
-          {
-            // every gather stencil inside the E/B window (checked builds)
-            const GatherAxis<R, ORDER> *ga[3] = {&gx, &gy, &gz};
-            constexpr int EW[3] = {G::EX, G::EY, G::EZ};
-            bool ok = true;
-#pragma unroll
-            for (int d = 0; d < DIM; ++d) {
-              const int lo = l[d] + (ga[d]->relp < ga[d]->reld ? ga[d]->relp : ga[d]->reld) + oE;
-              const int hi = l[d] + (ga[d]->relp > ga[d]->reld ? ga[d]->relp : ga[d]->reld) + oE + NS - 1;
-              ok = ok && lo >= 0 && hi < EW[d];
-            }
-            if (!PIC_CHECK(ok, a.ctr)) break;  // leaves the particle as it was
-          }
+        if (!PIC_CHECK(ok, a.ctr)) continue;
+      }
 #endif
-          const int xp = l[0] + gx.relp + oE, xd = l[0] + gx.reld + oE;
-          const int yp = (l[1] + gy.relp + oE) * G::EX, yd = (l[1] + gy.reld + oE) * G::EX;
-          const int zp = DIM == 3 ? (l[2] + gz.relp + oE) * G::EX * G::EY : 0;
-          const int zd = DIM == 3 ? (l[2] + gz.reld + oE) * G::EX * G::EY : 0;
-          constexpr int SY = G::EX, SZ = G::EX * G::EY;
-          R E[3], B[3];
-          E[0] = gsum<R, NS, DIM, SY, SZ>(sF + 0 * G::EN + xd + yp + zp, gx.wd, gy.wp, gz.wp);
-          E[1] = gsum<R, NS, DIM, SY, SZ>(sF + 1 * G::EN + xp + yd + zp, gx.wp, gy.wd, gz.wp);
-          E[2] = gsum<R, NS, DIM, SY, SZ>(sF + 2 * G::EN + xp + yp + zd, gx.wp, gy.wp, gz.wd);
-          B[0] = gsum<R, NS, DIM, SY, SZ>(sF + 3 * G::EN + xp + yd + zd, gx.wp, gy.wd, gz.wd);
-          B[1] = gsum<R, NS, DIM, SY, SZ>(sF + 4 * G::EN + xd + yp + zd, gx.wd, gy.wp, gz.wd);
-          B[2] = gsum<R, NS, DIM, SY, SZ>(sF + 5 * G::EN + xd + yd + zp, gx.wd, gy.wd, gz.wp);
-
-          // ---- Boris push (§2 eq. 3) and leap-frog move ----
-          R fn[3], ig;
-          int s[3];
-          push_move<R, ORDER, DIM>(a, u, E, B, f, fn, s, ig, my_clamp);
-          if (sizeof(R) == 4)
-            my_q1 += fabsf((float)sW[ep]) * fminf(1.f, sqrtf((float)(u[0] * u[0] + u[1] * u[1] + u[2] * u[2])));
-
-          if (!kSplit) {
-            bool done = false;
-            if constexpr (kSettled) {
-              const R vz = u[2] * ig;
-              done = deposit_settled<R, DIM, ORDER>(a, acc, l, s, f, fn, sW[ep], vz) ||
-                     dq_push<R>(dq, pack_job(l, s) | support_change<R, ORDER>(f, s, fn) << 22, f, fn, sW[ep], vz,
-                                DIM == 2);
-            }
-            if (!done && !deposit_particle<R, DIM, ORDER>(a, acc, l, s, f, fn, sW[ep], u[2] * ig))
-              break;  // (checked build) leaves the particle as it was
-          }
-
-          // ---- the new state ----
-          int nc = -1;  // removed at an absorbing wall after depositing its move
-          if (outside_walls<R>(a.absorb, ci[0] + s[0], fn[0], a.n[0])) {
-            ++my_absorbed;
-          } else {
-            nc = c;
-            const int i0 = ci[0] + s[0];
-            nc += s[0] + (i0 < 0 ? a.n[0] : (i0 >= a.n[0] ? -a.n[0] : 0));
-            const int i1 = ci[1] + s[1];
-            nc += (s[1] + (i1 < 0 ? a.n[1] : (i1 >= a.n[1] ? -a.n[1] : 0))) * a.n[0];
-            if (DIM == 3) {
-              const int i2 = ci[2] + s[2];
-              nc += (s[2] + (i2 < 0 ? a.n[2] : (i2 >= a.n[2] ? -a.n[2] : 0))) * a.n[0] * a.n[1];
-            }
-          }
-          if (kSplit) {
-            // Slot ep is this thread's own index: the state goes straight to
-            // global memory (coalesced).  The deposit job keeps the old
-            // offsets in sU (u is no longer needed there) and the new ones
-            // in sOff.
-            const int64_t p = c0 + ep;
-            a.cell[p] = nc;
-#pragma unroll
-            for (int d = 0; d < DIM; ++d) {
-              a.off[d][p] = fn[d];
-              sU[d * kThreads + ep] = f[d];
-              sOff[d * kThreads + ep] = fn[d];
-            }
-#pragma unroll
-            for (int d = 0; d < 3; ++d) a.u[d][p] = u[d];
-            job = pack_job(l, s);
-          } else {
-            // back into the staging slot, stored after the chunk
-#pragma unroll
-            for (int d = 0; d < DIM; ++d) sOff[d * kThreads + ep] = fn[d];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) sU[d * kThreads + ep] = u[d];
-            sCell[ep] = nc;
-          }
-        } while (0);
-      }
-      if (kSplit) sJob[ep] = job;
+      // does some lane of this warp use the last stencil node of an axis?
+      const unsigned act = __activemask();
+      const bool lx = __any_sync(act, X.S0[G::NW - 1] != R(0) || X.DS[G::NW - 1] != R(0));
+      const bool ly = __any_sync(act, Y.S0[G::NW - 1] != R(0) || Y.DS[G::NW - 1] != R(0));
+      const bool lz = DIM == 3 && __any_sync(act, Z.S0[G::NW - 1] != R(0) || Z.DS[G::NW - 1] != R(0));
+      deposit_win<R, ORDER, DIM, SY, SZ>(acc, bx + by * SY + bz * SZ, X, Y, Z, jf0 * w, jf1 * w, jf2 * w, qwvz, lx, ly,
+                                         lz);
     }
-    if (kSplit) {
-      __syncthreads();
-      // ---- Esirkepov deposit of slot e (3D) ----
-      if (e < cn) {
-        const int job = sJob[e];
-        if (job) {
-          int l[3], s[3];
-          unpack_job(job, l, s);
-          R f[3], fn[3];
-#pragma unroll
-          for (int d = 0; d < 3; ++d) {
-            f[d] = sU[d * kThreads + e];
-            fn[d] = sOff[d * kThreads + e];
-          }
-          bool done = false;
-          if constexpr (kSettled)
-            done = deposit_settled<R, DIM, ORDER>(a, acc, l, s, f, fn, sW[e], R(0)) ||
-                   dq_push<R>(dq, job | support_change<R, ORDER>(f, s, fn) << 22, f, fn, sW[e], R(0), false);
-          if (!done) deposit_particle<R, DIM, ORDER>(a, acc, l, s, f, fn, sW[e], R(0));
-        }
-      }
-    }
-    __syncthreads();
-    // coalesced store of the chunk (w is unchanged; 3D FP32 stored its state in phase 1)
-    if (!kSplit && tid < cn) {
-      const int64_t p = c0 + tid;
-      a.cell[p] = sCell[tid];
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) a.off[d][p] = sOff[d * kThreads + tid];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) a.u[d][p] = sU[d * kThreads + tid];
-    }
-    if constexpr (kSettled && MID) {
-      const int nq = *(volatile int *)dq.tail;  // read by every thread after the barrier above
-      const int inc = nq - q_prev;
-      if (nq + inc + inc / 2 > kQCap) {
-        if (tid == 0) atomicAdd(a.q_jobs, (unsigned long long)nq);
-        dq_drain<R, DIM, ORDER>(a, acc, dq, nq > kQCap ? kQCap : nq, sCell, true);
-        q_prev = 0;
-      } else {
-        q_prev = nq;
-      }
-    }
-  }
-  if constexpr (kSettled) {
-    // the deferred jobs still queued (the chunk loop ended on a barrier)
-    const int nq = *(volatile int *)dq.tail;
-    if (tid == 0 && nq > 0) atomicAdd(a.q_jobs, (unsigned long long)nq);
-    dq_drain<R, DIM, ORDER>(a, acc, dq, nq > kQCap ? kQCap : nq, sCell, false);
-  }
-
-  if (my_clamp) atomicAdd(&s_clamp, my_clamp);
-  if (my_absorbed) atomicAdd(&a.ctr->absorbed, (unsigned long long)my_absorbed);
-  if (sizeof(R) == 4) {
-    for (int o = 16; o > 0; o >>= 1) my_q1 += __shfl_down_sync(0xffffffffu, my_q1, o);
-    if ((tid & 31) == 0 && my_q1 > 0.f) atomicAdd(&s_q1, my_q1);
   }
   __syncthreads();
-  if (sizeof(R) == 4 && tid == 0) {
-    // bound inputs for the next step (the item keeps its slots until the next sort)
-    a.tq[2 * wi] = s_wsum;
-    a.tq[2 * wi + 1] = s_q1 * 1.0001f;
-  }
 
   // ---- flush the J window into global J ----
   if (sizeof(R) == 4 && (a.n[0] & 3) == 0) {
@@ -1103,26 +1033,26 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? (DIM == 2 ? 4 : (OR
     // aligned in global memory, one vector reduction each (every element
     // added atomically); a run reaching past the window's x ends adds zeros
     // there.  A run never straddles the periodic seam.
-    const int xs = t0[0] - G::D - G::LOJ;          // the window's first node, global x (unwrapped)
-    const int a0 = xs - (((xs % 4) + 4) & 3);      // the multiple of 4 at or below it
-    constexpr int NG = (G::JX + 6) / 4;            // runs per window row (the last may start past it)
-    for (int q = tid; q < NG * G::JY * G::JZ; q += kThreads) {
+    const int xs = t0[0] - G::O;               // the window's first node, global x (unwrapped)
+    const int a0 = xs - (((xs % 4) + 4) & 3);  // the multiple of 4 at or below it
+    constexpr int NG = (G::EX + 6) / 4;        // runs per window row (the last may start past it)
+    for (int q = tid; q < NG * G::EY * G::EZ; q += kThreads) {
       const int m = q % NG, row = q / NG;
-      const int y = row % G::JY, z = row / G::JY;
+      const int y = row % G::EY, z = row / G::EY;
       const int wx0 = a0 + 4 * m - xs;  // window x of the run's first node
-      if (wx0 >= G::JX) continue;
+      if (wx0 >= G::EX) continue;
       const int gi = wrap_near(a0 + 4 * m, a.n[0]);
-      const int gj = wrap_near(t0[1] - G::D - G::LOJ + y, a.n[1]);
-      const int gk = DIM == 3 ? wrap_near(t0[2] - G::D - G::LOJ + z, a.n[2]) : 0;
+      const int gj = wrap_near(t0[1] - G::O + y, a.n[1]);
+      const int gk = DIM == 3 ? wrap_near(t0[2] - G::O + z, a.n[2]) : 0;
       const int64_t g = gi + (int64_t)a.n[0] * (gj + (int64_t)a.n[1] * gk);
-      const int wrow = z * G::JP + y * G::JX;
+      const int wrow = z * SZ + y * SY;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         float v[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int wx = wx0 + e;
-          v[e] = (wx >= 0 && wx < G::JX) ? (float)acc.get(c, wrow + wx) : 0.f;
+          v[e] = (wx >= 0 && wx < G::EX) ? (float)acc.get(c, wrow + wx) : 0.f;
         }
         if (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f)
           asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a.J[c] + g), "f"(v[0]), "f"(v[1]),
@@ -1131,14 +1061,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? (DIM == 2 ? 4 : (OR
       }
     }
   } else {
-    for (int q = tid; q < G::JN; q += kThreads) {
-      const int z = q / G::JP;
-      const int x = (q - z * G::JP) % G::JX;
-      const int y = (q - z * G::JP) / G::JX;
-      if (y >= G::JY) continue;  // plane padding
-      const int gi = wrap_near(t0[0] - G::D - G::LOJ + x, a.n[0]);
-      const int gj = wrap_near(t0[1] - G::D - G::LOJ + y, a.n[1]);
-      const int gk = DIM == 3 ? wrap_near(t0[2] - G::D - G::LOJ + z, a.n[2]) : 0;
+    for (int q = tid; q < G::EN; q += kThreads) {
+      const int x = q % G::EX;
+      const int y = (q / G::EX) % G::EY;
+      const int z = q / SZ;
+      const int gi = wrap_near(t0[0] - G::O + x, a.n[0]);
+      const int gj = wrap_near(t0[1] - G::O + y, a.n[1]);
+      const int gk = DIM == 3 ? wrap_near(t0[2] - G::O + z, a.n[2]) : 0;
       const int64_t g = gi + (int64_t)a.n[0] * (gj + (int64_t)a.n[1] * gk);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -1147,7 +1076,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? (DIM == 2 ? 4 : (OR
       }
     }
   }
-  if (tid == 0 && s_clamp) atomicAdd(&a.ctr->clamped, (unsigned long long)s_clamp);
 }
 
 // Particles deferred by the tile kernel: the same gather / Boris / move /
@@ -1273,28 +1201,16 @@ __global__ void __launch_bounds__(kThreads) k_push_escaped(const PushArgs<R> a) 
   if (blockIdx.x == 0 && threadIdx.x == 0 && nesc) atomicAdd(&a.ctr->escaped, nesc);
 }
 
-template <class R, int DIM, int ORDER> constexpr size_t smem_bytes() {
-  using G = Geo<DIM, ORDER>;
-  // E, B window; J window; staging of cell, offsets, u, w; for FP32 3D the
-  // deposit jobs (a packed int per slot)
-  constexpr bool split = DIM == 3 && sizeof(R) == 4;
-  return (size_t)(6 * G::EN + (DIM + 4) * kThreads) * sizeof(R) + 24 * (size_t)G::JS +
-         (split ? 2 : 1) * kThreads * sizeof(int32_t) +
-         (sizeof(R) == 8 && DIM == 2 ? 0 : kQCap * (sizeof(int32_t) + 7 * sizeof(R)));
-}
-
 template <class R, int DIM, int ORDER>
 cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
-                     const int64_t *tile_start, const WorkSplit &ws, float *tq, int fresh, int32_t *esc_list,
-                     unsigned long long *esc_count, double q, double m, Counters *ctr, cudaStream_t st,
-                     int *nlaunch, bool mid_drain) {
+                     const int64_t *tile_start, const WorkSplit &ws, int32_t *esc_list, unsigned long long *esc_count,
+                     double q, double m, Counters *ctr, cudaStream_t st, int *nlaunch) {
+  if (ws.chunk > Lay<R, DIM, ORDER>::CAP) return cudaErrorInvalidValue;
   PushArgs<R> a;
   a.work_tile = ws.work_tile;
   a.work_pb = ws.work_pb;
   a.chunk = ws.chunk;
-  a.tq = tq;
-  a.fresh = fresh;
-  a.qabs = q < 0 ? -q : q;
+  a.qabs = (float)(q < 0 ? -q : q);
   for (int d = 0; d < 3; ++d) {
     a.n[d] = g.n[d];
     a.E[d] = static_cast<const R *>(E[d]);
@@ -1320,10 +1236,8 @@ cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *co
   a.absorb = g.absorb_lo || g.absorb_hi;
   a.ec = g.gather_ec;
   a.ctr = ctr;
-  constexpr size_t smem = smem_bytes<R, DIM, ORDER>();
-  // the variant that drains between chunks only where it can matter (3D;
-  // 2D targets queue few jobs)
-  auto fn = (DIM == 3 && mid_drain) ? k_push<R, DIM, ORDER, DIM == 3> : k_push<R, DIM, ORDER, false>;
+  constexpr size_t smem = Lay<R, DIM, ORDER>::kEnd;
+  auto fn = k_push<R, DIM, ORDER>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (ws.nwork > 0x7fffffff) return cudaErrorInvalidValue;
@@ -1564,30 +1478,34 @@ void push_tile_shape(int dims, int tile[3]) {
   tile[2] = dims == 3 ? Geo<3, 2>::TZ : 1;
 }
 
-size_t push_smem_bytes(const Grid &g) {
-  const int key = (g.prec == 1 ? 100 : 0) + g.dims * 10 + g.order;
-  switch (key) {
-    case 21: return smem_bytes<float, 2, 1>();
-    case 22: return smem_bytes<float, 2, 2>();
-    case 31: return smem_bytes<float, 3, 1>();
-    case 32: return smem_bytes<float, 3, 2>();
-    case 121: return smem_bytes<double, 2, 1>();
-    case 122: return smem_bytes<double, 2, 2>();
-    case 131: return smem_bytes<double, 3, 1>();
-    case 132: return smem_bytes<double, 3, 2>();
-    default: return 0;
+// The layout of the kernel that serves a grid: its shared memory, and the
+// most slots one of its work items may hold.
+template <class F> static auto with_layout(const Grid &g, F f) {
+  switch ((g.prec == 1 ? 100 : 0) + g.dims * 10 + g.order) {
+    case 21: return f(Lay<float, 2, 1>{});
+    case 22: return f(Lay<float, 2, 2>{});
+    case 31: return f(Lay<float, 3, 1>{});
+    case 121: return f(Lay<double, 2, 1>{});
+    case 122: return f(Lay<double, 2, 2>{});
+    case 131: return f(Lay<double, 3, 1>{});
+    case 132: return f(Lay<double, 3, 2>{});
+    default: return f(Lay<float, 3, 2>{});
   }
+}
+size_t push_smem_bytes(const Grid &g) {
+  return with_layout(g, [](auto l) { return (size_t)decltype(l)::kEnd; });
+}
+int64_t push_item_cap(const Grid &g) {
+  return with_layout(g, [](auto l) { return (int64_t)decltype(l)::CAP; });
 }
 
 cudaError_t launch_push(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
-                        const int64_t *tile_start, const WorkSplit &ws, float *tq, int fresh, int32_t *esc_list,
+                        const int64_t *tile_start, const WorkSplit &ws, int32_t *esc_list,
                         unsigned long long *esc_count, double q, double m, Counters *ctr, cudaStream_t st,
-                        int *nlaunch, int mid_drain) {
+                        int *nlaunch) {
   const int key = (g.prec == 1 ? 100 : 0) + g.dims * 10 + g.order;
-#define PIC_PUSH_CASE(K, R, D, O)                                                                        \
-  case K:                                                                                                \
-    return launch_t<R, D, O>(g, E, B, J, p, tile_start, ws, tq, fresh, esc_list, esc_count, q, m, ctr, st, \
-                             nlaunch, mid_drain != 0);
+#define PIC_PUSH_CASE(K, R, D, O) \
+  case K: return launch_t<R, D, O>(g, E, B, J, p, tile_start, ws, esc_list, esc_count, q, m, ctr, st, nlaunch);
   switch (key) {
     PIC_PUSH_CASE(21, float, 2, 1)
     PIC_PUSH_CASE(22, float, 2, 2)

@@ -150,7 +150,8 @@ __global__ void k_work_items(const int64_t *__restrict__ tile_start, int64_t nti
   }
   int64_t w = sh[threadIdx.x] - local;
   for (int64_t t = b; t < e; ++t) {
-    for (int64_t p = tile_start[t]; p < tile_start[t + 1]; p += chunk, ++w) {
+    const int64_t len = work_item_slots(tile_start[t + 1] - tile_start[t], chunk);
+    for (int64_t p = tile_start[t]; p < tile_start[t + 1]; p += len, ++w) {
       work_tile[w] = (int32_t)t;
       work_pb[w] = p;
     }
