@@ -651,14 +651,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_adj_push2d(cons
 }
 
 // Work items of a recorded particle buffer (the sort in effect when it was
-// recorded): item i covers the work_item_slots slots from work_pb[i] (fewer
-// at the end of the run) of tile t = work_tile[i] (-1: none); nsub blocks
-// share an item, kAdjSub slots each.
+// recorded): item i covers work_n[i] slots from work_pb[i] of tile
+// t = work_tile[i] (-1: none); nsub blocks share an item, kAdjSub slots each.
 struct AdjWork {
   const int32_t *work_tile;
   const int64_t *work_pb;
-  const int64_t *tile_start;
-  int64_t chunk;
+  const int32_t *work_n;
   int nsub;
   int nt0, t0, t1;
   unsigned long long *esc_total;  // running count of particles on the global path
@@ -679,10 +677,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
   const int item = blockIdx.x / w.nsub;
   const int t = w.work_tile[item];
   if (t < 0) return;
-  const int64_t te = w.tile_start[t + 1];
   const int64_t ib = w.work_pb[item];
-  const int64_t len = work_item_slots(te - w.tile_start[t], w.chunk);
-  const int64_t ie = ib + len < te ? ib + len : te;
+  const int64_t ie = ib + w.work_n[item];
   const int64_t pb = ib + (int64_t)(blockIdx.x % w.nsub) * kAdjSub;
   if (pb >= ie) return;
   const int64_t pe = pb + kAdjSub < ie ? pb + kAdjSub : ie;
@@ -908,8 +904,7 @@ static cudaError_t adj_push_t(const Grid &g, const Particles &tp, const int64_t 
   AdjWork w;
   w.work_tile = tt->work_tile;
   w.work_pb = tt->work_pb;
-  w.tile_start = tt->tile_start;
-  w.chunk = tt->chunk;
+  w.work_n = tt->work_n;
   w.nsub = (int)((tt->chunk + kAdjSub - 1) / kAdjSub);
   w.nt0 = g.ntile[0];
   w.t0 = g.tile[0];

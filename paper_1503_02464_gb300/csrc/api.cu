@@ -60,12 +60,12 @@ struct PCopy {
   int64_t *count = nullptr;
   // Tape entries: the work items of the sort in effect (tiled = false when
   // the species was unsorted at the copy).  meta is this copy's own buffer;
-  // work_pb, tile_start, work_tile point to it or, when the previous tape
-  // entry was recorded under the same sort, to that entry's arrays.
+  // work_pb, work_tile, work_n point to it or, when the previous tape entry
+  // was recorded under the same sort, to that entry's arrays.
   void *meta = nullptr;
   const int32_t *work_tile = nullptr;
   const int64_t *work_pb = nullptr;
-  const int64_t *tile_start = nullptr;
+  const int32_t *work_n = nullptr;
   int64_t nwork = 0, chunk = 0, sorts = -1;
   bool tiled = false;
 };
@@ -242,17 +242,14 @@ size_t particles_bytes(int64_t cap, size_t rs, int dims) {
   return align256(n * sizeof(int32_t)) + (size_t)(dims + 4) * align256(n * rs) + align256(n * sizeof(uint32_t));
 }
 
-// A sort's outputs in one allocation: work_pb[nwork], tile_start[ntiles + 1],
-// work_tile[nwork].
-size_t sort_meta_bytes(int64_t nwork, int64_t ntiles) {
-  return sizeof(int64_t) * (size_t)(nwork + ntiles + 1) + sizeof(int32_t) * (size_t)nwork;
-}
+// A sort's work items in one allocation (one copy for a tape entry):
+// work_pb[nwork], work_tile[nwork], work_n[nwork].
+size_t sort_meta_bytes(int64_t nwork) { return (sizeof(int64_t) + 2 * sizeof(int32_t)) * (size_t)nwork; }
 
-void set_sort_meta(void *base, int64_t nwork, int64_t ntiles, int64_t *&work_pb, int64_t *&tile_start,
-                   int32_t *&work_tile) {
+void set_sort_meta(void *base, int64_t nwork, int64_t *&work_pb, int32_t *&work_tile, int32_t *&work_n) {
   work_pb = static_cast<int64_t *>(base);
-  tile_start = work_pb + nwork;
-  work_tile = reinterpret_cast<int32_t *>(tile_start + ntiles + 1);
+  work_tile = reinterpret_cast<int32_t *>(work_pb + nwork);
+  work_n = work_tile + nwork;
 }
 
 void free_particles(Particles &p) {
@@ -382,7 +379,7 @@ cudaError_t alloc_snapshot(pic_handle *h, Snapshot &sn) {
   size_t total = align256(6 * fb);
   for (int i = 0; i < h->nsp; ++i)
     total += particles_bytes(h->sp[i].slots, h->rsize, h->g.dims) + 256 +
-             align256(sort_meta_bytes(h->sp[i].work.nwork, h->g.ntiles));
+             align256(sort_meta_bytes(h->sp[i].work.nwork));
   char *base = nullptr;
   const cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&base), total, h->st);
   if (e != cudaSuccess) return e;
@@ -400,7 +397,7 @@ cudaError_t alloc_snapshot(pic_handle *h, Snapshot &sn) {
     c.count = reinterpret_cast<int64_t *>(q);
     q += 256;
     c.meta = q;
-    q += align256(sort_meta_bytes(h->sp[i].work.nwork, h->g.ntiles));
+    q += align256(sort_meta_bytes(h->sp[i].work.nwork));
   }
   sn.allocated = true;
   sn.nsp = h->nsp;
@@ -441,17 +438,17 @@ cudaError_t save_snapshot(pic_handle *h, Snapshot &sn, bool tape = false, const 
     const PCopy *q = prev ? &prev->sp[i] : nullptr;
     if (q && q->tiled && q->sorts == s.sorts) {
       c.work_pb = q->work_pb;
-      c.tile_start = q->tile_start;
       c.work_tile = q->work_tile;
+      c.work_n = q->work_n;
     } else {
-      e = cudaMemcpyAsync(c.meta, s.work.work_pb, sort_meta_bytes(s.work.nwork, h->g.ntiles), cudaMemcpyDeviceToDevice,
+      e = cudaMemcpyAsync(c.meta, s.work.work_pb, sort_meta_bytes(s.work.nwork), cudaMemcpyDeviceToDevice,
                           h->st);
-      int64_t *pb = nullptr, *ts = nullptr;
-      int32_t *wt = nullptr;
-      set_sort_meta(c.meta, s.work.nwork, h->g.ntiles, pb, ts, wt);
+      int64_t *pb = nullptr;
+      int32_t *wt = nullptr, *wn = nullptr;
+      set_sort_meta(c.meta, s.work.nwork, pb, wt, wn);
       c.work_pb = pb;
-      c.tile_start = ts;
       c.work_tile = wt;
+      c.work_n = wn;
     }
   }
   sn.step = h->step;
@@ -613,7 +610,7 @@ int pic_create(const pic_config *cfg, pic_handle **out) {
        cudaMalloc(&h->keys, (size_t)nkeys * sizeof(int32_t)) == cudaSuccess &&
        cudaMalloc(&h->tile_tmp, (size_t)(g.ntiles + 1) * sizeof(int64_t)) == cudaSuccess &&
        cudaMalloc(&h->ctr, sizeof(Counters)) == cudaSuccess && cudaMalloc(&h->bad, sizeof(unsigned long long)) == cudaSuccess &&
-       cudaMalloc(&h->esc_count, 2 * sizeof(unsigned long long)) == cudaSuccess &&
+       cudaMalloc(&h->esc_count, 3 * sizeof(unsigned long long)) == cudaSuccess &&
        cudaMalloc(&h->mur, 8 * sizeof(double) * (size_t)g.n[1] * g.n[2]) == cudaSuccess;
   if (!ok) {
     pic_destroy(h);
@@ -672,7 +669,8 @@ int pic_destroy(pic_handle *h) {
     free_particles(s.buf[1]);
     cudaFree(s.d_count);
     cudaFree(s.rank);
-    cudaFree(s.work.work_pb);  // with tile_start and work_tile
+    cudaFree(s.tile_start);
+    cudaFree(s.work.work_pb);  // with work_tile and work_n
     cudaFreeHost(s.esc_host);
     if (s.esc_ev) cudaEventDestroy(s.esc_ev);
   }
@@ -730,23 +728,24 @@ int pic_add_species(pic_handle *h, double q, double m, int64_t capacity, int *sp
     chunk = chunk < 512 ? 512 : chunk;
     const int64_t cap = pic::push_item_cap(h->g);
     s.work.chunk = chunk > cap ? cap : chunk;
+    s.work.slots = s.slots;
     s.work.nwork = s.slots / s.work.chunk + 1 + h->g.ntiles;
   }
   if (e == cudaSuccess) e = cudaMallocHost(&s.esc_host, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.esc_ev, cudaEventDisableTiming);
-  // the sort's outputs in one allocation (one copy for a tape entry):
-  // work_pb[nwork], tile_start[ntiles + 1], work_tile[nwork]
+  if (e == cudaSuccess) e = cudaMalloc(&s.tile_start, sizeof(int64_t) * (size_t)(h->g.ntiles + 1));
   if (e == cudaSuccess) {
     void *meta = nullptr;
-    e = cudaMalloc(&meta, sort_meta_bytes(s.work.nwork, h->g.ntiles));
-    if (e == cudaSuccess) set_sort_meta(meta, s.work.nwork, h->g.ntiles, s.work.work_pb, s.tile_start, s.work.work_tile);
+    e = cudaMalloc(&meta, sort_meta_bytes(s.work.nwork));
+    if (e == cudaSuccess) set_sort_meta(meta, s.work.nwork, s.work.work_pb, s.work.work_tile, s.work.work_n);
   }
   if (e != cudaSuccess) {
     free_particles(s.buf[0]);
     free_particles(s.buf[1]);
     cudaFree(s.d_count);
     cudaFree(s.rank);
-    cudaFree(s.work.work_pb);  // with tile_start and work_tile
+    cudaFree(s.tile_start);
+    cudaFree(s.work.work_pb);  // with work_tile and work_n
     cudaFreeHost(s.esc_host);
     if (s.esc_ev) cudaEventDestroy(s.esc_ev);
     s = Species{};
@@ -1271,8 +1270,8 @@ int pic_step(pic_handle *h, int nsteps) {
       Timed tm(h, pic::KC_PUSH);
       int nl = 0;
       CK(h,
-         pic::launch_push(h->g, h->E, h->B, h->J, s.buf[s.cur], s.tile_start, s.work, s.rank, h->esc_count, s.q,
-                          s.m, h->ctr, h->st, &nl),
+         pic::launch_push(h->g, h->E, h->B, h->J, s.buf[s.cur], s.work, s.rank, h->esc_count, s.q, s.m, h->ctr,
+                          h->st, &nl),
          "push");
       h->launches += nl;
       if (s.crowded) h->crowded_pushes++;
@@ -1717,7 +1716,7 @@ int pic_adjoint_step(pic_handle *h, int nsteps) {
       pic::AdjTiles tt;
       tt.work_tile = c.work_tile;
       tt.work_pb = c.work_pb;
-      tt.tile_start = c.tile_start;
+      tt.work_n = c.work_n;
       tt.nwork = c.nwork;
       tt.chunk = c.chunk;
       tt.esc_total = h->adj_esc;

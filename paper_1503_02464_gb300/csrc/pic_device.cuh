@@ -196,14 +196,32 @@ template <class R, int ORDER> struct DepositAxis {
   }
 };
 
+// 1/sqrt(x) and 1/x for x >= 1 (infinite or NaN pass).  FP32: the hardware's
+// approximation and one Newton-Raphson step, y + y/2 (1 - x y^2) and
+// y + y (1 - x y), its residual in one FMA: within an ulp, like the IEEE root
+// and quotient it replaces, in a few instructions.  FP64: rsqrt (1 ulp, as
+// the root and quotient together) and the IEEE quotient.
+__device__ __forceinline__ float rsqrt_near(float x) {
+  const float y = rsqrtf(x);
+  const float e = x > 3.4e38f ? 0.f : fmaf(-x * y, y, 1.f);
+  return fmaf(0.5f * y, e, y);
+}
+__device__ __forceinline__ double rsqrt_near(double x) { return rsqrt(x); }
+__device__ __forceinline__ float rcp_near(float x) {
+  const float y = __fdividef(1.f, x);
+  const float e = x > 3.4e38f ? 0.f : fmaf(-x, y, 1.f);
+  return fmaf(y, e, y);
+}
+__device__ __forceinline__ double rcp_near(double x) { return 1.0 / x; }
+
 // Boris rotation in the variable u = gamma v (ref [8] of the paper; §2 eq. 3):
 // half electric kick, magnetic rotation, half electric kick.  h = q dt/(2m).
 template <class R>
 __device__ __forceinline__ void boris(R h, const R E[3], const R B[3], R u[3]) {
   const R umx = u[0] + h * E[0], umy = u[1] + h * E[1], umz = u[2] + h * E[2];
-  const R ig = R(1) / sqrt(R(1) + umx * umx + umy * umy + umz * umz);
+  const R ig = rsqrt_near(R(1) + umx * umx + umy * umy + umz * umz);
   const R tx = h * B[0] * ig, ty = h * B[1] * ig, tz = h * B[2] * ig;
-  const R sf = R(2) / (R(1) + tx * tx + ty * ty + tz * tz);
+  const R sf = R(2) * rcp_near(R(1) + tx * tx + ty * ty + tz * tz);
   const R sx = sf * tx, sy = sf * ty, sz = sf * tz;
   const R upx = umx + (umy * tz - umz * ty);
   const R upy = umy + (umz * tx - umx * tz);

@@ -129,33 +129,28 @@ size_t push_smem_bytes(const Grid &g);
 // Most slots a work item of the push may hold (its chunk is at most this).
 int64_t push_item_cap(const Grid &g);
 // Work items of the push kernel: each tile's slot run is cut into the fewest
-// pieces of at most `chunk` slots (a multiple of 4), all of them
-// work_item_slots(run, chunk) long but the last; item i starts at slot
-// work_pb[i] of tile work_tile[i] (-1: no work).  nwork bounds the item count
-// (slots / chunk + 1 + ntiles).
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline int64_t work_item_slots(int64_t run, int64_t chunk) {
-  const int64_t pieces = (run + chunk - 1) / chunk;
-  return pieces > 1 ? ((run + pieces - 1) / pieces + 3) / 4 * 4 : run;
-}
+// equal pieces (multiples of 4 slots; the last may be shorter) of at most
+// `chunk` slots; item i covers work_n[i] slots from work_pb[i] of tile
+// work_tile[i] (-1: no work, the list ends there).  nwork bounds the item
+// count (slots / chunk + 1 + ntiles).
 struct WorkSplit {
+  int64_t slots = 0;  // of the species
   int64_t chunk = 0;
   int64_t nwork = 0;
   int32_t *work_tile = nullptr;
   int64_t *work_pb = nullptr;
+  int32_t *work_n = nullptr;
 };
 
 // Tile kernel (one block per work item) + escape kernel.
 // esc_list (one int per slot) is scratch for particles deferred to the
-// escape kernel; esc_count (two counters) receives their number and the
-// number of particles whose shape support changed in the launch.
+// escape kernel; esc_count (three counters) receives their number and the
+// number of particles whose shape support changed in the launch, and counts
+// the work items that blocks took.
 constexpr int kCrowdedJobs = 168;  // such particles per work item above which a species counts as crowded (pic_diag)
 cudaError_t launch_push(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
-                        const int64_t *tile_start, const WorkSplit &ws, int32_t *esc_list,
-                        unsigned long long *esc_count, double q, double m, Counters *ctr, cudaStream_t st,
-                        int *nlaunch);
+                        const WorkSplit &ws, int32_t *esc_list, unsigned long long *esc_count, double q, double m,
+                        Counters *ctr, cudaStream_t st, int *nlaunch);
 
 // Diagnostics charge density of particles sorted by tile (exact 64-bit
 // fixed-point window sums; adds into rho).
@@ -248,7 +243,7 @@ cudaError_t launch_adj_mur(const Grid &g, void *const lE[3], double *pend, const
 struct AdjTiles {
   const int32_t *work_tile = nullptr;
   const int64_t *work_pb = nullptr;
-  const int64_t *tile_start = nullptr;
+  const int32_t *work_n = nullptr;
   int64_t nwork = 0, chunk = 0;
   unsigned long long *esc_total = nullptr;
 };

@@ -64,14 +64,18 @@ template <int DIM, int ORDER> struct Geo {
 // block keeps the deposit jobs of its whole item, so that the particles of
 // one node meet whatever their slots.  FP32 3D items hold a full 8x8x4 tile
 // of the 8-per-cell plasma with room to spare at two blocks per SM.
-constexpr int kTaskLen = 8;  // particles one thread sums at a time
 template <class R, int DIM, int ORDER> struct Lay {
   using G = Geo<DIM, ORDER>;
   static constexpr bool F32 = sizeof(R) == 4;
-  static constexpr int CAP = F32 ? (DIM == 3 ? 2176 : 2048) : (DIM == 3 ? 2432 : 1664);
-  static constexpr int BLOCKS = F32 ? (DIM == 3 ? 2 : 3) : (DIM == 3 ? 1 : 2);  // per SM
-  static constexpr int NJ = DIM == 3 ? 7 : 6;  // job: old and new offsets per axis, weight (2D3V: and vz)
-  static constexpr int MAXT = CAP / kTaskLen + G::KN;
+  static constexpr int CAP = F32 ? (DIM == 2 ? 1408 : ORDER == 1 ? 1216 : 2176) : (DIM == 3 ? 2432 : 1664);
+  // per SM (FP32: 2D at three 4 % slower, 3D CIC at two 19 %)
+  static constexpr int BLOCKS = F32 ? (DIM == 2 ? 4 : ORDER == 1 ? 3 : 2) : (DIM == 3 ? 1 : 2);
+  // a particle (offsets, momenta, weight), then its job (old and new offsets, 2D3V: vz, weight)
+  static constexpr int NJ = DIM == 3 ? 7 : 6;
+  // particles one thread sums at a time (3D: 6 beat 5, 7, 8, 12 and 16 by up
+  // to 5 %, two-stream 15 %; 2D: 8 beat 6 by 2 %)
+  static constexpr int TASK = DIM == 3 ? 6 : 8;
+  static constexpr int MAXT = CAP / TASK + G::KN;
   static constexpr size_t align16(size_t b) { return (b + 15) / 16 * 16; }
   // E and B, then (once every particle is pushed) the J window
   static constexpr size_t kWin = align16(6 * G::EN * sizeof(R) > 24 * G::JS ? 6 * G::EN * sizeof(R) : 24 * G::JS);
@@ -84,20 +88,22 @@ template <class R, int DIM, int ORDER> struct Lay {
   static_assert(G::KT < 1024 && CAP < 4096 && CAP % 32 == 0, "tag packing");
 };
 
-// Division by a runtime constant (Granlund-Montgomery): q = (umulhi(n,m) + n) >> l.
+// Division of n < 2^31 by a runtime constant d (Granlund-Montgomery):
+// q = umulhi(n, m) >> s with s = ceil(log2 d) - 1, m = ceil(2^(32 + s) / d)
+// (the excess e = m d - 2^(32 + s) < d <= 2^(s + 1), so e n < 2^(32 + s));
+// m = 0 stands for d = 1.
 struct FastDiv {
-  uint32_t m, l;
-  __device__ __forceinline__ uint32_t div(uint32_t n) const {
-    return (uint32_t)(((uint64_t)__umulhi(n, m) + n) >> l);
-  }
+  uint32_t m, s;
+  __device__ __forceinline__ uint32_t div(uint32_t n) const { return m ? __umulhi(n, m) >> s : n; }
 };
 
 FastDiv make_fastdiv(uint32_t d) {
-  FastDiv f;
+  FastDiv f{0, 0};
+  if (d < 2) return f;
   uint32_t l = 0;
   while ((1ull << l) < d) ++l;
-  f.l = l;
-  f.m = (uint32_t)(((1ull << 32) * ((1ull << l) - d)) / d + 1);
+  f.s = l - 1;
+  f.m = (uint32_t)(((1ull << (32 + f.s)) + d - 1) / d);
   return f;
 }
 
@@ -112,11 +118,13 @@ template <class R> struct PushArgs {
   R *off[3];
   R *u[3];
   const R *w;
-  const int64_t *tile_start;
   float qabs;                       // |q|
-  const int32_t *work_tile;         // work item -> tile (-1: none)
+  const int32_t *work_tile;         // work item -> tile (-1: none, nor any after it)
   const int64_t *work_pb;           // work item -> first slot
-  int64_t chunk;                    // slots per work item at most (work_item_slots)
+  const int32_t *work_n;            // work item -> slots
+  int nwork;                        // work items at most
+  int64_t slots;                    // slots of the species
+  unsigned long long *next_item;    // items taken beyond the first of every block
   int32_t *esc_list;                // slots deferred to k_push_escaped
   unsigned long long *esc_count;
   unsigned long long *q_jobs;       // particles of this launch whose shape support changes
@@ -125,7 +133,6 @@ template <class R> struct PushArgs {
   R jfac[3];  // -q dx_a / dt  (Esirkepov running-sum scale, times w)
   R qz;       // q            (2D3V: Jz = q w vz S)
   int absorb;  // absorbing x walls: remove particles leaving [kWallLo, n0 - kWallHiMargin)
-  int ec;      // energy-conserving gather
   Counters *ctr;
 };
 
@@ -139,7 +146,14 @@ template <class R> __device__ __forceinline__ bool outside_walls(int absorb, int
 
 template <class R> __device__ __forceinline__ R inv_sqrt(R x);
 template <> __device__ __forceinline__ float inv_sqrt<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double inv_sqrt<double>(double x) { return 1.0 / sqrt(x); }
+template <> __device__ __forceinline__ double inv_sqrt<double>(double x) { return rsqrt(x); }
+
+// One value copied from global to shared memory asynchronously.
+template <class R> __device__ __forceinline__ void copy_async(R *to, const R *from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from),
+               "n"((int)sizeof(R))
+               : "memory");
+}
 
 // Weighted sum of one field component over the gather stencil; the stencil
 // offsets are compile-time (row stride SY, plane stride SZ).
@@ -542,23 +556,70 @@ template <int JS> struct GroupSink<double, JS> {
 // A particle's tag, left by the push for the deposit: its group (10 bits),
 // for a particle whose support changes the move of its nearest node (CIC: of
 // its cell) as 1 + {-1, 0, 1} in 2 bits per axis, its rank within its sort
-// key (12 bits), and kTagChange or kTagIdle.
-constexpr uint32_t kTagChange = 1u << 30, kTagIdle = 1u << 31;
+// key (12 bits), and kTagChange; or kTagIdle, or kTagEscape (kTagIdle among
+// its bits).
+constexpr uint32_t kTagChange = 1u << 30, kTagIdle = 1u << 31, kTagEscape = kTagIdle | kTagChange;
 
-// How many deposit tasks a group of c particles makes: pieces of kTaskLen,
-// and one for the rest, counted by length class in 10-bit fields (class 0 the
-// longest).  The threads of a warp take tasks of one class, so that their
-// loops have about the same length.
-__device__ __forceinline__ int task_class(unsigned rest) {
-  return rest >= 6 ? 1 : rest == 5 ? 2 : rest == 4 ? 3 : rest >= 2 ? 4 : 5;
+// How many deposit tasks a group of c particles makes: pieces of T, and one
+// for the rest, counted by length class in 10-bit fields, the longest first
+// (T = 6: one class per length; T = 8: 8, 6 or 7, 5, 4, 2 or 3, 1).  The
+// threads of a warp take tasks of one class, so that their loops have the same
+// length.
+constexpr int kClasses = 6;
+template <int T> __device__ __forceinline__ int task_class(unsigned len) {
+  if (T == 6) return 6 - (int)len;
+  return len >= 8 ? 0 : len >= 6 ? 1 : len >= 5 ? 2 : len >= 4 ? 3 : len >= 2 ? 4 : 5;
 }
-__device__ __forceinline__ unsigned long long task_counts(unsigned c) {
-  const unsigned full = c / kTaskLen, rest = c % kTaskLen;
-  return (unsigned long long)full + (rest ? 1ull << (10 * task_class(rest)) : 0ull);
+template <int T> __device__ __forceinline__ unsigned long long task_counts(unsigned c) {
+  static_assert(T == 6 || T == 8, "classes");
+  const unsigned full = c / T, rest = c % T;
+  return (unsigned long long)full + (rest ? 1ull << (10 * task_class<T>(rest)) : 0ull);
+}
+
+// Ascending order of N = 8 values by Batcher's odd-even merge sort (19
+// compare-exchanges).
+__device__ __forceinline__ void sort8(uint32_t (&v)[8]) {
+#pragma unroll
+  for (int p = 1; p < 8; p *= 2)
+#pragma unroll
+    for (int k = p; k >= 1; k /= 2)
+#pragma unroll
+      for (int j = k % p; j + k < 8; j += 2 * k)
+#pragma unroll
+        for (int i = 0; i < k; ++i)
+          if (i + j + k < 8 && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+            const uint32_t lo = min(v[i + j], v[i + j + k]), hi = max(v[i + j], v[i + j + k]);
+            v[i + j] = lo;
+            v[i + j + k] = hi;
+          }
+}
+
+// A moved offset x (at most one cell away under the Courant limit) brought
+// back into [0, 1): the cell shift sh, and the offset.  A carry that rounds to
+// 1 is clamped and counted.
+template <class R> __device__ __forceinline__ R carry(R x, int &sh, unsigned &clamp);
+template <> __device__ __forceinline__ float carry<float>(float x, int &sh, unsigned &clamp) {
+  const float fl = floorf(x);
+  sh = (int)fl;
+  x -= fl;
+  if (x >= 1.f) {
+    x = below_one<float>();
+    ++clamp;
+  }
+  return x;
+}
+template <> __device__ __forceinline__ double carry<double>(double x, int &sh, unsigned &clamp) {
+  sh = (x >= 1.0) ? 1 : ((x < 0.0) ? -1 : 0);
+  x -= (double)sh;
+  if (x >= 1.0) {
+    x = below_one<double>();
+    ++clamp;
+  }
+  return x;
 }
 
 // The per-particle physics shared by the tile kernel and the escape kernel:
-// given gathered E, B, advance u, move, and build the deposit stencils.
+// given gathered E, B, advance u and move.
 template <class R, int ORDER, int DIM>
 __device__ __forceinline__ void push_move(const PushArgs<R> &a, R u[3], const R E[3], const R B[3], const R f[3],
                                           R fn[3], int s[3], R &ig, unsigned &clamp) {
@@ -570,40 +631,28 @@ __device__ __forceinline__ void push_move(const PushArgs<R> &a, R u[3], const R 
     s[d] = 0;
   }
 #pragma unroll
-  for (int d = 0; d < DIM; ++d) {
-    R x = f[d] + a.dtdx[d] * u[d] * ig;
-    const int sh = (x >= R(1)) ? 1 : ((x < R(0)) ? -1 : 0);
-    x -= R(sh);
-    if (x >= R(1)) {
-      x = below_one<R>();
-      ++clamp;
-    }
-    if (x < R(0)) {
-      x = R(0);
-      ++clamp;
-    }
-    fn[d] = x;
-    s[d] = sh;
-  }
+  for (int d = 0; d < DIM; ++d) fn[d] = carry<R>(f[d] + a.dtdx[d] * u[d] * ig, s[d], clamp);
 }
 
-// One block per work item.  In order: the E, B window is staged; every
-// particle of the item is gathered, pushed, moved and written back, leaving
-// its deposit job and tag in shared memory; the jobs are counting-sorted by
-// nearest node (indices only); the settled jobs are deposited a group at a
-// time, summed in registers, and those whose support changes one by one on
-// the general stencil; the J window is added to global J.
+// As many blocks as fit the GPU, each taking work items in turn.  For an item:
+// its particles and the E, B window are staged by asynchronous copies; every
+// particle is gathered, pushed, moved and written back, leaving its deposit
+// job and tag in its place; the jobs are counting-sorted by nearest node
+// (indices only); those whose support changes are deposited one by one on the
+// general stencil, the settled ones a group at a time, summed in registers;
+// the J window is added to global J while the next item's particles arrive.
 //
-// What bounds it: instruction issue and shared-memory wavefronts, not HBM.
-// Depositing each particle by itself cost 54 contributions of seven
-// instructions, two of them shared reductions of 3.2 wavefronts (1884
-// instructions per 32 particles, 36 % of the time in reductions); a group sum
-// costs one FMA per contribution and the seven instructions once per group of
-// up to kTaskLen particles.  3D TSC FP32 thermal plasma at 8 per cell, 16.8M
-// particles (ncu): 1.655 -> 1.110 ms, 1626 instructions, reduction wavefronts
-// 210 M -> 63 M; 256^3 (134M particles): 14.0 -> 9.4 ms per push; FP64 64^3:
-// 4.26 -> 3.03 ms (no compare-and-swap loop per contribution).
-template <class R, int DIM, int ORDER>
+// What bounds it: shared-memory wavefronts (69 % of the time at 128^3) and
+// instruction issue (61 %), not HBM.  Depositing each particle by itself cost
+// 54 contributions of seven instructions, two of them shared reductions of 3.2
+// wavefronts; a group sum costs one FMA per contribution and the seven
+// instructions once per group.  The gather's 162 shared loads per particle are
+// the largest part left.  3D TSC FP32 thermal plasma at 8 per cell, 16.8M
+// particles (ncu): 1.655 ms depositing particle by particle, 1.110 by groups,
+// 1.030 with asynchronous staging, blocks that stay, and tasks of six; 1884,
+// 1626 and 1520 instructions per 32 particles.  Two particles per thread in
+// packed FP32 (FFMA2) needed 16 % fewer instructions and the same time.
+template <class R, int DIM, int ORDER, bool EC>
 __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(const PushArgs<R> a) {
   using G = Geo<DIM, ORDER>;
   using L = Lay<R, DIM, ORDER>;
@@ -621,144 +670,177 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
   __shared__ float s_q;
   __shared__ unsigned int s_wsum[kThreads / 32];
   __shared__ unsigned long long s_wcls[kThreads / 32];
-
-  const int wi = blockIdx.x;  // work item
-  const int t = a.work_tile[wi];
-  if (t < 0) return;
-  const int64_t pb = a.work_pb[wi];
-  const int64_t run_b = a.tile_start[t], run_e = a.tile_start[t + 1];
-  const int64_t len = work_item_slots(run_e - run_b, a.chunk);
-  const int n = (int)(run_e - pb < len ? run_e - pb : len);
-  if (n <= 0) return;
+  __shared__ int64_t s_pb;  // the block's next item: first slot, slots, tile
+  __shared__ int s_n, s_tile;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int t0[3];
-  {
-    const int tx = t % a.ntile[0];
-    const int r = t / a.ntile[0];
-    t0[0] = tx * G::TX;
-    t0[1] = (r % a.ntile[1]) * G::TY;
-    t0[2] = (r / a.ntile[1]) * G::TZ;
-  }
-  // this thread's particles are slots tid, tid + 256, ...: each is loaded one
-  // pass ahead of its use
-  int c_next = -1;
-  R f_next[3], u_next[3], w_next = R(0);
+
+  // The item's particles, copied into their slots' places in shared memory
+  // (cell, offsets, momenta, weight: the arrays that their jobs will take),
+  // 16 bytes per asynchronous copy: runs and items start and end on multiples
+  // of four slots.
+  const auto stage_particles = [&](int64_t pb, int n) {
+    const auto copy = [&](void *to, const void *from, int bytes) {
+      const unsigned d = (unsigned)__cvta_generic_to_shared(to);
+      for (int i = tid * 16; i < bytes; i += kThreads * 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + i), "l"(static_cast<const char *>(from) + i)
+                     : "memory");
+    };
+    if (!PIC_CHECK(n >= 0 && n <= CAP && n % 4 == 0 && pb % 4 == 0 && pb >= 0 && pb + n <= a.slots, a.ctr)) return;
+    copy(sTag, a.cell + pb, n * (int)sizeof(int32_t));
 #pragma unroll
-  for (int d = 0; d < 3; ++d) f_next[d] = u_next[d] = R(0);
-  auto fetch = [&](int s) {
-    const int64_t p = pb + s;
-    c_next = a.cell[p];
+    for (int d = 0; d < DIM; ++d) copy(sJob + d * CAP, a.off[d] + pb, n * (int)sizeof(R));
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) f_next[d] = a.off[d][p];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) u_next[d] = a.u[d][p];
-    w_next = a.w[p];
+    for (int d = 0; d < 3; ++d) copy(sJob + (DIM + d) * CAP, a.u[d] + pb, n * (int)sizeof(R));
+    copy(sJob + (L::NJ - 1) * CAP, a.w + pb, n * (int)sizeof(R));
   };
-  if (tid < n) fetch(tid);
 
-  // ---- stage E, B of the tile + guard (periodic wrap of global indices) ----
-  for (int q = tid; q < G::EN; q += kThreads) {
-    const int x = q % G::EX;
-    const int y = (q / G::EX) % G::EY;
-    const int z = q / (G::EX * G::EY);
-    const int gi = wrap_near(t0[0] - G::O + x, a.n[0]);
-    const int gj = wrap_near(t0[1] - G::O + y, a.n[1]);
-    const int gk = DIM == 3 ? wrap_near(t0[2] - G::O + z, a.n[2]) : 0;
-    const int64_t g = gi + (int64_t)a.n[0] * (gj + (int64_t)a.n[1] * gk);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      sF[c * G::EN + q] = a.E[c][g];
-      sF[(3 + c) * G::EN + q] = a.B[c][g];
-    }
-  }
-  for (int q = tid; q < G::KT; q += kThreads) sCount[q] = 0;
-  if (tid == 0) {
-    s_clamp = s_absorbed = s_next = 0;
-    s_q = 0.f;
-  }
-  __syncthreads();
-
-  // ---- gather, Boris, move, write back; leave a deposit job and its tag.
-  // The slots are cell-sorted, so a warp's lanes sit in a few neighbouring
-  // cells and mostly read the same field nodes (shared-memory broadcasts).
-  unsigned my_clamp = 0, my_absorbed = 0;
-  float my_q = 0.f;  // bound on this thread's part of |J| at any node: sum |w| min(1, |u|)
-  for (int s = tid; s < n; s += kThreads) {
-    const int c = c_next;
-    R f[3], u[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      f[d] = f_next[d];
-      u[d] = u_next[d];
-    }
-    const R w = w_next;
-    if (s + kThreads < n) fetch(s + kThreads);
-    uint32_t tag = kTagIdle;
-    if (c >= 0) do {  // (a single pass, left early by particles that do not deposit)
-      const int64_t p = pb + s;
-      // decode the cell and its position relative to the tile
-      const uint32_t r0 = a.dn0.div((uint32_t)c);
-      int ci[3];
-      ci[0] = c - (int)r0 * a.n[0];
-      if (DIM == 3) {
-        const uint32_t r1 = a.dn1.div(r0);
-        ci[1] = (int)r0 - (int)r1 * a.n[1];
-        ci[2] = (int)r1;
-      } else {
-        ci[1] = (int)r0;
-        ci[2] = 0;
-      }
-      int l[3] = {0, 0, 0};
-      bool inw = true;
-      constexpr int TT[3] = {G::TX, G::TY, G::TZ};
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-        int dl = ci[d] - t0[d];
-        if (dl > TT[d] - 1 + G::D) dl -= a.n[d];
-        if (dl < -G::D) dl += a.n[d];
-        l[d] = dl;
-        inw = inw && dl >= -G::D && dl <= TT[d] - 1 + G::D;
-      }
-      R fn[3], ig = R(0), d0[3], d1[3];
-      int sh[3], k[3] = {0, 0, 0}, key[3] = {0, 0, 0};
-      if (inw) {
-        // ---- gather (§2: g-weighted average of the grid fields) ----
-        GatherAxis<R, ORDER> gx, gy, gz;
-        gx.set(f[0], a.ec);
-        gy.set(f[1], a.ec);
-        gz.set(f[2], a.ec);
+  int wi = blockIdx.x;
+  int t = wi < a.nwork ? a.work_tile[wi] : -1;
+  if (t < 0) return;
+  int64_t pb = a.work_pb[wi];
+  int n = a.work_n[wi];
+  stage_particles(pb, n);
+  while (t >= 0) {
 #ifdef PIC_CHECKED
-        {
-          // every gather stencil inside the E/B window (checked builds)
-          const GatherAxis<R, ORDER> *ga[3] = {&gx, &gy, &gz};
-          constexpr int EW[3] = {G::EX, G::EY, G::EZ};
-          bool ok = true;
-#pragma unroll
-          for (int d = 0; d < DIM; ++d) {
-            const int lo = l[d] + (ga[d]->relp < ga[d]->reld ? ga[d]->relp : ga[d]->reld) + G::O;
-            const int hi = l[d] + (ga[d]->relp > ga[d]->reld ? ga[d]->relp : ga[d]->reld) + G::O + NS - 1;
-            ok = ok && lo >= 0 && hi < EW[d];
-          }
-          if (!PIC_CHECK(ok, a.ctr)) break;  // leaves the particle as it was
-        }
+    if (!PIC_CHECK(n >= 0 && n <= CAP && n % 4 == 0 && pb % 4 == 0 && pb >= 0 && pb + n <= a.slots, a.ctr)) n = 0;
 #endif
-        const int xp = l[0] + gx.relp + G::O, xd = l[0] + gx.reld + G::O;
-        const int yp = (l[1] + gy.relp + G::O) * SY, yd = (l[1] + gy.reld + G::O) * SY;
-        const int zp = DIM == 3 ? (l[2] + gz.relp + G::O) * SZ : 0;
-        const int zd = DIM == 3 ? (l[2] + gz.reld + G::O) * SZ : 0;
-        R E[3], B[3];
-        E[0] = gsum<R, NS, DIM, SY, SZ>(sF + 0 * G::EN + xd + yp + zp, gx.wd, gy.wp, gz.wp);
-        E[1] = gsum<R, NS, DIM, SY, SZ>(sF + 1 * G::EN + xp + yd + zp, gx.wp, gy.wd, gz.wp);
-        E[2] = gsum<R, NS, DIM, SY, SZ>(sF + 2 * G::EN + xp + yp + zd, gx.wp, gy.wp, gz.wd);
-        B[0] = gsum<R, NS, DIM, SY, SZ>(sF + 3 * G::EN + xp + yd + zd, gx.wp, gy.wd, gz.wd);
-        B[1] = gsum<R, NS, DIM, SY, SZ>(sF + 4 * G::EN + xd + yp + zd, gx.wd, gy.wp, gz.wd);
-        B[2] = gsum<R, NS, DIM, SY, SZ>(sF + 5 * G::EN + xd + yd + zp, gx.wd, gy.wd, gz.wp);
+    int t0[3];
+    bool edge = false;  // the window crosses the grid's seam
+    {
+      const int tx = t % a.ntile[0];
+      const int r = t / a.ntile[0];
+      t0[0] = tx * G::TX;
+      t0[1] = (r % a.ntile[1]) * G::TY;
+      t0[2] = (r / a.ntile[1]) * G::TZ;
+      constexpr int EE[3] = {G::EX, G::EY, G::EZ};
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) edge = edge || t0[d] < G::O || t0[d] - G::O + EE[d] > a.n[d];
+    }
+    // ---- stage E, B of the tile + guard (periodic wrap of global indices), RL
+    // threads per row ----
+    {
+      constexpr int RL = G::EX <= 16 ? 16 : 32;
+      const int x = tid % RL;
+      if (x < G::EX) {
+        int gi = t0[0] - G::O + x;
+        if (edge) gi = wrap_near(gi, a.n[0]);
+        for (int r = tid / RL; r < G::EY * G::EZ; r += kThreads / RL) {
+          const int z = DIM == 3 ? r / G::EY : 0, y = r - z * G::EY;
+          int gj = t0[1] - G::O + y, gk = DIM == 3 ? t0[2] - G::O + z : 0;
+          if (edge) {
+            gj = wrap_near(gj, a.n[1]);
+            if (DIM == 3) gk = wrap_near(gk, a.n[2]);
+          }
+          const int g = gi + a.n[0] * (gj + a.n[1] * gk);  // (cells stay below 2^30)
+          const int q = x + r * G::EX;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            copy_async(sF + c * G::EN + q, a.E[c] + g);
+            copy_async(sF + (3 + c) * G::EN + q, a.B[c] + g);
+          }
+        }
+      }
+    }
+    for (int q = tid; q < G::KT; q += kThreads) sCount[q] = 0;
+    if (tid == 0) {
+      s_clamp = s_absorbed = s_next = 0;
+      s_q = 0.f;
+    }
+    unsigned long long taken = 0;
+    if (tid == 0) taken = atomicAdd(a.next_item, 1ull);  // (its result is first needed after the push)
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
 
-        // ---- Boris push (§2 eq. 3) and leap-frog move ----
+    // ---- gather, Boris, move, write back; leave a deposit job and its tag.
+    // The slots are cell-sorted, so a warp's lanes sit in a few neighbouring
+    // cells and mostly read the same field nodes (shared-memory broadcasts).
+    unsigned my_clamp = 0, my_absorbed = 0;
+    float my_q = 0.f;  // bound on this thread's part of |J| at any node: sum |w| |v|
+    for (int s = tid; s < n; s += kThreads) {
+      const int c = (int)sTag[s];
+      uint32_t tag = kTagIdle;
+      // (a single pass, left early by particles that do not deposit)
+      if (c >= 0 && PIC_CHECK(c / a.n[0] / a.n[1] < a.n[2], a.ctr)) do {
+        const int64_t p = pb + s;
+        // decode the cell and its position relative to the tile
+        const uint32_t r0 = a.dn0.div((uint32_t)c);
+        int ci[3];
+        ci[0] = c - (int)r0 * a.n[0];
+        if (DIM == 3) {
+          const uint32_t r1 = a.dn1.div(r0);
+          ci[1] = (int)r0 - (int)r1 * a.n[1];
+          ci[2] = (int)r1;
+        } else {
+          ci[1] = (int)r0;
+          ci[2] = 0;
+        }
+        int l[3] = {0, 0, 0};
+        bool inw = true;
+        constexpr int TT[3] = {G::TX, G::TY, G::TZ};
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+          int dl = ci[d] - t0[d];
+          if (edge) {
+            if (dl > TT[d] - 1 + G::D) dl -= a.n[d];
+            if (dl < -G::D) dl += a.n[d];
+          }
+          l[d] = dl;
+          inw = inw && (unsigned)(dl + G::D) < (unsigned)(TT[d] + 2 * G::D);
+        }
+        tag = kTagEscape;
+        if (!inw) break;
+        R f[3], u[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          f[d] = d < DIM ? sJob[d * CAP + s] : R(0);
+          u[d] = sJob[(DIM + d) * CAP + s];
+        }
+        const R w = sJob[(L::NJ - 1) * CAP + s];
+        // ---- gather (§2: g-weighted average of the grid fields) ----
+        R fn[3], ig;
+        int sh[3];
         unsigned clamp = 0;
-        push_move<R, ORDER, DIM>(a, u, E, B, f, fn, sh, ig, clamp);
-        // offsets from the nearest node (TSC) or in the cell (CIC), before
-        // and after, and how far that node or cell moved
+        {
+          GatherAxis<R, ORDER> gx, gy, gz;
+          gx.set(f[0], EC);
+          gy.set(f[1], EC);
+          gz.set(f[2], EC);
+#ifdef PIC_CHECKED
+          {
+            // every gather stencil inside the E/B window (checked builds)
+            const GatherAxis<R, ORDER> *ga[3] = {&gx, &gy, &gz};
+            constexpr int EW[3] = {G::EX, G::EY, G::EZ};
+            bool ok = true;
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) {
+              const int lo = l[d] + (ga[d]->relp < ga[d]->reld ? ga[d]->relp : ga[d]->reld) + G::O;
+              const int hi = l[d] + (ga[d]->relp > ga[d]->reld ? ga[d]->relp : ga[d]->reld) + G::O + NS - 1;
+              ok = ok && lo >= 0 && hi < EW[d];
+            }
+            if (!PIC_CHECK(ok, a.ctr)) {
+              tag = kTagIdle;
+              break;  // leaves the particle as it was
+            }
+          }
+#endif
+          const int xp = l[0] + gx.relp + G::O, xd = l[0] + gx.reld + G::O;
+          const int yp = (l[1] + gy.relp + G::O) * SY, yd = (l[1] + gy.reld + G::O) * SY;
+          const int zp = DIM == 3 ? (l[2] + gz.relp + G::O) * SZ : 0;
+          const int zd = DIM == 3 ? (l[2] + gz.reld + G::O) * SZ : 0;
+          R E[3], B[3];
+          E[0] = gsum<R, NS, DIM, SY, SZ>(sF + 0 * G::EN + xd + yp + zp, gx.wd, gy.wp, gz.wp);
+          E[1] = gsum<R, NS, DIM, SY, SZ>(sF + 1 * G::EN + xp + yd + zp, gx.wp, gy.wd, gz.wp);
+          E[2] = gsum<R, NS, DIM, SY, SZ>(sF + 2 * G::EN + xp + yp + zd, gx.wp, gy.wp, gz.wd);
+          B[0] = gsum<R, NS, DIM, SY, SZ>(sF + 3 * G::EN + xp + yd + zd, gx.wp, gy.wd, gz.wd);
+          B[1] = gsum<R, NS, DIM, SY, SZ>(sF + 4 * G::EN + xd + yp + zd, gx.wd, gy.wp, gz.wd);
+          B[2] = gsum<R, NS, DIM, SY, SZ>(sF + 5 * G::EN + xd + yd + zp, gx.wd, gy.wd, gz.wp);
+          // ---- Boris push (§2 eq. 3) and leap-frog move ----
+          push_move<R, ORDER, DIM>(a, u, E, B, f, fn, sh, ig, clamp);
+        }
+        // offsets from the nearest node (TSC) or in the cell (CIC), before and
+        // after, and how far that node or cell moved
+        R d0[3], d1[3];
+        int k[3] = {0, 0, 0}, key[3] = {0, 0, 0};
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
           if (d >= DIM) {
@@ -771,317 +853,374 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
           k[d] = sh[d] + h1 - h0;
           key[d] = l[d] + h0 + G::D;
           constexpr int KK[3] = {G::KX, G::KY, G::KZ};
-          inw = inw && key[d] + k[d] >= 0 && key[d] + k[d] < KK[d];
+          inw = inw && (unsigned)(key[d] + k[d]) < (unsigned)KK[d];
         }
-        if (inw) my_clamp += clamp;  // (the escape kernel counts its own)
-      }
-      if (!inw) {
-        // defer to k_push_escaped (state left untouched)
-        a.cell[p] = c | kEscFlag;
-        const unsigned act = __activemask();
-        const int leader = __ffs(act) - 1;
-        unsigned long long slot = 0;
-        if (lane == leader) slot = atomicAdd(a.esc_count, (unsigned long long)__popc(act));
-        slot = __shfl_sync(act, slot, leader) + __popc(act & ((1u << lane) - 1u));
-        a.esc_list[slot] = (int32_t)p;
-        break;
-      }
+        if (!inw) break;
+        tag = kTagIdle;
+        my_clamp += clamp;  // (the escape kernel counts its own)
 
-      // ---- the new state ----
-      int nc = -1;  // removed at an absorbing wall after depositing its move
-      if (outside_walls<R>(a.absorb, ci[0] + sh[0], fn[0], a.n[0])) {
-        ++my_absorbed;
-      } else {
-        nc = c;
-        const int i0 = ci[0] + sh[0];
-        nc += sh[0] + (i0 < 0 ? a.n[0] : (i0 >= a.n[0] ? -a.n[0] : 0));
-        const int i1 = ci[1] + sh[1];
-        nc += (sh[1] + (i1 < 0 ? a.n[1] : (i1 >= a.n[1] ? -a.n[1] : 0))) * a.n[0];
-        if (DIM == 3) {
-          const int i2 = ci[2] + sh[2];
-          nc += (sh[2] + (i2 < 0 ? a.n[2] : (i2 >= a.n[2] ? -a.n[2] : 0))) * a.n[0] * a.n[1];
+        // ---- the new state ----
+        int nc = c + sh[0] + a.n[0] * (DIM == 3 ? sh[1] + a.n[1] * sh[2] : sh[1]);
+        if (edge) {
+          int i[3];
+#pragma unroll
+          for (int d = 0; d < DIM; ++d) {
+            i[d] = ci[d] + sh[d];
+            if (i[d] < 0) i[d] = a.n[d] - 1;
+            if (i[d] >= a.n[d]) i[d] = 0;
+          }
+          nc = DIM == 3 ? i[0] + a.n[0] * (i[1] + a.n[1] * i[2]) : i[0] + a.n[0] * i[1];
+        }
+        if (outside_walls<R>(a.absorb, ci[0] + sh[0], fn[0], a.n[0])) {
+          nc = -1;  // removed at an absorbing wall after depositing its move
+          ++my_absorbed;
+        }
+        a.cell[p] = nc;
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) a.off[d][p] = fn[d];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) a.u[d][p] = u[d];
+
+        // ---- the deposit job ----
+        // A particle that keeps its place (and, in 2D3V, has vz = 0) or has no
+        // weight deposits nothing (a cold target before the pulse reaches it).
+        const R vz = u[2] * ig;
+        const bool change = (k[0] | k[1] | k[2]) != 0;
+        if (w == R(0) ||
+            !(change || d0[0] != d1[0] || d0[1] != d1[1] || (DIM == 3 ? d0[2] != d1[2] : vz != R(0))))
+          break;
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+          sJob[d * CAP + s] = d0[d];
+          sJob[(DIM + d) * CAP + s] = d1[d];
+        }
+        if (DIM == 2) sJob[4 * CAP + s] = vz;  // (the weight stays in its place)
+        const uint32_t group = (uint32_t)(key[0] + G::KX * (key[1] + G::KY * key[2]));
+        uint32_t sort_key = group;
+        tag = group;
+        if (change) {
+          sort_key = G::KN - 1 + (k[0] != 0) + 2 * (k[1] != 0) + 4 * (k[2] != 0);
+          tag |= (uint32_t)((k[0] + 1) << 10 | (k[1] + 1) << 12 | (k[2] + 1) << 14) | kTagChange;
+        }
+        tag |= atomicAdd(&sCount[sort_key], 1u) << 16;
+        // |v| <= min(1, |vx| + |vy| + |vz|)
+        if (sizeof(R) == 4)
+          my_q += fabsf((float)w) *
+                  fminf(1.f, (fabsf((float)u[0]) + fabsf((float)u[1]) + fabsf((float)u[2])) * (float)ig);
+      } while (0);
+      sTag[s] = tag;
+    }
+    if (sizeof(R) == 4) {
+      for (int o = 16; o > 0; o >>= 1) my_q += __shfl_xor_sync(0xffffffffu, my_q, o);
+      if (lane == 0 && my_q > 0.f) atomicAdd(&s_q, my_q);
+    }
+    if (my_clamp) atomicAdd(&s_clamp, my_clamp);
+    if (my_absorbed) atomicAdd(&s_absorbed, my_absorbed);
+    __syncthreads();
+    // the next item, read meanwhile
+    int t_next = -1, n_next = 0;
+    int64_t pb_next = 0;
+    if (tid == 0) {
+      if (s_clamp) atomicAdd(&a.ctr->clamped, (unsigned long long)s_clamp);
+      if (s_absorbed) atomicAdd(&a.ctr->absorbed, (unsigned long long)s_absorbed);
+      const unsigned long long next = taken + gridDim.x;
+      if (next < (unsigned long long)a.nwork) {
+        t_next = a.work_tile[next];
+        if (t_next >= 0) {
+          pb_next = a.work_pb[next];
+          n_next = a.work_n[next];
         }
       }
-      a.cell[p] = nc;
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) a.off[d][p] = fn[d];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) a.u[d][p] = u[d];
+    }
 
-      // ---- the deposit job ----
-      // A particle that keeps its place (and, in 2D3V, has vz = 0) or has no
-      // weight deposits nothing (a cold target before the pulse reaches it).
-      const R vz = u[2] * ig;
-      const bool change = (k[0] | k[1] | k[2]) != 0;
-      if (w == R(0) || !(change || d0[0] != d1[0] || d0[1] != d1[1] || (DIM == 3 ? d0[2] != d1[2] : vz != R(0)))) break;
-      sJob[0 * CAP + s] = d0[0];
-      sJob[1 * CAP + s] = d0[1];
-      sJob[2 * CAP + s] = d1[0];
-      sJob[3 * CAP + s] = d1[1];
-      sJob[4 * CAP + s] = w;
-      if (DIM == 3) {
-        sJob[5 * CAP + s] = d0[2];
-        sJob[(L::NJ - 1) * CAP + s] = d1[2];
-      } else {
-        sJob[5 * CAP + s] = vz;
-      }
-      const uint32_t group = (uint32_t)(key[0] + G::KX * (key[1] + G::KY * key[2]));
-      uint32_t sort_key = group;
-      tag = group;
-      if (change) {
-        sort_key = G::KN - 1 + (k[0] != 0) + 2 * (k[1] != 0) + 4 * (k[2] != 0);
-        tag |= (uint32_t)((k[0] + 1) << 10 | (k[1] + 1) << 12 | (k[2] + 1) << 14) | kTagChange;
-      }
-      tag |= atomicAdd(&sCount[sort_key], 1u) << 16;
-      if (sizeof(R) == 4)
-        my_q += fabsf((float)w) * fminf(1.f, sqrtf((float)(u[0] * u[0] + u[1] * u[1] + u[2] * u[2])));
-    } while (0);
-    sTag[s] = tag;
-  }
-  if (sizeof(R) == 4) {
-    for (int o = 16; o > 0; o >>= 1) my_q += __shfl_xor_sync(0xffffffffu, my_q, o);
-    if (lane == 0 && my_q > 0.f) atomicAdd(&s_q, my_q);
-  }
-  if (my_clamp) atomicAdd(&s_clamp, my_clamp);
-  if (my_absorbed) atomicAdd(&s_absorbed, my_absorbed);
-  __syncthreads();
-  if (tid == 0) {
-    if (s_clamp) atomicAdd(&a.ctr->clamped, (unsigned long long)s_clamp);
-    if (s_absorbed) atomicAdd(&a.ctr->absorbed, (unsigned long long)s_absorbed);
-  }
-
-  // ---- counting sort of the jobs: key starts, and the deposit tasks.  Each
-  // thread takes KPT consecutive keys; one block scan carries the job count
-  // and the task counts of every length class.
-  constexpr int KPT = (G::KT + kThreads - 1) / kThreads;
-  uint32_t cnt[KPT], sum = 0;
-  unsigned long long cls = 0;
-#pragma unroll
-  for (int i = 0; i < KPT; ++i) {
-    const int q = tid * KPT + i;
-    cnt[i] = q < G::KT ? sCount[q] : 0u;
-    sum += cnt[i];
-    if (q < G::KN) cls += task_counts(cnt[i]);
-  }
-  const uint32_t sum0 = sum;
-  const unsigned long long cls0 = cls;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t v = __shfl_up_sync(0xffffffffu, sum, o);
-    const unsigned long long x = __shfl_up_sync(0xffffffffu, cls, o);
-    if (lane >= o) {
-      sum += v;
-      cls += x;
-    }
-  }
-  if (lane == 31) {
-    s_wsum[warp] = sum;
-    s_wcls[warp] = cls;
-  }
-  // the J window replaces E and B
-  for (int q = tid; q < (int)(L::kWin / 16); q += kThreads) reinterpret_cast<int4 *>(smem_raw)[q] = int4{0, 0, 0, 0};
-  __syncthreads();
-  uint32_t at = sum - sum0, njob = 0;
-  unsigned long long pos = cls - cls0, all = 0;
-#pragma unroll
-  for (int i = 0; i < kThreads / 32; ++i) {
-    const uint32_t v = s_wsum[i];
-    const unsigned long long x = s_wcls[i];
-    if (i < warp) {
-      at += v;
-      pos += x;
-    }
-    njob += v;
-    all += x;
-  }
-  if (njob == 0) return;  // nothing moved: no current
-  int ntask = 0;
-  {
-    int first[6];  // this thread's next task of each class; a class follows the longer ones
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      first[q] = ntask + (int)((pos >> (10 * q)) & 1023u);
-      ntask += (int)((all >> (10 * q)) & 1023u);
-    }
+    // ---- counting sort of the jobs: key starts, and the deposit tasks.  Each
+    // thread takes KPT consecutive keys; one block scan carries the job count
+    // and the task counts of every length class.
+    constexpr int KPT = (G::KT + kThreads - 1) / kThreads;
+    uint32_t cnt[KPT], sum = 0;
+    unsigned long long cls = 0;
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
       const int q = tid * KPT + i;
-      if (q <= G::KT) sStart[q] = (uint16_t)at;
-      if (q < G::KN && cnt[i] > 0) {
-        const unsigned full = cnt[i] / kTaskLen, rest = cnt[i] % kTaskLen;
-        for (unsigned j = 0; j < full; ++j) sTask[first[0]++] = (uint16_t)((at + j * kTaskLen) | (kTaskLen - 1) << 12);
-        if (rest) {
-          const int cl = task_class(rest);
-          int where = 0;
+      cnt[i] = q < G::KT ? sCount[q] : 0u;
+      sum += cnt[i];
+      if (q < G::KN) cls += task_counts<L::TASK>(cnt[i]);
+    }
+    const uint32_t sum0 = sum;
+    const unsigned long long cls0 = cls;
 #pragma unroll
-          for (int z = 1; z < 6; ++z)
-            if (z == cl) where = first[z]++;
-          sTask[where] = (uint16_t)((at + full * kTaskLen) | (rest - 1) << 12);
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, sum, o);
+      const unsigned long long x = __shfl_up_sync(0xffffffffu, cls, o);
+      if (lane >= o) {
+        sum += v;
+        cls += x;
+      }
+    }
+    if (lane == 31) {
+      s_wsum[warp] = sum;
+      s_wcls[warp] = cls;
+    }
+    // the J window replaces E and B
+    for (int q = tid; q < (int)(L::kWin / 16); q += kThreads) reinterpret_cast<int4 *>(smem_raw)[q] = int4{0, 0, 0, 0};
+    __syncthreads();
+    // the warps' sums, scanned by the first lanes of every warp
+    uint32_t wv = s_wsum[lane % (kThreads / 32)];
+    unsigned long long wx = s_wcls[lane % (kThreads / 32)];
+#pragma unroll
+    for (int o = 1; o < kThreads / 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, wv, o);
+      const unsigned long long x = __shfl_up_sync(0xffffffffu, wx, o);
+      if (lane >= o) {
+        wv += v;
+        wx += x;
+      }
+    }
+    const uint32_t njob = __shfl_sync(0xffffffffu, wv, kThreads / 32 - 1);
+    const unsigned long long all = __shfl_sync(0xffffffffu, wx, kThreads / 32 - 1);
+    const int below = warp > 0 ? warp - 1 : 0;
+    const uint32_t vb = __shfl_sync(0xffffffffu, wv, below);
+    const unsigned long long xb = __shfl_sync(0xffffffffu, wx, below);
+    uint32_t at = sum - sum0 + (warp > 0 ? vb : 0u);
+    const unsigned long long pos = cls - cls0 + (warp > 0 ? xb : 0ull);
+    int ntask = 0;
+    {
+      int first[kClasses];  // this thread's next task of each class; a class follows the longer ones
+#pragma unroll
+      for (int q = 0; q < kClasses; ++q) {
+        first[q] = ntask + (int)((pos >> (10 * q)) & 1023u);
+        ntask += (int)((all >> (10 * q)) & 1023u);
+      }
+#pragma unroll
+      for (int i = 0; i < KPT; ++i) {
+        const int q = tid * KPT + i;
+        if (q <= G::KT) sStart[q] = (uint16_t)at;
+        if (q < G::KN) {
+          unsigned from = at, left = cnt[i];
+          for (; left >= L::TASK; left -= L::TASK, from += L::TASK)
+            sTask[first[0]++] = (uint16_t)(from | (L::TASK - 1) << 12);
+          if (left) {
+            const int cl = task_class<L::TASK>(left);
+            int where = 0;
+#pragma unroll
+            for (int z = 0; z < kClasses; ++z)
+              if (z == cl) where = first[z]++;
+            sTask[where] = (uint16_t)(from | (left - 1) << 12);
+          }
+        }
+        at += cnt[i];
+      }
+    }
+    if (tid == 0) {
+      s_tile = t_next;
+      s_pb = pb_next;
+      s_n = n_next;
+    }
+    __syncthreads();
+    // every thread takes part in every pass: a warp appends the particles that
+    // are left to k_push_escaped (state untouched) with one atomic
+    for (int s0 = 0; s0 < n; s0 += kThreads) {
+      const int s = s0 + tid;
+      const uint32_t tag = s < n ? sTag[s] : kTagIdle;
+      const unsigned esc = __ballot_sync(0xffffffffu, tag == kTagEscape);
+      if (esc) {
+        unsigned long long slot = 0;
+        if (lane == 0) slot = atomicAdd(a.esc_count, (unsigned long long)__popc(esc));
+        slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(esc & ((1u << lane) - 1u));
+        if (tag == kTagEscape && PIC_CHECK(slot < (unsigned long long)a.slots, a.ctr)) {
+          a.cell[pb + s] |= kEscFlag;
+          a.esc_list[slot] = (int32_t)(pb + s);
         }
       }
-      at += cnt[i];
+      if (tag & kTagIdle) continue;
+      uint32_t sort_key = tag & 1023u;
+      if (tag & kTagChange)
+        sort_key = G::KN - 1 + (((tag >> 10) & 3u) != 1u) + 2 * (((tag >> 12) & 3u) != 1u) +
+                   4 * (((tag >> 14) & 3u) != 1u);
+      const uint32_t q = sStart[sort_key] + ((tag >> 16) & 4095u);
+      if (!PIC_CHECK(q < (uint32_t)CAP, a.ctr)) continue;
+      sOrder[q] = (uint16_t)s;
     }
-  }
-  __syncthreads();
-  for (int s = tid; s < n; s += kThreads) {
-    const uint32_t tag = sTag[s];
-    if (tag & kTagIdle) continue;
-    uint32_t sort_key = tag & 1023u;
-    if (tag & kTagChange)
-      sort_key = G::KN - 1 + (((tag >> 10) & 3u) != 1u) + 2 * (((tag >> 12) & 3u) != 1u) + 4 * (((tag >> 14) & 3u) != 1u);
-    const uint32_t q = sStart[sort_key] + ((tag >> 16) & 4095u);
-    if (!PIC_CHECK(q < (uint32_t)CAP, a.ctr)) continue;
-    sOrder[q] = (uint16_t)s;
-  }
-  WinAcc<R> acc;
-  acc.w = reinterpret_cast<decltype(acc.w)>(smem_raw);
-  acc.jn = sizeof(R) == 4 ? G::JS : G::EN;
-  acc.dummy = G::EN + lane;
-  acc.scale = acc.unit = R(1);
-  if constexpr (sizeof(R) == 4) acc.set_scale(1.01f * a.qabs * s_q);  // 1.01: room for the FP32 rounding of the sum
-  __syncthreads();
+    WinAcc<R> acc;
+    acc.w = reinterpret_cast<decltype(acc.w)>(smem_raw);
+    acc.jn = sizeof(R) == 4 ? G::JS : G::EN;
+    acc.dummy = G::EN + lane;
+    acc.scale = acc.unit = R(1);
+    if constexpr (sizeof(R) == 4) acc.set_scale(1.01f * a.qabs * s_q);  // 1.01: room for the FP32 rounding of the sum
+    __syncthreads();
 
-  // ---- deposit: warps take the next 32 tasks, longest first, then the next
-  // 32 particles whose support changes (in order of the axes that do)
-  const int ntask32 = (ntask + 31) & ~31, nset = sStart[G::KN];
-  const int nunit = ntask32 + (int)njob - nset;
-  if (tid == 0 && (int)njob > nset) atomicAdd(a.q_jobs, (unsigned long long)((int)njob - nset));
-  const R jf0 = a.jfac[0] * acc.scale, jf1 = a.jfac[1] * acc.scale, jf2 = a.jfac[2] * acc.scale;
-  const R jz = a.qz * acc.scale;  // 2D3V
-  for (;;) {
-    unsigned base = 0;
-    if (lane == 0) base = atomicAdd(&s_next, 32u);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if ((int)base >= nunit) break;
-    const int unit = (int)base + lane;
-    if ((int)base < ntask32) {
-      if (unit >= ntask) continue;
-      const unsigned tk = sTask[unit];
-      int j = tk & 4095u;
-      const int je = j + (int)(tk >> 12) + 1;
-      int s = sOrder[j];
-      const uint32_t group = sTag[s] & 1023u;
-      const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
-      // the stencil's first node: one below the nearest node (TSC), the cell's (CIC)
-      constexpr int o = ORDER == 2 ? 0 : 1;
-      const int jb = (kx + o) + (ky + o) * SY + (DIM == 3 ? (kz + o) * SZ : 0);
-      GroupSum<R, DIM, ORDER> g;
-      g.clear();
-      while (true) {
-        SettledAxis<R, ORDER> X, Y, Z;
-        X.set(sJob[s], sJob[2 * CAP + s]);
-        Y.set(sJob[CAP + s], sJob[3 * CAP + s]);
-        const R w = sJob[4 * CAP + s];
-        R qwvz = R(0);
-        if (DIM == 3) Z.set(sJob[5 * CAP + s], sJob[(L::NJ - 1) * CAP + s]);
-        else qwvz = jz * w * sJob[5 * CAP + s];
-        if (++j < je) s = sOrder[j];
-        g.add(X, Y, Z, jf0 * w, jf1 * w, jf2 * w, qwvz);
-        if (j >= je) break;
-      }
-      GroupSink<R, sizeof(R) == 4 ? G::JS : G::EN> out;
-      if constexpr (sizeof(R) == 4) out.sb = (unsigned)__cvta_generic_to_shared(acc.w) + 4u * (unsigned)jb;
-      else out.w = acc.w + jb;
-      g.template flush<SY, SZ>(out);
-    } else {
-      if (unit >= nunit) continue;
-      const int s = sOrder[nset + unit - ntask32];
-      const uint32_t tag = sTag[s];
-      const int group = tag & 1023u;
-      const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
-      DepositAxis<R, ORDER> X, Y, Z;
-      X.set_nodes(sJob[s], (int)((tag >> 10) & 3u) - 1, sJob[2 * CAP + s]);
-      Y.set_nodes(sJob[CAP + s], (int)((tag >> 12) & 3u) - 1, sJob[3 * CAP + s]);
-      const R w = sJob[4 * CAP + s];
-      R qwvz = R(0);
-      if (DIM == 3) {
-        Z.set_nodes(sJob[5 * CAP + s], (int)((tag >> 14) & 3u) - 1, sJob[(L::NJ - 1) * CAP + s]);
+    // ---- deposit: warps take the next 32 particles whose support changes (the
+    // longest work, in order of the axes that do), then the next 32 tasks,
+    // longest first
+    const int nset = sStart[G::KN], nchg = (int)njob - nset, nchg32 = (nchg + 31) & ~31;
+    const int nunit = nchg32 + ntask;
+    if (tid == 0 && nchg > 0) atomicAdd(a.q_jobs, (unsigned long long)nchg);
+    const R jf0 = a.jfac[0] * acc.scale, jf1 = a.jfac[1] * acc.scale, jf2 = a.jfac[2] * acc.scale;
+    const R jz = a.qz * acc.scale;  // 2D3V
+    for (;;) {
+      unsigned base = 0;
+      if (lane == 0) base = atomicAdd(&s_next, 32u);
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if ((int)base >= nunit) break;
+      const int unit = (int)base + lane;
+      if ((int)base >= nchg32) {
+        if (unit >= nunit) continue;
+        const unsigned tk = sTask[unit - nchg32];
+        int j = tk & 4095u;
+        const int je = j + (int)(tk >> 12) + 1;
+        if constexpr (sizeof(R) == 4 && DIM == 2) {
+          // The job order within a group depends on the order in which warps
+          // reached its counter.  FP32 2D runs (those with an adjoint, whose
+          // segments are run twice) sum a task in the order of the old x
+          // offsets instead, so that a group of one task has one sum.
+          const int len = je - j;
+          if (len > 1) {
+            uint32_t v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const uint32_t o = i < len ? sOrder[j + i] : 0u;
+              v[i] = i < len ? (__float_as_uint((float)sJob[o] + 1.5f) << 9 & 0xfffff000u) | o : 0xffffffffu;
+            }
+            sort8(v);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (i < len) sOrder[j + i] = (uint16_t)(v[i] & 4095u);
+          }
+        }
+        int s = sOrder[j];
+        const uint32_t group = sTag[s] & 1023u;
+        const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
+        // the stencil's first node: one below the nearest node (TSC), the cell's (CIC)
+        constexpr int o = ORDER == 2 ? 0 : 1;
+        const int jb = (kx + o) + (ky + o) * SY + (DIM == 3 ? (kz + o) * SZ : 0);
+        GroupSum<R, DIM, ORDER> g;
+        g.clear();
+        while (true) {
+          SettledAxis<R, ORDER> X, Y, Z;
+          X.set(sJob[s], sJob[DIM * CAP + s]);
+          Y.set(sJob[CAP + s], sJob[(DIM + 1) * CAP + s]);
+          const R w = sJob[(L::NJ - 1) * CAP + s];
+          R qwvz = R(0);
+          if (DIM == 3) Z.set(sJob[2 * CAP + s], sJob[5 * CAP + s]);
+          else qwvz = jz * w * sJob[4 * CAP + s];
+          if (++j < je) s = sOrder[j];
+          g.add(X, Y, Z, jf0 * w, jf1 * w, jf2 * w, qwvz);
+          if (j >= je) break;
+        }
+        GroupSink<R, sizeof(R) == 4 ? G::JS : G::EN> out;
+        if constexpr (sizeof(R) == 4) out.sb = (unsigned)__cvta_generic_to_shared(acc.w) + 4u * (unsigned)jb;
+        else out.w = acc.w + jb;
+        g.template flush<SY, SZ>(out);
       } else {
-        Z.zero();
-        qwvz = jz * w * sJob[5 * CAP + s];
-      }
-      const int bx = kx + 1 + X.rel, by = ky + 1 + Y.rel, bz = DIM == 3 ? kz + 1 + Z.rel : 0;
+        // (lanes past the last one add nothing, so that the whole warp votes below)
+        bool have = unit < nchg;
+        const int s = sOrder[nset + (have ? unit : (int)base)];
+        const uint32_t tag = sTag[s];
+        const int group = tag & 1023u;
+        const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
+        DepositAxis<R, ORDER> X, Y, Z;
+        X.set_nodes(sJob[s], (int)((tag >> 10) & 3u) - 1, sJob[DIM * CAP + s]);
+        Y.set_nodes(sJob[CAP + s], (int)((tag >> 12) & 3u) - 1, sJob[(DIM + 1) * CAP + s]);
+        R w = sJob[(L::NJ - 1) * CAP + s];
+        R qwvz = R(0);
+        if (DIM == 3) {
+          Z.set_nodes(sJob[2 * CAP + s], (int)((tag >> 14) & 3u) - 1, sJob[5 * CAP + s]);
+        } else {
+          Z.zero();
+          qwvz = jz * w * sJob[4 * CAP + s];
+        }
+        const int bx = kx + 1 + X.rel, by = ky + 1 + Y.rel, bz = DIM == 3 ? kz + 1 + Z.rel : 0;
 #ifdef PIC_CHECKED
-      {
-        // the nodes that receive a current inside the window (checked builds)
-        const DepositAxis<R, ORDER> *da[3] = {&X, &Y, &Z};
-        const int b0[3] = {bx, by, bz};
-        constexpr int JW[3] = {G::EX, G::EY, G::EZ};
-        bool ok = true;
+        {
+          // the nodes that receive a current inside the window (checked builds)
+          const DepositAxis<R, ORDER> *da[3] = {&X, &Y, &Z};
+          const int b0[3] = {bx, by, bz};
+          constexpr int JW[3] = {G::EX, G::EY, G::EZ};
+          bool ok = true;
 #pragma unroll
-        for (int d = 0; d < DIM; ++d) {
-          const bool last = da[d]->S0[G::NW - 1] != R(0) || da[d]->DS[G::NW - 1] != R(0);
-          ok = ok && b0[d] >= 0 && b0[d] + G::NW - 2 + (last ? 1 : 0) < JW[d];
+          for (int d = 0; d < DIM; ++d) {
+            const bool last = da[d]->S0[G::NW - 1] != R(0) || da[d]->DS[G::NW - 1] != R(0);
+            ok = ok && b0[d] >= 0 && b0[d] + G::NW - 2 + (last ? 1 : 0) < JW[d];
+          }
+          if (!PIC_CHECK(ok, a.ctr)) have = false;
         }
-        if (!PIC_CHECK(ok, a.ctr)) continue;
-      }
 #endif
-      // does some lane of this warp use the last stencil node of an axis?
-      const unsigned act = __activemask();
-      const bool lx = __any_sync(act, X.S0[G::NW - 1] != R(0) || X.DS[G::NW - 1] != R(0));
-      const bool ly = __any_sync(act, Y.S0[G::NW - 1] != R(0) || Y.DS[G::NW - 1] != R(0));
-      const bool lz = DIM == 3 && __any_sync(act, Z.S0[G::NW - 1] != R(0) || Z.DS[G::NW - 1] != R(0));
-      deposit_win<R, ORDER, DIM, SY, SZ>(acc, bx + by * SY + bz * SZ, X, Y, Z, jf0 * w, jf1 * w, jf2 * w, qwvz, lx, ly,
-                                         lz);
+        if (!have) w = qwvz = R(0);
+        // does some lane of this warp use the last stencil node of an axis?
+        const bool lx = __any_sync(0xffffffffu, X.S0[G::NW - 1] != R(0) || X.DS[G::NW - 1] != R(0));
+        const bool ly = __any_sync(0xffffffffu, Y.S0[G::NW - 1] != R(0) || Y.DS[G::NW - 1] != R(0));
+        const bool lz = DIM == 3 && __any_sync(0xffffffffu, Z.S0[G::NW - 1] != R(0) || Z.DS[G::NW - 1] != R(0));
+        deposit_win<R, ORDER, DIM, SY, SZ>(acc, bx + by * SY + bz * SZ, X, Y, Z, jf0 * w, jf1 * w, jf2 * w, qwvz, lx, ly,
+                                           lz);
+      }
     }
-  }
-  __syncthreads();
+    __syncthreads();
 
-  // ---- flush the J window into global J ----
-  if (sizeof(R) == 4 && (a.n[0] & 3) == 0) {
-    // FP32 with rows of a multiple of four cells: runs of four nodes along x
-    // aligned in global memory, one vector reduction each (every element
-    // added atomically); a run reaching past the window's x ends adds zeros
-    // there.  A run never straddles the periodic seam.
-    const int xs = t0[0] - G::O;               // the window's first node, global x (unwrapped)
-    const int a0 = xs - (((xs % 4) + 4) & 3);  // the multiple of 4 at or below it
-    constexpr int NG = (G::EX + 6) / 4;        // runs per window row (the last may start past it)
-    for (int q = tid; q < NG * G::EY * G::EZ; q += kThreads) {
-      const int m = q % NG, row = q / NG;
-      const int y = row % G::EY, z = row / G::EY;
-      const int wx0 = a0 + 4 * m - xs;  // window x of the run's first node
-      if (wx0 >= G::EX) continue;
-      const int gi = wrap_near(a0 + 4 * m, a.n[0]);
-      const int gj = wrap_near(t0[1] - G::O + y, a.n[1]);
-      const int gk = DIM == 3 ? wrap_near(t0[2] - G::O + z, a.n[2]) : 0;
-      const int64_t g = gi + (int64_t)a.n[0] * (gj + (int64_t)a.n[1] * gk);
-      const int wrow = z * SZ + y * SY;
+    // ---- the next item's particles start on their way (their places are free)
+    t = s_tile;
+    pb = s_pb;
+    n = s_n;
+    if (t >= 0) stage_particles(pb, n);
+
+    // ---- flush the J window into global J (nothing moved: no current) ----
+    if (njob > 0) {
+    if (sizeof(R) == 4 && (a.n[0] & 3) == 0) {
+      // FP32 with rows of a multiple of four cells: runs of four nodes along x
+      // aligned in global memory, one vector reduction each (every element
+      // added atomically); a run reaching past the window's x ends adds zeros
+      // there.  A run never straddles the periodic seam.
+      const int xs = t0[0] - G::O;               // the window's first node, global x (unwrapped)
+      const int a0 = xs - (((xs % 4) + 4) & 3);  // the multiple of 4 at or below it
+      constexpr int NG = (G::EX + 6) / 4;        // runs per window row (the last may start past it)
+      for (int q = tid; q < NG * G::EY * G::EZ; q += kThreads) {
+        const int m = q % NG, row = q / NG;
+        const int y = row % G::EY, z = row / G::EY;
+        const int wx0 = a0 + 4 * m - xs;  // window x of the run's first node
+        if (wx0 >= G::EX) continue;
+        const int gi = wrap_near(a0 + 4 * m, a.n[0]);
+        const int gj = wrap_near(t0[1] - G::O + y, a.n[1]);
+        const int gk = DIM == 3 ? wrap_near(t0[2] - G::O + z, a.n[2]) : 0;
+        const int g = gi + a.n[0] * (gj + a.n[1] * gk);  // (cells stay below 2^30)
+        const int wrow = z * SZ + y * SY;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float v[4];
+        for (int c = 0; c < 3; ++c) {
+          float v[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int wx = wx0 + e;
-          v[e] = (wx >= 0 && wx < G::EX) ? (float)acc.get(c, wrow + wx) : 0.f;
+          for (int e = 0; e < 4; ++e) {
+            const int wx = wx0 + e;
+            v[e] = (wx >= 0 && wx < G::EX) ? (float)acc.get(c, wrow + wx) : 0.f;
+          }
+          if (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f)
+            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a.J[c] + g), "f"(v[0]), "f"(v[1]),
+                         "f"(v[2]), "f"(v[3])
+                         : "memory");
         }
-        if (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f)
-          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a.J[c] + g), "f"(v[0]), "f"(v[1]),
-                       "f"(v[2]), "f"(v[3])
-                       : "memory");
       }
-    }
-  } else {
-    for (int q = tid; q < G::EN; q += kThreads) {
-      const int x = q % G::EX;
-      const int y = (q / G::EX) % G::EY;
-      const int z = q / SZ;
-      const int gi = wrap_near(t0[0] - G::O + x, a.n[0]);
-      const int gj = wrap_near(t0[1] - G::O + y, a.n[1]);
-      const int gk = DIM == 3 ? wrap_near(t0[2] - G::O + z, a.n[2]) : 0;
-      const int64_t g = gi + (int64_t)a.n[0] * (gj + (int64_t)a.n[1] * gk);
+    } else {
+      for (int q = tid; q < G::EN; q += kThreads) {
+        const int x = q % G::EX;
+        const int y = (q / G::EX) % G::EY;
+        const int z = q / SZ;
+        const int gi = wrap_near(t0[0] - G::O + x, a.n[0]);
+        const int gj = wrap_near(t0[1] - G::O + y, a.n[1]);
+        const int gk = DIM == 3 ? wrap_near(t0[2] - G::O + z, a.n[2]) : 0;
+        const int g = gi + a.n[0] * (gj + a.n[1] * gk);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const R v = acc.get(c, q);
-        if (v != R(0)) atomicAdd(a.J[c] + g, v);
+        for (int c = 0; c < 3; ++c) {
+          const R v = acc.get(c, q);
+          if (v != R(0)) atomicAdd(a.J[c] + g, v);
+        }
       }
     }
+    }
+    __syncthreads();  // the window is free again
   }
 }
 
 // Particles deferred by the tile kernel: the same gather / Boris / move /
 // Esirkepov arithmetic, reading E, B from and adding J to global memory with
 // periodic index wrapping.
-template <class R, int DIM, int ORDER>
+template <class R, int DIM, int ORDER, bool EC>
 __global__ void __launch_bounds__(kThreads) k_push_escaped(const PushArgs<R> a) {
   constexpr int NS = ORDER + 1;
   constexpr int NW = ORDER + 2;
@@ -1090,7 +1229,9 @@ __global__ void __launch_bounds__(kThreads) k_push_escaped(const PushArgs<R> a) 
   for (unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; q < nesc;
        q += (unsigned long long)gridDim.x * blockDim.x) {
     const int64_t p = a.esc_list[q];
+    if (!PIC_CHECK(p >= 0 && p < a.slots, a.ctr)) continue;
     const int c = a.cell[p] & ~kEscFlag;
+    if (!PIC_CHECK(c >= 0 && c / a.n[0] / a.n[1] < a.n[2], a.ctr)) continue;
     int ci[3];
     ci[0] = c % a.n[0];
     ci[1] = (c / a.n[0]) % a.n[1];
@@ -1103,7 +1244,7 @@ __global__ void __launch_bounds__(kThreads) k_push_escaped(const PushArgs<R> a) 
     }
     GatherAxis<R, ORDER> ga[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) ga[d].set(f[d], a.ec);
+    for (int d = 0; d < 3; ++d) ga[d].set(f[d], EC);
     const int64_t sy = a.n[0], sz = (int64_t)a.n[0] * a.n[1];
     auto fetch = [&](const R *F, const bool dual[3]) {
       R acc = R(0);
@@ -1201,15 +1342,18 @@ __global__ void __launch_bounds__(kThreads) k_push_escaped(const PushArgs<R> a) 
   if (blockIdx.x == 0 && threadIdx.x == 0 && nesc) atomicAdd(&a.ctr->escaped, nesc);
 }
 
-template <class R, int DIM, int ORDER>
+template <class R, int DIM, int ORDER, bool EC>
 cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
-                     const int64_t *tile_start, const WorkSplit &ws, int32_t *esc_list, unsigned long long *esc_count,
-                     double q, double m, Counters *ctr, cudaStream_t st, int *nlaunch) {
-  if (ws.chunk > Lay<R, DIM, ORDER>::CAP) return cudaErrorInvalidValue;
+                     const WorkSplit &ws, int32_t *esc_list, unsigned long long *esc_count, double q, double m,
+                     Counters *ctr, cudaStream_t st, int *nlaunch) {
+  if (ws.chunk > Lay<R, DIM, ORDER>::CAP || ws.nwork > 0x7fffffff) return cudaErrorInvalidValue;
   PushArgs<R> a;
   a.work_tile = ws.work_tile;
   a.work_pb = ws.work_pb;
-  a.chunk = ws.chunk;
+  a.work_n = ws.work_n;
+  a.nwork = (int)ws.nwork;
+  a.slots = ws.slots;
+  a.next_item = esc_count + 2;
   a.qabs = (float)(q < 0 ? -q : q);
   for (int d = 0; d < 3; ++d) {
     a.n[d] = g.n[d];
@@ -1227,27 +1371,25 @@ cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *co
   a.dn1 = make_fastdiv((uint32_t)g.n[1]);
   a.cell = p.cell;
   a.w = static_cast<const R *>(p.w);
-  a.tile_start = tile_start;
   a.esc_list = esc_list;
   a.esc_count = esc_count;
   a.q_jobs = esc_count + 1;
   a.qmh = (R)(q * g.dt / (2.0 * m));
   a.qz = (R)q;
   a.absorb = g.absorb_lo || g.absorb_hi;
-  a.ec = g.gather_ec;
   a.ctr = ctr;
   constexpr size_t smem = Lay<R, DIM, ORDER>::kEnd;
-  auto fn = k_push<R, DIM, ORDER>;
+  auto fn = k_push<R, DIM, ORDER, EC>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  if (ws.nwork > 0x7fffffff) return cudaErrorInvalidValue;
-  e = cudaMemsetAsync(esc_count, 0, 2 * sizeof(unsigned long long), st);
+  e = cudaMemsetAsync(esc_count, 0, 3 * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  fn<<<(unsigned)ws.nwork, kThreads, smem, st>>>(a);
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  k_push_escaped<R, DIM, ORDER><<<nsm, kThreads, 0, st>>>(a);
+  const int64_t nb = (int64_t)nsm * Lay<R, DIM, ORDER>::BLOCKS;  // as many blocks as fit: they take items in turn
+  fn<<<(unsigned)(ws.nwork < nb ? ws.nwork : nb), kThreads, smem, st>>>(a);
+  k_push_escaped<R, DIM, ORDER, EC><<<nsm, kThreads, 0, st>>>(a);
   if (nlaunch) *nlaunch = 2;
   return cudaGetLastError();
 }
@@ -1500,12 +1642,13 @@ int64_t push_item_cap(const Grid &g) {
 }
 
 cudaError_t launch_push(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
-                        const int64_t *tile_start, const WorkSplit &ws, int32_t *esc_list,
-                        unsigned long long *esc_count, double q, double m, Counters *ctr, cudaStream_t st,
-                        int *nlaunch) {
+                        const WorkSplit &ws, int32_t *esc_list, unsigned long long *esc_count, double q, double m,
+                        Counters *ctr, cudaStream_t st, int *nlaunch) {
   const int key = (g.prec == 1 ? 100 : 0) + g.dims * 10 + g.order;
-#define PIC_PUSH_CASE(K, R, D, O) \
-  case K: return launch_t<R, D, O>(g, E, B, J, p, tile_start, ws, esc_list, esc_count, q, m, ctr, st, nlaunch);
+#define PIC_PUSH_CASE(K, R, D, O)                                                                        \
+  case K:                                                                                                \
+    return g.gather_ec ? launch_t<R, D, O, true>(g, E, B, J, p, ws, esc_list, esc_count, q, m, ctr, st, nlaunch) \
+                       : launch_t<R, D, O, false>(g, E, B, J, p, ws, esc_list, esc_count, q, m, ctr, st, nlaunch);
   switch (key) {
     PIC_PUSH_CASE(21, float, 2, 1)
     PIC_PUSH_CASE(22, float, 2, 2)

@@ -128,18 +128,29 @@ __global__ void k_offsets(int32_t *__restrict__ count, int64_t ntiles, int tc, c
   if (run + lane < tile_start[t + 1]) dst_cell[run + lane] = -1;
 }
 
+// Slots per work item of a tile's run: the fewest equal pieces of at most
+// `chunk` (runs and chunks are multiples of kTilePad, and so are the pieces).
+__device__ __forceinline__ int64_t item_slots(int64_t run, int64_t chunk) {
+  const int64_t pieces = (run + chunk - 1) / chunk;
+  return pieces > 1 ? ((run + pieces - 1) / pieces + kTilePad - 1) / kTilePad * kTilePad : run;
+}
+
 // Single block: cut every tile's slot run into items of at most `chunk`
 // slots.  Exclusive scan of the per-tile item counts, then each thread
 // writes the items of its own run of tiles.
 __global__ void k_work_items(const int64_t *__restrict__ tile_start, int64_t ntiles, int64_t chunk,
-                             int32_t *__restrict__ work_tile, int64_t *__restrict__ work_pb) {
+                             int32_t *__restrict__ work_tile, int64_t *__restrict__ work_pb,
+                             int32_t *__restrict__ work_n) {
   __shared__ int64_t sh[1024];
   const int T = blockDim.x;
   const int64_t per = (ntiles + T - 1) / T;
   const int64_t b = threadIdx.x * per;
   const int64_t e = b + per < ntiles ? b + per : ntiles;
   int64_t local = 0;
-  for (int64_t t = b; t < e; ++t) local += (tile_start[t + 1] - tile_start[t] + chunk - 1) / chunk;
+  for (int64_t t = b; t < e; ++t) {
+    const int64_t run = tile_start[t + 1] - tile_start[t];
+    if (run > 0) local += (run + item_slots(run, chunk) - 1) / item_slots(run, chunk);
+  }
   sh[threadIdx.x] = local;
   __syncthreads();
   for (int o = 1; o < T; o <<= 1) {
@@ -150,10 +161,11 @@ __global__ void k_work_items(const int64_t *__restrict__ tile_start, int64_t nti
   }
   int64_t w = sh[threadIdx.x] - local;
   for (int64_t t = b; t < e; ++t) {
-    const int64_t len = work_item_slots(tile_start[t + 1] - tile_start[t], chunk);
-    for (int64_t p = tile_start[t]; p < tile_start[t + 1]; p += len, ++w) {
+    const int64_t run = tile_start[t + 1] - tile_start[t], len = item_slots(run, chunk);
+    for (int64_t p = 0; p < run; p += len, ++w) {
       work_tile[w] = (int32_t)t;
-      work_pb[w] = p;
+      work_pb[w] = tile_start[t] + p;
+      work_n[w] = (int32_t)(run - p < len ? run - p : len);
     }
   }
 }
@@ -227,7 +239,7 @@ cudaError_t launch_sort(const Grid &g, const Particles &src, const Particles &ds
     k_gather<float><<<nb, 256, 0, st>>>(g.dims, src, dst, d_count, tile_tmp + g.ntiles, ctr);
   e = cudaMemsetAsync(ws.work_tile, 0xff, sizeof(int32_t) * (size_t)ws.nwork, st);  // -1: no work
   if (e != cudaSuccess) return e;
-  k_work_items<<<1, 1024, 0, st>>>(tile_start, g.ntiles, ws.chunk, ws.work_tile, ws.work_pb);
+  k_work_items<<<1, 1024, 0, st>>>(tile_start, g.ntiles, ws.chunk, ws.work_tile, ws.work_pb, ws.work_n);
   if (nlaunch) *nlaunch = 7;
   return cudaGetLastError();
 }
