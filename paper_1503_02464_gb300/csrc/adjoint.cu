@@ -306,7 +306,6 @@ constexpr int kAdjDrift = 4;                           // cells a particle may h
 constexpr int kAdjGuard = kAdjDrift + 2;               // window nodes below the tile (deposit reaches 2 below)
 constexpr int kAdjWin = kAdjTile + 2 * kAdjGuard + 1;  // window nodes per axis (and 3 above)
 constexpr int kAdjWinN = kAdjWin * kAdjWin;
-constexpr int kAdjSub = 512;                           // slots of a work item one block takes
 
 template <class R> struct WindowNodes {
   int wi, wj;  // the particle's cell in window coordinates
@@ -651,18 +650,18 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_adj_push2d(cons
 }
 
 // Work items of a recorded particle buffer (the sort in effect when it was
-// recorded): item i covers work_n[i] slots from work_pb[i] of tile
-// t = work_tile[i] (-1: none); nsub blocks share an item, kAdjSub slots each.
+// recorded): item i < *count covers work_n[i] <= kAdjItem slots from
+// work_pb[i] of tile t = work_tile[i], one block each.
 struct AdjWork {
+  const int32_t *count;
   const int32_t *work_tile;
   const int64_t *work_pb;
   const int32_t *work_n;
-  int nsub;
   int nt0, t0, t1;
   unsigned long long *esc_total;  // running count of particles on the global path
 };
 
-// The particle adjoint over kAdjSub slots of one work item, one block: E, B
+// The particle adjoint of one work item, one block: E, B
 // and lamJ of the item's tile window are staged in shared memory (lamE and
 // lamB are scattered to global memory).  A particle more than kAdjDrift
 // cells outside its tile since the sort is set aside and done at the end of
@@ -672,16 +671,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
     k_adj_push2d_win(const AdjPushArgs<R> a, const AdjWork w) {
   extern __shared__ __align__(16) unsigned char adj_smem[];
   R *s = reinterpret_cast<R *>(adj_smem);
-  __shared__ int s_esc[kAdjSub];
+  __shared__ int s_esc[kAdjItem];
   __shared__ int s_nesc;
-  const int item = blockIdx.x / w.nsub;
+  const int item = blockIdx.x;
+  if (item >= *w.count) return;
   const int t = w.work_tile[item];
-  if (t < 0) return;
-  const int64_t ib = w.work_pb[item];
-  const int64_t ie = ib + w.work_n[item];
-  const int64_t pb = ib + (int64_t)(blockIdx.x % w.nsub) * kAdjSub;
-  if (pb >= ie) return;
-  const int64_t pe = pb + kAdjSub < ie ? pb + kAdjSub : ie;
+  const int64_t pb = w.work_pb[item], pe = pb + w.work_n[item];
   const int n0 = a.n[0], n1 = a.n[1];
   const int tx = (t % w.nt0) * w.t0, ty = (t / w.nt0) * w.t1;  // the tile's first cell
   const int ox = tx - kAdjGuard, oy = ty - kAdjGuard;          // the window's first node
@@ -890,7 +885,7 @@ static cudaError_t adj_push_t(const Grid &g, const Particles &tp, const int64_t 
   a.err = err;
   a.qmh = (R)(q * g.dt / (2.0 * m));
   a.q = (R)q;
-  const bool win = tt && tt->work_tile && tt->nwork > 0 && g.tile[0] <= kAdjTile && g.tile[1] <= kAdjTile;
+  const bool win = tt && tt->items.nwork > 0 && g.tile[0] <= kAdjTile && g.tile[1] <= kAdjTile;
   if (!win) {
     k_adj_push2d<R><<<nblocks(nmax), 256, 0, st>>>(a);
     if (nlaunch) *nlaunch = 1;
@@ -902,17 +897,16 @@ static cudaError_t adj_push_t(const Grid &g, const Particles &tp, const int64_t 
     if (e != cudaSuccess) return e;
   }
   AdjWork w;
-  w.work_tile = tt->work_tile;
-  w.work_pb = tt->work_pb;
-  w.work_n = tt->work_n;
-  w.nsub = (int)((tt->chunk + kAdjSub - 1) / kAdjSub);
+  w.count = tt->items.count;
+  w.work_tile = tt->items.work_tile;
+  w.work_pb = tt->items.work_pb;
+  w.work_n = tt->items.work_n;
   w.nt0 = g.ntile[0];
   w.t0 = g.tile[0];
   w.t1 = g.tile[1];
   w.esc_total = tt->esc_total;
-  const int64_t nblk = tt->nwork * w.nsub;
-  if (nblk > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_adj_push2d_win<R><<<(unsigned)nblk, 256, smem, st>>>(a, w);
+  if (tt->items.nwork > 0x7fffffffLL) return cudaErrorInvalidValue;
+  k_adj_push2d_win<R><<<(unsigned)tt->items.nwork, 256, smem, st>>>(a, w);
   if (nlaunch) *nlaunch = 1;
   return cudaGetLastError();
 }

@@ -35,12 +35,13 @@ struct Species {
   int64_t h_count = 0;          // host mirror, valid while !stepped_since_count
   int32_t *rank = nullptr;
   int64_t *tile_start = nullptr;
-  pic::WorkSplit work;          // push work items (tile pieces of at most work.chunk slots)
+  pic::WorkSplit work;          // work items of the push and of the adjoint
   // escapes of the last push, read back without blocking (adaptive sort)
   unsigned long long *esc_host = nullptr;  // page-locked: [0] escapes, [1] particles whose support changed
   cudaEvent_t esc_ev = nullptr;
   bool esc_pending = false;
-  bool crowded = false;         // the last count read averaged more than kCrowdedJobs such particles per item
+  bool crowded = false;         // the last count read averaged more than kCrowdedJobs such particles per nominal item
+  int64_t nominal_items = 1;
   bool fast = false;            // the last escape count read was above 1/8 of the early-sort threshold
   int count_age = 0;            // steps since an escape count was last read
   int64_t esc_step = -1;        // step of the push whose escape count is being read back
@@ -58,15 +59,13 @@ struct TimerRec {
 struct PCopy {
   Particles p{};
   int64_t *count = nullptr;
-  // Tape entries: the work items of the sort in effect (tiled = false when
-  // the species was unsorted at the copy).  meta is this copy's own buffer;
-  // work_pb, work_tile, work_n point to it or, when the previous tape entry
-  // was recorded under the same sort, to that entry's arrays.
+  // Tape entries: the adjoint's work items of the sort in effect (tiled =
+  // false when the species was unsorted at the copy).  meta is this copy's own
+  // buffer; items lies in it or, when the previous tape entry was recorded
+  // under the same sort, in that entry's.
   void *meta = nullptr;
-  const int32_t *work_tile = nullptr;
-  const int64_t *work_pb = nullptr;
-  const int32_t *work_n = nullptr;
-  int64_t nwork = 0, chunk = 0, sorts = -1;
+  pic::WorkList items;
+  int64_t sorts = -1;
   bool tiled = false;
 };
 
@@ -111,7 +110,7 @@ struct pic_handle {
   double *rho_bg = nullptr, *rho = nullptr, *rho_prev = nullptr, *f64 = nullptr, *red = nullptr;
   int64_t rho_prev_step = -2;
   int32_t *keys = nullptr;
-  int64_t *tile_tmp = nullptr;
+  void *sort_tmp = nullptr;
   double *mur = nullptr;  // Mur wall planes (8 * n1 * n2)
   double *laser_prof = nullptr;  // laser profile P at the wall rows of the polarised component (n1 * n2)
   pic::Laser laser{};
@@ -242,14 +241,16 @@ size_t particles_bytes(int64_t cap, size_t rs, int dims) {
   return align256(n * sizeof(int32_t)) + (size_t)(dims + 4) * align256(n * rs) + align256(n * sizeof(uint32_t));
 }
 
-// A sort's work items in one allocation (one copy for a tape entry):
-// work_pb[nwork], work_tile[nwork], work_n[nwork].
-size_t sort_meta_bytes(int64_t nwork) { return (sizeof(int64_t) + 2 * sizeof(int32_t)) * (size_t)nwork; }
+// A work list of at most n items in one allocation (one copy for a tape
+// entry): count, work_pb[n], work_tile[n], work_n[n].
+size_t work_list_bytes(int64_t n) { return 16 + (sizeof(int64_t) + 2 * sizeof(int32_t)) * (size_t)n; }
 
-void set_sort_meta(void *base, int64_t nwork, int64_t *&work_pb, int32_t *&work_tile, int32_t *&work_n) {
-  work_pb = static_cast<int64_t *>(base);
-  work_tile = reinterpret_cast<int32_t *>(work_pb + nwork);
-  work_n = work_tile + nwork;
+void set_work_list(pic::WorkList &w, void *base, int64_t n) {
+  w.nwork = n;
+  w.count = static_cast<int32_t *>(base);
+  w.work_pb = reinterpret_cast<int64_t *>(static_cast<char *>(base) + 16);
+  w.work_tile = reinterpret_cast<int32_t *>(w.work_pb + n);
+  w.work_n = w.work_tile + n;
 }
 
 void free_particles(Particles &p) {
@@ -334,7 +335,7 @@ int sort_species(pic_handle *h, Species &s) {
   Timed tm(h, pic::KC_SORT);
   CK(h,
      pic::launch_sort(h->g, s.buf[s.cur], s.buf[1 - s.cur], s.d_count, s.slots, h->keys, s.rank, s.tile_start,
-                      h->tile_tmp, s.work, h->ctr, h->st, &nl),
+                      h->sort_tmp, s.work, h->ctr, h->st, &nl),
      "sort");
   h->launches += nl;
   s.cur = 1 - s.cur;
@@ -379,7 +380,7 @@ cudaError_t alloc_snapshot(pic_handle *h, Snapshot &sn) {
   size_t total = align256(6 * fb);
   for (int i = 0; i < h->nsp; ++i)
     total += particles_bytes(h->sp[i].slots, h->rsize, h->g.dims) + 256 +
-             align256(sort_meta_bytes(h->sp[i].work.nwork));
+             align256(work_list_bytes(h->sp[i].work.adj.nwork));
   char *base = nullptr;
   const cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&base), total, h->st);
   if (e != cudaSuccess) return e;
@@ -397,7 +398,7 @@ cudaError_t alloc_snapshot(pic_handle *h, Snapshot &sn) {
     c.count = reinterpret_cast<int64_t *>(q);
     q += 256;
     c.meta = q;
-    q += align256(sort_meta_bytes(h->sp[i].work.nwork));
+    q += align256(work_list_bytes(h->sp[i].work.adj.nwork));
   }
   sn.allocated = true;
   sn.nsp = h->nsp;
@@ -430,25 +431,16 @@ cudaError_t save_snapshot(pic_handle *h, Snapshot &sn, bool tape = false, const 
     PCopy &c = sn.sp[i];
     e = copy_particles(h, c.p, c.count, s.buf[s.cur], s.d_count, s.slots);
     // the slot order is that of the last sort unless a sort is pending
-    c.tiled = tape && !s.need_sort && s.work.nwork > 0;
-    c.nwork = s.work.nwork;
-    c.chunk = s.work.chunk;
+    c.tiled = tape && !s.need_sort && s.work.adj.nwork > 0;
     c.sorts = s.sorts;
     if (!c.tiled || e != cudaSuccess) continue;
     const PCopy *q = prev ? &prev->sp[i] : nullptr;
     if (q && q->tiled && q->sorts == s.sorts) {
-      c.work_pb = q->work_pb;
-      c.work_tile = q->work_tile;
-      c.work_n = q->work_n;
+      c.items = q->items;
     } else {
-      e = cudaMemcpyAsync(c.meta, s.work.work_pb, sort_meta_bytes(s.work.nwork), cudaMemcpyDeviceToDevice,
+      e = cudaMemcpyAsync(c.meta, s.work.adj.count, work_list_bytes(s.work.adj.nwork), cudaMemcpyDeviceToDevice,
                           h->st);
-      int64_t *pb = nullptr;
-      int32_t *wt = nullptr, *wn = nullptr;
-      set_sort_meta(c.meta, s.work.nwork, pb, wt, wn);
-      c.work_pb = pb;
-      c.work_tile = wt;
-      c.work_n = wn;
+      set_work_list(c.items, c.meta, s.work.adj.nwork);
     }
   }
   sn.step = h->step;
@@ -608,7 +600,7 @@ int pic_create(const pic_config *cfg, pic_handle **out) {
        cudaMalloc(&h->rho_prev, db) == cudaSuccess && cudaMalloc(&h->f64, db) == cudaSuccess &&
        cudaMalloc(&h->red, 16 * sizeof(double)) == cudaSuccess &&
        cudaMalloc(&h->keys, (size_t)nkeys * sizeof(int32_t)) == cudaSuccess &&
-       cudaMalloc(&h->tile_tmp, (size_t)(g.ntiles + 1) * sizeof(int64_t)) == cudaSuccess &&
+       cudaMalloc(&h->sort_tmp, pic::sort_tmp_bytes(g.ntiles)) == cudaSuccess &&
        cudaMalloc(&h->ctr, sizeof(Counters)) == cudaSuccess && cudaMalloc(&h->bad, sizeof(unsigned long long)) == cudaSuccess &&
        cudaMalloc(&h->esc_count, 3 * sizeof(unsigned long long)) == cudaSuccess &&
        cudaMalloc(&h->mur, 8 * sizeof(double) * (size_t)g.n[1] * g.n[2]) == cudaSuccess;
@@ -657,7 +649,7 @@ int pic_destroy(pic_handle *h) {
   cudaFree(h->f64);
   cudaFree(h->red);
   cudaFree(h->keys);
-  cudaFree(h->tile_tmp);
+  cudaFree(h->sort_tmp);
   cudaFree(h->ctr);
   cudaFree(h->bad);
   cudaFree(h->esc_count);
@@ -670,7 +662,8 @@ int pic_destroy(pic_handle *h) {
     cudaFree(s.d_count);
     cudaFree(s.rank);
     cudaFree(s.tile_start);
-    cudaFree(s.work.work_pb);  // with work_tile and work_n
+    cudaFree(s.work.count);  // the whole list
+    cudaFree(s.work.adj.count);
     cudaFreeHost(s.esc_host);
     if (s.esc_ev) cudaEventDestroy(s.esc_ev);
   }
@@ -715,37 +708,36 @@ int pic_add_species(pic_handle *h, double q, double m, int64_t capacity, int *sp
   if (e == cudaSuccess) e = alloc_particles(s.buf[1], s.slots, h->rsize, h->g.dims);
   if (e == cudaSuccess) e = cudaMalloc(&s.d_count, sizeof(int64_t));
   if (e == cudaSuccess) e = cudaMalloc(&s.rank, (size_t)(s.slots > 0 ? s.slots : 1) * sizeof(int32_t));
-  // Work items: pieces of at most `chunk` slots per tile, chunk sized so that
-  // a species spread over few tiles (a thin slab, a small grid) still gives
-  // about 16 blocks per SM, never below 512 slots and never above what the
-  // push kernel holds in shared memory.
+  s.work.slots = s.slots;
+  s.work.plan = pic::push_item_plan(h->g);
   {
-    int dev = 0, nsm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    int64_t chunk = s.slots / (16 * (int64_t)(nsm > 0 ? nsm : 1));
-    chunk = (chunk + 255) / 256 * 256;
-    chunk = chunk < 512 ? 512 : chunk;
-    const int64_t cap = pic::push_item_cap(h->g);
-    s.work.chunk = chunk > cap ? cap : chunk;
-    s.work.slots = s.slots;
-    s.work.nwork = s.slots / s.work.chunk + 1 + h->g.ntiles;
+    // what pic_diag's n_push_mid_drain takes for a species' work items: pieces
+    // for about 16 per SM, of at least 512 slots
+    int64_t piece = s.slots / (16 * (int64_t)s.work.plan.nsm);
+    piece = (piece + 255) / 256 * 256;
+    s.nominal_items = s.slots / (piece < 512 ? 512 : piece) + 1 + h->g.ntiles;
   }
   if (e == cudaSuccess) e = cudaMallocHost(&s.esc_host, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.esc_ev, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMalloc(&s.tile_start, sizeof(int64_t) * (size_t)(h->g.ntiles + 1));
-  if (e == cudaSuccess) {
-    void *meta = nullptr;
-    e = cudaMalloc(&meta, sort_meta_bytes(s.work.nwork));
-    if (e == cudaSuccess) set_sort_meta(meta, s.work.nwork, s.work.work_pb, s.work.work_tile, s.work.work_n);
-  }
+  // the sort's work items: a tile's run makes at most run / size + 1
+  const auto make_list = [&](pic::WorkList &w, int size) {
+    const int64_t n = s.slots / size + 1 + h->g.ntiles;
+    void *mem = nullptr;
+    if (e == cudaSuccess) e = cudaMalloc(&mem, work_list_bytes(n));
+    if (e == cudaSuccess) set_work_list(w, mem, n);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.count, 0, 16, h->st);
+  };
+  make_list(s.work, s.work.plan.cand[pic::kItemCands - 1]);
+  if (h->g.dims == 2) make_list(s.work.adj, pic::kAdjItem);
   if (e != cudaSuccess) {
     free_particles(s.buf[0]);
     free_particles(s.buf[1]);
     cudaFree(s.d_count);
     cudaFree(s.rank);
     cudaFree(s.tile_start);
-    cudaFree(s.work.work_pb);  // with work_tile and work_n
+    cudaFree(s.work.count);  // the whole list
+    cudaFree(s.work.adj.count);
     cudaFreeHost(s.esc_host);
     if (s.esc_ev) cudaEventDestroy(s.esc_ev);
     s = Species{};
@@ -1238,7 +1230,7 @@ int pic_step(pic_handle *h, int nsteps) {
           // (a count from before the last sort says nothing about the order now)
           many_escapes = s.esc_step >= s.sorted_at && s.esc_host[0] > lim;
           s.fast = s.esc_host[0] > lim / 8;
-          s.crowded = s.esc_host[1] > (unsigned long long)pic::kCrowdedJobs * (unsigned long long)s.work.nwork;
+          s.crowded = s.esc_host[1] > (unsigned long long)pic::kCrowdedJobs * (unsigned long long)s.nominal_items;
         } else {
           cudaGetLastError();  // not ready: not an error
           s.count_age++;
@@ -1714,11 +1706,7 @@ int pic_adjoint_step(pic_handle *h, int nsteps) {
       Timed tm(h, pic::KC_ADJ_PUSH, sa);
       const PCopy &c = en.sp[i];
       pic::AdjTiles tt;
-      tt.work_tile = c.work_tile;
-      tt.work_pb = c.work_pb;
-      tt.work_n = c.work_n;
-      tt.nwork = c.nwork;
-      tt.chunk = c.chunk;
+      tt.items = c.items;
       tt.esc_total = h->adj_esc;
       int nl = 0;
       CK(h,

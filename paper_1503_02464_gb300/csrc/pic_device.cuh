@@ -15,6 +15,25 @@ __device__ __forceinline__ int wrapi(int i, int n) {
   return i < 0 ? i + n : i;
 }
 
+// Division of n < 2^31 by a runtime constant d (Granlund-Montgomery):
+// q = umulhi(n, m) >> s with s = ceil(log2 d) - 1, m = ceil(2^(32 + s) / d)
+// (the excess e = m d - 2^(32 + s) < d <= 2^(s + 1), so e n < 2^(32 + s));
+// m = 0 stands for d = 1.
+struct FastDiv {
+  uint32_t m, s;
+  __device__ __forceinline__ uint32_t div(uint32_t n) const { return m ? __umulhi(n, m) >> s : n; }
+};
+
+inline FastDiv make_fastdiv(uint32_t d) {
+  FastDiv f{0, 0};
+  if (d < 2) return f;
+  uint32_t l = 0;
+  while ((1ull << l) < d) ++l;
+  f.s = l - 1;
+  f.m = (uint32_t)(((1ull << (32 + f.s)) + d - 1) / d);
+  return f;
+}
+
 // Largest value below one (offsets live in [0, 1)).
 template <class R> __device__ __forceinline__ R below_one();
 template <> __device__ __forceinline__ float below_one<float>() { return 0.99999994f; }

@@ -126,21 +126,33 @@ enum KernelClass {
 // drift allowance is one cell.
 void push_tile_shape(int dims, int tile[3]);
 size_t push_smem_bytes(const Grid &g);
-// Most slots a work item of the push may hold (its chunk is at most this).
-int64_t push_item_cap(const Grid &g);
-// Work items of the push kernel: each tile's slot run is cut into the fewest
-// equal pieces (multiples of 4 slots; the last may be shorter) of at most
-// `chunk` slots; item i covers work_n[i] slots from work_pb[i] of tile
-// work_tile[i] (-1: no work, the list ends there).  nwork bounds the item
-// count (slots / chunk + 1 + ntiles).
-struct WorkSplit {
-  int64_t slots = 0;  // of the species
-  int64_t chunk = 0;
-  int64_t nwork = 0;
+// How the sort cuts every tile's slot run into work items of the push: into
+// the fewest equal pieces (multiples of 4 slots; the last may be shorter) of
+// at most one of the candidate sizes, the largest of which is what the kernel
+// holds in shared memory.  The sort takes the candidate of the least estimated
+// time for the runs at hand: an item costs its slots and `fixed` more, and the
+// items run in rounds of `blocks` per SM on `nsm` SMs.
+constexpr int kItemCands = 8;
+struct ItemPlan {
+  int cand[kItemCands];  // descending multiples of 4
+  int blocks = 1, nsm = 1, fixed = 0;
+};
+ItemPlan push_item_plan(const Grid &g);
+// Work items: item i < *count covers work_n[i] slots from work_pb[i] of tile
+// work_tile[i].
+struct WorkList {
+  int64_t nwork = 0;  // items at most
+  int32_t *count = nullptr;
   int32_t *work_tile = nullptr;
   int64_t *work_pb = nullptr;
   int32_t *work_n = nullptr;
 };
+struct WorkSplit : WorkList {
+  int64_t slots = 0;  // of the species
+  ItemPlan plan;
+  WorkList adj;  // pieces of at most kAdjItem slots for the adjoint kernels (2D; else nwork = 0)
+};
+constexpr int kAdjItem = 512;
 
 // Tile kernel (one block per work item) + escape kernel.
 // esc_list (one int per slot) is scratch for particles deferred to the
@@ -160,11 +172,12 @@ cudaError_t launch_rho_tiled(const Grid &g, const Particles &p, const int64_t *t
 // ---- sort (sort.cu) ----
 // Counting sort of the slots [0, *d_count) of `src` by (tile, cell-in-tile),
 // dead slots dropped; result in `dst`, *d_count updated, tile_start[ntiles+1]
-// written.  Each tile's run is padded with dead slots to a multiple of
-// kTilePad.  `keys` has ntiles*tile_cells ints, `rank` one int per slot.
-
+// and the work items written.  Each tile's run is padded with dead slots to a
+// multiple of kTilePad.  `keys` has ntiles*tile_cells ints, `rank` one int per
+// slot, `tmp` sort_tmp_bytes.
+size_t sort_tmp_bytes(int64_t ntiles);
 cudaError_t launch_sort(const Grid &g, const Particles &src, const Particles &dst, int64_t *d_count,
-                        int64_t capacity, int32_t *keys, int32_t *rank, int64_t *tile_start, int64_t *tile_tmp,
+                        int64_t capacity, int32_t *keys, int32_t *rank, int64_t *tile_start, void *tmp,
                         const WorkSplit &ws, Counters *ctr, cudaStream_t st, int *nlaunch);
 
 // ---- fields and particle conversion (fields.cu) ----
@@ -237,14 +250,11 @@ cudaError_t launch_adj_yee_e(const Grid &g, void *const lE[3], void *const lB[3]
 cudaError_t launch_adj_mur(const Grid &g, void *const lE[3], double *pend, const LaserStep &ls_unit, double *da0,
                            cudaStream_t st);
 // Work items of a recorded particle buffer (those of the sort in effect when
-// it was recorded, see WorkSplit) for the windowed adjoint kernel;
+// it was recorded, see WorkSplit::adj) for the windowed adjoint kernel;
 // esc_total counts the particles that had drifted beyond their tile window
 // (a running sum).
 struct AdjTiles {
-  const int32_t *work_tile = nullptr;
-  const int64_t *work_pb = nullptr;
-  const int32_t *work_n = nullptr;
-  int64_t nwork = 0, chunk = 0;
+  WorkList items;
   unsigned long long *esc_total = nullptr;
 };
 // Per-particle adjoint of one recorded step (2D3V TSC only): tp/d_count

@@ -88,25 +88,6 @@ template <class R, int DIM, int ORDER> struct Lay {
   static_assert(G::KT < 1024 && CAP < 4096 && CAP % 32 == 0, "tag packing");
 };
 
-// Division of n < 2^31 by a runtime constant d (Granlund-Montgomery):
-// q = umulhi(n, m) >> s with s = ceil(log2 d) - 1, m = ceil(2^(32 + s) / d)
-// (the excess e = m d - 2^(32 + s) < d <= 2^(s + 1), so e n < 2^(32 + s));
-// m = 0 stands for d = 1.
-struct FastDiv {
-  uint32_t m, s;
-  __device__ __forceinline__ uint32_t div(uint32_t n) const { return m ? __umulhi(n, m) >> s : n; }
-};
-
-FastDiv make_fastdiv(uint32_t d) {
-  FastDiv f{0, 0};
-  if (d < 2) return f;
-  uint32_t l = 0;
-  while ((1ull << l) < d) ++l;
-  f.s = l - 1;
-  f.m = (uint32_t)(((1ull << (32 + f.s)) + d - 1) / d);
-  return f;
-}
-
 template <class R> struct PushArgs {
   int n[3];
   int ntile[2];
@@ -119,10 +100,10 @@ template <class R> struct PushArgs {
   R *u[3];
   const R *w;
   float qabs;                       // |q|
-  const int32_t *work_tile;         // work item -> tile (-1: none, nor any after it)
+  const int32_t *work_tile;         // work item -> tile
   const int64_t *work_pb;           // work item -> first slot
   const int32_t *work_n;            // work item -> slots
-  int nwork;                        // work items at most
+  const int32_t *nwork;             // work items
   int64_t slots;                    // slots of the species
   unsigned long long *next_item;    // items taken beyond the first of every block
   int32_t *esc_list;                // slots deferred to k_push_escaped
@@ -694,11 +675,11 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
     copy(sJob + (L::NJ - 1) * CAP, a.w + pb, n * (int)sizeof(R));
   };
 
-  int wi = blockIdx.x;
-  int t = wi < a.nwork ? a.work_tile[wi] : -1;
-  if (t < 0) return;
-  int64_t pb = a.work_pb[wi];
-  int n = a.work_n[wi];
+  const unsigned nwork = (unsigned)*a.nwork;
+  if (blockIdx.x >= nwork) return;
+  int t = a.work_tile[blockIdx.x];
+  int64_t pb = a.work_pb[blockIdx.x];
+  int n = a.work_n[blockIdx.x];
   stage_particles(pb, n);
   while (t >= 0) {
 #ifdef PIC_CHECKED
@@ -924,12 +905,10 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
       if (s_clamp) atomicAdd(&a.ctr->clamped, (unsigned long long)s_clamp);
       if (s_absorbed) atomicAdd(&a.ctr->absorbed, (unsigned long long)s_absorbed);
       const unsigned long long next = taken + gridDim.x;
-      if (next < (unsigned long long)a.nwork) {
+      if (next < nwork) {
         t_next = a.work_tile[next];
-        if (t_next >= 0) {
-          pb_next = a.work_pb[next];
-          n_next = a.work_n[next];
-        }
+        pb_next = a.work_pb[next];
+        n_next = a.work_n[next];
       }
     }
 
@@ -1346,12 +1325,12 @@ template <class R, int DIM, int ORDER, bool EC>
 cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
                      const WorkSplit &ws, int32_t *esc_list, unsigned long long *esc_count, double q, double m,
                      Counters *ctr, cudaStream_t st, int *nlaunch) {
-  if (ws.chunk > Lay<R, DIM, ORDER>::CAP || ws.nwork > 0x7fffffff) return cudaErrorInvalidValue;
+  if (ws.plan.cand[0] > Lay<R, DIM, ORDER>::CAP || ws.nwork > 0x7fffffff) return cudaErrorInvalidValue;
   PushArgs<R> a;
   a.work_tile = ws.work_tile;
   a.work_pb = ws.work_pb;
   a.work_n = ws.work_n;
-  a.nwork = (int)ws.nwork;
+  a.nwork = ws.count;
   a.slots = ws.slots;
   a.next_item = esc_count + 2;
   a.qabs = (float)(q < 0 ? -q : q);
@@ -1620,8 +1599,7 @@ void push_tile_shape(int dims, int tile[3]) {
   tile[2] = dims == 3 ? Geo<3, 2>::TZ : 1;
 }
 
-// The layout of the kernel that serves a grid: its shared memory, and the
-// most slots one of its work items may hold.
+// The layout of the kernel that serves a grid.
 template <class F> static auto with_layout(const Grid &g, F f) {
   switch ((g.prec == 1 ? 100 : 0) + g.dims * 10 + g.order) {
     case 21: return f(Lay<float, 2, 1>{});
@@ -1637,8 +1615,22 @@ template <class F> static auto with_layout(const Grid &g, F f) {
 size_t push_smem_bytes(const Grid &g) {
   return with_layout(g, [](auto l) { return (size_t)decltype(l)::kEnd; });
 }
-int64_t push_item_cap(const Grid &g) {
-  return with_layout(g, [](auto l) { return (int64_t)decltype(l)::CAP; });
+ItemPlan push_item_plan(const Grid &g) {
+  ItemPlan pl;
+  const int cap = with_layout(g, [](auto l) { return (int)decltype(l)::CAP; });
+  pl.blocks = with_layout(g, [](auto l) { return (int)decltype(l)::BLOCKS; });
+  // an item's own cost in slots, from the instructions of the same particles
+  // cut differently (2D: 434; 3D TSC: 345; FP64 particles cost far more each)
+  pl.fixed = g.prec == 1 ? 120 : 400;
+  for (int j = 0; j < kItemCands; ++j) {
+    const int c = cap * (kItemCands - j) / kItemCands / kTilePad * kTilePad;
+    pl.cand[j] = c > 256 ? c : 256;
+  }
+  int dev = 0;
+  pl.nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&pl.nsm, cudaDevAttrMultiProcessorCount, dev);
+  return pl;
 }
 
 cudaError_t launch_push(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
