@@ -12,6 +12,7 @@
 
 #include <cmath>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "pic.h"
@@ -24,6 +25,7 @@ using pic::Particles;
 namespace {
 
 constexpr int kMaxSpecies = 8;
+constexpr size_t kEscBytes = kMaxSpecies * pic::kEscCounters * sizeof(unsigned long long);
 
 struct Species {
   double q = 0, m = 1;
@@ -107,6 +109,9 @@ struct pic_handle {
   cudaStream_t st = nullptr;
   size_t rsize = 4;
   void *E[3] = {}, *B[3] = {}, *J[3] = {};
+  // 2D: the fields a step writes (then they trade places with E, B), and the
+  // J buffer of the next step, which is zero between steps
+  void *E2[3] = {}, *B2[3] = {}, *J2[3] = {};
   double *rho_bg = nullptr, *rho = nullptr, *rho_prev = nullptr, *f64 = nullptr, *red = nullptr;
   int64_t rho_prev_step = -2;
   int32_t *keys = nullptr;
@@ -114,7 +119,7 @@ struct pic_handle {
   double *mur = nullptr;  // Mur wall planes (8 * n1 * n2)
   double *laser_prof = nullptr;  // laser profile P at the wall rows of the polarised component (n1 * n2)
   pic::Laser laser{};
-  unsigned long long *esc_count = nullptr;
+  unsigned long long *esc_count = nullptr;  // kEscCounters per species, zero between steps
   Counters *ctr = nullptr;
   unsigned long long *bad = nullptr;
   Species sp[kMaxSpecies];
@@ -588,11 +593,17 @@ int pic_create(const pic_config *cfg, pic_handle **out) {
   // E, B in one block (a checkpoint copies them with one memcpy) and the
   // three J components in another (one memset clears J)
   bool ok = cudaMalloc(&h->E[0], 6 * fb) == cudaSuccess && cudaMalloc(&h->J[0], 3 * fb) == cudaSuccess;
+  if (g.dims == 2)
+    ok = ok && cudaMalloc(&h->E2[0], 6 * fb) == cudaSuccess && cudaMalloc(&h->J2[0], 3 * fb) == cudaSuccess;
   if (ok)
     for (int d = 0; d < 3; ++d) {
       h->E[d] = static_cast<char *>(h->E[0]) + d * fb;
       h->B[d] = static_cast<char *>(h->E[0]) + (3 + d) * fb;
       h->J[d] = static_cast<char *>(h->J[0]) + d * fb;
+      if (g.dims != 2) continue;
+      h->E2[d] = static_cast<char *>(h->E2[0]) + d * fb;
+      h->B2[d] = static_cast<char *>(h->E2[0]) + (3 + d) * fb;
+      h->J2[d] = static_cast<char *>(h->J2[0]) + d * fb;
     }
   const size_t db = (size_t)ncell * sizeof(double);
   const int64_t nkeys = g.ntiles * g.tile[0] * g.tile[1] * g.tile[2];
@@ -602,7 +613,7 @@ int pic_create(const pic_config *cfg, pic_handle **out) {
        cudaMalloc(&h->keys, (size_t)nkeys * sizeof(int32_t)) == cudaSuccess &&
        cudaMalloc(&h->sort_tmp, pic::sort_tmp_bytes(g.ntiles)) == cudaSuccess &&
        cudaMalloc(&h->ctr, sizeof(Counters)) == cudaSuccess && cudaMalloc(&h->bad, sizeof(unsigned long long)) == cudaSuccess &&
-       cudaMalloc(&h->esc_count, 3 * sizeof(unsigned long long)) == cudaSuccess &&
+       cudaMalloc(&h->esc_count, kEscBytes) == cudaSuccess &&
        cudaMalloc(&h->mur, 8 * sizeof(double) * (size_t)g.n[1] * g.n[2]) == cudaSuccess;
   if (!ok) {
     pic_destroy(h);
@@ -610,6 +621,8 @@ int pic_create(const pic_config *cfg, pic_handle **out) {
   }
   cudaMemsetAsync(h->E[0], 0, 6 * fb, h->st);
   cudaMemsetAsync(h->J[0], 0, 3 * fb, h->st);
+  if (h->J2[0]) cudaMemsetAsync(h->J2[0], 0, 3 * fb, h->st);
+  cudaMemsetAsync(h->esc_count, 0, kEscBytes, h->st);
   cudaMemsetAsync(h->rho_bg, 0, db, h->st);
   cudaMemsetAsync(h->ctr, 0, sizeof(Counters), h->st);
   // laser profile P = exp(-r^2/waist^2) at the wall rows of the polarised
@@ -643,6 +656,8 @@ int pic_destroy(pic_handle *h) {
   cudaStreamSynchronize(h->st);
   cudaFree(h->E[0]);  // E and B share one block
   cudaFree(h->J[0]);  // so do the three J components
+  cudaFree(h->E2[0]);
+  cudaFree(h->J2[0]);
   cudaFree(h->rho_bg);
   cudaFree(h->rho);
   cudaFree(h->rho_prev);
@@ -1211,7 +1226,8 @@ int pic_step(pic_handle *h, int nsteps) {
       // threshold waits for the count of its previous push; the others wait
       // once four steps have passed without a count, so that a long
       // pic_step call, whose host loop runs ahead of the device, still
-      // learns how the particles drift.  (On large grids a wait costs no
+      // learns how the particles drift; their counts are copied back every
+      // fourth step (a copy and an event cost 3 us, which small runs feel).  (On large grids a wait costs no
       // device time: the last step's field updates are still queued behind
       // the push when it ends.)
       bool many_escapes = false;
@@ -1253,23 +1269,29 @@ int pic_step(pic_handle *h, int nsteps) {
       }
       if (h->tape_len >= (int)tape.size()) h->taping = false;
     }
-    {
+    const bool walls = h->g.absorb_lo || h->g.absorb_hi;
+    if (h->g.dims == 2) {
+      // cleared by the field update of the step before
+      for (int d = 0; d < 3; ++d) std::swap(h->J[d], h->J2[d]);
+    } else {
       Timed tm(h, pic::KC_ZEROJ);
       CK(h, cudaMemsetAsync(h->J[0], 0, 3 * fb, h->st), "zero J");
+      CK(h, cudaMemsetAsync(h->esc_count, 0, kEscBytes, h->st), "zero counters");
     }
     for (int i = 0; i < h->nsp; ++i) {
       Species &s = h->sp[i];
       Timed tm(h, pic::KC_PUSH);
       int nl = 0;
       CK(h,
-         pic::launch_push(h->g, h->E, h->B, h->J, s.buf[s.cur], s.work, s.rank, h->esc_count, s.q, s.m, h->ctr,
-                          h->st, &nl),
+         pic::launch_push(h->g, h->E, h->B, h->J, s.buf[s.cur], s.work, s.rank, h->esc_count + i * pic::kEscCounters,
+                          s.q, s.m, h->ctr, h->st, &nl),
          "push");
       h->launches += nl;
       if (s.crowded) h->crowded_pushes++;
-      if (s.esc_host && !s.esc_pending) {
-        CK(h, cudaMemcpyAsync(s.esc_host, h->esc_count, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                              h->st),
+      // (a slow species' count is copied back every fourth step)
+      if (!s.esc_pending && (s.fast || s.esc_step < 0 || s.esc_step > h->step || h->step - s.esc_step >= 4)) {
+        CK(h, cudaMemcpyAsync(s.esc_host, h->esc_count + i * pic::kEscCounters, 2 * sizeof(unsigned long long),
+                              cudaMemcpyDeviceToHost, h->st),
            "escape count");
         CK(h, cudaEventRecord(s.esc_ev, h->st), "escape event");
         s.esc_pending = true;
@@ -1287,35 +1309,45 @@ int pic_step(pic_handle *h, int nsteps) {
         h->launches += nl;
       }
     }
-    {
-      Timed tm(h, pic::KC_YEE_B);
-      CK(h, pic::launch_yee_b(h->g, h->E, h->B, 0.5 * h->g.dt, h->st), "yee B");
-    }
-    const bool walls = h->g.absorb_lo || h->g.absorb_hi;
-    if (walls) {
-      Timed tm(h, pic::KC_BOUNDARY);
-      CK(h, pic::launch_mur_save(h->g, h->E, h->mur, h->st), "mur save");
-      h->launches++;
-    }
-    {
+    const pic::LaserStep wave = pic::laser_step(h->laser, h->laser_prof, h->laser.a0, h->g, h->step * h->g.dt,
+                                                (h->step + 1) * h->g.dt);
+    if (h->g.dims == 2) {
       Timed tm(h, pic::KC_YEE_E);
-      CK(h, pic::launch_yee_e(h->g, h->E, h->B, h->J, h->g.dt, h->st), "yee E");
-    }
-    if (walls) {
-      Timed tm(h, pic::KC_BOUNDARY);
       CK(h,
-         pic::launch_mur_apply(h->g, h->E, h->mur,
-                               pic::laser_step(h->laser, h->laser_prof, h->laser.a0, h->g, h->step * h->g.dt,
-                                               (h->step + 1) * h->g.dt),
-                               h->st),
-         "mur apply");
+         pic::launch_field_step2(h->g, h->E, h->B, h->J, h->E2, h->B2, h->J2, wave, h->esc_count,
+                                 kMaxSpecies * pic::kEscCounters, h->st),
+         "field step");
+      for (int d = 0; d < 3; ++d) {
+        std::swap(h->E[d], h->E2[d]);
+        std::swap(h->B[d], h->B2[d]);
+      }
       h->launches++;
+    } else {
+      {
+        Timed tm(h, pic::KC_YEE_B);
+        CK(h, pic::launch_yee_b(h->g, h->E, h->B, 0.5 * h->g.dt, h->st), "yee B");
+      }
+      if (walls) {
+        Timed tm(h, pic::KC_BOUNDARY);
+        CK(h, pic::launch_mur_save(h->g, h->E, h->mur, h->st), "mur save");
+        h->launches++;
+      }
+      {
+        Timed tm(h, pic::KC_YEE_E);
+        CK(h, pic::launch_yee_e(h->g, h->E, h->B, h->J, h->g.dt, h->st), "yee E");
+      }
+      if (walls) {
+        Timed tm(h, pic::KC_BOUNDARY);
+        CK(h,
+           pic::launch_mur_apply(h->g, h->E, h->mur, wave, h->st), "mur apply");
+        h->launches++;
+      }
+      {
+        Timed tm(h, pic::KC_YEE_B);
+        CK(h, pic::launch_yee_b(h->g, h->E, h->B, 0.5 * h->g.dt, h->st), "yee B");
+      }
+      h->launches += 3;
     }
-    {
-      Timed tm(h, pic::KC_YEE_B);
-      CK(h, pic::launch_yee_b(h->g, h->E, h->B, 0.5 * h->g.dt, h->st), "yee B");
-    }
-    h->launches += 3;
     h->step++;
     for (auto &o : h->outputs)
       if (o.active && pic_output_due(&o.req, h->step)) {

@@ -29,8 +29,9 @@ template <class R> struct YeeArgs {
   const R *J[3];
 };
 
+// 3D runs: the three updates as launches of their own (2D: k_field_step2).
 // B <- B - h curl E, curl E at the B locations.
-template <class R, int DIM>
+template <class R>
 __global__ void __launch_bounds__(256) k_yee_b(YeeArgs<R> a) {
   const int n0 = a.n[0], n1 = a.n[1], n2 = a.n[2];
   const int64_t ncell = (int64_t)n0 * n1 * n2;
@@ -46,11 +47,9 @@ __global__ void __launch_bounds__(256) k_yee_b(YeeArgs<R> a) {
     R cx = (a.E[2][cyp] - ez) * a.rdx[1];
     R cy = -(a.E[2][cxp] - ez) * a.rdx[0];
     const R cz = (a.E[1][cxp] - ey) * a.rdx[0] - (a.E[0][cyp] - ex) * a.rdx[1];
-    if (DIM == 3) {
-      const int64_t czp = c + (k + 1 < n2 ? sz : sz - sz * n2);
-      cx -= (a.E[1][czp] - ey) * a.rdx[2];
-      cy += (a.E[0][czp] - ex) * a.rdx[2];
-    }
+    const int64_t czp = c + (k + 1 < n2 ? sz : sz - sz * n2);
+    cx -= (a.E[1][czp] - ey) * a.rdx[2];
+    cy += (a.E[0][czp] - ex) * a.rdx[2];
     a.B[0][c] -= a.h * cx;
     if (a.absorb && i == n0 - 1) continue;  // By, Bz half a cell beyond the last node
     a.B[1][c] -= a.h * cy;
@@ -59,7 +58,7 @@ __global__ void __launch_bounds__(256) k_yee_b(YeeArgs<R> a) {
 }
 
 // E <- E + h (curl B - J), curl B at the E locations.
-template <class R, int DIM>
+template <class R>
 __global__ void __launch_bounds__(256) k_yee_e(YeeArgs<R> a) {
   const int n0 = a.n[0], n1 = a.n[1], n2 = a.n[2];
   const int64_t ncell = (int64_t)n0 * n1 * n2;
@@ -75,11 +74,9 @@ __global__ void __launch_bounds__(256) k_yee_e(YeeArgs<R> a) {
     R cx = (bz - a.B[2][cym]) * a.rdx[1];
     R cy = -(bz - a.B[2][cxm]) * a.rdx[0];
     const R cz = (by - a.B[1][cxm]) * a.rdx[0] - (bx - a.B[0][cym]) * a.rdx[1];
-    if (DIM == 3) {
-      const int64_t czm = c - (k > 0 ? sz : sz - sz * n2);
-      cx -= (by - a.B[1][czm]) * a.rdx[2];
-      cy += (bx - a.B[0][czm]) * a.rdx[2];
-    }
+    const int64_t czm = c - (k > 0 ? sz : sz - sz * n2);
+    cx -= (by - a.B[1][czm]) * a.rdx[2];
+    cy += (bx - a.B[0][czm]) * a.rdx[2];
     if (a.absorb && i == n0 - 1) continue;  // wall node (Mur) and Ex beyond the last node
     a.E[0][c] += a.h * (cx - a.J[0][c]);
     if (a.absorb && i == 0) continue;       // wall node (Mur)
@@ -103,7 +100,7 @@ template <class R> struct alignas(16) Pack {
 template <class R> __device__ __forceinline__ Pack<R> ldp(const R *p) { return *reinterpret_cast<const Pack<R> *>(p); }
 template <class R> __device__ __forceinline__ void stp(R *p, const Pack<R> &v) { *reinterpret_cast<Pack<R> *>(p) = v; }
 
-template <class R, int DIM>
+template <class R>
 __global__ void __launch_bounds__(256) k_yee_b_vec(YeeArgs<R> a) {
   constexpr int W = 16 / sizeof(R);
   const int n0 = a.n[0], n1 = a.n[1], n2 = a.n[2];
@@ -120,12 +117,9 @@ __global__ void __launch_bounds__(256) k_yee_b_vec(YeeArgs<R> a) {
   const Pack<R> ex = ldp(a.E[0] + c), ey = ldp(a.E[1] + c), ez = ldp(a.E[2] + c);
   const Pack<R> ex_yp = ldp(a.E[0] + cyp), ez_yp = ldp(a.E[2] + cyp);
   const R ey_xn = a.E[1][cxn], ez_xn = a.E[2][cxn];
-  Pack<R> ex_zp, ey_zp;
-  if (DIM == 3) {
-    const int64_t czp = k + 1 < n2 ? c + sz : c + sz - sz * n2;
-    ex_zp = ldp(a.E[0] + czp);
-    ey_zp = ldp(a.E[1] + czp);
-  }
+  const int64_t czp = k + 1 < n2 ? c + sz : c + sz - sz * n2;
+  const Pack<R> ex_zp = ldp(a.E[0] + czp);
+  const Pack<R> ey_zp = ldp(a.E[1] + czp);
   Pack<R> bx = ldp(a.B[0] + c), by = ldp(a.B[1] + c), bz = ldp(a.B[2] + c);
   // By, Bz half a cell beyond the last node stay as they are at absorbing walls
   const bool last = a.absorb && iq == nq - 1;
@@ -135,10 +129,8 @@ __global__ void __launch_bounds__(256) k_yee_b_vec(YeeArgs<R> a) {
     R cx = (ez_yp.v[w] - ez.v[w]) * a.rdx[1];
     R cy = -(ezx - ez.v[w]) * a.rdx[0];
     const R cz = (eyx - ey.v[w]) * a.rdx[0] - (ex_yp.v[w] - ex.v[w]) * a.rdx[1];
-    if (DIM == 3) {
-      cx -= (ey_zp.v[w] - ey.v[w]) * a.rdx[2];
-      cy += (ex_zp.v[w] - ex.v[w]) * a.rdx[2];
-    }
+    cx -= (ey_zp.v[w] - ey.v[w]) * a.rdx[2];
+    cy += (ex_zp.v[w] - ex.v[w]) * a.rdx[2];
     bx.v[w] -= a.h * cx;
     if (!(last && w == W - 1)) {
       by.v[w] -= a.h * cy;
@@ -150,7 +142,7 @@ __global__ void __launch_bounds__(256) k_yee_b_vec(YeeArgs<R> a) {
   stp(a.B[2] + c, bz);
 }
 
-template <class R, int DIM>
+template <class R>
 __global__ void __launch_bounds__(256) k_yee_e_vec(YeeArgs<R> a) {
   constexpr int W = 16 / sizeof(R);
   const int n0 = a.n[0], n1 = a.n[1], n2 = a.n[2];
@@ -167,12 +159,9 @@ __global__ void __launch_bounds__(256) k_yee_e_vec(YeeArgs<R> a) {
   const Pack<R> bx = ldp(a.B[0] + c), by = ldp(a.B[1] + c), bz = ldp(a.B[2] + c);
   const Pack<R> bx_ym = ldp(a.B[0] + cym), bz_ym = ldp(a.B[2] + cym);
   const R by_xp = a.B[1][cxp], bz_xp = a.B[2][cxp];
-  Pack<R> bx_zm, by_zm;
-  if (DIM == 3) {
-    const int64_t czm = k > 0 ? c - sz : c - sz + sz * n2;
-    bx_zm = ldp(a.B[0] + czm);
-    by_zm = ldp(a.B[1] + czm);
-  }
+  const int64_t czm = k > 0 ? c - sz : c - sz + sz * n2;
+  const Pack<R> bx_zm = ldp(a.B[0] + czm);
+  const Pack<R> by_zm = ldp(a.B[1] + czm);
   const Pack<R> jx = ldp(a.J[0] + c), jy = ldp(a.J[1] + c), jz = ldp(a.J[2] + c);
   Pack<R> ex = ldp(a.E[0] + c), ey = ldp(a.E[1] + c), ez = ldp(a.E[2] + c);
   // at absorbing walls the wall nodes belong to the Mur kernels, and Ex
@@ -184,10 +173,8 @@ __global__ void __launch_bounds__(256) k_yee_e_vec(YeeArgs<R> a) {
     R cx = (bz.v[w] - bz_ym.v[w]) * a.rdx[1];
     R cy = -(bz.v[w] - bzx) * a.rdx[0];
     const R cz = (by.v[w] - byx) * a.rdx[0] - (bx.v[w] - bx_ym.v[w]) * a.rdx[1];
-    if (DIM == 3) {
-      cx -= (by.v[w] - by_zm.v[w]) * a.rdx[2];
-      cy += (bx.v[w] - bx_zm.v[w]) * a.rdx[2];
-    }
+    cx -= (by.v[w] - by_zm.v[w]) * a.rdx[2];
+    cy += (bx.v[w] - bx_zm.v[w]) * a.rdx[2];
     const bool wall_hi = last && w == W - 1, wall_lo = first && w == 0;
     if (!wall_hi) ex.v[w] += a.h * (cx - jx.v[w]);
     if (!wall_hi && !wall_lo) {
@@ -286,6 +273,162 @@ YeeArgs<R> yee_args(const Grid &g, void *const E[3], void *const B[3], void *con
   }
   a.h = (R)h;
   return a;
+}
+
+// ---- the whole field update of a 2D step in one pass ----
+// B half, E (with the Mur walls and the incoming wave) and B half from the
+// fields E, B into E2, B2, and the next step's J cleared.  A warp takes a
+// strip of kStripW columns and `rows` rows, one lane per column with one lane
+// of halo below and two above, and marches along y: a row's y neighbours are
+// the registers of the passes before and after, its x neighbours come by
+// shuffle, so that there is no shared memory and no barrier.  The halo's
+// intermediate values are recomputed by every strip that needs them.
+//
+// Five launches with walls and 132 B per cell before (FP32), 72 B now with
+// the 12 that clear J.  Small grids are bound by launches and by the chain of
+// dependent passes, large ones by loads in flight: 2048 x 1024 FP32 with walls
+// 36 us (4.2 TB/s) where the launches took 55 and their gaps; 64 x 64 FP64 6.2
+// us (14.5).
+template <class R> struct FieldStep2 {
+  int n0, n1, absorb;
+  int width, rows;  // output columns and rows of a strip
+  unsigned strips;  // strips side by side
+  R rdx, rdy, h;    // h: the full step
+  const R *E[3], *B[3], *J[3];
+  R *E2[3], *B2[3], *Jn[3];
+  double kc;  // Mur: (dt - dx) / (dt + dx)
+  LaserStep ls;
+  unsigned long long *counters;  // escape counters cleared for the next step's pushes
+  int ncounters;
+};
+constexpr int kStripW = 29;
+
+template <class R> __global__ void __launch_bounds__(64) k_field_step2(const __grid_constant__ FieldStep2<R> a) {
+  const int lane = threadIdx.x & 31;
+  if (blockIdx.x == 0)
+    for (int k = threadIdx.x; k < a.ncounters; k += blockDim.x) a.counters[k] = 0;
+  const int x0 = (int)(blockIdx.x % a.strips) * a.width;
+  const int y0 = (int)((blockIdx.x / a.strips * (blockDim.x / 32) + (threadIdx.x >> 5)) * a.rows);
+  if (y0 >= a.n1) return;
+  const int rows = min(a.rows, a.n1 - y0);
+  int i = x0 - 1 + lane;  // this lane's column, wrapped
+  const bool mine = lane >= 1 && lane <= a.width && i < a.n0;
+  i %= a.n0;
+  if (i < 0) i += a.n0;
+  const bool wall_lo = a.absorb && i == 0, wall_hi = a.absorb && i == a.n0 - 1;
+  // the wave at the x = 0 wall: this strip's rows in groups of eight, four
+  // values of a row in four lanes (L0, L1 at the old and at the new time)
+  const bool wave = a.absorb && a.ls.pol != 0 && x0 == 0;
+  double wv = 0.0;
+  const bool has_lo = __any_sync(0xffffffffu, wall_lo), has_hi = __any_sync(0xffffffffu, wall_hi);
+  const auto row = [&](int j) {  // y0 + j, wrapped (rows -1 .. rows + 1 are asked for)
+    int y = y0 + j;
+    while (y >= a.n1) y -= a.n1;
+    return (y < 0 ? a.n1 - 1 : y) * a.n0 + i;  // (cells stay below 2^30)
+  };
+  R e[3], en[3], bh[3], bhm[3], ep[3], epm[3], bhp[3];
+  R b[3], jv[3], bn[3], jn[3], enn[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int g = row(-1), g1 = row(0);
+    e[c] = a.E[c][g];
+    en[c] = a.E[c][g1];
+    b[c] = a.B[c][g];
+    jv[c] = R(0);
+    bhm[c] = epm[c] = bhp[c] = R(0);
+  }
+  const R hh = R(0.5) * a.h;
+  for (int j = -1; j <= rows; ++j) {
+    // the next pass's loads first
+    if (j < rows) {
+      const int g1 = row(j + 1), g2 = row(j + 2);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        bn[c] = a.B[c][g1];
+        jn[c] = a.J[c][g1];
+        enn[c] = a.E[c][g2];
+      }
+    }
+    // B half: B - h/2 curl E (rows j, j + 1)
+    {
+      const R eyx = __shfl_down_sync(0xffffffffu, e[1], 1), ezx = __shfl_down_sync(0xffffffffu, e[2], 1);
+      const R cx = (en[2] - e[2]) * a.rdy;
+      const R cy = -(ezx - e[2]) * a.rdx;
+      const R cz = (eyx - e[1]) * a.rdx - (en[0] - e[0]) * a.rdy;
+      bh[0] = b[0] - hh * cx;
+      bh[1] = wall_hi ? b[1] : b[1] - hh * cy;  // By, Bz half a cell beyond the last node
+      bh[2] = wall_hi ? b[2] : b[2] - hh * cz;
+    }
+    // E: E + h (curl B - J) (rows j - 1, j)
+    const R byx = __shfl_up_sync(0xffffffffu, bh[1], 1), bzx = __shfl_up_sync(0xffffffffu, bh[2], 1);
+    if (j >= 0) {
+      const R cx = (bh[2] - bhm[2]) * a.rdy;
+      const R cy = -(bh[2] - bzx) * a.rdx;
+      const R cz = (bh[1] - byx) * a.rdx - (bh[0] - bhm[0]) * a.rdy;
+      ep[0] = wall_hi ? e[0] : e[0] + a.h * (cx - jv[0]);
+      ep[1] = wall_hi || wall_lo ? e[1] : e[1] + a.h * (cy - jv[1]);
+      ep[2] = wall_hi || wall_lo ? e[2] : e[2] + a.h * (cz - jv[2]);
+      if (a.absorb) {
+        if (wave && j % 8 == 0) {
+          // rows j .. j + 7: value lane % 4 of row lane / 4
+          const int y = (y0 + j + lane / 4) % a.n1;
+          const int v = lane % 4;
+          if (a.ls.oblique)
+            wv = laser_wave(a.ls, (v & 1) ? a.ls.dx : 0.0, (y + (a.ls.pol == 1 ? 0.5 : 0.0)) * a.ls.dy,
+                            a.ls.pol == 2 ? 0.5 * a.ls.dz : 0.0, v < 2 ? a.ls.t_old : a.ls.t_new);
+          else
+            wv = a.ls.prof[y] * a.ls.amp[v];
+        }
+        // (only the warps that hold a wall's column take these branches: left
+        // to every warp, the FP64 of the two lines cost three times the rest)
+        if (has_lo) {
+          double l[4];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) l[v] = __shfl_sync(0xffffffffu, wv, (j & 7) * 4 + v);
+#pragma unroll
+          for (int c = 1; c < 3; ++c) {
+            // the neighbour inside, at the old and at the new time
+            const R oi = __shfl_down_sync(0xffffffffu, e[c], 1), ni = __shfl_down_sync(0xffffffffu, ep[c], 1);
+            const bool in = wave && a.ls.pol == c;
+            const double s0o = (double)e[c] - (in ? l[0] : 0.0), s1o = (double)oi - (in ? l[1] : 0.0);
+            const double s1n = (double)ni - (in ? l[3] : 0.0);
+            if (wall_lo) ep[c] = (R)((in ? l[2] : 0.0) + s1o + a.kc * (s1n - s0o));
+          }
+        }
+        if (has_hi)
+#pragma unroll
+          for (int c = 1; c < 3; ++c) {
+            const R ox = __shfl_up_sync(0xffffffffu, e[c], 1), nx = __shfl_up_sync(0xffffffffu, ep[c], 1);
+            if (wall_hi) ep[c] = (R)((double)ox + a.kc * ((double)nx - (double)e[c]));
+          }
+      }
+    }
+    // B half of the row before: B - h/2 curl E (rows j - 1, j), and the results
+    const R eyx = __shfl_down_sync(0xffffffffu, epm[1], 1), ezx = __shfl_down_sync(0xffffffffu, epm[2], 1);
+    if (j >= 1 && mine) {
+      const R cx = (ep[2] - epm[2]) * a.rdy;
+      const R cy = -(ezx - epm[2]) * a.rdx;
+      const R cz = (eyx - epm[1]) * a.rdx - (ep[0] - epm[0]) * a.rdy;
+      const int g = (y0 + j - 1) * a.n0 + i;
+      a.B2[0][g] = bhp[0] - hh * cx;
+      a.B2[1][g] = wall_hi ? bhp[1] : bhp[1] - hh * cy;
+      a.B2[2][g] = wall_hi ? bhp[2] : bhp[2] - hh * cz;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        a.E2[c][g] = epm[c];
+        a.Jn[c][g] = R(0);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      bhm[c] = bhp[c] = bh[c];
+      epm[c] = ep[c];
+      e[c] = en[c];
+      en[c] = enn[c];
+      b[c] = bn[c];
+      jv[c] = jn[c];
+    }
+  }
 }
 
 // ---- particle load: global (x, y, z) -> (cell, offset) ----
@@ -638,12 +781,10 @@ template <class R> void yee_b_t(const Grid &g, void *const E[3], void *const B[3
   if (yee_vec_ok<R>(g, a, false)) {
     dim3 grid, block;
     yee_vec_shape<R>(g, grid, block);
-    if (g.dims == 3) k_yee_b_vec<R, 3><<<grid, block, 0, st>>>(a);
-    else k_yee_b_vec<R, 2><<<grid, block, 0, st>>>(a);
+    k_yee_b_vec<R><<<grid, block, 0, st>>>(a);
   } else {
     const int nb = grid_blocks(g.ncell, 256);
-    if (g.dims == 3) k_yee_b<R, 3><<<nb, 256, 0, st>>>(a);
-    else k_yee_b<R, 2><<<nb, 256, 0, st>>>(a);
+    k_yee_b<R><<<nb, 256, 0, st>>>(a);
   }
 }
 
@@ -653,12 +794,10 @@ void yee_e_t(const Grid &g, void *const E[3], void *const B[3], void *const J[3]
   if (yee_vec_ok<R>(g, a, true)) {
     dim3 grid, block;
     yee_vec_shape<R>(g, grid, block);
-    if (g.dims == 3) k_yee_e_vec<R, 3><<<grid, block, 0, st>>>(a);
-    else k_yee_e_vec<R, 2><<<grid, block, 0, st>>>(a);
+    k_yee_e_vec<R><<<grid, block, 0, st>>>(a);
   } else {
     const int nb = grid_blocks(g.ncell, 256);
-    if (g.dims == 3) k_yee_e<R, 3><<<nb, 256, 0, st>>>(a);
-    else k_yee_e<R, 2><<<nb, 256, 0, st>>>(a);
+    k_yee_e<R><<<nb, 256, 0, st>>>(a);
   }
 }
 
@@ -673,6 +812,56 @@ cudaError_t launch_yee_e(const Grid &g, void *const E[3], void *const B[3], void
   if (g.prec == 1) yee_e_t<double>(g, E, B, J, h, st);
   else yee_e_t<float>(g, E, B, J, h, st);
   return cudaGetLastError();
+}
+
+template <class R>
+static cudaError_t field_step2_t(const Grid &g, void *const E[3], void *const B[3], void *const J[3],
+                                 void *const E2[3], void *const B2[3], void *const Jn[3], const LaserStep &ls,
+                                 unsigned long long *counters, int ncounters, cudaStream_t st) {
+  FieldStep2<R> a;
+  a.n0 = g.n[0];
+  a.n1 = g.n[1];
+  a.absorb = g.absorb_lo || g.absorb_hi;
+  // (the right wall's node needs the column before it: not the first of a strip)
+  a.width = kStripW;
+  while (a.absorb && a.n0 % a.width == 1) --a.width;
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  // long strips recompute less (rows + 3 rows are read), short ones give more
+  // warps: the longest that make 64 warps per SM (2048 x 1024 FP32: 36 us, 47
+  // with 16 warps per SM), down to one row (64 x 64 FP64: 6.2 us, 9.1 with
+  // three).  An oblique wave is evaluated for eight rows at a time.
+  const int64_t strips = (a.n0 + a.width - 1) / a.width;
+  const int least = ls.oblique ? 7 : 1;
+  a.rows = 31;
+  while (a.rows > least && strips * ((a.n1 + a.rows - 1) / a.rows) < 64 * (int64_t)nsm) a.rows /= 2;
+  a.rdx = (R)(1.0 / g.dx[0]);
+  a.rdy = (R)(1.0 / g.dx[1]);
+  a.h = (R)g.dt;
+  for (int d = 0; d < 3; ++d) {
+    a.E[d] = static_cast<const R *>(E[d]);
+    a.B[d] = static_cast<const R *>(B[d]);
+    a.J[d] = static_cast<const R *>(J[d]);
+    a.E2[d] = static_cast<R *>(E2[d]);
+    a.B2[d] = static_cast<R *>(B2[d]);
+    a.Jn[d] = static_cast<R *>(Jn[d]);
+  }
+  a.kc = (g.dt - g.dx[0]) / (g.dt + g.dx[0]);
+  a.ls = ls;
+  a.counters = counters;
+  a.ncounters = ncounters;
+  a.strips = (unsigned)strips;
+  k_field_step2<R><<<(unsigned)(strips * ((a.n1 + 2 * a.rows - 1) / (2 * a.rows))), 64, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_field_step2(const Grid &g, void *const E[3], void *const B[3], void *const J[3], void *const E2[3],
+                               void *const B2[3], void *const Jn[3], const LaserStep &ls,
+                               unsigned long long *counters, int ncounters, cudaStream_t st) {
+  if (g.dims != 2) return cudaErrorInvalidValue;
+  if (g.prec == 1) return field_step2_t<double>(g, E, B, J, E2, B2, Jn, ls, counters, ncounters, st);
+  return field_step2_t<float>(g, E, B, J, E2, B2, Jn, ls, counters, ncounters, st);
 }
 
 cudaError_t launch_mur_save(const Grid &g, void *const E[3], double *buf, cudaStream_t st) {

@@ -235,12 +235,16 @@ __device__ __forceinline__ double rcp_near(double x) { return 1.0 / x; }
 
 // Boris rotation in the variable u = gamma v (ref [8] of the paper; §2 eq. 3):
 // half electric kick, magnetic rotation, half electric kick.  h = q dt/(2m).
-template <class R>
+// kIeee: with IEEE root and quotients, as the adjoint kernels recompute the
+// step (2D).
+template <class R, bool kIeee>
 __device__ __forceinline__ void boris(R h, const R E[3], const R B[3], R u[3]) {
   const R umx = u[0] + h * E[0], umy = u[1] + h * E[1], umz = u[2] + h * E[2];
-  const R ig = rsqrt_near(R(1) + umx * umx + umy * umy + umz * umz);
+  const R g2 = R(1) + umx * umx + umy * umy + umz * umz;
+  const R ig = kIeee ? R(1) / sqrt(g2) : rsqrt_near(g2);
   const R tx = h * B[0] * ig, ty = h * B[1] * ig, tz = h * B[2] * ig;
-  const R sf = R(2) * rcp_near(R(1) + tx * tx + ty * ty + tz * tz);
+  const R den = R(1) + tx * tx + ty * ty + tz * tz;
+  const R sf = kIeee ? R(2) / den : R(2) * rcp_near(den);
   const R sx = sf * tx, sy = sf * ty, sz = sf * tz;
   const R upx = umx + (umy * tz - umz * ty);
   const R upy = umy + (umz * tx - umx * tz);

@@ -156,9 +156,10 @@ constexpr int kAdjItem = 512;
 
 // Tile kernel (one block per work item) + escape kernel.
 // esc_list (one int per slot) is scratch for particles deferred to the
-// escape kernel; esc_count (three counters) receives their number and the
-// number of particles whose shape support changed in the launch, and counts
-// the work items that blocks took.
+// escape kernel; esc_count (kEscCounters counters, zero at the launch) receives
+// their number and the number of particles whose shape support changed, and
+// counts the work items that blocks took.
+constexpr int kEscCounters = 4;
 constexpr int kCrowdedJobs = 168;  // such particles per work item above which a species counts as crowded (pic_diag)
 cudaError_t launch_push(const Grid &g, void *const E[3], void *const B[3], void *const J[3], const Particles &p,
                         const WorkSplit &ws, int32_t *esc_list, unsigned long long *esc_count, double q, double m,
@@ -181,6 +182,7 @@ cudaError_t launch_sort(const Grid &g, const Particles &src, const Particles &ds
                         const WorkSplit &ws, Counters *ctr, cudaStream_t st, int *nlaunch);
 
 // ---- fields and particle conversion (fields.cu) ----
+// The updates of a 3D step.
 cudaError_t launch_yee_b(const Grid &g, void *const E[3], void *const B[3], double h, cudaStream_t st);
 cudaError_t launch_yee_e(const Grid &g, void *const E[3], void *const B[3], void *const J[3], double h,
                          cudaStream_t st);
@@ -190,6 +192,12 @@ cudaError_t launch_yee_e(const Grid &g, void *const E[3], void *const B[3], void
 cudaError_t launch_mur_save(const Grid &g, void *const E[3], double *buf, cudaStream_t st);
 cudaError_t launch_mur_apply(const Grid &g, void *const E[3], const double *buf, const LaserStep &ls,
                              cudaStream_t st);
+// The three updates of a 2D step, with the Mur walls and the incoming wave
+// (ls; pol = 0 without one), from E, B, J into E2, B2; Jn is cleared, and so
+// are the ncounters counters.
+cudaError_t launch_field_step2(const Grid &g, void *const E[3], void *const B[3], void *const J[3], void *const E2[3],
+                               void *const B2[3], void *const Jn[3], const LaserStep &ls,
+                               unsigned long long *counters, int ncounters, cudaStream_t st);
 // Load n particles into slots [offset, offset+n).
 cudaError_t launch_load(const Grid &g, const Particles &p, int64_t offset, int64_t n, const double *x,
                         const double *y, const double *z, const double *ux, const double *uy, const double *uz,

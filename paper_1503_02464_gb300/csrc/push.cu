@@ -16,6 +16,8 @@
 // k_push_escaped applies the same arithmetic on global memory afterwards.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "pic_device.cuh"
 
 namespace pic {
@@ -67,9 +69,9 @@ template <int DIM, int ORDER> struct Geo {
 template <class R, int DIM, int ORDER> struct Lay {
   using G = Geo<DIM, ORDER>;
   static constexpr bool F32 = sizeof(R) == 4;
-  static constexpr int CAP = F32 ? (DIM == 2 ? 1408 : ORDER == 1 ? 1216 : 2176) : (DIM == 3 ? 2432 : 1664);
-  // per SM (FP32: 2D at three 4 % slower, 3D CIC at two 19 %)
-  static constexpr int BLOCKS = F32 ? (DIM == 2 ? 4 : ORDER == 1 ? 3 : 2) : (DIM == 3 ? 1 : 2);
+  static constexpr int CAP = F32 ? (DIM == 2 ? 1920 : ORDER == 1 ? 1216 : 2176) : (DIM == 3 ? 2432 : 1664);
+  // per SM (FP32: 2D at four, with 64 registers, 10 % slower on the slab; 3D CIC at two 19 %)
+  static constexpr int BLOCKS = F32 ? (ORDER == 1 || DIM == 2 ? 3 : 2) : (DIM == 3 ? 1 : 2);
   // a particle (offsets, momenta, weight), then its job (old and new offsets, 2D3V: vz, weight)
   static constexpr int NJ = DIM == 3 ? 7 : 6;
   // particles one thread sums at a time (3D: 6 beat 5, 7, 8, 12 and 16 by up
@@ -382,6 +384,27 @@ template <class R, int ORDER> struct SettledAxis {
   }
 };
 
+// A running sum of contributions p q in registers.  FloatSum: one FMA.
+// FixedSum: the two fixed-point words of WinAcc<float>::add, so that the sum is
+// exact and does not depend on the order of the particles: what a 2D FP32 run
+// does (the runs with an adjoint, whose segments are run twice and have to
+// repeat themselves); its stencil has 21 sums where 3D TSC has 54.
+template <class R> struct FloatSum {
+  R v;
+  __device__ __forceinline__ void clear() { v = R(0); }
+  __device__ __forceinline__ void add(R p, R q) { v += p * q; }
+};
+struct FixedSum {
+  int hi, lo;
+  __device__ __forceinline__ void clear() { hi = lo = 0; }
+  __device__ __forceinline__ void add(float p, float q) {
+    const float y = fmaf(p, q, WinAcc<float>::kMagicHi);
+    const float z = fmaf(p, q, -(y - WinAcc<float>::kMagicHi)) + WinAcc<float>::kMagic;  // rounds to an integer
+    hi += __float_as_int(y) - __float_as_int(WinAcc<float>::kMagicHi);
+    lo += __float_as_int(z) - __float_as_int(WinAcc<float>::kMagic);
+  }
+};
+
 // The settled contributions of the particles of one node, summed in
 // registers: add() one particle, flush() the sums into the J window once per
 // group.  Same brackets as deposit_win: Jx gets
@@ -392,12 +415,16 @@ template <class R, int DIM, int ORDER> struct GroupSum {
   static constexpr int NS = ORDER + 1, M = ORDER;
   static constexpr int NA = DIM == 3 ? M * NS * NS : M * NS;  // Jx, Jy sums
   static constexpr int NZ = DIM == 3 ? M * NS * NS : NS * NS;  // Jz sums
-  R jx[NA], jy[NA], jz[NZ];
+  using S = typename std::conditional<sizeof(R) == 4 && DIM == 2, FixedSum, FloatSum<R>>::type;
+  S jx[NA], jy[NA], jz[NZ];
   __device__ __forceinline__ void clear() {
 #pragma unroll
-    for (int i = 0; i < NA; ++i) jx[i] = jy[i] = R(0);
+    for (int i = 0; i < NA; ++i) {
+      jx[i].clear();
+      jy[i].clear();
+    }
 #pragma unroll
-    for (int i = 0; i < NZ; ++i) jz[i] = R(0);
+    for (int i = 0; i < NZ; ++i) jz[i].clear();
   }
   __device__ __forceinline__ void add(const SettledAxis<R, ORDER> &X, const SettledAxis<R, ORDER> &Y,
                                       const SettledAxis<R, ORDER> &Z, R cx, R cy, R cz, R qwvz) {
@@ -434,7 +461,7 @@ template <class R, int DIM, int ORDER> struct GroupSum {
         for (int b = 0; b < NS; ++b) {
           const R br = Y.S0[b] * hz[c] + Y.DS[b] * tz[c];
 #pragma unroll
-          for (int a = 0; a < M; ++a) jx[(c * NS + b) * M + a] += Px[a] * br;
+          for (int a = 0; a < M; ++a) jx[(c * NS + b) * M + a].add(Px[a], br);
         }
 #pragma unroll
       for (int c = 0; c < NS; ++c)
@@ -442,7 +469,7 @@ template <class R, int DIM, int ORDER> struct GroupSum {
         for (int a = 0; a < NS; ++a) {
           const R br = Z.S0[c] * hx[a] + Z.DS[c] * tx[a];
 #pragma unroll
-          for (int b = 0; b < M; ++b) jy[(c * NS + a) * M + b] += Py[b] * br;
+          for (int b = 0; b < M; ++b) jy[(c * NS + a) * M + b].add(Py[b], br);
         }
 #pragma unroll
       for (int b = 0; b < NS; ++b) {
@@ -452,7 +479,7 @@ template <class R, int DIM, int ORDER> struct GroupSum {
         for (int a = 0; a < NS; ++a) {
           const R br = X.S0[a] * hy + X.DS[a] * ty;
 #pragma unroll
-          for (int c = 0; c < M; ++c) jz[(b * NS + a) * M + c] += Pz[c] * br;
+          for (int c = 0; c < M; ++c) jz[(b * NS + a) * M + c].add(Pz[c], br);
         }
       }
     } else {
@@ -461,15 +488,15 @@ template <class R, int DIM, int ORDER> struct GroupSum {
         const R hy = Y.S0[b] + R(0.5) * Y.DS[b];
         const R ty = R(0.5) * Y.S0[b] + Y.DS[b] * R(1.0 / 3.0);
 #pragma unroll
-        for (int a = 0; a < M; ++a) jx[b * M + a] += Px[a] * hy;
+        for (int a = 0; a < M; ++a) jx[b * M + a].add(Px[a], hy);
 #pragma unroll
-        for (int a = 0; a < NS; ++a) jz[b * NS + a] += qwvz * (X.S0[a] * hy + X.DS[a] * ty);
+        for (int a = 0; a < NS; ++a) jz[b * NS + a].add(qwvz, X.S0[a] * hy + X.DS[a] * ty);
       }
 #pragma unroll
       for (int a = 0; a < NS; ++a) {
         const R hx = X.S0[a] + R(0.5) * X.DS[a];
 #pragma unroll
-        for (int b = 0; b < M; ++b) jy[a * M + b] += Py[b] * hx;
+        for (int b = 0; b < M; ++b) jy[a * M + b].add(Py[b], hx);
       }
     }
   }
@@ -517,11 +544,14 @@ template <class R, int DIM, int ORDER> struct GroupSum {
 template <class R, int JS> struct GroupSink;
 template <int JS> struct GroupSink<float, JS> {
   unsigned sb;  // byte address of the Jx low word of the stencil's first node
-  __device__ __forceinline__ void add(int comp, int off, float v) const {
-    const float y = v + WinAcc<float>::kMagicHi;
+  __device__ __forceinline__ void add(int comp, int off, FixedSum s) const { put(comp, off, s.hi, s.lo); }
+  __device__ __forceinline__ void add(int comp, int off, FloatSum<float> s) const {
+    const float v = s.v, y = v + WinAcc<float>::kMagicHi;
     const float lf = v - (y - WinAcc<float>::kMagicHi);
     const int hi = __float_as_int(y) - __float_as_int(WinAcc<float>::kMagicHi);
-    const int lo = __float2int_rn(lf);
+    put(comp, off, hi, __float2int_rn(lf));
+  }
+  __device__ __forceinline__ void put(int comp, int off, int hi, int lo) const {
     const unsigned sa = sb + 8u * (unsigned)JS * (unsigned)comp + 4u * (unsigned)off;
     asm volatile("red.shared.add.s32 [%0], %1;\n\tred.shared.add.s32 [%2], %3;" ::"r"(sa), "r"(lo),
                  "r"(sa + 4u * (unsigned)JS), "r"(hi));
@@ -529,8 +559,8 @@ template <int JS> struct GroupSink<float, JS> {
 };
 template <int JS> struct GroupSink<double, JS> {
   double *w;  // Jx value of the stencil's first node (components JS doubles apart)
-  __device__ __forceinline__ void add(int comp, int off, double v) const {
-    if (v != 0.0) atomicAdd(w + comp * JS + off, v);
+  __device__ __forceinline__ void add(int comp, int off, FloatSum<double> s) const {
+    if (s.v != 0.0) atomicAdd(w + comp * JS + off, s.v);
   }
 };
 
@@ -555,24 +585,6 @@ template <int T> __device__ __forceinline__ unsigned long long task_counts(unsig
   static_assert(T == 6 || T == 8, "classes");
   const unsigned full = c / T, rest = c % T;
   return (unsigned long long)full + (rest ? 1ull << (10 * task_class<T>(rest)) : 0ull);
-}
-
-// Ascending order of N = 8 values by Batcher's odd-even merge sort (19
-// compare-exchanges).
-__device__ __forceinline__ void sort8(uint32_t (&v)[8]) {
-#pragma unroll
-  for (int p = 1; p < 8; p *= 2)
-#pragma unroll
-    for (int k = p; k >= 1; k /= 2)
-#pragma unroll
-      for (int j = k % p; j + k < 8; j += 2 * k)
-#pragma unroll
-        for (int i = 0; i < k; ++i)
-          if (i + j + k < 8 && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
-            const uint32_t lo = min(v[i + j], v[i + j + k]), hi = max(v[i + j], v[i + j + k]);
-            v[i + j] = lo;
-            v[i + j + k] = hi;
-          }
 }
 
 // A moved offset x (at most one cell away under the Courant limit) brought
@@ -604,7 +616,7 @@ template <> __device__ __forceinline__ double carry<double>(double x, int &sh, u
 template <class R, int ORDER, int DIM>
 __device__ __forceinline__ void push_move(const PushArgs<R> &a, R u[3], const R E[3], const R B[3], const R f[3],
                                           R fn[3], int s[3], R &ig, unsigned &clamp) {
-  boris<R>(a.qmh, E, B, u);
+  boris<R, DIM == 2>(a.qmh, E, B, u);
   ig = inv_sqrt<R>(R(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -1047,25 +1059,6 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
         const unsigned tk = sTask[unit - nchg32];
         int j = tk & 4095u;
         const int je = j + (int)(tk >> 12) + 1;
-        if constexpr (sizeof(R) == 4 && DIM == 2) {
-          // The job order within a group depends on the order in which warps
-          // reached its counter.  FP32 2D runs (those with an adjoint, whose
-          // segments are run twice) sum a task in the order of the old x
-          // offsets instead, so that a group of one task has one sum.
-          const int len = je - j;
-          if (len > 1) {
-            uint32_t v[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const uint32_t o = i < len ? sOrder[j + i] : 0u;
-              v[i] = i < len ? (__float_as_uint((float)sJob[o] + 1.5f) << 9 & 0xfffff000u) | o : 0xffffffffu;
-            }
-            sort8(v);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              if (i < len) sOrder[j + i] = (uint16_t)(v[i] & 4095u);
-          }
-        }
         int s = sOrder[j];
         const uint32_t group = sTag[s] & 1023u;
         const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
@@ -1360,8 +1353,6 @@ cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *co
   constexpr size_t smem = Lay<R, DIM, ORDER>::kEnd;
   auto fn = k_push<R, DIM, ORDER, EC>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(esc_count, 0, 3 * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
