@@ -110,7 +110,8 @@ struct pic_handle {
   size_t rsize = 4;
   void *E[3] = {}, *B[3] = {}, *J[3] = {};
   // 2D: the fields a step writes (then they trade places with E, B), and the
-  // J buffer of the next step, which is zero between steps
+  // J buffer of the next step, which is zero between steps; runs with current
+  // smoothing: J2 is its scratch (in 2D before the field update clears it)
   void *E2[3] = {}, *B2[3] = {}, *J2[3] = {};
   double *rho_bg = nullptr, *rho = nullptr, *rho_prev = nullptr, *f64 = nullptr, *red = nullptr;
   int64_t rho_prev_step = -2;
@@ -593,17 +594,17 @@ int pic_create(const pic_config *cfg, pic_handle **out) {
   // E, B in one block (a checkpoint copies them with one memcpy) and the
   // three J components in another (one memset clears J)
   bool ok = cudaMalloc(&h->E[0], 6 * fb) == cudaSuccess && cudaMalloc(&h->J[0], 3 * fb) == cudaSuccess;
-  if (g.dims == 2)
-    ok = ok && cudaMalloc(&h->E2[0], 6 * fb) == cudaSuccess && cudaMalloc(&h->J2[0], 3 * fb) == cudaSuccess;
+  if (g.dims == 2) ok = ok && cudaMalloc(&h->E2[0], 6 * fb) == cudaSuccess;
+  if (g.dims == 2 || c.filter_passes > 0) ok = ok && cudaMalloc(&h->J2[0], 3 * fb) == cudaSuccess;
   if (ok)
     for (int d = 0; d < 3; ++d) {
       h->E[d] = static_cast<char *>(h->E[0]) + d * fb;
       h->B[d] = static_cast<char *>(h->E[0]) + (3 + d) * fb;
       h->J[d] = static_cast<char *>(h->J[0]) + d * fb;
-      if (g.dims != 2) continue;
+      if (h->J2[0]) h->J2[d] = static_cast<char *>(h->J2[0]) + d * fb;
+      if (!h->E2[0]) continue;
       h->E2[d] = static_cast<char *>(h->E2[0]) + d * fb;
       h->B2[d] = static_cast<char *>(h->E2[0]) + (3 + d) * fb;
-      h->J2[d] = static_cast<char *>(h->J2[0]) + d * fb;
     }
   const size_t db = (size_t)ncell * sizeof(double);
   const int64_t nkeys = g.ntiles * g.tile[0] * g.tile[1] * g.tile[2];
@@ -1300,14 +1301,15 @@ int pic_step(pic_handle *h, int nsteps) {
     }
     if (h->cfg.filter_passes > 0) {
       Timed tm(h, pic::KC_FILTER);
-      for (int d = 0; d < 3; ++d) {
-        int nl = 0;
-        CK(h,
-           pic::launch_smooth(h->g, h->J[d], false, h->f64, h->cfg.filter_passes, h->cfg.filter_compensate, h->st,
-                              &nl),
-           "smooth J");
-        h->launches += nl;
-      }
+      int nl = 0;
+      bool in_tmp = false;
+      CK(h,
+         pic::launch_smooth(h->g, h->J[0], 3, false, h->J2[0], h->cfg.filter_passes, h->cfg.filter_compensate, h->st,
+                            &nl, &in_tmp),
+         "smooth J");
+      if (in_tmp)
+        for (int d = 0; d < 3; ++d) std::swap(h->J[d], h->J2[d]);
+      h->launches += nl;
     }
     const pic::LaserStep wave = pic::laser_step(h->laser, h->laser_prof, h->laser.a0, h->g, h->step * h->g.dt,
                                                 (h->step + 1) * h->g.dt);
@@ -1444,8 +1446,12 @@ int pic_diag(pic_handle *h, pic_diag_t *out) {
   if (h->cfg.filter_passes > 0) {
     // Gauss's law and continuity hold for the equally smoothed charge
     int nl = 0;
-    CK(h, pic::launch_smooth(h->g, h->rho, true, h->f64, h->cfg.filter_passes, h->cfg.filter_compensate, h->st, &nl),
+    bool in_tmp = false;
+    CK(h,
+       pic::launch_smooth(h->g, h->rho, 1, true, h->f64, h->cfg.filter_passes, h->cfg.filter_compensate, h->st, &nl,
+                          &in_tmp),
        "smooth rho");
+    if (in_tmp) std::swap(h->rho, h->f64);
     h->launches += nl;
   }
   CK(h, cudaMemsetAsync(h->red, 0, 16 * sizeof(double), h->st), "memset");

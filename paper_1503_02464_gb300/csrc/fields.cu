@@ -716,64 +716,90 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) atomicAdd(out + 2, v);
 }
 
-// One smoothing pass along `axis`: out = alpha in + side (in[-1] + in[+1]),
-// periodic (side = (1 - alpha)/2).  A Fourier mode exp(i k x) is multiplied
-// by alpha + (1 - alpha) cos(k dx).
-template <class R>
-__global__ void __launch_bounds__(256)
-    k_smooth_axis(const R *__restrict__ in, R *__restrict__ out, int n0, int n1, int n2, int axis, R alpha, R side) {
-  const int64_t ncell = (int64_t)n0 * n1 * n2;
-  const int64_t sy = n0, sz = (int64_t)n0 * n1;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
-    int64_t lo, hi;
-    if (axis == 0) {
-      const int i = (int)(c % n0);
-      lo = c + (i > 0 ? -1 : n0 - 1);
-      hi = c + (i + 1 < n0 ? 1 : 1 - n0);
-    } else if (axis == 1) {
-      const int j = (int)((c / n0) % n1);
-      lo = c + (j > 0 ? -sy : sy * (n1 - 1));
-      hi = c + (j + 1 < n1 ? sy : sy - sy * n1);
-    } else {
-      const int k = (int)(c / sz);
-      lo = c + (k > 0 ? -sz : sz * (n2 - 1));
-      hi = c + (k + 1 < n2 ? sz : sz - sz * n2);
+// All the smoothing passes along one axis at once: the taps of the passes
+// convolved, out = w[0] in + sum_k w[k] (in[-k] + in[+k]), periodic, on `ncomp`
+// fields back to back.  The passes of the axes commute, so a launch per axis
+// does what a launch per pass, axis and field did (27 launches for J in 3D with
+// two passes and compensation, 126 us on 75 x 50 x 43 FP32; three launches and
+// 13 us now).  The taps come from the cache: every value is read once per tap.
+constexpr int kSmoothRadius = 9;  // eight binomial passes and a compensating one
+template <class R> struct SmoothArgs {
+  const R *in;
+  R *out;
+  int n0, n1, n2, ncomp, axis, radius;
+  R w[kSmoothRadius + 1];
+};
+template <class R> __global__ void __launch_bounds__(256) k_smooth_axis(const __grid_constant__ SmoothArgs<R> a) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= a.n0) return;
+  const int len = a.axis == 0 ? a.n0 : a.axis == 1 ? a.n1 : a.n2;
+  const int64_t step = a.axis == 0 ? 1 : a.axis == 1 ? a.n0 : (int64_t)a.n0 * a.n1;
+  for (int64_t kc = blockIdx.z; kc < (int64_t)a.n2 * a.ncomp; kc += gridDim.z) {
+    for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < a.n1; j += gridDim.y * blockDim.y) {
+      const int64_t c = i + a.n0 * (j + a.n1 * kc);
+      const int at = a.axis == 0 ? i : a.axis == 1 ? j : (int)(kc % a.n2);
+      const R *line = a.in + (c - at * step);
+      R v = a.w[0] * a.in[c];
+      int lo = at, hi = at;
+      for (int k = 1; k <= a.radius; ++k) {
+        lo = lo > 0 ? lo - 1 : len - 1;
+        hi = hi + 1 < len ? hi + 1 : 0;
+        v += a.w[k] * (line[lo * step] + line[hi * step]);
+      }
+      a.out[c] = v;
     }
-    out[c] = alpha * in[c] + side * (in[lo] + in[hi]);
   }
 }
 
 template <class R>
-cudaError_t smooth_t(const Grid &g, R *f, R *tmp, int passes, int compensate, cudaStream_t st, int *nlaunch) {
-  const int nb = grid_blocks(g.ncell, 256);
-  R *src = f, *dst = tmp;
-  int nl = 0;
-  auto pass = [&](int axis, double alpha) {
-    k_smooth_axis<R><<<nb, 256, 0, st>>>(src, dst, g.n[0], g.n[1], g.n[2], axis, (R)alpha, (R)(0.5 * (1.0 - alpha)));
-    R *t = src;
-    src = dst;
-    dst = t;
-    ++nl;
+static cudaError_t smooth_t(const Grid &g, R *f, int ncomp, R *tmp, int passes, int compensate, cudaStream_t st,
+                            int *nlaunch, bool *in_tmp) {
+  // the taps at 0 .. radius of the passes (1/4, 1/2, 1/4) and (compensate) of
+  // (side, alpha, side), alpha = 1 + passes / 2, side = (1 - alpha) / 2
+  double w[kSmoothRadius + 2] = {1.0};
+  int radius = 0;
+  const auto convolve = [&](double alpha) {
+    const double side = 0.5 * (1.0 - alpha);
+    double o[kSmoothRadius + 2] = {};
+    for (int k = 0; k <= radius + 1; ++k)
+      o[k] = alpha * w[k] + side * ((k > 0 ? w[k - 1] : w[1]) + (k <= radius ? w[k + 1] : 0.0));
+    ++radius;
+    for (int k = 0; k <= radius; ++k) w[k] = o[k];
   };
-  for (int p = 0; p < passes; ++p)
-    for (int a = 0; a < g.dims; ++a) pass(a, 0.5);
-  if (compensate && passes > 0)
-    for (int a = 0; a < g.dims; ++a) pass(a, 1.0 + 0.5 * passes);
-  if (nlaunch) *nlaunch = nl;
-  if (src != f) {
-    const cudaError_t e = cudaMemcpyAsync(f, src, sizeof(R) * (size_t)g.ncell, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return e;
+  for (int p = 0; p < passes; ++p) convolve(0.5);
+  if (compensate) convolve(1.0 + 0.5 * passes);
+  SmoothArgs<R> a;
+  a.n0 = g.n[0];
+  a.n1 = g.n[1];
+  a.n2 = g.n[2];
+  a.ncomp = ncomp;
+  a.radius = radius;
+  for (int k = 0; k <= kSmoothRadius; ++k) a.w[k] = (R)(k <= radius ? w[k] : 0.0);
+  const dim3 block(64, 4, 1);
+  const int64_t planes = (int64_t)g.n[2] * ncomp;
+  const dim3 grid((a.n0 + 63) / 64, (a.n1 + 3) / 4 < 65535 ? (a.n1 + 3) / 4 : 65535, planes < 65535 ? planes : 65535);
+  for (a.axis = 0; a.axis < g.dims; ++a.axis) {
+    a.in = f;
+    a.out = tmp;
+    k_smooth_axis<R><<<grid, block, 0, st>>>(a);
+    R *t = f;
+    f = tmp;
+    tmp = t;
   }
+  if (nlaunch) *nlaunch = g.dims;
+  *in_tmp = g.dims % 2 == 1;
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_smooth(const Grid &g, void *f, bool f64, void *tmp, int passes, int compensate, cudaStream_t st,
-                          int *nlaunch) {
+cudaError_t launch_smooth(const Grid &g, void *f, int ncomp, bool f64, void *tmp, int passes, int compensate,
+                          cudaStream_t st, int *nlaunch, bool *in_tmp) {
   if (f64 || g.prec == 1)
-    return smooth_t<double>(g, static_cast<double *>(f), static_cast<double *>(tmp), passes, compensate, st, nlaunch);
-  return smooth_t<float>(g, static_cast<float *>(f), static_cast<float *>(tmp), passes, compensate, st, nlaunch);
+    return smooth_t<double>(g, static_cast<double *>(f), ncomp, static_cast<double *>(tmp), passes, compensate, st,
+                            nlaunch, in_tmp);
+  return smooth_t<float>(g, static_cast<float *>(f), ncomp, static_cast<float *>(tmp), passes, compensate, st, nlaunch,
+                         in_tmp);
 }
 
 template <class R> void yee_b_t(const Grid &g, void *const E[3], void *const B[3], double h, cudaStream_t st) {

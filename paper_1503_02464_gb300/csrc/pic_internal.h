@@ -225,12 +225,13 @@ cudaError_t launch_out_field(const Grid &g, const void *f, bool f64, const OutBo
 cudaError_t launch_out_particles(const Grid &g, const Particles &p, const int64_t *d_count, int64_t nmax,
                                  const OutBox &b, double *out, unsigned long long *count, int64_t cap,
                                  cudaStream_t st);
-// Current smoothing of one field in place: `passes` binomial passes along
-// every axis, then (compensate) one compensating pass.  f64 selects the
-// element type (double, else the grid's precision); tmp holds ncell elements
-// of that type.  *nlaunch receives the kernels launched.
-cudaError_t launch_smooth(const Grid &g, void *f, bool f64, void *tmp, int passes, int compensate, cudaStream_t st,
-                          int *nlaunch);
+// Current smoothing of ncomp fields back to back: `passes` binomial passes
+// along every axis, then (compensate) one compensating pass.  f64 selects the
+// element type (double, else the grid's precision); tmp holds as many elements
+// of that type, and the result where *in_tmp says so.  *nlaunch receives the
+// kernels launched.
+cudaError_t launch_smooth(const Grid &g, void *f, int ncomp, bool f64, void *tmp, int passes, int compensate,
+                          cudaStream_t st, int *nlaunch, bool *in_tmp);
 // n values between an array of the run's real type (prec: PIC_FP32 or
 // PIC_FP64) and FP64, on the device.
 cudaError_t launch_to_f64(int prec, const void *src, double *dst, int64_t n, cudaStream_t st);
