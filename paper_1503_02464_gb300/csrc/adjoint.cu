@@ -6,11 +6,12 @@
 //   gather F = G(x^n; E^n, B^n) -> Boris u^{n+1/2} -> move x^{n+1}
 //   -> Esirkepov J(x^n, x^{n+1}, w) -> B half / E (+ Mur walls, laser) / B half.
 // Reverse step n, given the adjoints of the state after the step:
-//   R5  adj_yee_b   lamE -= dt/2 C_B (M_B lamB)       (transpose of B half 2)
-//   R4  adj_mur     transpose of the Mur wall update; dF/da0 accumulates
-//   R3  adj_yee_e   lamJ = -dt M_E lamE; lamB += dt C_E (M_E lamE); + wall terms
-//   R1  adj_yee_b   lamE -= dt/2 C_B (M_B lamB)       (transpose of B half 1)
-//   P   adj_push    per particle: deposit^T, move^T, Boris^T, gather^T
+//   R5  lamE -= dt/2 C_B (M_B lamB)       (transpose of B half 2)
+//   R4  transpose of the Mur wall update; dF/da0 accumulates
+//   R3  lamJ = -dt M_E lamE; lamB += dt C_E (M_E lamE)
+//   R1  lamE -= dt/2 C_B (M_B lamB)       (transpose of B half 1); + wall terms
+//   P   per particle: deposit^T, move^T, Boris^T, gather^T
+// (R5 to R1 in k_adj_field_step, P in k_adj_push2d_win)
 // with C_B = C_E^T the Yee curls (curl B at E points, curl E at B points)
 // and M_B, M_E masks of the rows the forward updated.  Particle adjoints are
 // indexed by particle id; weight gradients accumulate in FP64.
@@ -31,148 +32,156 @@ int nblocks(int64_t n) {
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
-struct GridIdx {
-  int n0, n1, n2;
-  __device__ __forceinline__ void ijk(int64_t c, int &i, int &j, int &k) const {
-    i = (int)(c % n0);
-    const int64_t r = c / n0;
-    j = (int)(r % n1);
-    k = (int)(r / n1);
-  }
+// ---------------------------------------------------------------- fields
+// R5, R4, R3 and R1 of one reverse step in one pass, from lE, lB into lE2, lB2
+// and lJ: the transpose of the forward's fused update, built the same way (a
+// warp per strip of 29 columns and `rows` rows, one lane per column with two
+// lanes of halo below and one above, marching along y in registers).
+//   R5  lamE -= h/2 curl_at_E(M_B lamB): the transpose of "B -= h/2 curl_at_B(E)"
+//       over the rows the forward updated (By, Bz of the last x cell are not
+//       updated when the x walls absorb)
+//   R4  Mur walls (tangential components):  E0' = L0n + S1o + k (S1n - S0o),
+//       S = E - L (left, laser), E' = E(n0-2)o + k (E(n0-2)n - E(n0-1)o) (right).
+//       g = lamE(wall) is consumed (the wall value was overwritten), k g goes
+//       to the neighbour at the new time, g and -k g to the neighbour and the
+//       wall at the old time (with R1); dF/da0 += g dE0'/da0
+//   R3  lamJ = -h M_E lamE; lamB += h curl_at_B(M_E lamE)
+//   R1  as R5 with the new lamB, and R4's old-time terms
+// Four launches before, 37 us of the 256 x 256 FP32 run's reverse step with
+// their gaps; 10 us now.
+template <class R> struct AdjFieldStep {
+  int n0, n1, absorb, width, rows;
+  unsigned strips;
+  R rdx, rdy, h;
+  const R *lE[3], *lB[3];
+  R *lE2[3], *lB2[3], *lJ[3];
+  double kc;
+  LaserStep ls;  // unit amplitude
+  double *da0;
 };
 
-// ---------------------------------------------------------------- fields
-// lamE -= h * curl_at_E(M_B lamB): the transpose of "B -= h curl_at_B(E)"
-// over the rows the forward updated (By, Bz of the last x cell are not
-// updated when the x walls absorb).
-//
-// With `pend` (the second B half, R1), the Mur transpose's terms for the
-// old time level (R4, kept in `pend` by k_adj_mur) are added to lamEy,
-// lamEz at the wall nodes in the same pass: both updates only add to lamE.
-template <class R, int DIM>
-__global__ void __launch_bounds__(256)
-    k_adj_yee_b(GridIdx g, int absorb, R rdx, R rdy, R rdz, R h, R *lE0, R *lE1, R *lE2, const R *lB0, const R *lB1,
-                const R *lB2, const double *pend) {
-  const int64_t ncell = (int64_t)g.n0 * g.n1 * g.n2;
-  const int64_t sy = g.n0, sz = (int64_t)g.n0 * g.n1;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
-    int i, j, k;
-    g.ijk(c, i, j, k);
-    const int64_t cxm = c - (i > 0 ? 1 : 1 - g.n0);
-    const int64_t cym = c - (j > 0 ? sy : sy - sy * g.n1);
-    const bool mx0 = absorb && i == g.n0 - 1;        // row (i) of By, Bz masked
-    const bool mxm = absorb && (i == 0);             // row (i-1) wraps to the last x cell
-    const R bx = lB0[c], by = mx0 ? R(0) : lB1[c], bz = mx0 ? R(0) : lB2[c];
-    const R bzym = mx0 ? R(0) : lB2[cym];
-    const R byxm = mxm ? R(0) : lB1[cxm], bzxm = mxm ? R(0) : lB2[cxm];
-    const R bxym = lB0[cym];
-    R cx = (bz - bzym) * rdy;
-    R cy = -(bz - bzxm) * rdx;
-    const R cz = (by - byxm) * rdx - (bx - bxym) * rdy;
-    if (DIM == 3) {
-      const int64_t czm = c - (k > 0 ? sz : sz - sz * g.n2);
-      const R byzm = mx0 ? R(0) : lB1[czm];
-      cx -= (by - byzm) * rdz;
-      cy += (bx - lB0[czm]) * rdz;
-    }
-    R py = R(0), pz = R(0);
-    if (pend && (i < 2 || i >= g.n0 - 2)) {
-      // pend slots: nodes 0, 1, n0-2, n0-1 (for Ey, then for Ez), per row
-      const int64_t nyz = (int64_t)g.n1 * g.n2, jk = c / g.n0;
-      const int nodes[4] = {0, 1, g.n0 - 2, g.n0 - 1};
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (nodes[q] == i) {
-          py += (R)pend[q * nyz + jk];
-          pz += (R)pend[(4 + q) * nyz + jk];
-        }
-    }
-    lE0[c] -= h * cx;
-    lE1[c] += py - h * cy;
-    lE2[c] += pz - h * cz;
-  }
-}
-
-// lamJ = -h M_E lamE ; lamB += h * curl_at_B(M_E lamE): the transpose of
-// "E += h (curl_at_E(B) - J)" over the updated rows (with absorbing walls:
-// Ex of the last x cell, Ey and Ez of the first and last x cells are not).
-template <class R, int DIM>
-__global__ void __launch_bounds__(256)
-    k_adj_yee_e(GridIdx g, int absorb, R rdx, R rdy, R rdz, R h, const R *lE0, const R *lE1, const R *lE2, R *lB0,
-                R *lB1, R *lB2, R *lJ0, R *lJ1, R *lJ2) {
-  const int64_t ncell = (int64_t)g.n0 * g.n1 * g.n2;
-  const int64_t sy = g.n0, sz = (int64_t)g.n0 * g.n1;
-  auto mex = [&](int i) { return absorb && i == g.n0 - 1; };
-  auto meyz = [&](int i) { return absorb && (i == 0 || i == g.n0 - 1); };
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
-    int i, j, k;
-    g.ijk(c, i, j, k);
-    const int ip = i + 1 < g.n0 ? i + 1 : 0;
-    const int64_t cxp = c + (i + 1 < g.n0 ? 1 : 1 - g.n0);
-    const int64_t cyp = c + (j + 1 < g.n1 ? sy : sy - sy * g.n1);
-    const R ex = mex(i) ? R(0) : lE0[c], ey = meyz(i) ? R(0) : lE1[c], ez = meyz(i) ? R(0) : lE2[c];
-    lJ0[c] = -h * ex;
-    lJ1[c] = -h * ey;
-    lJ2[c] = -h * ez;
-    const R ezyp = meyz(i) ? R(0) : lE2[cyp];
-    const R ezxp = meyz(ip) ? R(0) : lE2[cxp];
-    const R eyxp = meyz(ip) ? R(0) : lE1[cxp];
-    const R exyp = mex(i) ? R(0) : lE0[cyp];
-    R cx = (ezyp - ez) * rdy;
-    R cy = -(ezxp - ez) * rdx;
-    const R cz = (eyxp - ey) * rdx - (exyp - ex) * rdy;
-    if (DIM == 3) {
-      const int64_t czp = c + (k + 1 < g.n2 ? sz : sz - sz * g.n2);
-      const R eyzp = meyz(i) ? R(0) : lE1[czp];
-      const R exzp = mex(i) ? R(0) : lE0[czp];
-      cx -= (eyzp - ey) * rdz;
-      cy += (exzp - ex) * rdz;
-    }
-    lB0[c] += h * cx;
-    lB1[c] += h * cy;
-    lB2[c] += h * cz;
-  }
-}
-
-// Transpose of the Mur wall update (tangential components y, z):
-//   E0' = L0n + S1o + k (S1n - S0o),  S = E - L     (left wall, laser)
-//   Ez' = E(n0-2)o + k (E(n0-2)n - E(n0-1)o)      (right wall)
-// g = lamE(wall) is consumed (the wall value was overwritten), k g goes to
-// the neighbour at the new time, and g, -k g are kept in `pend` for the old
-// time (added to lamE by the R1 pass of k_adj_yee_b).  dF/da0 += g dE0'/da0
-// (the laser terms over a0).
-template <class R>
-__global__ void k_adj_mur(int n0, int n1, int n2, double dx, double dt, R *lEy, R *lEz, double *pend, LaserStep ls,
-                          double *da0) {
-  __shared__ double sh[32];
-  const int64_t nyz = (int64_t)n1 * n2;
-  const double kc = (dt - dx) / (dt + dx);
+template <class R> __global__ void __launch_bounds__(64) k_adj_field_step(const __grid_constant__ AdjFieldStep<R> a) {
+  const int lane = threadIdx.x & 31;
+  const int x0 = (int)(blockIdx.x % a.strips) * a.width;
+  const int y0 = (int)((blockIdx.x / a.strips * (blockDim.x / 32) + (threadIdx.x >> 5)) * a.rows);
+  if (y0 >= a.n1) return;
+  const int rows = min(a.rows, a.n1 - y0);
+  int i = x0 - 2 + lane;  // this lane's column, wrapped
+  const bool mine = lane >= 2 && lane < 2 + a.width && i < a.n0;
+  i %= a.n0;
+  if (i < 0) i += a.n0;
+  const bool wall_lo = a.absorb && i == 0, wall_hi = a.absorb && i == a.n0 - 1;
+  const bool in_lo = a.absorb && i == 1, in_hi = a.absorb && i == a.n0 - 2;
+  const bool has_lo = __any_sync(0xffffffffu, wall_lo), has_hi = __any_sync(0xffffffffu, wall_hi);
+  const auto row = [&](int j) {
+    int y = y0 + j;
+    while (y >= a.n1) y -= a.n1;
+    while (y < 0) y += a.n1;
+    return y * a.n0 + i;
+  };
+  // curl at the E places of b (row j) and bm (row j - 1)
+  const auto curl_e = [&](const R (&b)[3], const R (&bm)[3], R (&c)[3]) {
+    R byx = __shfl_up_sync(0xffffffffu, b[1], 1), bzx = __shfl_up_sync(0xffffffffu, b[2], 1);
+    if (wall_lo) byx = bzx = R(0);  // the last x cell's, masked
+    c[0] = (b[2] - bm[2]) * a.rdy;
+    c[1] = -(b[2] - bzx) * a.rdx;
+    c[2] = (b[1] - byx) * a.rdx - (b[0] - bm[0]) * a.rdy;
+  };
+  const R hh = R(0.5) * a.h;
   double acc = 0.0;
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < 2 * nyz; q += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(q / nyz);
-    const int64_t jk = q % nyz;
-    R *E = c == 0 ? lEy : lEz;
-    double *pd = pend + (int64_t)c * 4 * nyz;  // slots: node 0, 1, n0-2, n0-1
-    const int64_t row = (int64_t)n0 * jk;
-    const double g0 = (double)E[row];
-    E[row] = R(0);
-    E[row + 1] += (R)(kc * g0);
-    pd[0 * nyz + jk] = -kc * g0;
-    pd[1 * nyz + jk] = g0;
-    if (ls.pol == c + 1) {
-      // unit-amplitude laser terms at the wall row: P(row) times the waveform
-      const double p = ls.prof[jk];
-      const double l0o = p * ls.amp[0], l1o = p * ls.amp[1], l0n = p * ls.amp[2], l1n = p * ls.amp[3];
-      acc += g0 * (l0n - l1o - kc * l1n + kc * l0o);
-    }
-    const double gr = (double)E[row + n0 - 1];
-    E[row + n0 - 1] = R(0);
-    E[row + n0 - 2] += (R)(kc * gr);
-    pd[2 * nyz + jk] = gr;
-    pd[3 * nyz + jk] = -kc * gr;
+  R b[3], bm[3], bn[3], braw[3], e[3], en[3];  // lamB of rows j, j - 1 (masked), j + 1, j - 1; lamE of rows j, j + 1
+  R em[3], mem[3], pm[3], bpm[3];  // row j - 1: lamE after R4, masked for R3, R4's old-time terms; row j - 2: new lamB, masked
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    bm[c] = c > 0 && wall_hi ? R(0) : a.lB[c][row(-2)];
+    b[c] = a.lB[c][row(-1)];
+    e[c] = a.lE[c][row(-1)];
+    braw[c] = em[c] = mem[c] = pm[c] = bpm[c] = R(0);
   }
-  const double v = block_sum(acc, sh);
-  if (threadIdx.x == 0 && v != 0.0) atomicAdd(da0, v);
+  for (int j = -1; j <= rows; ++j) {
+    if (j < rows) {
+      const int g = row(j + 1);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        bn[c] = a.lB[c][g];
+        en[c] = a.lE[c][g];
+      }
+    }
+    // R5
+    const R bk[3] = {b[0], wall_hi ? R(0) : b[1], wall_hi ? R(0) : b[2]};
+    R cu[3], eh[3], p[3] = {R(0), R(0), R(0)};
+    curl_e(bk, bm, cu);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) eh[c] = e[c] - hh * cu[c];
+    // R4 (only the warps that hold a wall's column)
+    if (has_lo)
+#pragma unroll
+      for (int c = 1; c < 3; ++c) {
+        const R up = __shfl_up_sync(0xffffffffu, eh[c], 1);
+        if (wall_lo) {
+          const double g = (double)eh[c];
+          if (mine && j >= 0 && j < rows && a.ls.pol == c) {
+            // unit-amplitude laser terms at the wall row: P(row) times the waveform
+            const double w = a.ls.prof[y0 + j];
+            acc += g * w * (a.ls.amp[2] - a.ls.amp[1] - a.kc * a.ls.amp[3] + a.kc * a.ls.amp[0]);
+          }
+          p[c] = (R)(-a.kc * g);
+          eh[c] = R(0);
+        }
+        if (in_lo) {
+          p[c] = up;
+          eh[c] += (R)(a.kc * (double)up);
+        }
+      }
+    if (has_hi)
+#pragma unroll
+      for (int c = 1; c < 3; ++c) {
+        const R dn = __shfl_down_sync(0xffffffffu, eh[c], 1);
+        if (wall_hi) {
+          p[c] = (R)(-a.kc * (double)eh[c]);
+          eh[c] = R(0);
+        }
+        if (in_hi) {
+          p[c] = dn;
+          eh[c] += (R)(a.kc * (double)dn);
+        }
+      }
+    const R me[3] = {wall_hi ? R(0) : eh[0], wall_lo || wall_hi ? R(0) : eh[1], wall_lo || wall_hi ? R(0) : eh[2]};
+    if (j >= 0) {
+      // R3 of row j - 1
+      const R eyx = __shfl_down_sync(0xffffffffu, mem[1], 1), ezx = __shfl_down_sync(0xffffffffu, mem[2], 1);
+      const R nb[3] = {braw[0] + a.h * ((me[2] - mem[2]) * a.rdy), braw[1] + a.h * (-(ezx - mem[2]) * a.rdx),
+                       braw[2] + a.h * ((eyx - mem[1]) * a.rdx - (me[0] - mem[0]) * a.rdy)};
+      // R1 of row j - 1
+      const R nk[3] = {nb[0], wall_hi ? R(0) : nb[1], wall_hi ? R(0) : nb[2]};
+      curl_e(nk, bpm, cu);
+      if (j >= 1 && mine) {
+        const int g = (y0 + j - 1) * a.n0 + i;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          a.lE2[c][g] = em[c] + (pm[c] - hh * cu[c]);
+          a.lB2[c][g] = nb[c];
+          a.lJ[c][g] = -a.h * mem[c];
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) bpm[c] = nk[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      bm[c] = bk[c];
+      braw[c] = b[c];
+      b[c] = bn[c];
+      e[c] = en[c];
+      em[c] = eh[c];
+      mem[c] = me[c];
+      pm[c] = p[c];
+    }
+  }
+  if (has_lo) {
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0 && acc != 0.0) atomicAdd(a.da0, acc);
+  }
 }
 
 // ---------------------------------------------------------------- particles
@@ -259,18 +268,26 @@ template <> __device__ __forceinline__ double inv_sqrt_fwd<double>(double x) { r
 
 // The forward Boris step (the push's arithmetic) with its intermediates:
 // u- = u0 + h E, t = h B / gamma-, s = 2 t / (1 + t^2), u' = u- + u- x t,
-// u+ = u- + u' x s, uo = u+ + h E.
-template <class R>
-__device__ __forceinline__ void boris_fwd(R h, const R u0[3], const R F[6], R um[3], R t[3], R sv[3], R up[3],
-                                          R uo[3]) {
+// u+ = u- + u' x s, uo = u+ + h E.  rg = 1 / gamma- and sf = 2 / (1 + t^2) are
+// computed by boris_roots once and kept: the transpose needs no other quotient.
+template <class R> __device__ __forceinline__ void boris_roots(R h, const R u0[3], const R F[6], R &rg, R &sf) {
+  R um[3], t[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) um[d] = u0[d] + h * F[d];
-  const R gm = sqrt(R(1) + um[0] * um[0] + um[1] * um[1] + um[2] * um[2]);
+  rg = R(1) / sqrt(R(1) + um[0] * um[0] + um[1] * um[1] + um[2] * um[2]);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) t[d] = h * F[3 + d] / gm;
-  const R den = R(1) + t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
+  for (int d = 0; d < 3; ++d) t[d] = h * F[3 + d] * rg;
+  sf = R(2) / (R(1) + t[0] * t[0] + t[1] * t[1] + t[2] * t[2]);
+}
+template <class R>
+__device__ __forceinline__ void boris_fwd(R h, const R u0[3], const R F[6], R rg, R sf, R um[3], R t[3], R sv[3],
+                                          R up[3], R uo[3]) {
 #pragma unroll
-  for (int d = 0; d < 3; ++d) sv[d] = R(2) * t[d] / den;
+  for (int d = 0; d < 3; ++d) {
+    um[d] = u0[d] + h * F[d];
+    t[d] = h * F[3 + d] * rg;
+    sv[d] = sf * t[d];
+  }
   up[0] = um[0] + (um[1] * t[2] - um[2] * t[1]);
   up[1] = um[1] + (um[2] * t[0] - um[0] * t[2]);
   up[2] = um[2] + (um[0] * t[1] - um[1] * t[0]);
@@ -369,10 +386,11 @@ __device__ __forceinline__ void adj_particle(const AdjPushArgs<R> &a, const Node
     // Boris.  Its intermediate values are recomputed from u0 and F for the
     // transpose further down, rather than kept live through deposit^T.
     const R h = a.qmh;
-    R uo[3];
+    R uo[3], rg, sf;
+    boris_roots<R>(h, u0, F, rg, sf);
     {
       R um[3], t[3], sv[3], up[3];
-      boris_fwd<R>(h, u0, F, um, t, sv, up, uo);
+      boris_fwd<R>(h, u0, F, rg, sf, um, t, sv, up, uo);
     }
     // move
     const R ig = inv_sqrt_fwd<R>(R(1) + uo[0] * uo[0] + uo[1] * uo[1] + uo[2] * uo[2]);
@@ -527,10 +545,8 @@ __device__ __forceinline__ void adj_particle(const AdjPushArgs<R> &a, const Node
     R um[3], t[3], sv[3], up[3];
     {
       R uo_[3];
-      boris_fwd<R>(h, u0, F, um, t, sv, up, uo_);
+      boris_fwd<R>(h, u0, F, rg, sf, um, t, sv, up, uo_);
     }
-    const R gm = sqrt(R(1) + um[0] * um[0] + um[1] * um[1] + um[2] * um[2]);
-    const R den = R(1) + t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
     R lF[6];
 #pragma unroll
     for (int d = 0; d < 3; ++d) lF[d] = h * lu[d];  // u_out = u+' + h E
@@ -544,12 +560,12 @@ __device__ __forceinline__ void adj_particle(const AdjPushArgs<R> &a, const Node
     lsv[0] = lu[1] * up[2] - lu[2] * up[1];
     lsv[1] = lu[2] * up[0] - lu[0] * up[2];
     lsv[2] = lu[0] * up[1] - lu[1] * up[0];
-    // sv = 2 t / (1 + t^2)
+    // sv = 2 t / (1 + t^2) = sf t
     R lt[3];
     {
       const R tl = t[0] * lsv[0] + t[1] * lsv[1] + t[2] * lsv[2];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) lt[d] = R(2) / den * lsv[d] - R(4) * t[d] * tl / (den * den);
+      for (int d = 0; d < 3; ++d) lt[d] = sf * (lsv[d] - sv[d] * tl);
     }
     // up = um + um x t: lambda_um += lup + t x lup ; lambda_t += lup x um
 #pragma unroll
@@ -560,16 +576,17 @@ __device__ __forceinline__ void adj_particle(const AdjPushArgs<R> &a, const Node
     lt[0] += lup[1] * um[2] - lup[2] * um[1];
     lt[1] += lup[2] * um[0] - lup[0] * um[2];
     lt[2] += lup[0] * um[1] - lup[1] * um[0];
-    // t = h B / gm
+    // t = h B rg
     R lgm = 0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      lF[3 + d] = h / gm * lt[d];
-      lgm -= h * F[3 + d] / (gm * gm) * lt[d];
+      lF[3 + d] = h * rg * lt[d];
+      lgm -= t[d] * lt[d];
     }
-    // gm = sqrt(1 + um^2)
+    // 1 / rg = sqrt(1 + um^2); lgm so far is times 1 / rg
+    lgm *= rg * rg;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) lum[d] += lgm * um[d] / gm;
+    for (int d = 0; d < 3; ++d) lum[d] += lgm * um[d];
     // um = u + h E
     R lu0[3];
 #pragma unroll
@@ -602,16 +619,21 @@ __device__ __forceinline__ void adj_particle(const AdjPushArgs<R> &a, const Node
         const int rx = dx_[cc] ? gx.reld : gx.relp, ry = dy_[cc] ? gy.reld : gy.relp;
         const R *wx = dx_[cc] ? gx.wd : gx.wp, *dwx = dx_[cc] ? gx.dwd : gx.dwp;
         const R *wy = dy_[cc] ? gy.wd : gy.wp, *dwy = dy_[cc] ? gy.dwd : gy.dwp;
+        const R lw[3] = {lF[cc] * wx[0], lF[cc] * wx[1], lF[cc] * wx[2]};
         R sx = 0, sy = 0;
 #pragma unroll
-        for (int b = 0; b < 3; ++b)
+        for (int b = 0; b < 3; ++b) {
+          R rx0 = 0, ry0 = 0;
 #pragma unroll
           for (int aa = 0; aa < 3; ++aa) {
             const R v = G[ix[aa] + iy[b]];
-            sx += v * dwx[aa] * wy[b];
-            sy += v * wx[aa] * dwy[b];
-            atomicAdd(LG + nd.sx(rx + aa) + nd.sy(ry + b), lF[cc] * wx[aa] * wy[b]);
+            rx0 += v * dwx[aa];
+            ry0 += v * wx[aa];
+            atomicAdd(LG + nd.sx(rx + aa) + nd.sy(ry + b), lw[aa] * wy[b]);
           }
+          sx += rx0 * wy[b];
+          sy += ry0 * dwy[b];
+        }
         lX[0] += lF[cc] * sx;
         lX[1] += lF[cc] * sy;
       }
@@ -667,7 +689,9 @@ struct AdjWork {
 // cells outside its tile since the sort is set aside and done at the end of
 // the block with all its nodes in global memory.
 template <class R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
+// (FP64: one block per SM and no spills, 106 us per launch of the 120 x 64 run;
+// two blocks at 128 registers 115 us.  FP32: two blocks per SM 7 % slower.)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1)
     k_adj_push2d_win(const AdjPushArgs<R> a, const AdjWork w) {
   extern __shared__ __align__(16) unsigned char adj_smem[];
   R *s = reinterpret_cast<R *>(adj_smem);
@@ -783,75 +807,49 @@ __global__ void k_adj_seed(int n0, const int32_t *cell, const R *u0, const R *u1
   if (threadIdx.x == 0 && v != 0.0) atomicAdd(F, v);
 }
 
-template <class R> GridIdx gidx(const Grid &g) { return GridIdx{g.n[0], g.n[1], g.n[2]}; }
-
 }  // namespace
 
-cudaError_t launch_adj_yee_b(const Grid &g, void *const lE[3], void *const lB[3], double h, const double *pend,
-                             cudaStream_t st) {
-  const int nb = nblocks(g.ncell);
-  const int absorb = g.absorb_lo || g.absorb_hi;
-  if (g.prec == 1) {
-    auto E = [&](int c) { return static_cast<double *>(lE[c]); };
-    auto B = [&](int c) { return static_cast<const double *>(lB[c]); };
-    if (g.dims == 3)
-      k_adj_yee_b<double, 3><<<nb, 256, 0, st>>>(gidx<double>(g), absorb, 1.0 / g.dx[0], 1.0 / g.dx[1], 1.0 / g.dx[2],
-                                                 h, E(0), E(1), E(2), B(0), B(1), B(2), pend);
-    else
-      k_adj_yee_b<double, 2><<<nb, 256, 0, st>>>(gidx<double>(g), absorb, 1.0 / g.dx[0], 1.0 / g.dx[1], 1.0 / g.dx[2],
-                                                 h, E(0), E(1), E(2), B(0), B(1), B(2), pend);
-  } else {
-    auto E = [&](int c) { return static_cast<float *>(lE[c]); };
-    auto B = [&](int c) { return static_cast<const float *>(lB[c]); };
-    if (g.dims == 3)
-      k_adj_yee_b<float, 3><<<nb, 256, 0, st>>>(gidx<float>(g), absorb, (float)(1.0 / g.dx[0]), (float)(1.0 / g.dx[1]),
-                                                (float)(1.0 / g.dx[2]), (float)h, E(0), E(1), E(2), B(0), B(1), B(2), pend);
-    else
-      k_adj_yee_b<float, 2><<<nb, 256, 0, st>>>(gidx<float>(g), absorb, (float)(1.0 / g.dx[0]), (float)(1.0 / g.dx[1]),
-                                                (float)(1.0 / g.dx[2]), (float)h, E(0), E(1), E(2), B(0), B(1), B(2), pend);
+template <class R>
+static cudaError_t adj_field_t(const Grid &g, void *const lE[3], void *const lB[3], void *const lE2[3],
+                               void *const lB2[3], void *const lJ[3], const LaserStep &ls_unit, double *da0,
+                               cudaStream_t st) {
+  AdjFieldStep<R> a;
+  a.n0 = g.n[0];
+  a.n1 = g.n[1];
+  a.absorb = g.absorb_lo || g.absorb_hi;
+  // (the last node but one needs the wall's value: not alone past a strip's end)
+  a.width = 29;
+  while (a.absorb && a.n0 % a.width == 2) --a.width;
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t strips = (a.n0 + a.width - 1) / a.width;
+  a.rows = 31;  // as the forward's update (launch_field_step2)
+  while (a.rows > 1 && strips * ((a.n1 + a.rows - 1) / a.rows) < 64 * (int64_t)nsm) a.rows /= 2;
+  a.strips = (unsigned)strips;
+  a.rdx = (R)(1.0 / g.dx[0]);
+  a.rdy = (R)(1.0 / g.dx[1]);
+  a.h = (R)g.dt;
+  for (int d = 0; d < 3; ++d) {
+    a.lE[d] = static_cast<const R *>(lE[d]);
+    a.lB[d] = static_cast<const R *>(lB[d]);
+    a.lE2[d] = static_cast<R *>(lE2[d]);
+    a.lB2[d] = static_cast<R *>(lB2[d]);
+    a.lJ[d] = static_cast<R *>(lJ[d]);
   }
+  a.kc = (g.dt - g.dx[0]) / (g.dt + g.dx[0]);
+  a.ls = ls_unit;
+  a.da0 = da0;
+  k_adj_field_step<R><<<(unsigned)(strips * ((a.n1 + 2 * a.rows - 1) / (2 * a.rows))), 64, 0, st>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_adj_yee_e(const Grid &g, void *const lE[3], void *const lB[3], void *const lJ[3], double h,
+cudaError_t launch_adj_field(const Grid &g, void *const lE[3], void *const lB[3], void *const lE2[3],
+                             void *const lB2[3], void *const lJ[3], const LaserStep &ls_unit, double *da0,
                              cudaStream_t st) {
-  const int nb = nblocks(g.ncell);
-  const int absorb = g.absorb_lo || g.absorb_hi;
-  if (g.prec == 1) {
-    auto E = [&](int c) { return static_cast<const double *>(lE[c]); };
-    auto B = [&](int c) { return static_cast<double *>(lB[c]); };
-    auto J = [&](int c) { return static_cast<double *>(lJ[c]); };
-    if (g.dims == 3)
-      k_adj_yee_e<double, 3><<<nb, 256, 0, st>>>(gidx<double>(g), absorb, 1.0 / g.dx[0], 1.0 / g.dx[1], 1.0 / g.dx[2],
-                                                 h, E(0), E(1), E(2), B(0), B(1), B(2), J(0), J(1), J(2));
-    else
-      k_adj_yee_e<double, 2><<<nb, 256, 0, st>>>(gidx<double>(g), absorb, 1.0 / g.dx[0], 1.0 / g.dx[1], 1.0 / g.dx[2],
-                                                 h, E(0), E(1), E(2), B(0), B(1), B(2), J(0), J(1), J(2));
-  } else {
-    auto E = [&](int c) { return static_cast<const float *>(lE[c]); };
-    auto B = [&](int c) { return static_cast<float *>(lB[c]); };
-    auto J = [&](int c) { return static_cast<float *>(lJ[c]); };
-    const float r0 = (float)(1.0 / g.dx[0]), r1 = (float)(1.0 / g.dx[1]), r2 = (float)(1.0 / g.dx[2]);
-    if (g.dims == 3)
-      k_adj_yee_e<float, 3><<<nb, 256, 0, st>>>(gidx<float>(g), absorb, r0, r1, r2, (float)h, E(0), E(1), E(2), B(0),
-                                                B(1), B(2), J(0), J(1), J(2));
-    else
-      k_adj_yee_e<float, 2><<<nb, 256, 0, st>>>(gidx<float>(g), absorb, r0, r1, r2, (float)h, E(0), E(1), E(2), B(0),
-                                                B(1), B(2), J(0), J(1), J(2));
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_adj_mur(const Grid &g, void *const lE[3], double *pend, const LaserStep &ls_unit, double *da0,
-                           cudaStream_t st) {
-  const int nb = nblocks(2LL * g.n[1] * g.n[2]);
-  if (g.prec == 1)
-    k_adj_mur<double><<<nb, 256, 0, st>>>(g.n[0], g.n[1], g.n[2], g.dx[0], g.dt, static_cast<double *>(lE[1]),
-                                          static_cast<double *>(lE[2]), pend, ls_unit, da0);
-  else
-    k_adj_mur<float><<<nb, 256, 0, st>>>(g.n[0], g.n[1], g.n[2], g.dx[0], g.dt, static_cast<float *>(lE[1]),
-                                         static_cast<float *>(lE[2]), pend, ls_unit, da0);
-  return cudaGetLastError();
+  if (g.dims != 2) return cudaErrorInvalidValue;
+  if (g.prec == 1) return adj_field_t<double>(g, lE, lB, lE2, lB2, lJ, ls_unit, da0, st);
+  return adj_field_t<float>(g, lE, lB, lE2, lB2, lJ, ls_unit, da0, st);
 }
 
 template <class R>

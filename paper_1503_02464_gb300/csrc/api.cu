@@ -59,12 +59,15 @@ struct TimerRec {
 
 // Device copy of one species' particle state (and its slot count).
 struct PCopy {
-  Particles p{};
+  Particles own{};               // this copy's own buffer
+  int64_t *own_count = nullptr;
+  Particles p{};                 // the copy (see below: w and id may be an earlier entry's)
   int64_t *count = nullptr;
   // Tape entries: the adjoint's work items of the sort in effect (tiled =
   // false when the species was unsorted at the copy).  meta is this copy's own
   // buffer; items lies in it or, when the previous tape entry was recorded
-  // under the same sort, in that entry's.
+  // under the same sort, in that entry's; so do the weights, the ids and the
+  // slot count, which only a sort changes.
   void *meta = nullptr;
   pic::WorkList items;
   int64_t sorts = -1;
@@ -148,7 +151,8 @@ struct pic_handle {
   bool adj_ready = false;
   int64_t id_cap = 0;
   void *lE[3] = {}, *lB[3] = {}, *lJ[3] = {};
-  double *pend = nullptr, *da0 = nullptr, *objF = nullptr;
+  void *lE2[3] = {}, *lB2[3] = {};  // what a reverse step's field update writes (then they trade places)
+  double *da0 = nullptr, *objF = nullptr;
   double *adj_stage = nullptr;  // FP64 staging of id-indexed adjoint arrays (id_cap doubles)
   unsigned long long *adj_err = nullptr;
   unsigned long long *adj_esc = nullptr;  // particle adjoints on the global-memory path since pic_adjoint_begin
@@ -399,9 +403,9 @@ cudaError_t alloc_snapshot(pic_handle *h, Snapshot &sn) {
   char *q = base + align256(6 * fb);
   for (int i = 0; i < h->nsp; ++i) {
     PCopy &c = sn.sp[i];
-    carve_particles(c.p, q, h->sp[i].slots, h->rsize, h->g.dims);
+    carve_particles(c.own, q, h->sp[i].slots, h->rsize, h->g.dims);
     q += particles_bytes(h->sp[i].slots, h->rsize, h->g.dims);
-    c.count = reinterpret_cast<int64_t *>(q);
+    c.own_count = reinterpret_cast<int64_t *>(q);
     q += 256;
     c.meta = q;
     q += align256(work_list_bytes(h->sp[i].work.adj.nwork));
@@ -435,19 +439,28 @@ cudaError_t save_snapshot(pic_handle *h, Snapshot &sn, bool tape = false, const 
   for (int i = 0; i < h->nsp && e == cudaSuccess; ++i) {
     Species &s = h->sp[i];
     PCopy &c = sn.sp[i];
-    e = copy_particles(h, c.p, c.count, s.buf[s.cur], s.d_count, s.slots);
+    const Particles &src = s.buf[s.cur];
+    c.p = c.own;
+    c.count = c.own_count;
     // the slot order is that of the last sort unless a sort is pending
     c.tiled = tape && !s.need_sort && s.work.adj.nwork > 0;
     c.sorts = s.sorts;
-    if (!c.tiled || e != cudaSuccess) continue;
-    const PCopy *q = prev ? &prev->sp[i] : nullptr;
+    const PCopy *q = c.tiled && prev ? &prev->sp[i] : nullptr;
     if (q && q->tiled && q->sorts == s.sorts) {
+      // cell, offsets and momenta lie in front of w and id: one copy, a quarter
+      // shorter (256 x 256 FP32 run: 13 us a step instead of 17 and a copy less)
+      c.p.w = q->p.w;
+      c.p.id = q->p.id;
+      c.count = q->count;
       c.items = q->items;
-    } else {
-      e = cudaMemcpyAsync(c.meta, s.work.adj.count, work_list_bytes(s.work.adj.nwork), cudaMemcpyDeviceToDevice,
-                          h->st);
-      set_work_list(c.items, c.meta, s.work.adj.nwork);
+      e = cudaMemcpyAsync(c.p.cell, src.cell, static_cast<char *>(src.w) - reinterpret_cast<char *>(src.cell),
+                          cudaMemcpyDeviceToDevice, h->st);
+      continue;
     }
+    e = copy_particles(h, c.p, c.count, src, s.d_count, s.slots);
+    if (!c.tiled || e != cudaSuccess) continue;
+    e = cudaMemcpyAsync(c.meta, s.work.adj.count, work_list_bytes(s.work.adj.nwork), cudaMemcpyDeviceToDevice, h->st);
+    set_work_list(c.items, c.meta, s.work.adj.nwork);
   }
   sn.step = h->step;
   return e;
@@ -458,15 +471,16 @@ void free_adjoint(pic_handle *h) {
     cudaFree(h->lE[d]);
     cudaFree(h->lB[d]);
     cudaFree(h->lJ[d]);
-    h->lE[d] = h->lB[d] = h->lJ[d] = nullptr;
+    cudaFree(h->lE2[d]);
+    cudaFree(h->lB2[d]);
+    h->lE[d] = h->lB[d] = h->lJ[d] = h->lE2[d] = h->lB2[d] = nullptr;
   }
-  cudaFree(h->pend);
   cudaFree(h->da0);
   cudaFree(h->objF);
   cudaFree(h->adj_err);
   cudaFree(h->adj_stage);
   cudaFree(h->adj_esc);
-  h->pend = h->da0 = h->objF = h->adj_stage = nullptr;
+  h->da0 = h->objF = h->adj_stage = nullptr;
   h->adj_err = nullptr;
   h->adj_esc = nullptr;
   for (int i = 0; i < kMaxSpecies; ++i) {
@@ -1648,9 +1662,9 @@ int pic_adjoint_begin(pic_handle *h, int64_t id_capacity) {
     bool ok = true;
     for (int d = 0; d < 3 && ok; ++d)
       ok = cudaMalloc(&h->lE[d], fb) == cudaSuccess && cudaMalloc(&h->lB[d], fb) == cudaSuccess &&
-           cudaMalloc(&h->lJ[d], fb) == cudaSuccess;
-    ok = ok && cudaMalloc(&h->pend, 8 * sizeof(double) * (size_t)h->g.n[1] * h->g.n[2]) == cudaSuccess &&
-         cudaMalloc(&h->da0, sizeof(double)) == cudaSuccess && cudaMalloc(&h->objF, sizeof(double)) == cudaSuccess &&
+           cudaMalloc(&h->lJ[d], fb) == cudaSuccess && cudaMalloc(&h->lE2[d], fb) == cudaSuccess &&
+           cudaMalloc(&h->lB2[d], fb) == cudaSuccess;
+    ok = ok && cudaMalloc(&h->da0, sizeof(double)) == cudaSuccess && cudaMalloc(&h->objF, sizeof(double)) == cudaSuccess &&
          cudaMalloc(&h->adj_err, sizeof(unsigned long long)) == cudaSuccess &&
          cudaMalloc(&h->adj_esc, sizeof(unsigned long long)) == cudaSuccess &&
          cudaMalloc(&h->adj_stage, (size_t)id_capacity * sizeof(double)) == cudaSuccess;
@@ -1714,7 +1728,6 @@ int pic_adjoint_seed_kinetic(pic_handle *h, int species, int col_lo, int col_hi,
 int pic_adjoint_step(pic_handle *h, int nsteps) {
   if (!h || !h->adj_ready) return fail(h, PIC_EINVAL, "call pic_adjoint_begin first");
   if (nsteps < 0 || nsteps > h->tape_len) return fail(h, PIC_EINVAL, "more adjoint steps than recorded steps");
-  const bool walls = h->g.absorb_lo || h->g.absorb_hi;
   // The reversal runs on st_adj after everything enqueued on st so far (the
   // tape's recording, seeds, adjoint writes), so that st can go on with the
   // next segment's recomputation meanwhile.
@@ -1727,18 +1740,16 @@ int pic_adjoint_step(pic_handle *h, int nsteps) {
     const double t_old = en.step * h->g.dt, t_new = (en.step + 1) * h->g.dt;
     {
       Timed tm(h, pic::KC_ADJ_FIELD, sa);
-      CK(h, pic::launch_adj_yee_b(h->g, h->lE, h->lB, 0.5 * h->g.dt, nullptr, sa), "adjoint B half");
-      if (walls)
-        CK(h,
-           pic::launch_adj_mur(h->g, h->lE, h->pend,
+      CK(h,
+         pic::launch_adj_field(h->g, h->lE, h->lB, h->lE2, h->lB2, h->lJ,
                                pic::laser_step(h->laser, h->laser_prof, 1.0, h->g, t_old, t_new), h->da0, sa),
-           "adjoint Mur");
-      CK(h, pic::launch_adj_yee_e(h->g, h->lE, h->lB, h->lJ, h->g.dt, sa), "adjoint E");
-      // the second B half also adds the Mur transpose's old-time terms
-      CK(h, pic::launch_adj_yee_b(h->g, h->lE, h->lB, 0.5 * h->g.dt, walls ? h->pend : nullptr, sa),
-         "adjoint B half");
+         "adjoint fields");
+      for (int d = 0; d < 3; ++d) {
+        std::swap(h->lE[d], h->lE2[d]);
+        std::swap(h->lB[d], h->lB2[d]);
+      }
     }
-    h->launches += walls ? 4 : 3;
+    h->launches++;
     for (int i = 0; i < h->nsp; ++i) {
       Species &s = h->sp[i];
       Timed tm(h, pic::KC_ADJ_PUSH, sa);

@@ -250,14 +250,12 @@ cudaError_t launch_particle_diag(const Grid &g, const Particles &p, const int64_
                                  double *out, cudaStream_t st);
 
 // ---- adjoint (adjoint.cu) ----
-// pend (may be null): the Mur transpose's old-time terms, added to lamE at the
-// wall nodes in the same pass (the second B half of the reversed step).
-cudaError_t launch_adj_yee_b(const Grid &g, void *const lE[3], void *const lB[3], double h, const double *pend,
+// The field part of a reverse step (2D) from lE, lB into lE2, lB2 and lJ;
+// ls_unit: the incoming wave of unit amplitude, whose share of the Mur
+// transpose is added to *da0.
+cudaError_t launch_adj_field(const Grid &g, void *const lE[3], void *const lB[3], void *const lE2[3],
+                             void *const lB2[3], void *const lJ[3], const LaserStep &ls_unit, double *da0,
                              cudaStream_t st);
-cudaError_t launch_adj_yee_e(const Grid &g, void *const lE[3], void *const lB[3], void *const lJ[3], double h,
-                             cudaStream_t st);
-cudaError_t launch_adj_mur(const Grid &g, void *const lE[3], double *pend, const LaserStep &ls_unit, double *da0,
-                           cudaStream_t st);
 // Work items of a recorded particle buffer (those of the sort in effect when
 // it was recorded, see WorkSplit::adj) for the windowed adjoint kernel;
 // esc_total counts the particles that had drifted beyond their tile window

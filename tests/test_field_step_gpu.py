@@ -79,3 +79,42 @@ def test_smoothing_wraps(dims, n, passes, comp):
     jf = j_floor(wl, [p]) * ((1 + 0.5 * passes) ** dims if comp else 1.0)
     fe = compare_fields(o, s, j_abs=jf)
     assert max(fe.values()) <= 2e-12, fe
+
+
+@pytest.mark.parametrize("walls", [False, True], ids=["periodic", "mur_walls"])
+@pytest.mark.parametrize("n", [(16, 1), (28, 3), (29, 2), (30, 5), (31, 9), (58, 4), (59, 1), (60, 33), (814, 2)])
+def test_reversed_field_step_is_the_transpose(n, walls):
+    """<A x, y> = <x, A^T y> for one field step without particles, the adjoint's
+    strips having their halo on the other side."""
+    d = 0.1
+    s = Simulation(2, n, (d, d), 0.9 * synth.courant_limit((d, d), 2), 2, "fp64", absorbing_x=walls)
+    rng = np.random.default_rng(17)
+    x = [rng.normal(size=s.shape3) for _ in range(6)]
+    y = [rng.normal(size=s.shape3) for _ in range(6)]
+    for c in range(6):
+        s.set_field(c, x[c])
+    s.tape_begin(1)
+    s.step(1)
+    ax = [s.field(c) for c in range(6)]
+    s.adjoint_begin(1)
+    for c in range(6):
+        s.adjoint_set_field(c, y[c])
+    s.adjoint_step(1)
+    aty = [s.adjoint_field(c) for c in range(6)]
+    lhs = sum(float((p * q).sum()) for p, q in zip(ax, y))
+    rhs = sum(float((p * q).sum()) for p, q in zip(x, aty))
+    scale = sum(float(np.abs(p * q).sum()) for p, q in zip(ax, y))
+    assert abs(lhs - rhs) <= 1e-13 * scale, (lhs, rhs, scale)
+    # (the sum could hide an entry: one unit seed per wall column)
+    for c in (1, 2):
+        for col in (0, 1, n[0] - 2, n[0] - 1):
+            s.tape_begin(1)
+            s.step(0)
+            s.tape_record()
+            s.adjoint_begin(1)
+            seed = np.zeros(s.shape3)
+            seed[0, 0, col] = 1.0
+            s.adjoint_set_field(c, seed)
+            s.adjoint_step(1)
+            got = sum(float((p * s.adjoint_field(k)).sum()) for k, p in enumerate(x))
+            assert abs(got - ax[c][0, 0, col]) <= 1e-13 * 30, (c, col)
