@@ -26,6 +26,8 @@ namespace {
 
 constexpr int kMaxSpecies = 8;
 constexpr size_t kEscBytes = kMaxSpecies * pic::kEscCounters * sizeof(unsigned long long);
+// Species up to this size have their escape count read back less often (a push of 2M takes about 0.1 ms).
+constexpr int64_t kSmallSpecies = int64_t(1) << 21;
 
 struct Species {
   double q = 0, m = 1;
@@ -1241,8 +1243,7 @@ int pic_step(pic_handle *h, int nsteps) {
       // threshold waits for the count of its previous push; the others wait
       // once four steps have passed without a count, so that a long
       // pic_step call, whose host loop runs ahead of the device, still
-      // learns how the particles drift; their counts are copied back every
-      // fourth step (a copy and an event cost 3 us, which small runs feel).  (On large grids a wait costs no
+      // learns how the particles drift.  (On large grids a wait costs no
       // device time: the last step's field updates are still queued behind
       // the push when it ends.)
       bool many_escapes = false;
@@ -1303,8 +1304,14 @@ int pic_step(pic_handle *h, int nsteps) {
          "push");
       h->launches += nl;
       if (s.crowded) h->crowded_pushes++;
-      // (a slow species' count is copied back every fourth step)
-      if (!s.esc_pending && (s.fast || s.esc_step < 0 || s.esc_step > h->step || h->step - s.esc_step >= 4)) {
+      // A copy and an event cost 3 us, which small species feel: a slow one's
+      // count comes back every fourth step.  A large one, whose push takes far
+      // longer, asks at every step: its escapes cost more than the copy
+      // (beams of 28M particles, first steps: escape kernel 0.9 -> 4.5 ms when
+      // the early sort came up to three steps later).
+      const bool ask = s.fast || s.h_count > kSmallSpecies || s.esc_step < 0 || s.esc_step > h->step ||
+                       h->step - s.esc_step >= 4;
+      if (!s.esc_pending && ask) {
         CK(h, cudaMemcpyAsync(s.esc_host, h->esc_count + i * pic::kEscCounters, 2 * sizeof(unsigned long long),
                               cudaMemcpyDeviceToHost, h->st),
            "escape count");
