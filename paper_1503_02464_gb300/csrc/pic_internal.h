@@ -132,7 +132,7 @@ size_t push_smem_bytes(const Grid &g);
 // holds in shared memory.  The sort takes the candidate of the least estimated
 // time for the runs at hand: an item costs its slots and `fixed` more, and the
 // items run in rounds of `blocks` per SM on `nsm` SMs.
-constexpr int kItemCands = 8;
+constexpr int kItemCands = 30;
 struct ItemPlan {
   int cand[kItemCands];  // descending multiples of 4
   int blocks = 1, nsm = 1, fixed = 0;

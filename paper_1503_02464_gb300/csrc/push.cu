@@ -16,6 +16,7 @@
 // k_push_escaped applies the same arithmetic on global memory afterwards.
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <type_traits>
 
 #include "pic_device.cuh"
@@ -1614,8 +1615,11 @@ ItemPlan push_item_plan(const Grid &g) {
   // cut differently (2D: 434; 3D TSC: 345; FP64 particles cost far more each)
   pl.fixed = g.prec == 1 ? 120 : 400;
   for (int j = 0; j < kItemCands; ++j) {
-    const int c = cap * (kItemCands - j) / kItemCands / kTilePad * kTilePad;
-    pl.cand[j] = c > 256 ? c : 256;
+    // eight sizes per halving, down to a twelfth: close enough that the items of
+    // few tiles can fill the SMs' last round (eight sizes, none below 256,
+    // against these: 64^2 FP64 CIC push 39.5 -> 37.3 us, 75 x 50 x 43 FP32 CIC
+    // 105 -> 93 us, 2D foil of 0.33M particles 27.8 -> 20.9 us)
+    pl.cand[j] = (int)(cap * std::exp2(-j / 8.0)) / kTilePad * kTilePad;
   }
   int dev = 0;
   pl.nsm = 1;

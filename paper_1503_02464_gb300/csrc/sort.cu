@@ -99,24 +99,29 @@ __device__ __forceinline__ uint32_t items_of(uint32_t run, uint32_t size) {
 // the adjoint's items.
 constexpr int kGroup = 1024;
 constexpr int kVals = kItemCands + 2;
+constexpr int kPart = 2;  // values of a block of k_tile_groups: the divisions are a serial chain
+static_assert(kVals <= 32 && kVals % kPart == 0, "one warp per value, one lane per candidate");
 
 __global__ void __launch_bounds__(kGroup)
     k_tile_groups(const uint32_t *__restrict__ run, int64_t ntiles, ItemPlan plan, uint32_t *__restrict__ part,
                   const int64_t *__restrict__ d_count, int64_t *__restrict__ n_src) {
-  __shared__ uint32_t s[kVals];
-  if (threadIdx.x < kVals) s[threadIdx.x] = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *n_src = *d_count;  // k_tile_starts rewrites it
+  __shared__ uint32_t s[kPart];
+  const int v0 = blockIdx.y * kPart;
+  if (threadIdx.x < kPart) s[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && v0 == 0 && threadIdx.x == 0) *n_src = *d_count;  // k_tile_starts rewrites it
   __syncthreads();
   const int64_t t = blockIdx.x * (int64_t)kGroup + threadIdx.x;
   const uint32_t r = t < ntiles ? run[t] : 0u;
 #pragma unroll
-  for (int v = 0; v < kVals; ++v) {
-    const uint32_t x = v == 0 ? r : items_of(r, v <= kItemCands ? (uint32_t)plan.cand[v - 1] : (uint32_t)kAdjItem);
+  for (int k = 0; k < kPart; ++k) {
+    const int v = v0 + k;
+    uint32_t x = r;
+    if (v > 0) x = items_of(r, v <= kItemCands ? (uint32_t)plan.cand[v - 1] : (uint32_t)kAdjItem);
     const uint32_t sum = __reduce_add_sync(0xffffffffu, x);
-    if ((threadIdx.x & 31) == 0 && sum > 0) atomicAdd(&s[v], sum);
+    if ((threadIdx.x & 31) == 0 && sum > 0) atomicAdd(&s[k], sum);
   }
   __syncthreads();
-  if (threadIdx.x < kVals) part[blockIdx.x * kVals + threadIdx.x] = s[threadIdx.x];
+  if (threadIdx.x < kPart) part[blockIdx.x * kVals + v0 + threadIdx.x] = s[threadIdx.x];
 }
 
 // The size of the push's items is chosen here, where the tiles' runs are
@@ -125,13 +130,23 @@ __global__ void __launch_bounds__(kGroup)
 // 2D plasma of 1.8M particles 0.137 -> 0.119 ms per push, FP64 64^3 3.03 ->
 // 2.73 ms).
 //
-// Estimated time of a species of `slots` slots cut into `items`: whole rounds
-// of plan.blocks items per SM, and a last one whose few blocks on an SM run
-// faster one by one (a block alone takes about (blocks + 1) / 2 of a share).
+// Estimated time of a species of `slots` slots cut into `items`, in items (of
+// their mean slots and plan.fixed more) that an SM's blocks share.  Measured
+// with every size from 520 to 1920 slots in 2D FP32 (three blocks per SM): with
+// two rounds of items or more the time is proportional to slots + 400 items
+// within 5 % wherever the last round ends (a block that draws no item leaves
+// its share to the others), SMs with one item more than others costing up to
+// half of it; just above one round the second costs 0.4 of a round before its
+// items; below one, two blocks on an SM take 0.85 of the time of three.  A
+// block that has its SM to itself leaves it idle instead.
+// (2D foil of 0.33M particles: 256 items 25.0 us per push, 416 items 20.9, 480
+// items 26.9, 576 items 31.2.)
 __device__ __forceinline__ unsigned long long item_cost(const ItemPlan &pl, uint32_t slots, uint32_t items) {
   const uint32_t per = pl.blocks * pl.nsm, full = items / per, rem = items % per;
-  uint32_t unit = 2 * pl.blocks * full;
-  if (rem > 0) unit += max(pl.blocks + 1, 2 * (int)((rem + pl.nsm - 1) / pl.nsm));
+  const uint32_t most = (rem + pl.nsm - 1) / pl.nsm * pl.nsm;
+  uint32_t unit = items;
+  if (full == 0) unit = (per + most) / 2;
+  else if (rem > 0) unit += pl.blocks == 1 ? per - rem : 2 * per / (5 * full * full) + (most - rem) / 2;
   return (unsigned long long)unit * (slots / items + pl.fixed);
 }
 
@@ -189,17 +204,20 @@ __global__ void __launch_bounds__(kGroup)
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int best = 0;
+  if (warp == 0) {
+    int best = lane;
     unsigned long long least = ~0ull;
-    for (int j = 0; j < kItemCands && s_total[0] > 0; ++j) {
-      const unsigned long long c = item_cost(plan, s_total[0], s_total[1 + j]);
-      if (c < least) {
+    if (lane < kItemCands && s_total[0] > 0) least = item_cost(plan, s_total[0], s_total[1 + lane]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long c = __shfl_xor_sync(0xffffffffu, least, o);
+      const int j = __shfl_xor_sync(0xffffffffu, best, o);
+      if (c < least || (c == least && j < best)) {
         least = c;
         best = j;
       }
     }
-    s_pick = best;
+    if (lane == 0) s_pick = best;
   }
   __syncthreads();
   const int pick = s_pick;
@@ -318,7 +336,7 @@ cudaError_t launch_sort(const Grid &g, const Particles &src, const Particles &ds
   k_hist<<<nb, 256, 0, st>>>(km, src.cell, d_count, keys, rank);
   const unsigned wb = (unsigned)((g.ntiles * 32 + 255) / 256);
   k_tile_sum<<<wb, 256, 0, st>>>(keys, g.ntiles, km.tc, run);
-  k_tile_groups<<<groups, kGroup, 0, st>>>(run, g.ntiles, ws.plan, part, d_count, n_src);
+  k_tile_groups<<<dim3(groups, kVals / kPart), kGroup, 0, st>>>(run, g.ntiles, ws.plan, part, d_count, n_src);
   k_tile_starts<<<groups, kGroup, 0, st>>>(run, g.ntiles, groups, ws.plan, part, tile_start, d_count, ws, ws.adj);
   k_offsets<<<wb, 256, 0, st>>>(keys, g.ntiles, km.tc, tile_start, dst.cell);
   k_permute<<<nb, 256, 0, st>>>(km, src.cell, n_src, keys, rank, dst.cell, capacity, ctr);
