@@ -33,6 +33,7 @@ template <class R> struct YeeArgs {
 // B <- B - h curl E, curl E at the B locations.
 template <class R>
 __global__ void __launch_bounds__(256) k_yee_b(YeeArgs<R> a) {
+  after_previous();
   const int n0 = a.n[0], n1 = a.n[1], n2 = a.n[2];
   const int64_t ncell = (int64_t)n0 * n1 * n2;
   const int64_t sy = n0, sz = (int64_t)n0 * n1;
@@ -60,6 +61,7 @@ __global__ void __launch_bounds__(256) k_yee_b(YeeArgs<R> a) {
 // E <- E + h (curl B - J), curl B at the E locations.
 template <class R>
 __global__ void __launch_bounds__(256) k_yee_e(YeeArgs<R> a) {
+  after_previous();
   const int n0 = a.n[0], n1 = a.n[1], n2 = a.n[2];
   const int64_t ncell = (int64_t)n0 * n1 * n2;
   const int64_t sy = n0, sz = (int64_t)n0 * n1;
@@ -102,6 +104,7 @@ template <class R> __device__ __forceinline__ void stp(R *p, const Pack<R> &v) {
 
 template <class R>
 __global__ void __launch_bounds__(256) k_yee_b_vec(YeeArgs<R> a) {
+  after_previous();
   constexpr int W = 16 / sizeof(R);
   const int n0 = a.n[0], n1 = a.n[1], n2 = a.n[2];
   const int nq = n0 / W;
@@ -144,6 +147,7 @@ __global__ void __launch_bounds__(256) k_yee_b_vec(YeeArgs<R> a) {
 
 template <class R>
 __global__ void __launch_bounds__(256) k_yee_e_vec(YeeArgs<R> a) {
+  after_previous();
   constexpr int W = 16 / sizeof(R);
   const int n0 = a.n[0], n1 = a.n[1], n2 = a.n[2];
   const int nq = n0 / W;
@@ -208,6 +212,7 @@ template <class R> void yee_vec_shape(const Grid &g, dim3 &grid, dim3 &block) {
 
 template <class R>
 __global__ void k_mur_save(int n0, int n1, int n2, const R *Ey, const R *Ez, double *buf) {
+  after_previous();
   const int64_t nyz = (int64_t)n1 * n2;
   const int nodes[4] = {0, 1, n0 - 2, n0 - 1};
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < 8 * nyz; q += (int64_t)gridDim.x * blockDim.x) {
@@ -224,6 +229,7 @@ __global__ void k_mur_save(int n0, int n1, int n2, const R *Ey, const R *Ez, dou
 template <class R>
 __global__ void k_mur_apply(int n0, int n1, int n2, double dx, double dt, R *Ey, R *Ez, const double *buf,
                             LaserStep ls) {
+  after_previous();
   const int64_t nyz = (int64_t)n1 * n2;
   const double kc = (dt - dx) / (dt + dx);
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < 2 * nyz; q += (int64_t)gridDim.x * blockDim.x) {
@@ -304,6 +310,7 @@ template <class R> struct FieldStep2 {
 constexpr int kStripW = 29;
 
 template <class R> __global__ void __launch_bounds__(64) k_field_step2(const __grid_constant__ FieldStep2<R> a) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   if (blockIdx.x == 0)
     for (int k = threadIdx.x; k < a.ncounters; k += blockDim.x) a.counters[k] = 0;
@@ -721,7 +728,7 @@ __global__ void __launch_bounds__(256)
 // fields back to back.  The passes of the axes commute, so a launch per axis
 // does what a launch per pass, axis and field did (27 launches for J in 3D with
 // two passes and compensation, 126 us on 75 x 50 x 43 FP32; three launches and
-// 13 us now).  The taps come from the cache: every value is read once per tap.
+// 26 us now).  The taps come from the cache: every value is read once per tap.
 constexpr int kSmoothRadius = 9;  // eight binomial passes and a compensating one
 template <class R> struct SmoothArgs {
   const R *in;
@@ -730,6 +737,7 @@ template <class R> struct SmoothArgs {
   R w[kSmoothRadius + 1];
 };
 template <class R> __global__ void __launch_bounds__(256) k_smooth_axis(const __grid_constant__ SmoothArgs<R> a) {
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.n0) return;
   const int len = a.axis == 0 ? a.n0 : a.axis == 1 ? a.n1 : a.n2;
@@ -781,7 +789,7 @@ static cudaError_t smooth_t(const Grid &g, R *f, int ncomp, R *tmp, int passes, 
   for (a.axis = 0; a.axis < g.dims; ++a.axis) {
     a.in = f;
     a.out = tmp;
-    k_smooth_axis<R><<<grid, block, 0, st>>>(a);
+    launch_next(k_smooth_axis<R>, grid, block, 0, st, a);
     R *t = f;
     f = tmp;
     tmp = t;
@@ -807,10 +815,10 @@ template <class R> void yee_b_t(const Grid &g, void *const E[3], void *const B[3
   if (yee_vec_ok<R>(g, a, false)) {
     dim3 grid, block;
     yee_vec_shape<R>(g, grid, block);
-    k_yee_b_vec<R><<<grid, block, 0, st>>>(a);
+    launch_next(k_yee_b_vec<R>, grid, block, 0, st, a);
   } else {
     const int nb = grid_blocks(g.ncell, 256);
-    k_yee_b<R><<<nb, 256, 0, st>>>(a);
+    launch_next(k_yee_b<R>, nb, 256, 0, st, a);
   }
 }
 
@@ -820,10 +828,10 @@ void yee_e_t(const Grid &g, void *const E[3], void *const B[3], void *const J[3]
   if (yee_vec_ok<R>(g, a, true)) {
     dim3 grid, block;
     yee_vec_shape<R>(g, grid, block);
-    k_yee_e_vec<R><<<grid, block, 0, st>>>(a);
+    launch_next(k_yee_e_vec<R>, grid, block, 0, st, a);
   } else {
     const int nb = grid_blocks(g.ncell, 256);
-    k_yee_e<R><<<nb, 256, 0, st>>>(a);
+    launch_next(k_yee_e<R>, nb, 256, 0, st, a);
   }
 }
 
@@ -878,7 +886,7 @@ static cudaError_t field_step2_t(const Grid &g, void *const E[3], void *const B[
   a.counters = counters;
   a.ncounters = ncounters;
   a.strips = (unsigned)strips;
-  k_field_step2<R><<<(unsigned)(strips * ((a.n1 + 2 * a.rows - 1) / (2 * a.rows))), 64, 0, st>>>(a);
+  launch_next(k_field_step2<R>, (unsigned)(strips * ((a.n1 + 2 * a.rows - 1) / (2 * a.rows))), 64, 0, st, a);
   return cudaGetLastError();
 }
 
@@ -893,11 +901,11 @@ cudaError_t launch_field_step2(const Grid &g, void *const E[3], void *const B[3]
 cudaError_t launch_mur_save(const Grid &g, void *const E[3], double *buf, cudaStream_t st) {
   const int nb = grid_blocks(8LL * g.n[1] * g.n[2], 256);
   if (g.prec == 1)
-    k_mur_save<double><<<nb, 256, 0, st>>>(g.n[0], g.n[1], g.n[2], static_cast<const double *>(E[1]),
-                                           static_cast<const double *>(E[2]), buf);
+    launch_next(k_mur_save<double>, nb, 256, 0, st, g.n[0], g.n[1], g.n[2], static_cast<const double *>(E[1]),
+                static_cast<const double *>(E[2]), buf);
   else
-    k_mur_save<float><<<nb, 256, 0, st>>>(g.n[0], g.n[1], g.n[2], static_cast<const float *>(E[1]),
-                                          static_cast<const float *>(E[2]), buf);
+    launch_next(k_mur_save<float>, nb, 256, 0, st, g.n[0], g.n[1], g.n[2], static_cast<const float *>(E[1]),
+                static_cast<const float *>(E[2]), buf);
   return cudaGetLastError();
 }
 
@@ -941,11 +949,11 @@ cudaError_t launch_mur_apply(const Grid &g, void *const E[3], const double *buf,
                              cudaStream_t st) {
   const int nb = grid_blocks(2LL * g.n[1] * g.n[2], 256);
   if (g.prec == 1)
-    k_mur_apply<double><<<nb, 256, 0, st>>>(g.n[0], g.n[1], g.n[2], g.dx[0], g.dt, static_cast<double *>(E[1]),
-                                            static_cast<double *>(E[2]), buf, ls);
+    launch_next(k_mur_apply<double>, nb, 256, 0, st, g.n[0], g.n[1], g.n[2], g.dx[0], g.dt,
+                static_cast<double *>(E[1]), static_cast<double *>(E[2]), buf, ls);
   else
-    k_mur_apply<float><<<nb, 256, 0, st>>>(g.n[0], g.n[1], g.n[2], g.dx[0], g.dt, static_cast<float *>(E[1]),
-                                           static_cast<float *>(E[2]), buf, ls);
+    launch_next(k_mur_apply<float>, nb, 256, 0, st, g.n[0], g.n[1], g.n[2], g.dx[0], g.dt,
+                static_cast<float *>(E[1]), static_cast<float *>(E[2]), buf, ls);
   return cudaGetLastError();
 }
 

@@ -15,6 +15,40 @@ __device__ __forceinline__ int wrapi(int i, int n) {
   return i < 0 ? i + n : i;
 }
 
+// The kernels of a step follow each other on one stream, each reading what the
+// one before wrote.  launch_next launches a kernel so that its blocks may be
+// set up while the kernel before it drains, and after_previous, the first
+// thing every thread of such a kernel does, waits until that kernel has ended
+// and its writes are visible, then lets the kernel after it be set up (once
+// every block of this one has come so far).  After anything but a kernel it is
+// a plain launch.  It saves one to two microseconds per launch: 64^2 FP64
+// plasma 59 -> 52 us per step (three launches), 75 x 50 x 43 smoothed plasma
+// 212 -> 193, 2D foil with two species 147 -> 133.  Not in the reverse sweep,
+// which shares the SMs with the recomputation's stream: blocks set up early
+// there hold places that the other stream could use (256 x 256 gradient 35.5
+// ms without, 36.9 with).
+template <class... P, class... A>
+inline cudaError_t launch_next(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = attr;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
+// next_early: whether the kernel after this one may be set up before every
+// block of this one has ended.
+template <bool next_early = true> __device__ __forceinline__ void after_previous() {
+  cudaGridDependencySynchronize();
+  if (next_early) cudaTriggerProgrammaticLaunchCompletion();
+}
+
 // Division of n < 2^31 by a runtime constant d (Granlund-Montgomery):
 // q = umulhi(n, m) >> s with s = ceil(log2 d) - 1, m = ceil(2^(32 + s) / d)
 // (the excess e = m d - 2^(32 + s) < d <= 2^(s + 1), so e n < 2^(32 + s));

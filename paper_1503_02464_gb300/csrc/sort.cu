@@ -52,6 +52,7 @@ struct KeyMap {
 
 __global__ void k_hist(KeyMap km, const int32_t *__restrict__ cell, const int64_t *__restrict__ d_count,
                        int32_t *__restrict__ count, int32_t *__restrict__ rank) {
+  after_previous();
   const int64_t n = *d_count;
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -72,6 +73,7 @@ __global__ void k_hist(KeyMap km, const int32_t *__restrict__ cell, const int64_
 
 // one warp per tile
 __global__ void k_tile_sum(const int32_t *__restrict__ count, int64_t ntiles, int tc, uint32_t *__restrict__ run) {
+  after_previous();
   const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= ntiles) return;
@@ -105,6 +107,7 @@ static_assert(kVals <= 32 && kVals % kPart == 0, "one warp per value, one lane p
 __global__ void __launch_bounds__(kGroup)
     k_tile_groups(const uint32_t *__restrict__ run, int64_t ntiles, ItemPlan plan, uint32_t *__restrict__ part,
                   const int64_t *__restrict__ d_count, int64_t *__restrict__ n_src) {
+  after_previous();
   __shared__ uint32_t s[kPart];
   const int v0 = blockIdx.y * kPart;
   if (threadIdx.x < kPart) s[threadIdx.x] = 0;
@@ -186,6 +189,7 @@ __global__ void __launch_bounds__(kGroup)
     k_tile_starts(const uint32_t *__restrict__ run, int64_t ntiles, int ngroups, ItemPlan plan,
                   const uint32_t *__restrict__ part, int64_t *__restrict__ tile_start, int64_t *__restrict__ d_count,
                   WorkList push, WorkList adj) {
+  after_previous();
   __shared__ uint32_t s_before[kVals], s_total[kVals], s_scan[32][3];
   __shared__ int s_pick;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -249,6 +253,7 @@ __global__ void __launch_bounds__(kGroup)
 // tile's padding slots in the destination are marked dead
 __global__ void k_offsets(int32_t *__restrict__ count, int64_t ntiles, int tc, const int64_t *__restrict__ tile_start,
                           int32_t *__restrict__ dst_cell) {
+  after_previous();
   const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= ntiles) return;
@@ -271,6 +276,7 @@ __global__ void k_offsets(int32_t *__restrict__ count, int64_t ntiles, int tc, c
 __global__ void k_permute(KeyMap km, const int32_t *__restrict__ cell, const int64_t *__restrict__ n_src,
                           const int32_t *__restrict__ count, const int32_t *__restrict__ rank,
                           int32_t *__restrict__ dst_cell, int64_t capacity, Counters *ctr) {
+  after_previous();
   const int64_t n = *n_src;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
     const int r = rank[p];
@@ -284,6 +290,7 @@ __global__ void k_permute(KeyMap km, const int32_t *__restrict__ cell, const int
 template <class R>
 __global__ void k_gather(int dims, Particles src, Particles dst, const int64_t *__restrict__ n_dst,
                          const int64_t *__restrict__ n_src, Counters *ctr) {
+  after_previous();
   const int64_t n = *n_dst;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
     const int p = dst.cell[q];
@@ -333,17 +340,19 @@ cudaError_t launch_sort(const Grid &g, const Particles &src, const Particles &ds
   const int nsm = ws.plan.nsm;
   const int64_t want = (capacity + 255) / 256;
   const int nb = (int)(want < (int64_t)nsm * 16 ? (want > 0 ? want : 1) : (int64_t)nsm * 16);
-  k_hist<<<nb, 256, 0, st>>>(km, src.cell, d_count, keys, rank);
+  launch_next(k_hist, nb, 256, 0, st, km, src.cell, d_count, keys, rank);
   const unsigned wb = (unsigned)((g.ntiles * 32 + 255) / 256);
-  k_tile_sum<<<wb, 256, 0, st>>>(keys, g.ntiles, km.tc, run);
-  k_tile_groups<<<dim3(groups, kVals / kPart), kGroup, 0, st>>>(run, g.ntiles, ws.plan, part, d_count, n_src);
-  k_tile_starts<<<groups, kGroup, 0, st>>>(run, g.ntiles, groups, ws.plan, part, tile_start, d_count, ws, ws.adj);
-  k_offsets<<<wb, 256, 0, st>>>(keys, g.ntiles, km.tc, tile_start, dst.cell);
-  k_permute<<<nb, 256, 0, st>>>(km, src.cell, n_src, keys, rank, dst.cell, capacity, ctr);
+  launch_next(k_tile_sum, wb, 256, 0, st, keys, g.ntiles, km.tc, run);
+  launch_next(k_tile_groups, dim3(groups, kVals / kPart), kGroup, 0, st, run, g.ntiles, ws.plan, part, d_count,
+              n_src);
+  launch_next(k_tile_starts, groups, kGroup, 0, st, run, g.ntiles, groups, ws.plan, part, tile_start, d_count, ws,
+              ws.adj);
+  launch_next(k_offsets, wb, 256, 0, st, keys, g.ntiles, km.tc, tile_start, dst.cell);
+  launch_next(k_permute, nb, 256, 0, st, km, src.cell, n_src, keys, rank, dst.cell, capacity, ctr);
   if (g.prec == 1)
-    k_gather<double><<<nb, 256, 0, st>>>(g.dims, src, dst, d_count, n_src, ctr);
+    launch_next(k_gather<double>, nb, 256, 0, st, g.dims, src, dst, d_count, n_src, ctr);
   else
-    k_gather<float><<<nb, 256, 0, st>>>(g.dims, src, dst, d_count, n_src, ctr);
+    launch_next(k_gather<float>, nb, 256, 0, st, g.dims, src, dst, d_count, n_src, ctr);
   if (nlaunch) *nlaunch = 7;
   return cudaGetLastError();
 }
