@@ -61,6 +61,7 @@ template <class R> struct AdjFieldStep {
 };
 
 template <class R> __global__ void __launch_bounds__(64) k_adj_field_step(const __grid_constant__ AdjFieldStep<R> a) {
+  after_previous<false>();
   const int lane = threadIdx.x & 31;
   const int x0 = (int)(blockIdx.x % a.strips) * a.width;
   const int y0 = (int)((blockIdx.x / a.strips * (blockDim.x / 32) + (threadIdx.x >> 5)) * a.rows);
@@ -654,6 +655,7 @@ __device__ __forceinline__ void adj_particle(const AdjPushArgs<R> &a, const Node
 // for FP64) trades spills for occupancy.
 template <class R>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_adj_push2d(const AdjPushArgs<R> a) {
+  after_previous<false>();
   const int n0 = a.n[0], n1 = a.n[1];
   const int64_t n = *a.d_count;
   const R *F[6] = {a.E[0], a.E[1], a.E[2], a.B[0], a.B[1], a.B[2]};
@@ -693,6 +695,7 @@ template <class R>
 // two blocks at 128 registers 115 us.  FP32: two blocks per SM 7 % slower.)
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1)
     k_adj_push2d_win(const AdjPushArgs<R> a, const AdjWork w) {
+  after_previous<false>();
   extern __shared__ __align__(16) unsigned char adj_smem[];
   R *s = reinterpret_cast<R *>(adj_smem);
   __shared__ int s_esc[kAdjItem];
@@ -840,7 +843,7 @@ static cudaError_t adj_field_t(const Grid &g, void *const lE[3], void *const lB[
   a.kc = (g.dt - g.dx[0]) / (g.dt + g.dx[0]);
   a.ls = ls_unit;
   a.da0 = da0;
-  k_adj_field_step<R><<<(unsigned)(strips * ((a.n1 + 2 * a.rows - 1) / (2 * a.rows))), 64, 0, st>>>(a);
+  launch_next(k_adj_field_step<R>, (unsigned)(strips * ((a.n1 + 2 * a.rows - 1) / (2 * a.rows))), 64, 0, st, a);
   return cudaGetLastError();
 }
 
@@ -885,7 +888,7 @@ static cudaError_t adj_push_t(const Grid &g, const Particles &tp, const int64_t 
   a.q = (R)q;
   const bool win = tt && tt->items.nwork > 0 && g.tile[0] <= kAdjTile && g.tile[1] <= kAdjTile;
   if (!win) {
-    k_adj_push2d<R><<<nblocks(nmax), 256, 0, st>>>(a);
+    launch_next(k_adj_push2d<R>, nblocks(nmax), 256, 0, st, a);
     if (nlaunch) *nlaunch = 1;
     return cudaGetLastError();
   }
@@ -904,7 +907,7 @@ static cudaError_t adj_push_t(const Grid &g, const Particles &tp, const int64_t 
   w.t1 = g.tile[1];
   w.esc_total = tt->esc_total;
   if (tt->items.nwork > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_adj_push2d_win<R><<<(unsigned)tt->items.nwork, 256, smem, st>>>(a, w);
+  launch_next(k_adj_push2d_win<R>, (unsigned)tt->items.nwork, 256, smem, st, a, w);
   if (nlaunch) *nlaunch = 1;
   return cudaGetLastError();
 }

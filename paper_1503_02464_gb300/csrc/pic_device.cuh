@@ -23,10 +23,10 @@ __device__ __forceinline__ int wrapi(int i, int n) {
 // every block of this one has come so far).  After anything but a kernel it is
 // a plain launch.  It saves one to two microseconds per launch: 64^2 FP64
 // plasma 59 -> 52 us per step (three launches), 75 x 50 x 43 smoothed plasma
-// 212 -> 193, 2D foil with two species 147 -> 133.  Not in the reverse sweep,
-// which shares the SMs with the recomputation's stream: blocks set up early
-// there hold places that the other stream could use (256 x 256 gradient 35.5
-// ms without, 36.9 with).
+// 212 -> 193, 2D foil with two species 147 -> 133.  The kernels of the reverse
+// sweep do not let their successors be set up early: they share the SMs with
+// the recomputation's stream, and such blocks hold places that it could use
+// (256 x 256 gradient 36.9 ms; without it 35.2, and 35.5 with plain launches).
 template <class... P, class... A>
 inline cudaError_t launch_next(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchAttribute attr[1];
