@@ -1291,8 +1291,8 @@ int pic_step(pic_handle *h, int nsteps) {
       for (int d = 0; d < 3; ++d) std::swap(h->J[d], h->J2[d]);
     } else {
       Timed tm(h, pic::KC_ZEROJ);
-      CK(h, cudaMemsetAsync(h->J[0], 0, 3 * fb, h->st), "zero J");
-      CK(h, cudaMemsetAsync(h->esc_count, 0, kEscBytes, h->st), "zero counters");
+      CK(h, pic::launch_clear(h->J[0], 3 * fb, h->esc_count, kMaxSpecies * pic::kEscCounters, h->st), "zero J");
+      h->launches++;
     }
     for (int i = 0; i < h->nsp; ++i) {
       Species &s = h->sp[i];

@@ -118,3 +118,18 @@ def test_reversed_field_step_is_the_transpose(n, walls):
             s.adjoint_step(1)
             got = sum(float((p * s.adjoint_field(k)).sum()) for k, p in enumerate(x))
             assert abs(got - ax[c][0, 0, col]) <= 1e-13 * 30, (c, col)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [(9, 7, 5), (10, 7, 5), (11, 7, 5), (8, 8, 8), (75, 50, 43)])
+def test_current_cleared_before_a_3d_step(n, precision):
+    """J starts every step at zero up to its last value, whatever its bytes
+    leave of the 16-byte stores (exact: nothing deposits)."""
+    wl = synth.small(3, n, 2, 1, 0.1, 11)
+    s = Simulation.from_workload(wl, precision=precision)
+    for step in range(2):
+        for c in (6, 7, 8):
+            s.set_field(c, 1.0 + step)
+        s.step(1)
+        for c in range(9):
+            assert not s.field(c).any(), (n, c)
