@@ -636,15 +636,16 @@ __device__ __forceinline__ void push_move(const PushArgs<R> &a, R u[3], const R 
 // general stencil, the settled ones a group at a time, summed in registers;
 // the J window is added to global J while the next item's particles arrive.
 //
-// What bounds it: shared-memory wavefronts (69 % of the time at 128^3) and
-// instruction issue (61 %), not HBM.  Depositing each particle by itself cost
+// What bounds it: shared-memory wavefronts (70 % of the time at 128^3) and
+// instruction issue (64 %), not HBM.  Depositing each particle by itself cost
 // 54 contributions of seven instructions, two of them shared reductions of 3.2
 // wavefronts; a group sum costs one FMA per contribution and the seven
 // instructions once per group.  The gather's 162 shared loads per particle are
 // the largest part left.  3D TSC FP32 thermal plasma at 8 per cell, 16.8M
 // particles (ncu): 1.655 ms depositing particle by particle, 1.110 by groups,
-// 1.030 with asynchronous staging, blocks that stay, and tasks of six; 1884,
-// 1626 and 1520 instructions per 32 particles.  Two particles per thread in
+// 1.030 with asynchronous staging, blocks that stay, and tasks of six, 1.010
+// with the sort's item sizes; 1884, 1626, 1520 and 1520 instructions per 32
+// particles.  Two particles per thread in
 // packed FP32 (FFMA2) needed 16 % fewer instructions and the same time.
 template <class R, int DIM, int ORDER, bool EC>
 __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(const PushArgs<R> a) {
