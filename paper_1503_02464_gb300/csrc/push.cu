@@ -1627,6 +1627,11 @@ ItemPlan push_item_plan(const Grid &g) {
     // against these: 64^2 FP64 CIC push 39.5 -> 37.3 us, 75 x 50 x 43 FP32 CIC
     // 105 -> 93 us, 2D foil of 0.33M particles 27.8 -> 20.9 us)
     pl.cand[j] = (int)(cap * std::exp2(-j / 8.0)) / kTilePad * kTilePad;
+    // 2D FP32: a tile of up to 512 slots stays whole.  The windows of its and
+    // its neighbours' items are added to J in any order, and with one item per
+    // tile most nodes receive two values at most, whose sum has no order: small
+    // differentiable runs repeat themselves.
+    if (g.dims == 2 && g.prec == 0 && pl.cand[j] < 512) pl.cand[j] = 512;
   }
   int dev = 0;
   pl.nsm = 1;
