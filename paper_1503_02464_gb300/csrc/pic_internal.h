@@ -183,6 +183,8 @@ cudaError_t launch_sort(const Grid &g, const Particles &src, const Particles &ds
 
 // ---- fields and particle conversion (fields.cu) ----
 // The updates of a 3D step.
+// Copies two blocks (16-byte aligned, multiples of 4 bytes).
+cudaError_t launch_copy(void *const dst[2], const void *const src[2], const size_t bytes[2], cudaStream_t st);
 // Clears `bytes` (a multiple of 4) at mem (16-byte aligned) and the counters.
 cudaError_t launch_clear(void *mem, size_t bytes, unsigned long long *counters, int ncounters, cudaStream_t st);
 cudaError_t launch_yee_b(const Grid &g, void *const E[3], void *const B[3], double h, cudaStream_t st);
