@@ -102,7 +102,7 @@ template <class R> struct PushArgs {
   R *off[3];
   R *u[3];
   const R *w;
-  float qabs;                       // |q|
+  float reach;                      // FP32: the largest of the factors dt / dx_a and (2D3V) 1, see WinAcc
   const int32_t *work_tile;         // work item -> tile
   const int64_t *work_pb;           // work item -> first slot
   const int32_t *work_n;            // work item -> slots
@@ -115,6 +115,7 @@ template <class R> struct PushArgs {
   R qmh;      // q dt / (2 m)
   R dtdx[3];  // dt / dx_a
   R jfac[3];  // -q dx_a / dt  (Esirkepov running-sum scale, times w)
+  float jhi[3], jlo[3];  // FP32: the factor of the window's J_a, and what its rounding left out
   R qz;       // q            (2D3V: Jz = q w vz S)
   int absorb;  // absorbing x walls: remove particles leaving [kWallLo, n0 - kWallHiMargin)
   Counters *ctr;
@@ -163,19 +164,28 @@ __device__ __forceinline__ R gsum(const R *__restrict__ F, const R *wx, const R 
 // Shared-memory J window.  FP32 runs accumulate in fixed point: FP32 shared
 // atomics are compare-and-swap loops costing several shared-memory
 // wavefronts each, integer shared atomics are single native operations, and
-// integer sums are exact and independent of order.  A contribution v becomes
-// the integer X = rint(v * 2^K), K chosen per work item from a bound on |J|
-// at any node: each Esirkepov contribution of a particle satisfies
-// |v| <= |q w| |v_p|, so |J_node| <= Q = sum over the item's particles of
-// |q w| min(1, |u|) with u the momentum after the push; 2^K keeps Q 2^K below
-// 2^kLimitLog2.  X is kept as two signed 32-bit words, X = hi * 2^16 + lo
-// with |lo| <= 2^15, both found with FP32 FMAs and adds only (adding
-// 1.5 * 2^(23 + s) rounds a float of magnitude below 2^(22 + s) to a multiple
-// of 2^s held in the low mantissa bits), because float-to-64-bit conversions
-// run on the slow FP64 pipe.  With |X| < 2^37 the hi sums cannot overflow, and
-// the lo sums cannot overflow for fewer than 65,536 contributions per node (an
-// item holds at most Lay::CAP particles).  FP64 runs use plain double shared
-// atomics, keeping FP64 rounding.
+// integer sums are exact and independent of order.  The window holds J without
+// its factor -q dx_a / dt (2D3V Jz: q), which the flush multiplies in, to more
+// than FP32's precision (rounded to FP32 and multiplied into every particle's
+// weight it left up to an ulp in J).  A contribution v becomes
+// the integer X = rint(v * 2^K), K chosen per work item: each Esirkepov
+// contribution of a particle is at most |w| |v_a| dt / dx_a (2D3V Jz:
+// |w| |v_z|), so at most its q = |w| min(1, |vx| + |vy| + |vz|), with the
+// velocity after the push, times the largest of those factors.  2^K keeps what
+// is added at a time, up to Lay::TASK particles of one node, below
+// 2^kLimitLog2: at most Q = min(TASK max q, sum of q) over the item's jobs.
+// (From the sum of q alone the quantum was up to 2^8 coarser and as large an
+// error of J as all other roundings: rms 1.3e-7 instead of 7.8e-8 with 8 per
+// cell, and 2.3e-6 instead of 9e-8 in the transverse components of beams of 27
+// per cell.)  X is kept as two signed 32-bit words, X = hi * 2^16 + lo with
+// |lo| <= 2^15, both found with FP32 FMAs and adds only (adding 1.5 * 2^(23 + s)
+// rounds a float of magnitude below 2^(22 + s) to a multiple of 2^s held in the
+// low mantissa bits), because float-to-64-bit conversions run on the slow FP64
+// pipe.  With |X| < 2^37 per addition (the split holds to 2^38: a stored move of
+// less than an ulp of its offset may be twice v dt) an item's hi sums stay below
+// 2^30, and the lo sums cannot overflow for fewer than 65,536 contributions per
+// node (an item holds at most Lay::CAP particles).  FP64 runs use plain double
+// shared atomics, keeping FP64 rounding.
 template <class R> struct WinAcc;
 template <> struct WinAcc<float> {
   int *w;       // [3][2][jn]: per component lo words, then hi words
@@ -218,9 +228,11 @@ template <> struct WinAcc<float> {
     scale = __int_as_float((127 + K) << 23);
     unit = __int_as_float((127 - K) << 23);
   }
-  __device__ __forceinline__ float get(int comp, int idx) const {
+  // The node's J: the sum times the component's factor jhi + jlo.
+  __device__ __forceinline__ float get(int comp, int idx, float jhi, float jlo) const {
     const int *b = w + comp * 2 * jn + idx;
-    return fmaf((float)b[jn], 65536.0f * unit, (float)b[0] * unit);
+    const float hi = (float)b[jn];
+    return fmaf(hi, 65536.0f * unit * jhi, fmaf(hi, 65536.0f * unit * jlo, (float)b[0] * (unit * jhi)));
   }
 };
 template <> struct WinAcc<double> {
@@ -233,7 +245,7 @@ template <> struct WinAcc<double> {
     const double x = p * q;
     if (x != 0.0) atomicAdd(w + comp * jn + idx, x);
   }
-  __device__ __forceinline__ double get(int comp, int idx) const { return w[comp * jn + idx]; }
+  __device__ __forceinline__ double get(int comp, int idx, float, float) const { return w[comp * jn + idx]; }
 };
 
 // Esirkepov deposit into the shared J window (compile-time strides).
@@ -385,15 +397,39 @@ template <class R, int ORDER> struct SettledAxis {
   }
 };
 
-// A running sum of contributions p q in registers.  FloatSum: one FMA.
-// FixedSum: the two fixed-point words of WinAcc<float>::add, so that the sum is
-// exact and does not depend on the order of the particles: what a 2D FP32 run
-// does (the runs with an adjoint, whose segments are run twice and have to
-// repeat themselves); its stencil has 21 sums where 3D TSC has 54.
-template <class R> struct FloatSum {
-  R v;
-  __device__ __forceinline__ void clear() { v = R(0); }
-  __device__ __forceinline__ void add(R p, R q) { v += p * q; }
+// A running sum of contributions p q in registers.
+// DoubleSum: one FMA (FP64 runs).
+// PairSum: FP32 in 3D.  hi starts at WinAcc<float>::kMagicHi, so that every FMA
+// rounds its sum to a multiple of 2^16 (|sum| < 2^38, see WinAcc); how far it
+// moved is exact, and a second FMA gives what the contribution was short of
+// that, at most 2^15, which lo sums.  lo keeps 2^-6 of a unit, and is rounded to
+// a whole one when the window takes the sum: finer than the window, which rounds
+// every contribution by itself.  Two registers, and four instructions for two
+// sums in packed FP32.  (3D TSC takes its 54 sums in two passes over the tasks,
+// Jx and Jy and then Jz, to stay within 128 registers.)  One FP32 value (one
+// FMA) loses what cancels within a group, and J had 5 to 13 % more error (rms
+// against the 64-bit current of the same moves, 48 x 40 x 32 cells with 1 to 32
+// particles each).  256^3 plasma of 8 per cell, 20 steps: 200.5 ms with one FP32
+// value, 209.1 with the pair, 214.5 with its four instructions unpacked.
+// FixedSum: FP32 in 2D.  The two fixed-point words of WinAcc<float>::add, so that
+// the sum of a given scale does not depend on the order of the particles at all;
+// its stencil has 21 sums where 3D TSC has 54.
+struct DoubleSum {
+  double v;
+  __device__ __forceinline__ void clear() { v = 0.0; }
+  __device__ __forceinline__ void add(double p, double q) { v += p * q; }
+};
+struct PairSum {
+  float hi, lo;
+  __device__ __forceinline__ void clear() {
+    hi = WinAcc<float>::kMagicHi;
+    lo = 0.f;
+  }
+  __device__ __forceinline__ void add(float p, float q) {
+    const float y = fmaf(p, q, hi);
+    lo += fmaf(p, q, hi - y);
+    hi = y;
+  }
 };
 struct FixedSum {
   int hi, lo;
@@ -406,26 +442,54 @@ struct FixedSum {
   }
 };
 
+// M sums with a common factor q.
+template <int M, class S, class R> __device__ __forceinline__ void add_each(S *s, const R *p, R q) {
+#pragma unroll
+  for (int k = 0; k < M; ++k) s[k].add(p[k], q);
+}
+// Two PairSums in packed FP32: the same four operations on both at once.
+template <> __device__ __forceinline__ void add_each<2, PairSum, float>(PairSum *s, const float *p, float q) {
+  asm("{\n\t"
+      ".reg .b64 p, q, h, l, y, d;\n\t"
+      "mov.b64 p, {%4, %5};\n\t"
+      "mov.b64 q, {%6, %6};\n\t"
+      "mov.b64 h, {%0, %1};\n\t"
+      "mov.b64 l, {%2, %3};\n\t"
+      "fma.rn.f32x2 y, p, q, h;\n\t"
+      "sub.rn.f32x2 d, h, y;\n\t"
+      "fma.rn.f32x2 d, p, q, d;\n\t"
+      "add.rn.f32x2 l, l, d;\n\t"
+      "mov.b64 {%0, %1}, y;\n\t"
+      "mov.b64 {%2, %3}, l;\n\t"
+      "}"
+      : "+f"(s[0].hi), "+f"(s[1].hi), "+f"(s[0].lo), "+f"(s[1].lo)
+      : "f"(p[0]), "f"(p[1]), "f"(q));
+}
+
 // The settled contributions of the particles of one node, summed in
 // registers: add() one particle, flush() the sums into the J window once per
 // group.  Same brackets as deposit_win: Jx gets
 // Px (S0y S0z + DSy S0z/2 + S0y DSz/2 + DSy DSz/3), cyclic; in 2D3V
 // Jz = q w vz (S0x S0y + DSx S0y/2 + S0x DSy/2 + DSx DSy/3).  The running
 // sums of DS along an axis end at -DS[last] (the whole sum vanishes).
-template <class R, int DIM, int ORDER> struct GroupSum {
+// COMPS: the components summed (bit c: J_c); the others' sums take no registers.
+template <class R, int DIM, int ORDER, int COMPS> struct GroupSum {
   static constexpr int NS = ORDER + 1, M = ORDER;
   static constexpr int NA = DIM == 3 ? M * NS * NS : M * NS;  // Jx, Jy sums
   static constexpr int NZ = DIM == 3 ? M * NS * NS : NS * NS;  // Jz sums
-  using S = typename std::conditional<sizeof(R) == 4 && DIM == 2, FixedSum, FloatSum<R>>::type;
+  static constexpr bool kX = COMPS & 1, kY = COMPS & 2, kZ = COMPS & 4;
+  using S = typename std::conditional<sizeof(R) == 8, DoubleSum,
+                                      typename std::conditional<DIM == 2, FixedSum, PairSum>::type>::type;
   S jx[NA], jy[NA], jz[NZ];
   __device__ __forceinline__ void clear() {
 #pragma unroll
     for (int i = 0; i < NA; ++i) {
-      jx[i].clear();
-      jy[i].clear();
+      if (kX) jx[i].clear();
+      if (kY) jy[i].clear();
     }
 #pragma unroll
-    for (int i = 0; i < NZ; ++i) jz[i].clear();
+    for (int i = 0; i < NZ; ++i)
+      if (kZ) jz[i].clear();
   }
   __device__ __forceinline__ void add(const SettledAxis<R, ORDER> &X, const SettledAxis<R, ORDER> &Y,
                                       const SettledAxis<R, ORDER> &Z, R cx, R cy, R cz, R qwvz) {
@@ -457,30 +521,27 @@ template <class R, int DIM, int ORDER> struct GroupSum {
         tx[k] = R(0.5) * X.S0[k] + X.DS[k] * R(1.0 / 3.0);
       }
 #pragma unroll
-      for (int c = 0; c < NS; ++c)
+      for (int c = 0; c < (kX ? NS : 0); ++c)
 #pragma unroll
         for (int b = 0; b < NS; ++b) {
           const R br = Y.S0[b] * hz[c] + Y.DS[b] * tz[c];
-#pragma unroll
-          for (int a = 0; a < M; ++a) jx[(c * NS + b) * M + a].add(Px[a], br);
+          add_each<M>(jx + (c * NS + b) * M, Px, br);
         }
 #pragma unroll
-      for (int c = 0; c < NS; ++c)
+      for (int c = 0; c < (kY ? NS : 0); ++c)
 #pragma unroll
         for (int a = 0; a < NS; ++a) {
           const R br = Z.S0[c] * hx[a] + Z.DS[c] * tx[a];
-#pragma unroll
-          for (int b = 0; b < M; ++b) jy[(c * NS + a) * M + b].add(Py[b], br);
+          add_each<M>(jy + (c * NS + a) * M, Py, br);
         }
 #pragma unroll
-      for (int b = 0; b < NS; ++b) {
+      for (int b = 0; b < (kZ ? NS : 0); ++b) {
         const R hy = Y.S0[b] + R(0.5) * Y.DS[b];
         const R ty = R(0.5) * Y.S0[b] + Y.DS[b] * R(1.0 / 3.0);
 #pragma unroll
         for (int a = 0; a < NS; ++a) {
           const R br = X.S0[a] * hy + X.DS[a] * ty;
-#pragma unroll
-          for (int c = 0; c < M; ++c) jz[(b * NS + a) * M + c].add(Pz[c], br);
+          add_each<M>(jz + (b * NS + a) * M, Pz, br);
         }
       }
     } else {
@@ -506,19 +567,19 @@ template <class R, int DIM, int ORDER> struct GroupSum {
   template <int SY, int SZ, class Sink> __device__ __forceinline__ void flush(const Sink &out) const {
     if constexpr (DIM == 3) {
 #pragma unroll
-      for (int c = 0; c < NS; ++c)
+      for (int c = 0; c < (kX ? NS : 0); ++c)
 #pragma unroll
         for (int b = 0; b < NS; ++b)
 #pragma unroll
           for (int a = 0; a < M; ++a) out.add(0, c * SZ + b * SY + a, jx[(c * NS + b) * M + a]);
 #pragma unroll
-      for (int c = 0; c < NS; ++c)
+      for (int c = 0; c < (kY ? NS : 0); ++c)
 #pragma unroll
         for (int a = 0; a < NS; ++a)
 #pragma unroll
           for (int b = 0; b < M; ++b) out.add(1, c * SZ + b * SY + a, jy[(c * NS + a) * M + b]);
 #pragma unroll
-      for (int b = 0; b < NS; ++b)
+      for (int b = 0; b < (kZ ? NS : 0); ++b)
 #pragma unroll
         for (int a = 0; a < NS; ++a)
 #pragma unroll
@@ -546,11 +607,8 @@ template <class R, int JS> struct GroupSink;
 template <int JS> struct GroupSink<float, JS> {
   unsigned sb;  // byte address of the Jx low word of the stencil's first node
   __device__ __forceinline__ void add(int comp, int off, FixedSum s) const { put(comp, off, s.hi, s.lo); }
-  __device__ __forceinline__ void add(int comp, int off, FloatSum<float> s) const {
-    const float v = s.v, y = v + WinAcc<float>::kMagicHi;
-    const float lf = v - (y - WinAcc<float>::kMagicHi);
-    const int hi = __float_as_int(y) - __float_as_int(WinAcc<float>::kMagicHi);
-    put(comp, off, hi, __float2int_rn(lf));
+  __device__ __forceinline__ void add(int comp, int off, PairSum s) const {
+    put(comp, off, __float_as_int(s.hi) - __float_as_int(WinAcc<float>::kMagicHi), __float2int_rn(s.lo));
   }
   __device__ __forceinline__ void put(int comp, int off, int hi, int lo) const {
     const unsigned sa = sb + 8u * (unsigned)JS * (unsigned)comp + 4u * (unsigned)off;
@@ -560,10 +618,47 @@ template <int JS> struct GroupSink<float, JS> {
 };
 template <int JS> struct GroupSink<double, JS> {
   double *w;  // Jx value of the stencil's first node (components JS doubles apart)
-  __device__ __forceinline__ void add(int comp, int off, FloatSum<double> s) const {
+  __device__ __forceinline__ void add(int comp, int off, DoubleSum s) const {
     if (s.v != 0.0) atomicAdd(w + comp * JS + off, s.v);
   }
 };
+
+// A deposit task: up to TASK settled particles of one group, from position
+// tk % 4096 of the job order, their sums added to the window.  scale: of Jx, Jy,
+// Jz, and (2D3V) of q vz w.
+template <class R, int DIM, int ORDER, int COMPS>
+__device__ __forceinline__ void deposit_task(const WinAcc<R> &acc, const R *sJob, const uint16_t *sOrder,
+                                             const uint32_t *sTag, unsigned tk, const R (&scale)[4]) {
+  using G = Geo<DIM, ORDER>;
+  using L = Lay<R, DIM, ORDER>;
+  constexpr int CAP = L::CAP, SY = G::EX, SZ = G::EX * G::EY;
+  int j = tk & 4095u;
+  const int je = j + (int)(tk >> 12) + 1;
+  int s = sOrder[j];
+  const uint32_t group = sTag[s] & 1023u;
+  const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
+  // the stencil's first node: one below the nearest node (TSC), the cell's (CIC)
+  constexpr int o = ORDER == 2 ? 0 : 1;
+  const int jb = (kx + o) + (ky + o) * SY + (DIM == 3 ? (kz + o) * SZ : 0);
+  GroupSum<R, DIM, ORDER, COMPS> g;
+  g.clear();
+  while (true) {
+    SettledAxis<R, ORDER> X, Y, Z;
+    X.set(sJob[s], sJob[DIM * CAP + s]);
+    Y.set(sJob[CAP + s], sJob[(DIM + 1) * CAP + s]);
+    const R w = sJob[(L::NJ - 1) * CAP + s];
+    R qwvz = R(0);
+    if (DIM == 3) Z.set(sJob[2 * CAP + s], sJob[5 * CAP + s]);
+    else qwvz = scale[3] * w * sJob[4 * CAP + s];
+    if (++j < je) s = sOrder[j];
+    g.add(X, Y, Z, scale[0] * w, scale[1] * w, scale[2] * w, qwvz);
+    if (j >= je) break;
+  }
+  GroupSink<R, sizeof(R) == 4 ? G::JS : G::EN> out;
+  if constexpr (sizeof(R) == 4) out.sb = (unsigned)__cvta_generic_to_shared(acc.w) + 4u * (unsigned)jb;
+  else out.w = acc.w + jb;
+  g.template flush<SY, SZ>(out);
+}
 
 // A particle's tag, left by the push for the deposit: its group (10 bits),
 // for a particle whose support changes the move of its nearest node (CIC: of
@@ -636,16 +731,17 @@ __device__ __forceinline__ void push_move(const PushArgs<R> &a, R u[3], const R 
 // general stencil, the settled ones a group at a time, summed in registers;
 // the J window is added to global J while the next item's particles arrive.
 //
-// What bounds it: shared-memory wavefronts (70 % of the time at 128^3) and
-// instruction issue (64 %), not HBM.  Depositing each particle by itself cost
+// What bounds it: shared-memory wavefronts (72 % of the time at 128^3) and
+// instruction issue (66 %), not HBM.  Depositing each particle by itself cost
 // 54 contributions of seven instructions, two of them shared reductions of 3.2
-// wavefronts; a group sum costs one FMA per contribution and the seven
-// instructions once per group.  The gather's 162 shared loads per particle are
+// wavefronts; a group sum costs two packed instructions per contribution and the
+// reductions once per group.  The gather's 162 shared loads per particle are
 // the largest part left.  3D TSC FP32 thermal plasma at 8 per cell, 16.8M
 // particles (ncu): 1.655 ms depositing particle by particle, 1.110 by groups,
 // 1.030 with asynchronous staging, blocks that stay, and tasks of six, 1.010
-// with the sort's item sizes; 1884, 1626, 1520 and 1520 instructions per 32
-// particles.  Two particles per thread in
+// with the sort's item sizes, 1.069 with the sums kept exact (the group sums
+// before were one FP32 value); 1884, 1626, 1520, 1520 and 1666 instructions per
+// 32 particles.  Two particles per thread in
 // packed FP32 (FFMA2) needed 16 % fewer instructions and the same time.
 template <class R, int DIM, int ORDER, bool EC>
 __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(const PushArgs<R> a) {
@@ -665,7 +761,8 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
   uint16_t *sStart = reinterpret_cast<uint16_t *>(smem_raw + L::kCount);  // over the counts, once read
   uint16_t *sTask = reinterpret_cast<uint16_t *>(smem_raw + L::kTask);
   __shared__ unsigned int s_clamp, s_absorbed, s_next;
-  __shared__ float s_q;
+  __shared__ float s_q;          // sum and (as bits) maximum of q, see WinAcc
+  __shared__ unsigned int s_qmax;
   __shared__ unsigned int s_wsum[kThreads / 32];
   __shared__ unsigned long long s_wcls[kThreads / 32];
   __shared__ int64_t s_pb;  // the block's next item: first slot, slots, tile
@@ -743,6 +840,7 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
     if (tid == 0) {
       s_clamp = s_absorbed = s_next = 0;
       s_q = 0.f;
+      s_qmax = 0;
     }
     unsigned long long taken = 0;
     if (tid == 0) taken = atomicAdd(a.next_item, 1ull);  // (its result is first needed after the push)
@@ -753,7 +851,7 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
     // The slots are cell-sorted, so a warp's lanes sit in a few neighbouring
     // cells and mostly read the same field nodes (shared-memory broadcasts).
     unsigned my_clamp = 0, my_absorbed = 0;
-    float my_q = 0.f;  // bound on this thread's part of |J| at any node: sum |w| |v|
+    float my_q = 0.f, my_qmax = 0.f;
     for (int s = tid; s < n; s += kThreads) {
       const int c = (int)sTag[s];
       uint32_t tag = kTagIdle;
@@ -902,15 +1000,22 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
         }
         tag |= atomicAdd(&sCount[sort_key], 1u) << 16;
         // |v| <= min(1, |vx| + |vy| + |vz|)
-        if (sizeof(R) == 4)
-          my_q += fabsf((float)w) *
-                  fminf(1.f, (fabsf((float)u[0]) + fabsf((float)u[1]) + fabsf((float)u[2])) * (float)ig);
+        if (sizeof(R) == 4) {
+          const float q = fabsf((float)w) *
+                          fminf(1.f, (fabsf((float)u[0]) + fabsf((float)u[1]) + fabsf((float)u[2])) * (float)ig);
+          my_q += q;
+          my_qmax = fmaxf(my_qmax, q);
+        }
       } while (0);
       sTag[s] = tag;
     }
     if (sizeof(R) == 4) {
       for (int o = 16; o > 0; o >>= 1) my_q += __shfl_xor_sync(0xffffffffu, my_q, o);
-      if (lane == 0 && my_q > 0.f) atomicAdd(&s_q, my_q);
+      const unsigned qmax = __reduce_max_sync(0xffffffffu, __float_as_uint(my_qmax));
+      if (lane == 0 && my_q > 0.f) {
+        atomicAdd(&s_q, my_q);
+        atomicMax(&s_qmax, qmax);
+      }
     }
     if (my_clamp) atomicAdd(&s_clamp, my_clamp);
     if (my_absorbed) atomicAdd(&s_absorbed, my_absorbed);
@@ -1042,17 +1147,21 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
     acc.jn = sizeof(R) == 4 ? G::JS : G::EN;
     acc.dummy = G::EN + lane;
     acc.scale = acc.unit = R(1);
-    if constexpr (sizeof(R) == 4) acc.set_scale(1.01f * a.qabs * s_q);  // 1.01: room for the FP32 rounding of the sum
+    if constexpr (sizeof(R) == 4)  // 1.01: room for the FP32 rounding of the sum
+      acc.set_scale(1.01f * a.reach * fminf(L::TASK * __uint_as_float(s_qmax), s_q));
     __syncthreads();
 
     // ---- deposit: warps take the next 32 particles whose support changes (the
     // longest work, in order of the axes that do), then the next 32 tasks,
-    // longest first
+    // longest first (kParts = 2: all of them for Jx and Jy, then again for Jz)
+    constexpr int kParts = DIM == 3 && ORDER == 2 && L::F32 ? 2 : 1;
     const int nset = sStart[G::KN], nchg = (int)njob - nset, nchg32 = (nchg + 31) & ~31;
-    const int nunit = nchg32 + ntask;
+    const int ntask32 = (ntask + 31) & ~31;
+    const int nunit = nchg32 + (kParts == 2 ? ntask32 : 0) + ntask;
     if (tid == 0 && nchg > 0) atomicAdd(a.q_jobs, (unsigned long long)nchg);
-    const R jf0 = a.jfac[0] * acc.scale, jf1 = a.jfac[1] * acc.scale, jf2 = a.jfac[2] * acc.scale;
-    const R jz = a.qz * acc.scale;  // 2D3V
+    // (FP32: the factors come in with the flush, and the scale is a power of two)
+    const R jf0 = L::F32 ? acc.scale : a.jfac[0], jf1 = L::F32 ? acc.scale : a.jfac[1];
+    const R jf2 = L::F32 ? acc.scale : a.jfac[2], jz = L::F32 ? acc.scale : a.qz;  // jz: 2D3V
     for (;;) {
       unsigned base = 0;
       if (lane == 0) base = atomicAdd(&s_next, 32u);
@@ -1060,34 +1169,13 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
       if ((int)base >= nunit) break;
       const int unit = (int)base + lane;
       if ((int)base >= nchg32) {
-        if (unit >= nunit) continue;
-        const unsigned tk = sTask[unit - nchg32];
-        int j = tk & 4095u;
-        const int je = j + (int)(tk >> 12) + 1;
-        int s = sOrder[j];
-        const uint32_t group = sTag[s] & 1023u;
-        const int kx = group % G::KX, ky = group / G::KX % G::KY, kz = DIM == 3 ? group / (G::KX * G::KY) : 0;
-        // the stencil's first node: one below the nearest node (TSC), the cell's (CIC)
-        constexpr int o = ORDER == 2 ? 0 : 1;
-        const int jb = (kx + o) + (ky + o) * SY + (DIM == 3 ? (kz + o) * SZ : 0);
-        GroupSum<R, DIM, ORDER> g;
-        g.clear();
-        while (true) {
-          SettledAxis<R, ORDER> X, Y, Z;
-          X.set(sJob[s], sJob[DIM * CAP + s]);
-          Y.set(sJob[CAP + s], sJob[(DIM + 1) * CAP + s]);
-          const R w = sJob[(L::NJ - 1) * CAP + s];
-          R qwvz = R(0);
-          if (DIM == 3) Z.set(sJob[2 * CAP + s], sJob[5 * CAP + s]);
-          else qwvz = jz * w * sJob[4 * CAP + s];
-          if (++j < je) s = sOrder[j];
-          g.add(X, Y, Z, jf0 * w, jf1 * w, jf2 * w, qwvz);
-          if (j >= je) break;
-        }
-        GroupSink<R, sizeof(R) == 4 ? G::JS : G::EN> out;
-        if constexpr (sizeof(R) == 4) out.sb = (unsigned)__cvta_generic_to_shared(acc.w) + 4u * (unsigned)jb;
-        else out.w = acc.w + jb;
-        g.template flush<SY, SZ>(out);
+        const bool second = kParts == 2 && (int)base >= nchg32 + ntask32;
+        const int i = unit - nchg32 - (second ? ntask32 : 0);
+        if (i >= ntask) continue;
+        const R c[4] = {jf0, jf1, jf2, jz};
+        if (kParts == 1) deposit_task<R, DIM, ORDER, 7>(acc, sJob, sOrder, sTag, sTask[i], c);
+        else if (second) deposit_task<R, DIM, ORDER, 4>(acc, sJob, sOrder, sTag, sTask[i], c);
+        else deposit_task<R, DIM, ORDER, 3>(acc, sJob, sOrder, sTag, sTask[i], c);
       } else {
         // (lanes past the last one add nothing, so that the whole warp votes below)
         bool have = unit < nchg;
@@ -1165,7 +1253,7 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const int wx = wx0 + e;
-            v[e] = (wx >= 0 && wx < G::EX) ? (float)acc.get(c, wrow + wx) : 0.f;
+            v[e] = (wx >= 0 && wx < G::EX) ? (float)acc.get(c, wrow + wx, a.jhi[c], a.jlo[c]) : 0.f;
           }
           if (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f)
             asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a.J[c] + g), "f"(v[0]), "f"(v[1]),
@@ -1184,7 +1272,7 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
         const int g = gi + a.n[0] * (gj + a.n[1] * gk);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const R v = acc.get(c, q);
+          const R v = acc.get(c, q, a.jhi[c], a.jlo[c]);
           if (v != R(0)) atomicAdd(a.J[c] + g, v);
         }
       }
@@ -1332,7 +1420,7 @@ cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *co
   a.nwork = ws.count;
   a.slots = ws.slots;
   a.next_item = esc_count + 2;
-  a.qabs = (float)(q < 0 ? -q : q);
+  a.reach = DIM == 2 ? 1.f : 0.f;
   for (int d = 0; d < 3; ++d) {
     a.n[d] = g.n[d];
     a.E[d] = static_cast<const R *>(E[d]);
@@ -1341,7 +1429,11 @@ cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *co
     a.off[d] = static_cast<R *>(p.off[d]);
     a.u[d] = static_cast<R *>(p.u[d]);
     a.dtdx[d] = (R)(g.dt / g.dx[d]);
-    a.jfac[d] = (R)(-q * g.dx[d] / g.dt);
+    const double jfac = -q * g.dx[d] / g.dt, jwin = DIM == 2 && d == 2 ? q : jfac;
+    a.jfac[d] = (R)jfac;
+    a.jhi[d] = (float)jwin;
+    a.jlo[d] = (float)(jwin - (double)a.jhi[d]);
+    if (d < DIM) a.reach = std::fmax(a.reach, (float)(g.dt / g.dx[d]) * 1.000001f);
   }
   a.ntile[0] = g.ntile[0];
   a.ntile[1] = g.ntile[1];
