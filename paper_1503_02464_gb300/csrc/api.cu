@@ -26,8 +26,6 @@ namespace {
 
 constexpr int kMaxSpecies = 8;
 constexpr size_t kEscBytes = kMaxSpecies * pic::kEscCounters * sizeof(unsigned long long);
-// Species up to this size have their escape count read back less often (a push of 2M takes about 0.1 ms).
-constexpr int64_t kSmallSpecies = int64_t(1) << 21;
 
 struct Species {
   double q = 0, m = 1;
@@ -1312,14 +1310,11 @@ int pic_step(pic_handle *h, int nsteps) {
          "push");
       h->launches += nl;
       if (s.crowded) h->crowded_pushes++;
-      // A copy and an event cost 3 us, which small species feel: a slow one's
-      // count comes back every fourth step.  A large one, whose push takes far
-      // longer, asks at every step: its escapes cost more than the copy
-      // (beams of 28M particles, first steps: escape kernel 0.9 -> 4.5 ms when
-      // the early sort came up to three steps later).
-      const bool ask = s.fast || s.h_count > kSmallSpecies || s.esc_step < 0 || s.esc_step > h->step ||
-                       h->step - s.esc_step >= 4;
-      if (!s.esc_pending && ask) {
+      // Every push's count comes back, unless one is on its way still: the next
+      // step sorts early by it.  (The copy and the event take 3 us of a small
+      // species' step; asked for every fourth step, a beam whose particles leave
+      // their tiles together was sorted up to three steps late.)
+      if (!s.esc_pending) {
         CK(h, cudaMemcpyAsync(s.esc_host, h->esc_count + i * pic::kEscCounters, 2 * sizeof(unsigned long long),
                               cudaMemcpyDeviceToHost, h->st),
            "escape count");
