@@ -262,11 +262,6 @@ template <class R> struct AdjPushArgs {
   R qmh, dtdx[3], cxu[3], q;
 };
 
-// The move's 1/gamma exactly as the forward push computes it.
-template <class R> __device__ __forceinline__ R inv_sqrt_fwd(R x);
-template <> __device__ __forceinline__ float inv_sqrt_fwd<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double inv_sqrt_fwd<double>(double x) { return 1.0 / sqrt(x); }
-
 // The forward Boris step (the push's arithmetic) with its intermediates:
 // u- = u0 + h E, t = h B / gamma-, s = 2 t / (1 + t^2), u' = u- + u- x t,
 // u+ = u- + u' x s, uo = u+ + h E.  rg = 1 / gamma- and sf = 2 / (1 + t^2) are
@@ -394,7 +389,7 @@ __device__ __forceinline__ void adj_particle(const AdjPushArgs<R> &a, const Node
       boris_fwd<R>(h, u0, F, rg, sf, um, t, sv, up, uo);
     }
     // move
-    const R ig = inv_sqrt_fwd<R>(R(1) + uo[0] * uo[0] + uo[1] * uo[1] + uo[2] * uo[2]);
+    const R ig = inv_gamma<R>(uo);
     R fn[2];
     int sh[2];
 #pragma unroll

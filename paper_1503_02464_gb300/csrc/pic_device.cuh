@@ -249,6 +249,17 @@ template <class R, int ORDER> struct DepositAxis {
   }
 };
 
+// The move's 1 / gamma, of the push and of the adjoint kernels' recomputation
+// of it: one function, so that the same momentum gives both the same move (a
+// particle on a cell face or between two nodes has to take the same side).
+// FP64: rsqrt, off by at most 1.01 2^-53 of itself on 4M values in [1, 10^6],
+// where the IEEE root and quotient were by 1.50.
+__device__ __forceinline__ float rsqrt_move(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_move(double x) { return rsqrt(x); }
+template <class R> __device__ __forceinline__ R inv_gamma(const R u[3]) {
+  return rsqrt_move(R(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+}
+
 // 1/sqrt(x) and 1/x for x >= 1 (infinite or NaN pass).  FP32: the hardware's
 // approximation and one Newton-Raphson step, y + y/2 (1 - x y^2) and
 // y + y (1 - x y), its residual in one FMA: within an ulp, like the IEEE root

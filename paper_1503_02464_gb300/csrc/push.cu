@@ -129,10 +129,6 @@ template <class R> __device__ __forceinline__ bool outside_walls(int absorb, int
   return X < (R)kWallLo || X >= (R)(n0 - kWallHiMargin);
 }
 
-template <class R> __device__ __forceinline__ R inv_sqrt(R x);
-template <> __device__ __forceinline__ float inv_sqrt<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double inv_sqrt<double>(double x) { return rsqrt(x); }
-
 // One value copied from global to shared memory asynchronously.
 template <class R> __device__ __forceinline__ void copy_async(R *to, const R *from) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from),
@@ -713,7 +709,7 @@ template <class R, int ORDER, int DIM>
 __device__ __forceinline__ void push_move(const PushArgs<R> &a, R u[3], const R E[3], const R B[3], const R f[3],
                                           R fn[3], int s[3], R &ig, unsigned &clamp) {
   boris<R, DIM == 2>(a.qmh, E, B, u);
-  ig = inv_sqrt<R>(R(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+  ig = inv_gamma<R>(u);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     fn[d] = R(0);
