@@ -166,7 +166,10 @@ typedef struct {
   int64_t n_push_mid_drain; /* species pushes made while the species' last count
                              read back averaged more than 168 particles per
                              work item changing their shape support (e.g. fast
-                             beams)                                            */
+                             beams).  Work items as counted here: the capacity
+                             in 16 pieces per SM, of at least 512 slots, and
+                             one per cell tile.  A statistic only: no kernel
+                             is chosen by it                                   */
   int64_t n_adj_escaped;  /* particle adjoints since pic_adjoint_begin computed
                              on the global-memory path: the particle had moved
                              more than 2 cells out of the tile it was sorted
@@ -190,7 +193,9 @@ typedef struct pic_handle pic_handle;
 /* Create a simulation.  Validates sizes, shape order, precision, boundary
  * kinds and the Courant condition of the Yee scheme (§2 states dx_i >= c dt;
  * the limit enforced is the sharper (sum dx_i^-2)^(-1/2)).  Allocates and
- * zeroes E, B, J.  Returns PIC_EINVAL / PIC_ECOURANT / PIC_ENOMEM / PIC_ECUDA.
+ * zeroes E, B, J; 2D runs hold a second set of the nine (a step's field update
+ * writes one from the other), and 3D runs with current smoothing a second J.
+ * Returns PIC_EINVAL / PIC_ECOURANT / PIC_ENOMEM / PIC_ECUDA.
  * On failure *out is NULL.  Checkpoints, tape entries and load staging are
  * stream-ordered allocations from the device's default memory pool; the
  * first pic_create of the process lets that pool keep up to a quarter of
@@ -248,7 +253,9 @@ int pic_set_background(pic_handle *h, const double *rho_bg, int mem_kind);
 /* Advance nsteps PIC cycles (enqueued on the stream; asynchronous).
  * Per step: sort (every sort_every steps) -> J = 0 -> per species one fused
  * gather/Boris/move/deposit launch -> Yee B half step -> E step -> B half
- * step (-> wall and laser boundary kernels when enabled). */
+ * step (-> wall and laser boundary kernels when enabled).  In 2D one launch
+ * makes the field updates, walls and wave included, and clears the next
+ * step's J. */
 int pic_step(pic_handle *h, int nsteps);
 
 /* Copy one field (PIC_EX .. PIC_RHO) as FP64 into out (n[0]*n[1]*n[2]
@@ -288,7 +295,8 @@ int pic_sync(pic_handle *h);
  * entries (either may be NULL); class order: 0 sort, 1 zero J, 2 push,
  * 3 Yee B, 4 Yee E, 5 boundary, 6 current smoothing, 7 adjoint field
  * updates, 8 adjoint particle kernel, 9 checkpoint, restore and tape copies
- * (device-to-device).  The number of classes written goes
+ * (device-to-device).  In 2D a step's one field launch counts as class 4;
+ * classes 1, 3 and 5 stay at zero.  The number of classes written goes
  * to *ncls (NULL allowed).  PIC_EINVAL for a NULL handle. */
 int pic_profile(pic_handle *h, int enable);
 int pic_timings(pic_handle *h, double *ms, int64_t *launches, int nmax, int *ncls);

@@ -686,8 +686,9 @@ struct AdjWork {
 // cells outside its tile since the sort is set aside and done at the end of
 // the block with all its nodes in global memory.
 template <class R>
-// (FP64: one block per SM and no spills, 106 us per launch of the 120 x 64 run;
-// two blocks at 128 registers 115 us.  FP32: two blocks per SM 7 % slower.)
+// (FP64: one block per SM at 255 registers, 352 B of spill stores, 106 us per
+// launch of the 120 x 64 run; two blocks at 128 registers 115 us.  FP32: 80
+// registers, 444 B of spill stores; two blocks per SM 7 % slower.)
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1)
     k_adj_push2d_win(const AdjPushArgs<R> a, const AdjWork w) {
   after_previous<false>();

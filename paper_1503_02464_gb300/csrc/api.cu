@@ -614,7 +614,7 @@ int pic_create(const pic_config *cfg, pic_handle **out) {
   }
   const size_t fb = (size_t)ncell * h->rsize;
   // E, B in one block (a checkpoint copies them with one memcpy) and the
-  // three J components in another (one memset clears J)
+  // three J components in another (k_clear or, in 2D, the field update clears it)
   bool ok = cudaMalloc(&h->E[0], 6 * fb) == cudaSuccess && cudaMalloc(&h->J[0], 3 * fb) == cudaSuccess;
   if (g.dims == 2) ok = ok && cudaMalloc(&h->E2[0], 6 * fb) == cudaSuccess;
   if (g.dims == 2 || c.filter_passes > 0) ok = ok && cudaMalloc(&h->J2[0], 3 * fb) == cudaSuccess;

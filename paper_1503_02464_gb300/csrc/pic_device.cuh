@@ -23,7 +23,8 @@ __device__ __forceinline__ int wrapi(int i, int n) {
 // every block of this one has come so far).  After anything but a kernel it is
 // a plain launch.  It saves one to two microseconds per launch: 64^2 FP64
 // plasma 59 -> 52 us per step (three launches), 75 x 50 x 43 smoothed plasma
-// 212 -> 193, 2D foil with two species 147 -> 133.  The kernels of the reverse
+// 212 -> 193, 2D foil with two species 147 -> 133 (steps as long as the host
+// lets them be: 135 to 152 on other boxes).  The kernels of the reverse
 // sweep do not let their successors be set up early: they share the SMs with
 // the recomputation's stream, and such blocks hold places that it could use
 // (256 x 256 gradient 36.9 ms; without it 35.2, and 35.5 with plain launches).
@@ -262,9 +263,11 @@ template <class R> __device__ __forceinline__ R inv_gamma(const R u[3]) {
 
 // 1/sqrt(x) and 1/x for x >= 1 (infinite or NaN pass).  FP32: the hardware's
 // approximation and one Newton-Raphson step, y + y/2 (1 - x y^2) and
-// y + y (1 - x y), its residual in one FMA: within an ulp, like the IEEE root
-// and quotient it replaces, in a few instructions.  FP64: rsqrt (1 ulp, as
-// the root and quotient together) and the IEEE quotient.
+// y + y (1 - x y), its residual in one FMA, in a few instructions.  Against 64
+// bits on 4M values each in [1, 2], [1, 100] and [1, 10^6], in 2^-24 of the
+// value: the root is off by at most 1.24 (rms 0.47), the IEEE root and quotient
+// by 1.50 (0.60); the reciprocal equals the IEEE quotient on all of them.  FP64:
+// rsqrt (see inv_gamma) and the IEEE quotient.
 __device__ __forceinline__ float rsqrt_near(float x) {
   const float y = rsqrtf(x);
   const float e = x > 3.4e38f ? 0.f : fmaf(-x * y, y, 1.f);

@@ -154,7 +154,7 @@ struct WorkSplit : WorkList {
 };
 constexpr int kAdjItem = 512;
 
-// Tile kernel (one block per work item) + escape kernel.
+// Tile kernel (blocks that stay and draw work items in turn) + escape kernel.
 // esc_list (one int per slot) is scratch for particles deferred to the
 // escape kernel; esc_count (kEscCounters counters, zero at the launch) receives
 // their number and the number of particles whose shape support changed, and
@@ -182,11 +182,11 @@ cudaError_t launch_sort(const Grid &g, const Particles &src, const Particles &ds
                         const WorkSplit &ws, Counters *ctr, cudaStream_t st, int *nlaunch);
 
 // ---- fields and particle conversion (fields.cu) ----
-// The updates of a 3D step.
 // Copies two blocks (16-byte aligned, multiples of 4 bytes).
 cudaError_t launch_copy(void *const dst[2], const void *const src[2], const size_t bytes[2], cudaStream_t st);
 // Clears `bytes` (a multiple of 4) at mem (16-byte aligned) and the counters.
 cudaError_t launch_clear(void *mem, size_t bytes, unsigned long long *counters, int ncounters, cudaStream_t st);
+// The updates of a 3D step.
 cudaError_t launch_yee_b(const Grid &g, void *const E[3], void *const B[3], double h, cudaStream_t st);
 cudaError_t launch_yee_e(const Grid &g, void *const E[3], void *const B[3], void *const J[3], double h,
                          cudaStream_t st);

@@ -5,11 +5,11 @@
 //
 // Cell tiles are 8x8x4 in 3D, 16x16 in 2D.  The sort keeps each tile's
 // particles in one contiguous, 4-aligned slot range and cuts that range into
-// work items of bounded size; one thread block takes one work item.  The
-// block stages E and B of the tile plus guard cells in shared memory, pushes
-// all its particles, and then deposits them by groups that share a nearest
-// node (see k_push) into a J window in shared memory (fixed point in FP32
-// runs), which it adds to the global J.
+// work items of bounded size, which the resident thread blocks take in turn.
+// For an item a block stages E and B of the tile plus guard cells in shared
+// memory, pushes all its particles, and then deposits them by groups that
+// share a nearest node (see k_push) into a J window in shared memory (fixed
+// point in FP32 runs), which it adds to the global J.
 //
 // A particle that has drifted more than D = 1 cell outside its tile since the
 // last sort is not handled here: its slot is appended to an escape list and
@@ -1715,10 +1715,13 @@ ItemPlan push_item_plan(const Grid &g) {
     // against these: 64^2 FP64 CIC push 39.5 -> 37.3 us, 75 x 50 x 43 FP32 CIC
     // 105 -> 93 us, 2D foil of 0.33M particles 27.8 -> 20.9 us)
     pl.cand[j] = (int)(cap * std::exp2(-j / 8.0)) / kTilePad * kTilePad;
-    // 2D FP32: a tile of up to 512 slots stays whole.  The windows of its and
-    // its neighbours' items are added to J in any order, and with one item per
-    // tile most nodes receive two values at most, whose sum has no order: small
-    // differentiable runs repeat themselves.
+    // 2D FP32: a tile of up to 512 slots stays whole.  An item's window does not
+    // depend on the order of its particles, but the windows of its and its
+    // neighbours' items are added to J in any order: with one item per tile most
+    // nodes receive two values at most, whose sum has no order, so that small
+    // differentiable runs mostly repeat themselves to the last bit.  Nodes near a
+    // tile's corner receive up to four, escaped particles add theirs by
+    // themselves, and larger tiles may be cut: there nothing promises it.
     if (g.dims == 2 && g.prec == 0 && pl.cand[j] < 512) pl.cand[j] = 512;
   }
   int dev = 0;

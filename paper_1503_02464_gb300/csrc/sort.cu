@@ -143,7 +143,11 @@ __global__ void __launch_bounds__(kGroup)
 // items; below one, two blocks on an SM take 0.85 of the time of three.  A
 // block that has its SM to itself leaves it idle instead.
 // (2D foil of 0.33M particles: 256 items 25.0 us per push, 416 items 20.9, 480
-// items 26.9, 576 items 31.2.)
+// items 26.9, 576 items 31.2.)  3D and FP64 runs are ranked by the same form: on
+// nine of ten of them, 3D FP32 and FP64 and 2D FP64, CIC and TSC, every second
+// size forced in turn, the choice was within 1 % of the fastest (FP64 40^3 of 8
+// per cell 819 us, 838 to 1544 with the others; 64^3 FP32 180 and 229 to 611), and
+// 5 % slower on one (48 x 40 x 32 TSC FP32 of 27 per cell, 156 us and 149).
 __device__ __forceinline__ unsigned long long item_cost(const ItemPlan &pl, uint32_t slots, uint32_t items) {
   const uint32_t per = pl.blocks * pl.nsm, full = items / per, rem = items % per;
   const uint32_t most = (rem + pl.nsm - 1) / pl.nsm * pl.nsm;
