@@ -115,6 +115,7 @@ template <class R> struct PushArgs {
   R qmh;      // q dt / (2 m)
   R dtdx[3];  // dt / dx_a
   R jfac[3];  // -q dx_a / dt  (Esirkepov running-sum scale, times w)
+  float pre[3];          // FP32: powers of two that even out the components of the window, see WinAcc
   float jhi[3], jlo[3];  // FP32: the factor of the window's J_a, and what its rounding left out
   R qz;       // q            (2D3V: Jz = q w vz S)
   int absorb;  // absorbing x walls: remove particles leaving [kWallLo, n0 - kWallHiMargin)
@@ -167,7 +168,9 @@ __device__ __forceinline__ R gsum(const R *__restrict__ F, const R *wx, const R 
 // the integer X = rint(v * 2^K), K chosen per work item: each Esirkepov
 // contribution of a particle is at most |w| |v_a| dt / dx_a (2D3V Jz:
 // |w| |v_z|), so at most its q = |w| min(1, |vx| + |vy| + |vz|), with the
-// velocity after the push, times the largest of those factors.  2^K keeps what
+// velocity after the push, times the largest of those factors.  (A component of
+// a smaller factor is held times a power of two that makes up for it, so that
+// flat cells or a small dt cost no bits.)  2^K keeps what
 // is added at a time, up to Lay::TASK particles of one node, below
 // 2^kLimitLog2: at most Q = min(TASK max q, sum of q) over the item's jobs.
 // (From the sum of q alone the quantum was up to 2^8 coarser and as large an
@@ -1155,9 +1158,9 @@ __global__ void __launch_bounds__(kThreads, Lay<R, DIM, ORDER>::BLOCKS) k_push(c
     const int ntask32 = (ntask + 31) & ~31;
     const int nunit = nchg32 + (kParts == 2 ? ntask32 : 0) + ntask;
     if (tid == 0 && nchg > 0) atomicAdd(a.q_jobs, (unsigned long long)nchg);
-    // (FP32: the factors come in with the flush, and the scale is a power of two)
-    const R jf0 = L::F32 ? acc.scale : a.jfac[0], jf1 = L::F32 ? acc.scale : a.jfac[1];
-    const R jf2 = L::F32 ? acc.scale : a.jfac[2], jz = L::F32 ? acc.scale : a.qz;  // jz: 2D3V
+    // (FP32: the factors come in with the flush, and the scales are powers of two)
+    const R jf0 = L::F32 ? acc.scale * a.pre[0] : a.jfac[0], jf1 = L::F32 ? acc.scale * a.pre[1] : a.jfac[1];
+    const R jf2 = L::F32 ? acc.scale * a.pre[2] : a.jfac[2], jz = L::F32 ? jf2 : a.qz;  // jz: 2D3V
     for (;;) {
       unsigned base = 0;
       if (lane == 0) base = atomicAdd(&s_next, 32u);
@@ -1425,11 +1428,17 @@ cudaError_t launch_t(const Grid &g, void *const E[3], void *const B[3], void *co
     a.off[d] = static_cast<R *>(p.off[d]);
     a.u[d] = static_cast<R *>(p.u[d]);
     a.dtdx[d] = (R)(g.dt / g.dx[d]);
-    const double jfac = -q * g.dx[d] / g.dt, jwin = DIM == 2 && d == 2 ? q : jfac;
-    a.jfac[d] = (R)jfac;
+    a.jfac[d] = (R)(-q * g.dx[d] / g.dt);
+    if (d < DIM) a.reach = std::fmax(a.reach, (float)(g.dt / g.dx[d]) * 1.000001f);
+  }
+  for (int d = 0; d < 3; ++d) {
+    const bool z2 = DIM == 2 && d == 2;
+    // the power of two next below what J_d's factor dt / dx_d lacks to the largest (at least 1)
+    const double lacks = a.reach / (z2 ? 1.0 : g.dt / g.dx[d]);
+    a.pre[d] = (float)std::exp2(std::floor(std::log2(std::fmin(lacks, 16777216.0))));
+    const double jwin = (z2 ? q : -q * g.dx[d] / g.dt) / a.pre[d];
     a.jhi[d] = (float)jwin;
     a.jlo[d] = (float)(jwin - (double)a.jhi[d]);
-    if (d < DIM) a.reach = std::fmax(a.reach, (float)(g.dt / g.dx[d]) * 1.000001f);
   }
   a.ntile[0] = g.ntile[0];
   a.ntile[1] = g.ntile[1];
