@@ -166,7 +166,8 @@ typedef struct {
   int64_t n_push_mid_drain; /* species pushes made while the species' last count
                              read back averaged more than 168 particles per
                              work item changing their shape support (e.g. fast
-                             beams).  Work items as counted here: the capacity
+                             beams; those without weight, which deposit nothing,
+                             aside).  Work items as counted here: the capacity
                              in 16 pieces per SM, of at least 512 slots, and
                              one per cell tile.  A statistic only: no kernel
                              is chosen by it                                   */
