@@ -118,7 +118,9 @@ typedef struct {
                           of its particles down the escape path               */
   int tile[3];         /* cell-tile shape of the push kernel (0 = default)     */
   int drift_guard;     /* cells a particle may stray from its tile between sorts
-                          and still use the tile's shared-memory window (0 = 1) */
+                          and still use the tile's shared-memory window, its
+                          cell (CIC) or nearest node (TSC) after the move
+                          included (0 = 1)                                     */
   pic_laser laser;
   void *stream;        /* cudaStream_t                                         */
   /* Current smoothing after the deposit, before the E update (a standard

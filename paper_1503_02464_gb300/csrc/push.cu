@@ -12,8 +12,9 @@
 // point in FP32 runs), which it adds to the global J.
 //
 // A particle that has drifted more than D = 1 cell outside its tile since the
-// last sort is not handled here: its slot is appended to an escape list and
-// k_push_escaped applies the same arithmetic on global memory afterwards.
+// last sort, or whose cell (CIC) or nearest node (TSC) does in this move, is not
+// handled here: its slot is appended to an escape list and k_push_escaped
+// applies the same arithmetic on global memory afterwards.
 #include <cuda_runtime.h>
 
 #include <cmath>
